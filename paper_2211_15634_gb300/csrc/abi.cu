@@ -808,9 +808,9 @@ static int check_2d(const void *T2, const void *T, const void *Ci, double lam, d
 static int mode_2d(int dtype, unsigned flags, StepCoef c) {
     if (dtype == PS_F32) return Z_F32;
     if (flags & PS_RUN_CI_SCALED) return Z_F64_SCALED;
-    const double K = c.dtlam * c.ax;
-    if (c.ax == c.ay && K > 2.2250738585072014e-308 && K < 1e300) return Z_F64_EMU_ISO_DMUL;
-    return Z_F64_NATIVE;
+    for (const double K : {c.dtlam * c.ax, c.dtlam * c.ay})
+        if (!(K > 2.2250738585072014e-308 && K < 1e300)) return Z_F64_NATIVE;
+    return c.ax == c.ay ? Z_F64_EMU_ISO_DMUL : Z_F64_EMU_ANISO;
 }
 
 int ps_diffusion2d_step(void *T2, const void *T, const void *Ci, double lam, double dt, double _dx,

@@ -43,6 +43,10 @@ struct M2D<Z_F64_EMU_ISO_DMUL> {
     using E = double;
 };
 template <>
+struct M2D<Z_F64_EMU_ANISO> {
+    using E = double;
+};
+template <>
 struct M2D<Z_F64_NATIVE> {
     using E = double;
 };
@@ -54,8 +58,11 @@ __device__ __forceinline__ E node2d(E c, E xm, E xp, E ym, E yp, E ci, const P2D
     } else if constexpr (MODE == Z_F64_SCALED) {
         return f64s_node(c, xm, xp, ym, yp, c, c, ci);
     } else if constexpr (MODE == Z_F64_EMU_ISO_DMUL) {
-        return emu_step_node<true, true>(dbits(c), dbits(xm), dbits(xp), dbits(ym), dbits(yp), dbits(c),
-                                         dbits(c), ci, p.ek);
+        return emu_step_node<AX_ISO, true>(dbits(c), dbits(xm), dbits(xp), dbits(ym), dbits(yp), dbits(c),
+                                           dbits(c), ci, p.ek);
+    } else if constexpr (MODE == Z_F64_EMU_ANISO) {
+        return emu_step_node<AX_COMMON, false, 2>(dbits(c), dbits(xm), dbits(xp), dbits(ym), dbits(yp), dbits(c),
+                                                  dbits(c), ci, p.ek);
     } else {
         const double d2x = (xp - c) - (c - xm), d2y = (yp - c) - (c - ym);
         return c + p.ek.dtlam * (ci * (d2x * p.ek.ax + d2y * p.ek.ay));
@@ -153,7 +160,7 @@ k_ymarch2d(typename M2D<MODE>::E *__restrict__ T2, const typename M2D<MODE>::E *
         if (lane == 31) right = hr;
         E out[PX];
         bool warp_fast = false;
-        if constexpr (MODE == Z_F64_SCALED || MODE == Z_F64_EMU_ISO_DMUL) {
+        if constexpr (MODE == Z_F64_SCALED || MODE == Z_F64_EMU_ISO_DMUL || MODE == Z_F64_EMU_ANISO) {
             // one same-binade check over this lane's distinct values (words of nodes that
             // are not written replaced by the reference, so they cannot force the general
             // path); the whole warp takes the short path together when all lanes pass
@@ -189,8 +196,15 @@ k_ymarch2d(typename M2D<MODE>::E *__restrict__ T2, const typename M2D<MODE>::E *
                 }
             } else if constexpr (MODE == Z_F64_EMU_ISO_DMUL) {
                 if (warp_fast) {
-                    out[i] = emu_fast_node<true, true>(dbits(c[i]), dbits(xm), dbits(xp), dbits(up[i]),
-                                                       dbits(dn[i]), dbits(c[i]), dbits(c[i]), ci[i], p.ek);
+                    out[i] = emu_fast_node<AX_ISO, true>(dbits(c[i]), dbits(xm), dbits(xp), dbits(up[i]),
+                                                         dbits(dn[i]), dbits(c[i]), dbits(c[i]), ci[i], p.ek);
+                    continue;
+                }
+            } else if constexpr (MODE == Z_F64_EMU_ANISO) {
+                if (warp_fast) {
+                    out[i] = emu_fast_node<AX_COMMON, false, 2>(dbits(c[i]), dbits(xm), dbits(xp), dbits(up[i]),
+                                                                dbits(dn[i]), dbits(c[i]), dbits(c[i]), ci[i],
+                                                                p.ek);
                     continue;
                 }
             }
@@ -279,15 +293,16 @@ static cudaError_t launch_2d_t(void *T2, const void *T, const void *Ci, P2D p, i
 }
 
 // mode: Z_F32, Z_F64_SCALED (Ci holds dt*lam*_dx^2*Ci, equal spacings), Z_F64_EMU_ISO_DMUL
-// (equal spacings, positive coefficient) or Z_F64_NATIVE (anything else in FP64)
+// (equal spacings, positive coefficient), Z_F64_EMU_ANISO (unequal ones within a factor of
+// 16) or Z_F64_NATIVE (anything else in FP64)
 cudaError_t launch_step2d(int mode, void *T2, const void *T, const void *Ci, StepCoef c, int64_t nx,
                           int64_t ny, cudaStream_t s) {
     P2D p{};
     p.fdtlam = (float)c.dtlam;
     p.fax = (float)c.ax;
     p.fay = (float)c.ay;
-    p.ek = EmuCoef{emu_const(c.dtlam * c.ax), emu_const(c.dtlam * c.ay), emu_const(c.dtlam * c.ax),
-                   c.dtlam, c.ax, c.ay, 0.0, c.dtlam * c.ax};
+    p.ek = emu_coef(c.dtlam, c.ax, c.ay, c.ax);  // the z term is not used
+    p.ek.az = 0.0;                               // (and vanishes in the general path's plain form)
     const int esz = mode == Z_F32 ? 4 : 8;
     const bool vec = ((nx * esz) % 16 == 0) && ((((uintptr_t)T2 | (uintptr_t)T | (uintptr_t)Ci) & 15u) == 0);
     switch (mode) {
@@ -304,10 +319,17 @@ cudaError_t launch_step2d(int mode, void *T2, const void *T, const void *Ci, Ste
         case Z_F64_EMU_ISO_DMUL:
             return vec ? launch_2d_t<Z_F64_EMU_ISO_DMUL, 4, 2>(T2, T, Ci, p, nx, ny, s)
                        : launch_2d_t<Z_F64_EMU_ISO_DMUL, 1>(T2, T, Ci, p, nx, ny, s);
+        // spacings within a factor of 16 of each other; beyond that plain FP64, whose products
+        // lose nothing at any ratio
+        case Z_F64_EMU_ANISO:
+            if (!p.ek.common) break;
+            return vec ? launch_2d_t<Z_F64_EMU_ANISO, 4, 2>(T2, T, Ci, p, nx, ny, s)
+                       : launch_2d_t<Z_F64_EMU_ANISO, 1>(T2, T, Ci, p, nx, ny, s);
         default:
-            return vec ? launch_2d_t<Z_F64_NATIVE, 4, 2>(T2, T, Ci, p, nx, ny, s)
-                       : launch_2d_t<Z_F64_NATIVE, 1>(T2, T, Ci, p, nx, ny, s);
+            break;
     }
+    return vec ? launch_2d_t<Z_F64_NATIVE, 4, 2>(T2, T, Ci, p, nx, ny, s)
+               : launch_2d_t<Z_F64_NATIVE, 1>(T2, T, Ci, p, nx, ny, s);
 }
 
 cudaError_t launch_copy_edges2d(void *T2, const void *T, int64_t nx, int64_t ny, int esz, cudaStream_t s) {

@@ -11,7 +11,8 @@
 // where S is the sum of the six neighbours minus six times the centre (or one
 // such sum per axis), formed EXACTLY in 64-bit integer arithmetic, K =
 // dt*lam*_d^2 is a host constant, and the product K*S is formed with a 64x64
-// bit high multiply and packed into an FP64 bit pattern with integer ops.
+// bit high multiply and packed into an FP64 bit pattern with integer ops
+// (unequal spacings: the axes' products summed as integers first, emu_L_common).
 // The kDmul variant instead packs S exactly and spends a second FP64
 // instruction on Ci*K:  T2 = fma(Ci*K, S*2^sc, T).
 //
@@ -61,7 +62,36 @@ struct EmuCoef {
     EmuK kx, ky, kz;  // dt*lam*_d^2 per axis as integer mantissa and exponent
     double dtlam, ax, ay, az;
     double Kx;        // dt*lam*_dx^2 (the kDmul variant, iso grids)
+    // the three K as integers at one exponent, K_d = r_d * 2^re (emu_set_common); common: whether
+    // that is exact, i.e. the K lie within a factor of 2^8 (spacings within 16)
+    unsigned long long rx, ry, rz;
+    int re, common;
 };
+
+// How a node's Laplacian combines its axes: one K (equal spacings), one K per axis as
+// integers at a common exponent, or one K per axis at its own exponent (spacings so unequal
+// that the small K would lose bits at the large one's exponent).
+enum EmuAxes { AX_COMMON = 0, AX_ISO = 1, AX_FAR = 2 };
+
+// Sets common, re and r_d from the three K.
+__host__ __device__ inline void emu_set_common(EmuCoef &c) {
+    const int exy = c.kx.e > c.ky.e ? c.kx.e : c.ky.e, e = exy > c.kz.e ? exy : c.kz.e;
+    // mantissas are multiples of 2^10: after a shift by at most 8 still of 4 (emu_L_common)
+    c.common = e - c.kx.e <= 8 && e - c.ky.e <= 8 && e - c.kz.e <= 8;
+    if (!c.common) return;
+    c.re = e;
+    c.rx = c.kx.m >> (e - c.kx.e);
+    c.ry = c.ky.m >> (e - c.ky.e);
+    c.rz = c.kz.m >> (e - c.kz.e);
+}
+
+// K_d = dtlam * a_d (positive normal, or the emulated forms are not run).
+inline EmuCoef emu_coef(double dtlam, double ax, double ay, double az) {
+    EmuCoef c{emu_const(dtlam * ax), emu_const(dtlam * ay), emu_const(dtlam * az), dtlam, ax, ay, az,
+              dtlam * ax, 0ull, 0ull, 0ull, 0, 0};
+    emu_set_common(c);
+    return c;
+}
 
 __device__ __forceinline__ unsigned long long dbits(double d) {
     return (unsigned long long)__double_as_longlong(d);
@@ -178,14 +208,60 @@ __device__ __forceinline__ bool emu_same_binade(unsigned long long c, unsigned l
     return ((d & 0xfff00000u) == 0u) && emu_fast_exponent(hc);
 }
 
+// (sum_d r_d * S_d) * 2^(sc + re) for exact per-axis sums |S_d| <= 2^61: the sums are shifted
+// left together until the largest fills 62 bits, biased by 2^62 to be unsigned, multiplied by
+// the 63-bit r_d keeping the top 64 bits of each product (three 32 x 32-bit multiplies with
+// the accumulation inside; the dropped low product is below one unit), added, unbiased
+// (sum r_d / 4, exact as r_d % 4 == 0) and converted once: one rounding to 53 bits of a value
+// known to about 2^-59 of its largest term.  A node then needs two FP64-pipe instructions
+// (the conversion and the final DFMA), which the pipe serves in about the time HBM needs, and
+// about 110 integer ones, which bind.  Measured, us a step: 512 x 384 x 256 nodes 280 (443
+// with one product, pack and FP64 sum per axis, three FP64 instructions and less exact; 307
+// with the integer pack in place of the conversion); 2-D 8192 x 6000 255 (878 in plain FP64,
+// ten FP64 instructions per node; 274 with the integer pack).
+// kDim = 2: the z sum is not there.
+template <int kDim>
+__device__ __forceinline__ double emu_L_common(long long sx, long long sy, long long sz, int sc,
+                                               unsigned long long flip, const EmuCoef &k) {
+    unsigned long long m = (unsigned long long)(sx ^ (sx >> 63)) | (unsigned long long)(sy ^ (sy >> 63));
+    if (kDim == 3) m |= (unsigned long long)(sz ^ (sz >> 63));
+    // 2m + 1 scales with the sums bit for bit (also where one is -1), so the same real sums
+    // at another scale 2^sc give the same result
+    const int n = __clzll((long long)(2ull * m + 1ull)) - 1;
+    auto term = [n](long long s, unsigned long long r) -> unsigned long long {
+        const unsigned long long u = ((unsigned long long)s << n) + (1ull << 62);  // [0, 2^63)
+        const unsigned uh = (unsigned)(u >> 32), ul = (unsigned)u;
+        const unsigned rh = (unsigned)(r >> 32), rl = (unsigned)r;
+        const unsigned long long cross = (unsigned long long)uh * rl + (unsigned long long)ul * rh;  // < 2^64
+        return (unsigned long long)uh * rh + (cross >> 32);
+    };
+    unsigned long long q = term(sx, k.rx) + term(sy, k.ry);  // < 3 * 2^62 in all
+    unsigned long long bias = (k.rx >> 2) + (k.ry >> 2);
+    if (kDim == 3) {
+        q += term(sz, k.rz);
+        bias += k.rz >> 2;
+    }
+    const long long v = (long long)(q - bias);
+    const int t = sc + k.re + 64 - n;  // L = v * 2^t
+    if (t >= -1022 && t <= 960) {      // v as FP64 times 2^t is normal (or v = 0)
+        const unsigned long long b = dbits(__ll2double_rn(v)) + ((unsigned long long)(unsigned)(t << 20) << 32);
+        return bitsd((v == 0ll ? 0ull : b) ^ flip);
+    }
+    unsigned long long sg;
+    const unsigned long long a = emu_abs(v, &sg);
+    return bitsd((a == 0ull ? 0ull : emu_pack_mag(a, t)) | (sg ^ flip));
+}
+
 // L (as FP64 bits, with sign) from exact per-axis sums at scale 2^sc.
-template <bool kIso>
+template <int kAx, int kDim = 3>
 __device__ __forceinline__ double emu_L(long long sx, long long sy, long long sz, int sc,
                                         unsigned long long flip, const EmuCoef &k) {
     unsigned long long sg;
-    if (kIso) {
+    if (kAx == AX_ISO) {
         const unsigned long long a = emu_abs(sx + sy + sz, &sg);
         return bitsd(emu_scaled_mag(a, sc, k.kx) | (sg ^ flip));
+    } else if (kAx == AX_COMMON) {
+        return emu_L_common<kDim>(sx, sy, sz, sc, flip, k);
     } else {
         unsigned long long s1, s2, s3;
         const unsigned long long ax = emu_abs(sx, &s1), ay = emu_abs(sy, &s2), az = emu_abs(sz, &s3);
@@ -196,8 +272,20 @@ __device__ __forceinline__ double emu_L(long long sx, long long sy, long long sz
     }
 }
 
+// emu_L of signed sums (the general path).  AX_COMMON truncates its products, so the sums
+// are first taken with the centre's sign, as the fast and window paths have them: every path
+// of a node then gives the same bits, and a field of the other sign exactly the other sign.
+template <int kAx, int kDim = 3>
+__device__ __forceinline__ double emu_L_signed(long long sx, long long sy, long long sz, int sc,
+                                               unsigned long long c, const EmuCoef &k) {
+    if (kAx != AX_COMMON) return emu_L<kAx, kDim>(sx, sy, sz, sc, 0ull, k);
+    const long long neg = (long long)c >> 63;  // conditional negation: (s ^ neg) - neg
+    return emu_L<kAx, kDim>((sx ^ neg) - neg, (sy ^ neg) - neg, (sz ^ neg) - neg, sc,
+                            c & 0x8000000000000000ull, k);
+}
+
 // Fast path (caller checked emu_same_binade).
-template <bool kIso, bool kDmul>
+template <int kAx, bool kDmul, int kDim = 3>
 __device__ __forceinline__ double emu_fast_node(unsigned long long c, unsigned long long xm,
                                                 unsigned long long xp, unsigned long long ym,
                                                 unsigned long long yp, unsigned long long zm,
@@ -207,17 +295,17 @@ __device__ __forceinline__ double emu_fast_node(unsigned long long c, unsigned l
     const unsigned long long c2 = c + c;
     const long long sx = (long long)(xm + xp - c2);
     const long long sy = (long long)(ym + yp - c2);
-    const long long sz = (long long)(zm + zp - c2);
+    const long long sz = kDim == 3 ? (long long)(zm + zp - c2) : 0ll;
     const int e = emu_exp(c);
     const int sc = (e ? e : 1) - 1075;
     const unsigned long long flip = c & 0x8000000000000000ull;  // negative values: minus
-    if (kDmul && kIso) {
+    if (kDmul && kAx == AX_ISO) {
         unsigned long long sg;
         const unsigned long long a = emu_abs(sx + sy + sz, &sg);
         const double Sd = bitsd(emu_pack_mag_normal(a, sc) | (sg ^ flip));
         return fma(ci * k.Kx, Sd, bitsd(c));
     }
-    return fma(ci, emu_L<kIso>(sx, sy, sz, sc, flip, k), bitsd(c));
+    return fma(ci, emu_L<kAx, kDim>(sx, sy, sz, sc, flip, k), bitsd(c));
 }
 
 // Signed fixed-point value of FP64 bits v at scale 2^(Emax' - 1079), where
@@ -233,7 +321,7 @@ __device__ __forceinline__ long long emu_fixed(unsigned long long v, int emax1) 
 }
 
 // General path: any signs and exponents (rare for smooth fields).
-template <bool kIso>
+template <int kAx, int kDim = 3>
 __device__ __noinline__ double emu_general_node(unsigned long long c, unsigned long long xm,
                                                 unsigned long long xp, unsigned long long ym,
                                                 unsigned long long yp, unsigned long long zm,
@@ -255,7 +343,7 @@ __device__ __noinline__ double emu_general_node(unsigned long long c, unsigned l
     const long long sx = emu_fixed(xm, em1) + emu_fixed(xp, em1) - fc2;
     const long long sy = emu_fixed(ym, em1) + emu_fixed(yp, em1) - fc2;
     const long long sz = emu_fixed(zm, em1) + emu_fixed(zp, em1) - fc2;
-    return fma(ci, emu_L<kIso>(sx, sy, sz, em1 - 1079, 0ull, k), bitsd(c));
+    return fma(ci, emu_L_signed<kAx, kDim>(sx, sy, sz, em1 - 1079, c, k), bitsd(c));
 }
 
 // Exact per-axis second-difference sums of seven arbitrary finite FP64 values
@@ -343,8 +431,8 @@ __device__ __forceinline__ double emu_step_node_scaled(unsigned long long c, uns
 // bit for bit those of the per-node general path that the fused-pair and column
 // kernels take.  Inf/NaN among a node's values: plain FP64, which propagates it.
 //   kScaled: out = fma(cs, S*2^sc, c) with ci = cs (pre-scaled coefficient);
-//   else:    out = fma(ci, L, c), L = emu_L<kIso>(per-axis sums).
-template <int PX, bool kScaled, bool kIso>
+//   else:    out = fma(ci, L, c), L = emu_L_signed<kAx>(per-axis sums).
+template <int PX, bool kScaled, int kAx>
 __device__ __forceinline__ void emu_lane_general(const unsigned long long (&c)[PX], unsigned long long xl,
                                                  unsigned long long xr, const unsigned long long (&ym)[PX],
                                                  const unsigned long long (&yp)[PX],
@@ -360,7 +448,7 @@ __device__ __forceinline__ void emu_lane_general(const unsigned long long (&c)[P
             if (kScaled)
                 out[i] = fma(ci[i], emu_pack(sx + sy + sz, sc), bitsd(c[i]));
             else
-                out[i] = fma(ci[i], emu_L<kIso>(sx, sy, sz, sc, 0ull, k), bitsd(c[i]));
+                out[i] = fma(ci[i], emu_L_signed<kAx>(sx, sy, sz, sc, c[i], k), bitsd(c[i]));
         } else {  // Inf / NaN
             const double cc = bitsd(c[i]);
             if (kScaled) {
@@ -413,7 +501,7 @@ __device__ __forceinline__ long long emu_window_units(unsigned long long v, unsi
 // instructions (|value| < 2^57 units, so the sums of seven stay below 2^61), the sums
 // are exact, and the node finishes as on the general path (same real sum, same rounding: bit for
 // bit emu_lane_general's result) at about half its cost.  flip: the values' sign.
-template <int PX, bool kScaled, bool kIso>
+template <int PX, bool kScaled, int kAx>
 __device__ __forceinline__ void emu_lane_window(const unsigned long long (&c)[PX], unsigned long long xl,
                                                 unsigned long long xr, const unsigned long long (&ym)[PX],
                                                 const unsigned long long (&yp)[PX],
@@ -438,21 +526,21 @@ __device__ __forceinline__ void emu_lane_window(const unsigned long long (&c)[PX
             const unsigned long long a = emu_abs(sx + sy + sz, &sg);
             out[i] = fma(ci[i], bitsd(emu_pack_mag_normal(a, sc) | (sg ^ flip)), bitsd(c[i]));
         } else {
-            out[i] = fma(ci[i], emu_L<kIso>(sx, sy, sz, sc, flip, k), bitsd(c[i]));
+            out[i] = fma(ci[i], emu_L<kAx>(sx, sy, sz, sc, flip, k), bitsd(c[i]));
         }
     }
 }
 
 // One node, either path (per-lane branch).
-template <bool kIso, bool kDmul>
+template <int kAx, bool kDmul, int kDim = 3>
 __device__ __forceinline__ double emu_step_node(unsigned long long c, unsigned long long xm,
                                                 unsigned long long xp, unsigned long long ym,
                                                 unsigned long long yp, unsigned long long zm,
                                                 unsigned long long zp, double ci,
                                                 const EmuCoef &k) {
     if (emu_same_binade(c, xm, xp, ym, yp, zm, zp))
-        return emu_fast_node<kIso, kDmul>(c, xm, xp, ym, yp, zm, zp, ci, k);
-    return emu_general_node<kIso>(c, xm, xp, ym, yp, zm, zp, ci, k);
+        return emu_fast_node<kAx, kDmul, kDim>(c, xm, xp, ym, yp, zm, zp, ci, k);
+    return emu_general_node<kAx, kDim>(c, xm, xp, ym, yp, zm, zp, ci, k);
 }
 
 }  // namespace psd

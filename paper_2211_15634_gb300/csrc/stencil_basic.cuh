@@ -20,7 +20,7 @@ struct CoefT {
 
 // Same column march for FP64 data with the one-DFMA emulated arithmetic of
 // emu64.cuh (used when the TMA kernel cannot serve the grid, e.g. odd nx).
-template <bool kIso, bool kScaled>
+template <int kAx, bool kScaled>
 __global__ void __launch_bounds__(256)
 k_step_basic_emu(double *__restrict__ T2, const double *__restrict__ T,
                  const double *__restrict__ Ci, EmuCoef c, int64_t nx, int64_t ny, int64_t nz,
@@ -40,7 +40,7 @@ k_step_basic_emu(double *__restrict__ T2, const double *__restrict__ T,
         if (kScaled)  // Ci holds dt*lam*_d^2*Ci (isotropic grid)
             T2[p] = emu_step_node_scaled(tc, Tb[p - 1], Tb[p + 1], Tb[p - sy], Tb[p + sy], tm, tp, Ci[p]);
         else
-            T2[p] = emu_step_node<kIso, false>(tc, Tb[p - 1], Tb[p + 1], Tb[p - sy], Tb[p + sy], tm,
+            T2[p] = emu_step_node<kAx, false>(tc, Tb[p - 1], Tb[p + 1], Tb[p - sy], Tb[p + sy], tm,
                                                tp, Ci[p], c);
         tm = tc;
         tc = tp;
@@ -59,11 +59,13 @@ inline cudaError_t launch_step_basic_emu(double *T2, const double *T, const doub
     if (gx > 0x7fffffff || gy > 65535 || gz > 65535) return cudaErrorInvalidConfiguration;
     const dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)gz);
     if (scaled)
-        k_step_basic_emu<true, true><<<grid, block, 0, s>>>(T2, T, Ci, c, nx, ny, nz, (int)kchunk);
+        k_step_basic_emu<AX_ISO, true><<<grid, block, 0, s>>>(T2, T, Ci, c, nx, ny, nz, (int)kchunk);
     else if (iso)
-        k_step_basic_emu<true, false><<<grid, block, 0, s>>>(T2, T, Ci, c, nx, ny, nz, (int)kchunk);
+        k_step_basic_emu<AX_ISO, false><<<grid, block, 0, s>>>(T2, T, Ci, c, nx, ny, nz, (int)kchunk);
+    else if (c.common)
+        k_step_basic_emu<AX_COMMON, false><<<grid, block, 0, s>>>(T2, T, Ci, c, nx, ny, nz, (int)kchunk);
     else
-        k_step_basic_emu<false, false><<<grid, block, 0, s>>>(T2, T, Ci, c, nx, ny, nz, (int)kchunk);
+        k_step_basic_emu<AX_FAR, false><<<grid, block, 0, s>>>(T2, T, Ci, c, nx, ny, nz, (int)kchunk);
     return cudaGetLastError();
 }
 

@@ -30,8 +30,7 @@ cudaError_t launch_step_f64_fast(double *T2, const double *T, const double *Ci, 
     if (step_tma_ok(g, 8, T2, T, Ci))
         return launch_zmarch(iso ? Z_F64_EMU_ISO : Z_F64_EMU_ANISO, T2, T, nullptr, nullptr, Ci, c, g, s,
                              write_bnd);
-    const EmuCoef ek{emu_const(c.dtlam * c.ax), emu_const(c.dtlam * c.ay), emu_const(c.dtlam * c.az),
-                     c.dtlam, c.ax, c.ay, c.az, c.dtlam * c.ax};
+    const EmuCoef ek = emu_coef(c.dtlam, c.ax, c.ay, c.az);
     return launch_step_basic_emu(T2, T, Ci, ek, iso, g.nx, g.ny, g.nz, sm_count(), s);
 }
 

@@ -10,13 +10,14 @@ namespace psd {
 
 enum ZMode {
     Z_F64_EMU_ISO = 0,       // one DFMA per node, 64x64 high multiply by K
-    Z_F64_EMU_ANISO = 1,     // as above, one product per axis
+    Z_F64_EMU_ANISO = 1,     // as above, the axes' K as integers at one exponent
     Z_F64_NATIVE = 2,        // plain FP64 instructions
     Z_F32 = 3,
     Z_F32_COMP = 4,
     Z_F64_EMU_ISO_DMUL = 5,  // two FP64 ops per node: fma(Ci*K, S, T)
     Z_F64_SCALED = 6,        // Ci already holds dt*lam*_d^2*Ci: fma(Cs, S, T)
     Z_F64_SCALED4 = 7,       // as Z_F64_SCALED, four nodes per thread (32-byte accesses)
+    Z_F64_EMU_ANISO_FAR = 8,  // spacings more than 16 apart: one rounded product per axis
 };
 
 struct ZParams {

@@ -38,6 +38,8 @@ struct ZTraits<Z_F64_EMU_ISO> {
 template <>
 struct ZTraits<Z_F64_EMU_ANISO> : ZTraits<Z_F64_EMU_ISO> {};
 template <>
+struct ZTraits<Z_F64_EMU_ANISO_FAR> : ZTraits<Z_F64_EMU_ISO> {};
+template <>
 struct ZTraits<Z_F64_NATIVE> : ZTraits<Z_F64_EMU_ISO> {};
 template <>
 struct ZTraits<Z_F64_EMU_ISO_DMUL> : ZTraits<Z_F64_EMU_ISO> {};
@@ -185,9 +187,10 @@ __device__ __forceinline__ void zmarch_tile(const CUtensorMap *tmT, const CUtens
         if (row_ok) {
             V cv{};  // E2 at the own nodes (two-float state)
             V out;
-            if constexpr (MODE == Z_F64_EMU_ISO || MODE == Z_F64_EMU_ANISO ||
+            if constexpr (MODE == Z_F64_EMU_ISO || MODE == Z_F64_EMU_ANISO || MODE == Z_F64_EMU_ANISO_FAR ||
                           MODE == Z_F64_EMU_ISO_DMUL || MODE == Z_F64_SCALED || MODE == Z_F64_SCALED4) {
-                constexpr bool kIso = MODE != Z_F64_EMU_ANISO;
+                constexpr int kAx = MODE == Z_F64_EMU_ANISO ? AX_COMMON
+                                    : MODE == Z_F64_EMU_ANISO_FAR ? AX_FAR : AX_ISO;
                 constexpr bool kDmul = MODE == Z_F64_EMU_ISO_DMUL;
                 constexpr bool kScaled = MODE == Z_F64_SCALED || MODE == Z_F64_SCALED4;
                 unsigned long long c[PX], xm[PX], xp[PX], ym[PX], yp[PX], zm[PX], zp[PX];
@@ -256,7 +259,7 @@ __device__ __forceinline__ void zmarch_tile(const CUtensorMap *tmT, const CUtens
                             reinterpret_cast<E *>(&out)[i] =
                                 emu_fast_node_scaled(c[i], xm[i], xp[i], ym[i], yp[i], zm[i], zp[i], ci);
                         else
-                            reinterpret_cast<E *>(&out)[i] = emu_fast_node<kIso, kDmul>(
+                            reinterpret_cast<E *>(&out)[i] = emu_fast_node<kAx, kDmul>(
                                 c[i], xm[i], xp[i], ym[i], yp[i], zm[i], zp[i], ci, p.ek);
                     }
                 } else {
@@ -269,10 +272,10 @@ __device__ __forceinline__ void zmarch_tile(const CUtensorMap *tmT, const CUtens
                     unsigned ewin;
                     const bool near = emu_window_hi(hw, hc, &ewin);
                     if (__all_sync(rmask, near))
-                        emu_lane_window<PX, kScaled, kIso>(c, xm[0], xp[PX - 1], ym, yp, zm, zp, ci, p.ek,
+                        emu_lane_window<PX, kScaled, kAx>(c, xm[0], xp[PX - 1], ym, yp, zm, zp, ci, p.ek,
                                                            ewin, o);
                     else
-                        emu_lane_general<PX, kScaled, kIso>(c, xm[0], xp[PX - 1], ym, yp, zm, zp, ci,
+                        emu_lane_general<PX, kScaled, kAx>(c, xm[0], xp[PX - 1], ym, yp, zm, zp, ci,
                                                             p.ek, o);
 #pragma unroll
                     for (int i = 0; i < PX; ++i) reinterpret_cast<E *>(&out)[i] = o[i];
