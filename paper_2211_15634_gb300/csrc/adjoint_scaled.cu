@@ -24,6 +24,11 @@
 // the same-binade fast path (one DFMA); w = Cs*ybar costs one DMUL per tile
 // value.  Csbar of plane k is loaded at the top of iteration k so that its
 // latency hides behind the w tile work.
+//
+// The same kernel takes Ci as given (kAx, kGiven below).  Measured at 256^3 against the
+// z-march it replaced there (adjoint_zmarch.cu: w values spread over the threads, two
+// barriers per plane, one pack and one FP64 product per axis): equal spacings 184 against
+// 244 us, unequal 240 against 362; 512 x 384 x 256 unequal 693 against 1014.
 #include <cudaTypedefs.h>
 
 
@@ -40,6 +45,7 @@ __device__ unsigned g_adjs_error;  // set when an mbarrier wait times out
 struct AdjSParams {
     int64_t nx, ny, nz;
     int kchunk, ntx;
+    EmuCoef ek;  // AX_COMMON: dt*lam*_d^2 of the axes at one exponent
 };
 
 // Fixed-point value of FP64 bits v at scale 2^(E-1079) (E >= the exponent of v).
@@ -59,18 +65,33 @@ __device__ __forceinline__ double adjs_pack_normal(long long S, int sc) {
     return bitsd(emu_pack_mag_normal(a, sc) | sg);
 }
 
+template <int kAx>
 static __device__ __noinline__ double adjs_lap_general(unsigned long long c, unsigned long long xm,
                                                        unsigned long long xp, unsigned long long ym,
                                                        unsigned long long yp, unsigned long long zm,
-                                                       unsigned long long zp) {
+                                                       unsigned long long zp, const EmuCoef &k) {
     long long sx, sy, sz;
     int sc;
-    if (emu_sums_general(c, xm, xp, ym, yp, zm, zp, sx, sy, sz, sc)) return emu_pack(sx + sy + sz, sc);
-    const double cc = bitsd(c);  // Inf / NaN: plain FP64 propagates it
+    const double cc = bitsd(c);
+    if (emu_sums_general(c, xm, xp, ym, yp, zm, zp, sx, sy, sz, sc)) {
+        if constexpr (kAx == AX_COMMON) return emu_L_signed<AX_COMMON>(sx, sy, sz, sc, c, k);
+        return emu_pack(sx + sy + sz, sc);
+    }
+    // Inf / NaN: plain FP64 propagates it
+    if constexpr (kAx == AX_COMMON) {
+        const double d2x = (bitsd(xp) - cc) - (cc - bitsd(xm)), d2y = (bitsd(yp) - cc) - (cc - bitsd(ym)),
+                     d2z = (bitsd(zp) - cc) - (cc - bitsd(zm));
+        return k.dtlam * ((d2x * k.ax + d2y * k.ay) + d2z * k.az);
+    }
     return (((bitsd(xm) + bitsd(xp)) + (bitsd(ym) + bitsd(yp))) + (bitsd(zm) + bitsd(zp))) - 6.0 * cc;
 }
 
-template <int BY, int NST>
+// kAx, kGiven: AX_ISO on the pre-scaled coefficient; AX_ISO and kGiven, Ci as given on equal
+// spacings: w = Ci*ybar, the one dt*lam*_d^2 multiplied in last (Tbar by the DFMA that
+// replaces the DADD, Cibar by one more DMUL); AX_COMMON, Ci as given on unequal spacings: w =
+// Ci*ybar, Tbar = ybar + L(w) and Cibar += ybar*L(T) with L = sum_d dt*lam*_d^2 * (second
+// difference along d), the axes' exact sums combined as integers (emu_L_common).
+template <int BY, int NST, int kAx, bool kGiven>
 __global__ void __launch_bounds__(32 * BY, 3)
 k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmY,
                  const __grid_constant__ CUtensorMap tmC, double *__restrict__ Tbar,
@@ -255,18 +276,26 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
             const long long wl = wk[row * W + col - 1], wr = wk[row * W + col + PX];
             const longlong2 wu = *(const longlong2 *)(wk + (row - 1) * W + col);
             const longlong2 wd = *(const longlong2 *)(wk + (row + 1) * W + col);
-            const long long S0 = ((wl + wc1) + (wu.x + wd.x)) + (wm0 + wp0) - 6 * wc0;
-            const long long S1 = ((wc0 + wr) + (wu.y + wd.y)) + (wm1 + wp1) - 6 * wc1;
             const int sc = Esc - 1079;
             double2 tb;
-            if (Esc >= 57 && Esc <= 2042) {  // CTA-uniform: the packed sums are normal
-                tb.x = yc.x + adjs_pack_normal(S0, sc);
-                tb.y = yc.y + adjs_pack_normal(S1, sc);
+            const long long S0 = ((wl + wc1) + (wu.x + wd.x)) + (wm0 + wp0) - 6 * wc0;
+            const long long S1 = ((wc0 + wr) + (wu.y + wd.y)) + (wm1 + wp1) - 6 * wc1;
+            if constexpr (kAx == AX_COMMON) {
+                if (Esc == 0x7ff) {  // a non-finite w in this CTA's march: report NaN
+                    tb.x = tb.y = __longlong_as_double(0x7ff8000000000000ll);
+                } else {
+                    const long long a2 = 2 * wc0, b2 = 2 * wc1;
+                    tb.x = yc.x + emu_L_common<3>(wl + wc1 - a2, wu.x + wd.x - a2, wm0 + wp0 - a2, sc, 0ull, p.ek);
+                    tb.y = yc.y + emu_L_common<3>(wc0 + wr - b2, wu.y + wd.y - b2, wm1 + wp1 - b2, sc, 0ull, p.ek);
+                }
+            } else if (Esc >= 57 && Esc <= 2042) {  // CTA-uniform: the packed sums are normal
+                tb.x = kGiven ? fma(p.ek.Kx, adjs_pack_normal(S0, sc), yc.x) : yc.x + adjs_pack_normal(S0, sc);
+                tb.y = kGiven ? fma(p.ek.Kx, adjs_pack_normal(S1, sc), yc.y) : yc.y + adjs_pack_normal(S1, sc);
             } else if (Esc == 0x7ff) {  // a non-finite w in this CTA's march: report NaN
                 tb.x = tb.y = __longlong_as_double(0x7ff8000000000000ll);
             } else {
-                tb.x = yc.x + adjs_pack(S0, sc);
-                tb.y = yc.y + adjs_pack(S1, sc);
+                tb.x = kGiven ? fma(p.ek.Kx, adjs_pack(S0, sc), yc.x) : yc.x + adjs_pack(S0, sc);
+                tb.y = kGiven ? fma(p.ek.Kx, adjs_pack(S1, sc), yc.y) : yc.y + adjs_pack(S1, sc);
             }
             if (all_x) {
                 *(double2 *)(Tbar + base) = tb;
@@ -302,7 +331,15 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
                 }
                 const bool fast = emu_same_binade_hi(hw, hc0);
                 double L0, L1;
-                if (__all_sync(0xffffffffu, fast)) {
+                if (kAx == AX_COMMON && __all_sync(0xffffffffu, fast)) {
+                    const unsigned long long a2 = 2ull * c0, b2 = 2ull * c1;
+                    const int sct = emu_exp(c0) - 1075;
+                    const unsigned long long flip = c0 & 0x8000000000000000ull;  // negative: minus
+                    L0 = emu_L_common<3>((long long)(xl + c1 - a2), (long long)(u0 + d0 - a2),
+                                         (long long)(m0b + p0 - a2), sct, flip, p.ek);
+                    L1 = emu_L_common<3>((long long)(c0 + xr - b2), (long long)(u1 + d1 - b2),
+                                         (long long)(m1b + p1 - b2), sct, flip, p.ek);
+                } else if (kAx != AX_COMMON && __all_sync(0xffffffffu, fast)) {
                     const long long S0t = (long long)(((xl + c1) + (u0 + d0)) + (m0b + p0) - 6ull * c0);
                     const long long S1t = (long long)(((c0 + xr) + (u1 + d1)) + (m1b + p1) - 6ull * c1);
                     const int e = emu_exp(c0);
@@ -313,11 +350,11 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
                     L0 = bitsd(emu_pack_mag_normal(a0, sct) | (g0 ^ flip));
                     L1 = bitsd(emu_pack_mag_normal(a1, sct) | (g1 ^ flip));
                 } else {
-                    L0 = m0 ? adjs_lap_general(c0, xl, c1, u0, d0, m0b, p0) : 0.0;
-                    L1 = m1 ? adjs_lap_general(c1, c0, xr, u1, d1, m1b, p1) : 0.0;
+                    L0 = m0 ? adjs_lap_general<kAx>(c0, xl, c1, u0, d0, m0b, p0, p.ek) : 0.0;
+                    L1 = m1 ? adjs_lap_general<kAx>(c1, c0, xr, u1, d1, m1b, p1, p.ek) : 0.0;
                 }
-                cb.x = fma(yc.x, L0, cb.x);
-                cb.y = fma(yc.y, L1, cb.y);
+                cb.x = fma(kAx == AX_ISO && kGiven ? p.ek.Kx * yc.x : yc.x, L0, cb.x);
+                cb.y = fma(kAx == AX_ISO && kGiven ? p.ek.Kx * yc.y : yc.y, L1, cb.y);
                 if (all_in) {
                     *(double2 *)(Csbar + base) = cb;
                 } else {
@@ -340,14 +377,15 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
     }
 }
 
-cudaError_t launch_adjoint_scaled(double *Tbar, double *Csbar, const double *ybar, const double *T,
-                                  const double *Cs, Grid3 g, cudaStream_t s) {
+template <int kAx, bool kGiven>
+static cudaError_t launch_adjs(double *Tbar, double *Csbar, const double *ybar, const double *T,
+                               const double *Cs, const EmuCoef &ek, Grid3 g, cudaStream_t s) {
     constexpr int BY = 8, NST = 3, PX = 2, BX = 32 * PX, W = BX + 2 * PX, H = BY + 2;
     constexpr unsigned TBA = (W * H * 8 + 127) / 128 * 128;
     constexpr size_t smem = 3 * NST * TBA + 3 * TBA + NST * 8;
     static unsigned attr_gen[64] = {0};
     cudaError_t ae;
-    if (!set_smem_attr_once((const void *)k_adjoint_scaled<BY, NST>, (int)smem, attr_gen, &ae)) return ae;
+    if (!set_smem_attr_once((const void *)k_adjoint_scaled<BY, NST, kAx, kGiven>, (int)smem, attr_gen, &ae)) return ae;
     CUtensorMap mT, mY, mC;
     if (!make_tensor_map_3d(&mT, T, 8, g, W, H) || !make_tensor_map_3d(&mY, ybar, 8, g, W, H) ||
         !make_tensor_map_3d(&mC, Cs, 8, g, W, H))
@@ -379,9 +417,21 @@ cudaError_t launch_adjoint_scaled(double *Tbar, double *Csbar, const double *yba
     }
     const int64_t gz = (g.nz + kchunk - 1) / kchunk;
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
-    AdjSParams p{g.nx, g.ny, g.nz, kchunk, (int)ntx};
-    return launch_pdl(k_adjoint_scaled<BY, NST>, dim3((unsigned)tiles, (unsigned)gz, 1), dim3(32 * BY), smem, s,
+    AdjSParams p{g.nx, g.ny, g.nz, kchunk, (int)ntx, ek};
+    return launch_pdl(k_adjoint_scaled<BY, NST, kAx, kGiven>, dim3((unsigned)tiles, (unsigned)gz, 1), dim3(32 * BY), smem, s,
                       mT, mY, mC, Tbar, Csbar, p);
+}
+
+cudaError_t launch_adjoint_scaled(double *Tbar, double *Csbar, const double *ybar, const double *T,
+                                  const double *Cs, Grid3 g, cudaStream_t s) {
+    return launch_adjs<AX_ISO, false>(Tbar, Csbar, ybar, T, Cs, EmuCoef{}, g, s);
+}
+
+cudaError_t launch_adjoint_given(double *Tbar, double *Cibar, const double *ybar, const double *T,
+                                 const double *Ci, const EmuCoef &ek, Grid3 g, cudaStream_t s) {
+    if (ek.ax == ek.ay && ek.ay == ek.az)
+        return launch_adjs<AX_ISO, true>(Tbar, Cibar, ybar, T, Ci, ek, g, s);
+    return launch_adjs<AX_COMMON, true>(Tbar, Cibar, ybar, T, Ci, ek, g, s);
 }
 
 unsigned adjoint_scaled_device_error(bool clear) {

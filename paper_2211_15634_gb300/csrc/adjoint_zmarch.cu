@@ -1,4 +1,6 @@
-// FP64 transposed step (adjoint) on Ci as given, as a TMA-fed z-march.
+// FP64 transposed step (adjoint) on Ci as given, as a TMA-fed z-march, for coefficients
+// that adjoint_scaled.cu does not take: spacings more than 16 apart, or a dt*lam that is not
+// positive (256^3 on unequal spacings: 362 us here, 240 there).
 //
 // For ybar = dL/dT_{t+1} and the state T = T_t the forward step read:
 //   w[q]      = Ci[q]*ybar[q] at interior q, 0 elsewhere (and outside the grid),
@@ -51,7 +53,7 @@ __device__ __forceinline__ E aget(const V &v, int i) {
     return reinterpret_cast<const E *>(&v)[i];
 }
 
-template <typename E, bool kIso, int BY, int NST>
+template <typename E, int BY, int NST>
 __global__ void __launch_bounds__(32 * BY, 3)
 k_adjoint_zmarch(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmY,
                  const __grid_constant__ CUtensorMap tmC, E *__restrict__ Tbar,
@@ -271,7 +273,7 @@ k_adjoint_zmarch(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
                 // a non-finite w anywhere in this CTA's march: report NaN, not garbage
                 reinterpret_cast<E *>(&tb)[i] =
                     Esc == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
-                                 : emu_axpy3<kIso>(yb, sx, sy, sz, Esc - 1079, p.Kx, p.Ky, p.Kz);
+                                 : emu_axpy3(yb, sx, sy, sz, Esc - 1079, p.Kx, p.Ky, p.Kz);
             }
             // ---- Cibar: T-Laplacian, same-binade fast path when the whole warp allows it
             if (do_ci) {
@@ -337,10 +339,10 @@ k_adjoint_zmarch(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
                         }
                         const int e = emu_exp(c[i]);
                         sc = (e ? e : 1) - 1075;
-                        L = emu_axpy3<kIso>(0.0, sx, sy, sz, sc, p.Kx, p.Ky, p.Kz);
+                        L = emu_axpy3(0.0, sx, sy, sz, sc, p.Kx, p.Ky, p.Kz);
                     } else if (emu_sums_general(c[i], xm[i], xp[i], ym[i], yp[i], zm[i], zp[i],
                                                 sx, sy, sz, sc)) {
-                        L = emu_axpy3<kIso>(0.0, sx, sy, sz, sc, p.Kx, p.Ky, p.Kz);
+                        L = emu_axpy3(0.0, sx, sy, sz, sc, p.Kx, p.Ky, p.Kz);
                     } else {
                         const double cc = bitsd(c[i]);
                         L = (p.Kx * ((bitsd(xm[i]) - cc) - (cc - bitsd(xp[i]))) +
@@ -380,7 +382,7 @@ k_adjoint_zmarch(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
     }
 }
 
-template <typename E, bool kIso, int BY, int NST>
+template <typename E, int BY, int NST>
 static cudaError_t launch_adj_t(E *Tbar, E *Cibar, const E *ybar, const E *T, const E *Ci, Grid3 g,
                                 AdjParams p, int kchunk, cudaStream_t s) {
     constexpr int PX = ATraits<E>::PX, BX = 32 * PX, W = BX + 2 * PX, H = BY + 2;
@@ -388,7 +390,7 @@ static cudaError_t launch_adj_t(E *Tbar, E *Cibar, const E *ybar, const E *T, co
     constexpr size_t smem = 3 * NST * TBA + 3 * TBA + NST * 8;
     static unsigned attr_gen[64] = {0};
     cudaError_t ae;
-    if (!set_smem_attr_once((const void *)k_adjoint_zmarch<E, kIso, BY, NST>, (int)smem, attr_gen, &ae)) return ae;
+    if (!set_smem_attr_once((const void *)k_adjoint_zmarch<E, BY, NST>, (int)smem, attr_gen, &ae)) return ae;
     CUtensorMap mT, mY, mC;
     if (!make_tensor_map_3d(&mT, T, sizeof(E), g, W, H) || !make_tensor_map_3d(&mY, ybar, sizeof(E), g, W, H) ||
         !make_tensor_map_3d(&mC, Ci, sizeof(E), g, W, H))
@@ -407,7 +409,7 @@ static cudaError_t launch_adj_t(E *Tbar, E *Cibar, const E *ybar, const E *T, co
     p.nz = g.nz;
     p.ntx = (int)ntx;
     p.kchunk = kchunk;
-    return launch_pdl(k_adjoint_zmarch<E, kIso, BY, NST>, dim3((unsigned)tiles, (unsigned)gz, 1), dim3(32 * BY), smem,
+    return launch_pdl(k_adjoint_zmarch<E, BY, NST>, dim3((unsigned)tiles, (unsigned)gz, 1), dim3(32 * BY), smem,
                       s, mT, mY, mC, Tbar, Cibar, p);
 }
 
@@ -428,9 +430,11 @@ cudaError_t launch_adjoint_zmarch(E *Tbar, E *Cibar, const E *ybar, const E *T, 
     p.Ky = c.dtlam * c.ay;
     p.Kz = c.dtlam * c.az;
     const int kchunk = launch_override(PS_OVERRIDE_ADJ_KCHUNK);
-    const bool iso = c.ax == c.ay && c.ay == c.az;
-    if (iso) return launch_adj_t<E, true, 8, 3>(Tbar, Cibar, ybar, T, Ci, g, p, kchunk, s);
-    return launch_adj_t<E, false, 8, 3>(Tbar, Cibar, ybar, T, Ci, g, p, kchunk, s);
+    if (emu_ok(c)) {
+        const EmuCoef ek = emu_coef(c.dtlam, c.ax, c.ay, c.az);
+        if (ek.common) return launch_adjoint_given(Tbar, Cibar, ybar, T, Ci, ek, g, s);
+    }
+    return launch_adj_t<E, 8, 3>(Tbar, Cibar, ybar, T, Ci, g, p, kchunk, s);
 }
 
 template cudaError_t launch_adjoint_zmarch<double>(double *, double *, const double *, const double *,

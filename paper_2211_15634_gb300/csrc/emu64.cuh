@@ -375,12 +375,9 @@ __device__ __forceinline__ double emu_pack(long long S, int sc) {
     return bitsd(emu_pack_mag(a, sc) | sg);
 }
 
-// base + sum_d K_d * S_d * 2^sc with one DFMA per distinct coefficient
-// (one in total when the grid is isotropic).  Kx/Ky/Kz are FP64 constants.
-template <bool kIso>
+// base + sum_d K_d * S_d * 2^sc with one DFMA per axis.  Kx/Ky/Kz are FP64 constants.
 __device__ __forceinline__ double emu_axpy3(double base, long long sx, long long sy, long long sz,
                                             int sc, double Kx, double Ky, double Kz) {
-    if (kIso) return fma(Kx, emu_pack(sx + sy + sz, sc), base);
     return fma(Kz, emu_pack(sz, sc), fma(Ky, emu_pack(sy, sc), fma(Kx, emu_pack(sx, sc), base)));
 }
 

@@ -16,7 +16,7 @@ cudaError_t launch_step_f64_native(double *T2, const double *T, const double *Ci
                                             sm_count(), s);
 }
 
-static bool emu_ok(StepCoef c) {
+bool emu_ok(StepCoef c) {
     const double k[3] = {c.dtlam * c.ax, c.dtlam * c.ay, c.dtlam * c.az};
     for (double v : k)
         if (!(v > 2.2250738585072014e-308 && v < 1e300)) return false;  // positive normal

@@ -54,6 +54,12 @@ unsigned adjoint_device_error(bool clear);
 // TMA-fed transposed step on the pre-scaled coefficient (adjoint_scaled.cu).
 cudaError_t launch_adjoint_scaled(double *Tbar, double *Csbar, const double *ybar, const double *T,
                                   const double *Cs, Grid3 g, cudaStream_t s);
+// The same kernel on Ci as given: equal spacings, or the axes' coefficients at one exponent
+// (ek.common).
+cudaError_t launch_adjoint_given(double *Tbar, double *Cibar, const double *ybar, const double *T,
+                                 const double *Ci, const EmuCoef &ek, Grid3 g, cudaStream_t s);
+// True when dt*lam*_d^2 is positive and normal on every axis (the emulated FP64 forms).
+bool emu_ok(StepCoef c);
 // One step of the TMA z-march in `mode`; E2 / Ein: the correction fields of the
 // two-float state (Z_F32_COMP only, else unused).  write_bnd: also store the x and y
 // boundary nodes of planes 1 .. nz-2 as copies of T's (not with Z_F32_COMP).

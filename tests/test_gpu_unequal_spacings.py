@@ -73,3 +73,22 @@ def test_2d_matches_oracle(ratios, shape):
         T = to_dev(T0)
         got = to_host(api.run2d(T, torch.empty_like(T), to_dev(Ci), 1.0, dt, inv[:2], 5))
         assert rel_linf(got, oracle.run2d(T0, Ci, 1.0, dt, *inv[:2], 5)) <= 1e-12
+
+
+@pytest.mark.parametrize("ratios", ["equal"] + list(RATIOS))
+@pytest.mark.parametrize("values", ["smooth", "many_binades"])
+@pytest.mark.parametrize("shape", [(3, 3, 3), (68, 19, 13), (132, 21, 17)])
+def test_transposed_step_matches_oracle(ratios, values, shape):
+    """Ci as given: one coefficient (equal), integers at one exponent, one product per axis."""
+    nx, ny, nz = shape
+    T = inputs.t0_gaussian(nx, ny, nz) if values == "smooth" else field(values, shape)
+    Ci, ybar = inputs.ci_random(nx, ny, nz), inputs.random_field((nz, ny, nx), 31, -1.0, 1.0)
+    inv, d2 = ((nx - 1.0,) * 3, 1.0 / (nx - 1.0) ** 2) if ratios == "equal" else inverse_spacings(ratios, nx)
+    dt = d2 / Ci.max() / 6.1
+    ref_c = np.zeros_like(T)
+    ref_t = oracle.adjoint_step(ybar, T, Ci, ref_c, 1.0, dt, *inv)
+    tbar, cibar = to_dev(np.full_like(T, np.nan)), to_dev(np.zeros_like(T))
+    api.adjoint(tbar, cibar, to_dev(ybar), to_dev(T), to_dev(Ci), 1.0, dt, inv)
+    assert rel_linf(to_host(tbar), ref_t) <= 1e-14
+    assert rel_linf(to_host(cibar), ref_c) <= 1e-14
+    assert api.device_error() == 0
