@@ -178,28 +178,32 @@ static int check_step_args(const void *T2, const void *T, const void *Ci, double
 }
 
 // One step; E2 / E: correction fields of the two-float state (PS_RUN_COMPENSATED).
-// write_bnd: the step also stores T's x and y boundary nodes of planes 1 .. nz-2 into T2
-// where the z-march serves it (step_writes_xy_boundary; not with PS_RUN_COMPENSATED).
+// in_loop: one of a time loop's steps (internal.h).  write_bnd: the step also stores T's x
+// and y boundary nodes of planes 1 .. nz-2 into T2 (not with PS_RUN_COMPENSATED).
 static cudaError_t enqueue_step(void *T2, const void *T, void *E2, const void *E, const void *Ci,
                                 StepCoef c, Grid3 g, int dtype, unsigned flags, cudaStream_t s,
-                                bool write_bnd = false) {
+                                bool in_loop = false, bool write_bnd = false) {
     if (dtype == PS_F64) {
         if (flags & PS_RUN_CI_SCALED)
             return launch_step_f64_scaled((double *)T2, (const double *)T, (const double *)Ci, g, s,
-                                          write_bnd);
+                                          write_bnd, in_loop);
         if (flags & PS_RUN_NATIVE_F64)
-            return launch_step_f64_native((double *)T2, (const double *)T, (const double *)Ci, c, g, s);
-        return launch_step_f64_fast((double *)T2, (const double *)T, (const double *)Ci, c, g, s, write_bnd);
+            return launch_step_f64_native((double *)T2, (const double *)T, (const double *)Ci, c, g, s, write_bnd);
+        return launch_step_f64_fast((double *)T2, (const double *)T, (const double *)Ci, c, g, s, write_bnd, in_loop);
     }
     if (flags & PS_RUN_COMPENSATED)
         return launch_step_f32_comp((float *)T2, (const float *)T, (float *)E2, (const float *)E,
-                                    (const float *)Ci, c, g, s);
-    return launch_step_f32((float *)T2, (const float *)T, (const float *)Ci, c, g, s, write_bnd);
+                                    (const float *)Ci, c, g, s, in_loop);
+    return launch_step_f32((float *)T2, (const float *)T, (const float *)Ci, c, g, s, write_bnd, in_loop);
 }
 
-// True when PS_RUN_TEMPORAL2 can fuse step pairs for these arguments (the mode
-// is checked by the caller: FP32 plain, or FP64 on the pre-scaled coefficient).
-static bool temporal2_ok(Grid3 g, int dtype, const void *T, const void *T2, const void *Ci) {
+// True when PS_RUN_TEMPORAL2 fuses step pairs for these arguments (the mode is checked by the
+// caller: FP32 plain, or FP64 on the pre-scaled coefficient).  FP32 pairs leave small grids
+// to the single steps' column kernel, which is faster there (us a step, pairs against single
+// steps: 64^3 4.6 / 2.2, 192^3 17 / 14), unless a z-chunk is set for them.  states: pairs that
+// keep both states, see states_column.
+static bool temporal2_ok(Grid3 g, int dtype, const void *T, const void *T2, const void *Ci, bool states = false) {
+    if (dtype == PS_F32 && (!states || (double)g.n() <= 2.2e6) && step_small(g, Z_F32) && launch_override(PS_OVERRIDE_KCHUNK2) <= 0) return false;
     return zmarch2_supported(g, elem_bytes(dtype), T, T2, Ci) &&
            zmarch2_supported(g, elem_bytes(dtype), T2, T, Ci);
 }
@@ -235,7 +239,7 @@ static cudaError_t enqueue_run(void *T, void *T2, void *comp, const void *Ci, St
         void *dst = (it & 1) ? T : T2;
         e = it < pairs ? enqueue_step2(dst, src, Ci, c, g, dtype, s)
                        : enqueue_step(dst, src, (it & 1) ? EA : EB, (it & 1) ? EB : EA, Ci, c, g, dtype,
-                                      flags, s);
+                                      flags, s, true);
     }
     return e;
 }
@@ -510,13 +514,21 @@ static int plan_states(int nt, int every, bool pairs, std::vector<StatesOp> *ops
     return cur_slot;
 }
 
+// Whether a state-keeping loop's single steps may take the column kernel on a small grid.
+// FP32 only up to 2.2 million nodes: beyond, pairs that write both states are faster, and
+// beside a reverse sweep the march's few CTAs leave the transposed steps more of each SM
+// (192^3, nt = 64, checkpoints every 8: the gradient 3.87 ms, 4.28 with the column kernel).
+static bool states_column(int dtype, Grid3 g) {
+    return dtype == PS_F64 || (double)g.n() <= 2.2e6;
+}
+
 // Whether PS_RUN_TEMPORAL2 runs fused pairs for this state-keeping loop (at least two
 // grids): FP32 where the pair kernel serves every grid (all 16-byte aligned at one
 // stride, so T0 and the first two grids decide).
 static bool states_pairs(unsigned flags, int dtype, int nt, Grid3 g, const void *T0, const void *grid0,
                          const void *grid1, const void *Ci) {
-    return (flags & PS_RUN_TEMPORAL2) && dtype == PS_F32 && nt >= 2 && temporal2_ok(g, dtype, T0, grid0, Ci) &&
-           temporal2_ok(g, dtype, grid0, grid1, Ci);
+    return (flags & PS_RUN_TEMPORAL2) && dtype == PS_F32 && nt >= 2 && temporal2_ok(g, dtype, T0, grid0, Ci, true) &&
+           temporal2_ok(g, dtype, grid0, grid1, Ci, true);
 }
 
 static cudaError_t enqueue_run_states(const void *T0, char *base, int64_t grid_stride, size_t esz, int every,
@@ -525,24 +537,20 @@ static cudaError_t enqueue_run_states(const void *T0, char *base, int64_t grid_s
     const int nslots = nt / every, nwork = (every > 1 && nt > 0) ? 2 : 0;
     auto grid = [&](int slot) { return (void *)(base + (size_t)slot * (size_t)grid_stride * esz); };
     auto slot_grid = [&](int slot) { return slot >= 0 ? grid(slot) : grid(nslots + (-1 - slot)); };
-    // The boundary of every grid this call writes is T0's.  Where the z-march serves the
-    // steps they store the x and y faces themselves (in their coalesced row stores), so
-    // only the two z faces of each grid are copied here; else the whole boundary is.
-    const bool scaled = (flags & PS_RUN_CI_SCALED) != 0, native = (flags & PS_RUN_NATIVE_F64) != 0;
+    // The boundary of every grid this call writes is T0's.  The steps store the x and y faces
+    // themselves (beside their own row stores), so only the two z faces of each grid are
+    // copied here.
     const int ngrids = nslots + nwork;
-    bool steps_bnd = true;
-    for (int k = 0; k < ngrids && steps_bnd; ++k)
-        steps_bnd = step_writes_xy_boundary(dtype, scaled, native, c, g, grid(k), T0, Ci) &&
-                    step_writes_xy_boundary(dtype, scaled, native, c, g, grid(k), grid(k), Ci);
     // PS_RUN_TEMPORAL2 (FP32): fused pairs.  With every = 1 they keep both states and
     // store both states' x and y faces; with every > 1 they keep only their second state
     // and write interior nodes only, so the whole boundary is copied then.
     const bool pairs = ngrids >= 2 && states_pairs(flags, dtype, nt, g, T0, grid(0), grid(1), Ci);
-    const bool faces_by_steps = steps_bnd && !(pairs && every > 1);
+    const bool faces_by_steps = !(pairs && every > 1);
     if (nt > 0 && ngrids > 0) {
         cudaError_t e = launch_copy_boundary_many(base, ngrids, grid_stride, T0, g, (int)esz, s, faces_by_steps);
         if (e != cudaSuccess) return e;
     }
+    const bool in_loop = states_column(dtype, g);
     std::vector<StatesOp> ops;
     plan_states(nt, every, pairs, &ops);
     const void *cur = T0;
@@ -555,7 +563,7 @@ static cudaError_t enqueue_run_states(const void *T0, char *base, int64_t grid_s
         else if (op.steps == 2)
             e = enqueue_step2(dst, cur, Ci, c, g, dtype, s);
         else
-            e = enqueue_step(dst, cur, nullptr, nullptr, Ci, c, g, dtype, flags, s, faces_by_steps);
+            e = enqueue_step(dst, cur, nullptr, nullptr, Ci, c, g, dtype, flags, s, in_loop, faces_by_steps);
         if (e != cudaSuccess) return e;
         cur = dst;
     }

@@ -1,15 +1,27 @@
 // Plain 7-point step kernels: one thread per interior (i, j) column,
 // marching along z with a three-value register queue.  x/y neighbours are
-// read through the L1/L2 caches.  These are the straightforward kernels
-// (FP64 instructions for FP64 data); the tiled kernels replace them on the
-// hot path.
+// read through the L1/L2 caches.
+//
+// They serve two kinds of grid.  Small ones inside a time loop (step_small, zmarch.cu): a
+// march of 1 .. 16 planes per thread keeps a step at a few memory round trips, where the TMA
+// z-march waits for 8 planes of copies one after the other.  Measured, us a step in a
+// captured loop (march as it was / this): FP64 pre-scaled 32^3 7.4 / 1.5, 64^3 7.4 / 3.0, 96^3
+// 8.9 / 6.1, 128^3 14.8 / 10.4, 192^3 41 / 39, 208^3 48 / 52; FP32 32^3 4.2 / 1.5, 64^3
+// 4.3 / 2.2, 96^3 4.4 / 3.6, 160^3 10.9 / 8.8, 192^3 14.3 / 13.7, 208^3 19 / 22.  And grids
+// that the march cannot take (2^31 nodes and more on ragged rows, spacings more than 16
+// apart on odd nx, plain FP64, the two-float step on ragged rows).
+// The next step's CTAs are let in at the end of the march, not at its start: with one wave of
+// CTAs or less they would fill whatever slots are free and leave the SMs unevenly loaded
+// (FP32 160 x 63 x 311: 9.0 us against 7.5).
 #pragma once
 
 #include <cuda_runtime.h>
 #include <cstdint>
 
 #include "emu64.cuh"
+#include "internal.h"
 #include "node.cuh"
+#include "pdl.cuh"
 
 namespace psd {
 
@@ -18,13 +30,38 @@ struct CoefT {
     F dtlam, ax, ay, az;
 };
 
-// Same column march for FP64 data with the one-DFMA emulated arithmetic of
-// emu64.cuh (used when the TMA kernel cannot serve the grid, e.g. odd nx).
-template <int kAx, bool kScaled>
+// kBnd: the columns beside the x and y faces store T's boundary values of the planes [k0, k1)
+// they have marched (the corners by the column in the corner).  A loop of its own: inside the
+// march it held registers the arithmetic needs (spills at 64).
+template <typename F>
+__device__ __forceinline__ void column_boundary(F *__restrict__ T2, const F *__restrict__ T, int64_t i, int64_t j,
+                                                int64_t k0, int64_t k1, int64_t nx, int64_t ny) {
+    const bool l = i == 1, r = i == nx - 2, d = j == 1, u = j == ny - 2;
+    if (!(l || r || d || u)) return;
+#pragma unroll 1
+    for (int64_t k = k0; k < k1; ++k) {
+        const int64_t p = i + nx * (j + ny * k);
+        auto put = [&](bool on, int64_t q) {
+            if (on) T2[q] = T[q];
+        };
+        put(l, p - 1);
+        put(r, p + 1);
+        put(d, p - nx);
+        put(u, p + nx);
+        put(l && d, p - nx - 1);
+        put(r && d, p - nx + 1);
+        put(l && u, p + nx - 1);
+        put(r && u, p + nx + 1);
+    }
+}
+
+// FP64 data with the one-DFMA emulated arithmetic of emu64.cuh.
+template <int kAx, bool kScaled, bool kBnd>
 __global__ void __launch_bounds__(256)
 k_step_basic_emu(double *__restrict__ T2, const double *__restrict__ T,
                  const double *__restrict__ Ci, EmuCoef c, int64_t nx, int64_t ny, int64_t nz,
                  int kchunk) {
+    grid_dep_wait();  // the previous step's writes (and its reads of T2) are complete
     const int64_t i = 1 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t j = 1 + (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
     if (i > nx - 2 || j > ny - 2) return;
@@ -45,39 +82,20 @@ k_step_basic_emu(double *__restrict__ T2, const double *__restrict__ T,
         tm = tc;
         tc = tp;
     }
-}
-
-inline cudaError_t launch_step_basic_emu(double *T2, const double *T, const double *Ci,
-                                         const EmuCoef &c, bool iso, int64_t nx, int64_t ny,
-                                         int64_t nz, int nsm, cudaStream_t s, bool scaled = false) {
-    const dim3 block(32, 8, 1);
-    const int64_t gx = (nx - 2 + block.x - 1) / block.x, gy = (ny - 2 + block.y - 1) / block.y;
-    int64_t want = (8LL * nsm + gx * gy - 1) / (gx * gy);
-    int64_t kchunk = (nz - 2 + want - 1) / want;
-    if (kchunk < 16) kchunk = 16;
-    const int64_t gz = (nz - 2 + kchunk - 1) / kchunk;
-    if (gx > 0x7fffffff || gy > 65535 || gz > 65535) return cudaErrorInvalidConfiguration;
-    const dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)gz);
-    if (scaled)
-        k_step_basic_emu<AX_ISO, true><<<grid, block, 0, s>>>(T2, T, Ci, c, nx, ny, nz, (int)kchunk);
-    else if (iso)
-        k_step_basic_emu<AX_ISO, false><<<grid, block, 0, s>>>(T2, T, Ci, c, nx, ny, nz, (int)kchunk);
-    else if (c.common)
-        k_step_basic_emu<AX_COMMON, false><<<grid, block, 0, s>>>(T2, T, Ci, c, nx, ny, nz, (int)kchunk);
-    else
-        k_step_basic_emu<AX_FAR, false><<<grid, block, 0, s>>>(T2, T, Ci, c, nx, ny, nz, (int)kchunk);
-    return cudaGetLastError();
+    grid_dep_launch();
+    if constexpr (kBnd) column_boundary(T2, T, i, j, k0, k1, nx, ny);
 }
 
 // Fig. 1 step!: T2 = T + dt*lam*Ci*((d2x*_dx^2 + d2y*_dy^2) + d2z*_dz^2) at
-// interior nodes; the z-range of this block is [k0, k1).  kComp (FP32): the state
-// is the two-float pair (T, E) and (T2, E2) receives the compensated step
-// (comp32_node, node.cuh).
-template <typename F, bool kComp>
+// interior nodes; the z-range of this block is [k0, k1).  FP32: f32_node's roundings.
+// kComp (FP32): the state is the two-float pair (T, E) and (T2, E2) receives the
+// compensated step (comp32_node, node.cuh).
+template <typename F, bool kComp, bool kBnd>
 __global__ void __launch_bounds__(256)
 k_step_basic(F *__restrict__ T2, const F *__restrict__ T, F *__restrict__ E2,
              const F *__restrict__ E, const F *__restrict__ Ci, CoefT<F> c, int64_t nx, int64_t ny,
              int64_t nz, int kchunk) {
+    grid_dep_wait();
     const int64_t i = 1 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t j = 1 + (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
     if (i > nx - 2 || j > ny - 2) return;
@@ -95,6 +113,9 @@ k_step_basic(F *__restrict__ T2, const F *__restrict__ T, F *__restrict__ E2,
                                 E[p + 1], E[p - sy], E[p + sy], E[p - sz], E[p + sz], Ci[p], c.dtlam,
                                 c.ax, c.ay, c.az, &e2);
             E2[p] = e2;
+        } else if constexpr (sizeof(F) == 4) {
+            T2[p] = f32_node(tc, T[p - 1], T[p + 1], T[p - sy], T[p + sy], tm, tp, Ci[p], c.dtlam, c.ax, c.ay,
+                             c.az);
         } else {
             const F d2x = (T[p + 1] - tc) - (tc - T[p - 1]);
             const F d2y = (T[p + sy] - tc) - (tc - T[p - sy]);
@@ -105,22 +126,71 @@ k_step_basic(F *__restrict__ T2, const F *__restrict__ T, F *__restrict__ E2,
         tm = tc;
         tc = tp;
     }
+    grid_dep_launch();
+    if constexpr (kBnd) column_boundary(T2, T, i, j, k0, k1, nx, ny);
+}
+
+// Launch shape of the column kernels: 32 x 8 columns per CTA and kchunk planes.  false: the
+// grid does not fit a launch.
+inline bool column_shape(int64_t nx, int64_t ny, int64_t nz, bool f32, bool small, dim3 *grid, int *kchunk) {
+    const int64_t gx = (nx - 2 + 31) / 32, gy = (ny - 2 + 7) / 8;
+    // about 8 blocks per SM, each chunk at least 16 planes
+    const int64_t want = (8LL * sm_count() + gx * gy - 1) / (gx * gy);
+    int64_t kc = (nz - 2 + want - 1) / want;
+    if (kc < 16) kc = 16;
+    if (small) {
+        // FP64 and the two-float step: about eight CTAs per SM, 1 to 8 planes.  FP32: the
+        // planes of a chunk are loaded four at a time (the compiler's unrolling), so 4, 8 or
+        // the long chunks, and 1 where even that leaves SMs idle.  Sweeps at 32^3 .. 192^3:
+        // within 10% of the best chunk at each.
+        const int64_t planes = gx * gy * (nz - 2);  // CTAs at one plane each
+        if (f32) {
+            const double r = (double)planes / (2.0 * sm_count());
+            if (r < 17.0) kc = r < 1.0 ? 1 : (r < 6.0 ? 4 : 8);
+        } else {
+            kc = planes / (8LL * sm_count());
+            kc = kc < 1 ? 1 : (kc > 8 ? 8 : kc);
+        }
+    }
+    const int64_t gz = (nz - 2 + kc - 1) / kc;
+    if (gx > 0x7fffffff || gy > 65535 || gz > 65535) return false;
+    *grid = dim3((unsigned)gx, (unsigned)gy, (unsigned)gz);
+    *kchunk = (int)kc;
+    return true;
+}
+
+template <int kAx, bool kScaled>
+inline cudaError_t launch_basic_emu_t(double *T2, const double *T, const double *Ci, const EmuCoef &c, Grid3 g,
+                                      cudaStream_t s, bool write_bnd, bool small) {
+    dim3 grid;
+    int kc;
+    if (!column_shape(g.nx, g.ny, g.nz, false, small, &grid, &kc)) return cudaErrorInvalidConfiguration;
+    if (write_bnd)
+        return launch_pdl(k_step_basic_emu<kAx, kScaled, true>, grid, dim3(32, 8), 0, s, T2, T, Ci, c, g.nx, g.ny,
+                          g.nz, kc);
+    return launch_pdl(k_step_basic_emu<kAx, kScaled, false>, grid, dim3(32, 8), 0, s, T2, T, Ci, c, g.nx, g.ny,
+                      g.nz, kc);
+}
+
+inline cudaError_t launch_step_basic_emu(double *T2, const double *T, const double *Ci, const EmuCoef &c, bool iso,
+                                         Grid3 g, cudaStream_t s, bool scaled, bool write_bnd, bool small) {
+    if (scaled) return launch_basic_emu_t<AX_ISO, true>(T2, T, Ci, c, g, s, write_bnd, small);
+    if (iso) return launch_basic_emu_t<AX_ISO, false>(T2, T, Ci, c, g, s, write_bnd, small);
+    if (c.common) return launch_basic_emu_t<AX_COMMON, false>(T2, T, Ci, c, g, s, write_bnd, small);
+    return launch_basic_emu_t<AX_FAR, false>(T2, T, Ci, c, g, s, write_bnd, small);
 }
 
 template <typename F, bool kComp>
-cudaError_t launch_step_basic(F *T2, const F *T, F *E2, const F *E, const F *Ci, CoefT<F> c, int64_t nx,
-                              int64_t ny, int64_t nz, int nsm, cudaStream_t s) {
-    const dim3 block(32, 8, 1);
-    const int64_t gx = (nx - 2 + block.x - 1) / block.x, gy = (ny - 2 + block.y - 1) / block.y;
-    // enough z-chunks for about 8 blocks per SM, each chunk at least 16 planes
-    int64_t want = (8LL * nsm + gx * gy - 1) / (gx * gy);
-    int64_t kchunk = (nz - 2 + want - 1) / want;
-    if (kchunk < 16) kchunk = 16;
-    const int64_t gz = (nz - 2 + kchunk - 1) / kchunk;
-    if (gx > 0x7fffffff || gy > 65535 || gz > 65535) return cudaErrorInvalidConfiguration;
-    k_step_basic<F, kComp><<<dim3((unsigned)gx, (unsigned)gy, (unsigned)gz), block, 0, s>>>(
-        T2, T, E2, E, Ci, c, nx, ny, nz, (int)kchunk);
-    return cudaGetLastError();
+cudaError_t launch_step_basic(F *T2, const F *T, F *E2, const F *E, const F *Ci, CoefT<F> c, Grid3 g,
+                              cudaStream_t s, bool write_bnd, bool small) {
+    dim3 grid;
+    int kc;
+    if (!column_shape(g.nx, g.ny, g.nz, sizeof(F) == 4 && !kComp, small, &grid, &kc)) return cudaErrorInvalidConfiguration;
+    if (!kComp && write_bnd)
+        return launch_pdl(k_step_basic<F, kComp, !kComp>, grid, dim3(32, 8), 0, s, T2, T, E2, E, Ci, c, g.nx, g.ny,
+                          g.nz, kc);
+    return launch_pdl(k_step_basic<F, kComp, false>, grid, dim3(32, 8), 0, s, T2, T, E2, E, Ci, c, g.nx, g.ny, g.nz,
+                      kc);
 }
 
 }  // namespace psd

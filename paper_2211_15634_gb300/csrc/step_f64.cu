@@ -1,6 +1,8 @@
 // FP64 forward step dispatch.
-//   fast:   TMA z-march with one-DFMA emulated arithmetic (even nx), else the
-//           plain column march with the same arithmetic;
+//   fast:   TMA z-march with one-DFMA emulated arithmetic (even nx), its row-by-row form
+//           (odd nx below 2^31 nodes, spacings within 16 of each other), else the plain
+//           column march with the same arithmetic;
+//           Small grids inside a time loop take the column march (stencil_basic.cuh).
 //   native: plain column march with ordinary FP64 instructions.
 #include "internal.h"
 #include "stencil_basic.cuh"
@@ -11,9 +13,8 @@ namespace psd {
 static CoefT<double> coef_f64(StepCoef c) { return CoefT<double>{c.dtlam, c.ax, c.ay, c.az}; }
 
 cudaError_t launch_step_f64_native(double *T2, const double *T, const double *Ci, StepCoef c,
-                                   Grid3 g, cudaStream_t s) {
-    return launch_step_basic<double, false>(T2, T, nullptr, nullptr, Ci, coef_f64(c), g.nx, g.ny, g.nz,
-                                            sm_count(), s);
+                                   Grid3 g, cudaStream_t s, bool write_bnd) {
+    return launch_step_basic<double, false>(T2, T, nullptr, nullptr, Ci, coef_f64(c), g, s, write_bnd, false);
 }
 
 bool emu_ok(StepCoef c) {
@@ -24,43 +25,46 @@ bool emu_ok(StepCoef c) {
 }
 
 cudaError_t launch_step_f64_fast(double *T2, const double *T, const double *Ci, StepCoef c,
-                                 Grid3 g, cudaStream_t s, bool write_bnd) {
-    if (!emu_ok(c)) return launch_step_f64_native(T2, T, Ci, c, g, s);
+                                 Grid3 g, cudaStream_t s, bool write_bnd, bool in_loop) {
+    if (!emu_ok(c)) return launch_step_f64_native(T2, T, Ci, c, g, s, write_bnd);
     const bool iso = c.ax == c.ay && c.ay == c.az;
+    const EmuCoef ek = emu_coef(c.dtlam, c.ax, c.ay, c.az);
+    // equal spacings keep the march: its one-binade form multiplies Ci by K first, which
+    // rounds another way than the column kernel's K*S
+    if (in_loop && !iso && step_small(g, Z_F64_EMU_ANISO)) return launch_step_basic_emu(T2, T, Ci, ek, iso, g, s, false, write_bnd, true);
     if (step_tma_ok(g, 8, T2, T, Ci))
         return launch_zmarch(iso ? Z_F64_EMU_ISO : Z_F64_EMU_ANISO, T2, T, nullptr, nullptr, Ci, c, g, s,
                              write_bnd);
-    const EmuCoef ek = emu_coef(c.dtlam, c.ax, c.ay, c.az);
-    return launch_step_basic_emu(T2, T, Ci, ek, iso, g.nx, g.ny, g.nz, sm_count(), s);
+    if (ek.common && step_ragged_ok(g, 8, T2, T, Ci))
+        return launch_zmarch_ragged(iso ? Z_F64_EMU_ISO_DMUL : Z_F64_EMU_ANISO, T2, T, Ci, c, g, s, write_bnd);
+    return launch_step_basic_emu(T2, T, Ci, ek, iso, g, s, false, write_bnd, false);
 }
 
 // Ci already scaled to dt*lam*_dx^2*Ci (isotropic grids): one DFMA per node.
 cudaError_t launch_step_f64_scaled(double *T2, const double *T, const double *Cs, Grid3 g,
-                                   cudaStream_t s, bool write_bnd) {
+                                   cudaStream_t s, bool write_bnd, bool in_loop) {
     const StepCoef dummy{1.0, 1.0, 1.0, 1.0};
+    const EmuCoef ek{};
+    if (in_loop && step_small(g, Z_F64_SCALED)) return launch_step_basic_emu(T2, T, Cs, ek, true, g, s, true, write_bnd, true);
     if (step_tma_ok(g, 8, T2, T, Cs))
         return launch_zmarch(Z_F64_SCALED, T2, T, nullptr, nullptr, Cs, dummy, g, s, write_bnd);
-    const EmuCoef ek{};
-    return launch_step_basic_emu(T2, T, Cs, ek, true, g.nx, g.ny, g.nz, sm_count(), s, true);
-}
-
-bool step_writes_xy_boundary(int dtype, bool scaled, bool native, StepCoef c, Grid3 g, const void *T2,
-                             const void *T, const void *Ci) {
-    if (dtype != PS_F64) return step_tma_ok(g, 4, T2, T, Ci);  // launch_step_f32
-    if (scaled) return step_tma_ok(g, 8, T2, T, Ci);           // launch_step_f64_scaled
-    if (native || !emu_ok(c)) return false;                     // the plain column kernel
-    return step_tma_ok(g, 8, T2, T, Ci);                        // launch_step_f64_fast
+    if (step_ragged_ok(g, 8, T2, T, Cs))
+        return launch_zmarch_ragged(Z_F64_SCALED, T2, T, Cs, dummy, g, s, write_bnd);
+    return launch_step_basic_emu(T2, T, Cs, ek, true, g, s, true, write_bnd, false);
 }
 
 const char *step_f64_kernel_name(Grid3 g, const void *T2, const void *T, const void *Ci, StepCoef c,
                                  bool scaled) {
     if (scaled) {
+        if (step_ragged_ok(g, 8, T2, T, Ci)) return "k_zmarch_rag<F64_SCALED>";
         if (!step_tma_ok(g, 8, T2, T, Ci)) return "k_step_basic_emu";
         return f64_scaled_wide(g, T2, T, Ci) ? "k_zmarch<F64_SCALED4>" : "k_zmarch<F64_SCALED>";
     }
     if (!emu_ok(c)) return "k_step_basic<double>";
     const bool iso = c.ax == c.ay && c.ay == c.az;
     if (step_tma_ok(g, 8, T2, T, Ci)) return iso ? "k_zmarch<F64_EMU_ISO>" : "k_zmarch<F64_EMU_ANISO>";
+    if (emu_coef(c.dtlam, c.ax, c.ay, c.az).common && step_ragged_ok(g, 8, T2, T, Ci))
+        return iso ? "k_zmarch_rag<F64_EMU_ISO>" : "k_zmarch_rag<F64_EMU_ANISO>";
     return "k_step_basic_emu";
 }
 

@@ -18,6 +18,7 @@
 #include "tma.cuh"
 #include "zmarch.h"
 #include "zmarch_tile.cuh"
+#include "zrag_tile.cuh"
 
 namespace psd {
 
@@ -35,6 +36,20 @@ k_zmarch(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtens
     const int k0 = 1 + (int)blockIdx.y * p.kchunk;
     const int k1 = (int)min((int64_t)k0 + p.kchunk, p.nz - 1);  // output planes [k0, k1)
     zmarch_tile<MODE, BY, NST, 32, kBnd>(&tmT, &tmC, T2v, E2v, p, X0, Y0, k0, k1, &g_zmarch_error, &tmE);
+}
+
+// The same on ragged rows (zrag_tile.cuh).
+template <int MODE, int PX, int BY, int NST, int MINB, bool kBnd>
+__global__ void __launch_bounds__(32 * BY, MINB)
+k_zmarch_rag(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmC,
+             void *__restrict__ T2v, const ZParams p) {
+    grid_dep_wait();
+    grid_dep_launch();
+    const int X0 = 1 + (int)(blockIdx.x % p.ntx) * (32 * PX);
+    const int Y0 = 1 + (int)(blockIdx.x / p.ntx) * BY;
+    const int k0 = 1 + (int)blockIdx.y * p.kchunk;
+    const int k1 = (int)min((int64_t)k0 + p.kchunk, p.nz - 1);
+    zrag_tile<MODE, PX, BY, NST, kBnd>(&tmT, &tmC, T2v, p, X0, Y0, k0, k1, &g_zmarch_error);
 }
 
 // Failure-path self-test: one CTA waits on an mbarrier that nothing ever arrives on.
@@ -91,6 +106,31 @@ bool make_tensor_map_3d_pitch(CUtensorMap *m, const void *ptr, int esz, Grid3 g,
     return r == CUDA_SUCCESS;
 }
 
+bool make_tensor_map_rows(CUtensorMap *m, const void *ptr, int esz, int64_t n, int64_t rowlen, unsigned bx,
+                          unsigned by) {
+    auto fn = encode_fn();
+    if (!fn) return false;
+    const bool line = by == 0;  // one line of n elements
+    const cuuint64_t dims[2] = {(cuuint64_t)(line ? n : rowlen), (cuuint64_t)(line ? 1 : n / rowlen)};
+    const cuuint64_t strides[1] = {line ? 0 : (cuuint64_t)(rowlen * esz)};
+    const cuuint32_t box[2] = {bx, line ? 1u : by}, estr[2] = {1, 1};
+    const CUresult r = fn(m, esz == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
+                          line ? 1 : 2, const_cast<void *>(ptr), dims, strides, box, estr,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS;
+}
+
+bool ragged_supported(Grid3 g, const void *a, const void *b, const void *c) {
+    if (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c) & 15u) return false;
+    // element coordinates of planes -1 .. nz, tiles past the grid included, fit 32 bits
+    // (FP32; FP64's row-pair coordinates then do)
+    if (g.nx > (1LL << 30) || g.ny > (1LL << 30)) return false;
+    const double plane = (double)g.nx * ((double)g.ny + 64.0);
+    if (plane * ((double)g.nz + 2.0) + 4096.0 >= 2147483647.0) return false;
+    return encode_fn() != nullptr;
+}
+
 bool zmarch_supported(Grid3 g, int esz, const void *a, const void *b, const void *c) {
     if ((g.nx * esz) % 16 != 0) return false;
     if (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c) & 15u) return false;
@@ -98,8 +138,61 @@ bool zmarch_supported(Grid3 g, int esz, const void *a, const void *b, const void
     return encode_fn() != nullptr;
 }
 
+bool step_small(Grid3 g, int mode) {
+    // a set z-chunk or nodes-per-thread override asks for the march
+    if (launch_override(PS_OVERRIDE_KCHUNK) > 0 || launch_override(PS_OVERRIDE_F64_PX2) == 1) return false;
+    const double n = (double)g.nx * (double)g.ny * (double)g.nz;
+    // The line lies where the march catches up (us a step, column / march).
+    const bool aligned = (g.nx * (mode == Z_F32 || mode == Z_F32_COMP ? 4 : 8)) % 16 == 0;
+    // rows that fill the march's 128-node tiles by 77% or more favour it
+    const bool full = (double)g.nx >= 0.77 * 128.0 * (double)((g.nx + 127) / 128);
+    switch (mode) {
+        case Z_F32:  // full rows 5e5 nodes 3.0 / 2.9, 1e6 4.1 / 3.7; 192^3 13.1 / 14.3, 200^3 16 / 16;
+                     // ragged 205^3 20.8 / 21.7, 211^3 25.5 / 23.8
+            return n <= (aligned ? (full ? 6e5 : 7.5e6) : 8.8e6);
+        case Z_F32_COMP:  // 160^3 14 / 19, 176^3 25 / 25; ragged rows have no march: only the
+                          // column kernel's chunks differ (343 x 96 x 95: 12.0 us, long ones 11.6)
+            return n <= (aligned ? 4.3e6 : 2.5e6);
+        case Z_F64_EMU_ANISO:  // 192^3 37 / 41, 200^3 53 / 49; ragged 219^3 61 / 64, 227^3 71 / 69
+            return n <= (aligned ? 7.5e6 : 1.05e7);
+        default: {
+            // by the share of useful lanes in the march's 64-node tiles (four nodes per thread:
+            // where as good): 128 x 321 x 75 (1) 23 / 21, 128^3 (1) 10 / 15; 160^3 (0.83) 21 / 24,
+            // 176^3 (0.92) 32 / 29; 200^3 (0.78) 50 / 45
+            const double lanes = aligned ? (double)g.nx / (64.0 * (double)((g.nx + 63) / 64))
+                                         : (double)(g.nx - 2) / (64.0 * (double)((g.nx - 2 + 63) / 64));
+            return n <= (lanes >= 0.87 ? 2.2e6 : (lanes >= 0.8 ? 4.3e6 : 7.5e6));
+        }
+    }
+}
+
+bool step_ragged_ok(Grid3 g, int esz, const void *a, const void *b, const void *c) {
+    if (launch_override(PS_OVERRIDE_STEP_PLAIN) == 1 || (g.nx * esz) % 16 == 0) return false;
+    // FP32 rows that leave more than 40% of its 128-node tiles idle: the column kernel is as
+    // fast (151 x 367 x 271, 0.58 in use: 44.5 us a step here, 43.6 there)
+    if (esz == 4 && (double)(g.nx - 2) < 0.6 * 128.0 * (double)((g.nx - 2 + 127) / 128) &&
+        launch_override(PS_OVERRIDE_KCHUNK) <= 0)
+        return false;
+    return ragged_supported(g, a, b, c);
+}
+
 bool step_tma_ok(Grid3 g, int esz, const void *a, const void *b, const void *c) {
     return launch_override(PS_OVERRIDE_STEP_PLAIN) != 1 && zmarch_supported(g, esz, a, b, c);
+}
+
+// Planes per CTA of the one-step march.
+static int step_kchunk(int esz, Grid3 g, int64_t tiles) {
+    // Short chunks keep many CTAs in flight (no wave tail) while consecutive
+    // CTAs - neighbouring tiles of one chunk - share their halo planes in L2;
+    // each chunk pays two extra planes.  Measured (sweeps at 256^3 and 512^3):
+    // FP32 is fastest at 8 planes; FP64 at 8 planes on small grids and flat from
+    // 24 to 40 planes at 512^3, so about 64 CTAs per SM between 8 and 32 planes.
+    // FP32 grids up to 3 million nodes (a few CTAs per SM): 3 planes (128^3 5.1 against 5.6 us).
+    if (esz == 4 && (double)g.nx * (double)g.ny * (double)g.nz <= 3e6) return 3;
+    const int64_t target = 64LL * sm_count();
+    const int64_t kmax = esz == 8 ? 32 : 8;
+    const int64_t kc = (g.nz - 2) * tiles / target;
+    return (int)(kc < 8 ? 8 : (kc > kmax ? kmax : kc));
 }
 
 template <int MODE, int BY, int NST, bool kBnd = false>
@@ -125,17 +218,7 @@ static cudaError_t launch_zmarch_t(void *T2, const void *T, void *E2, const void
     }
     const int64_t ntx = (g.nx + BX - 1) / BX, nty = (g.ny + BY - 1) / BY;
     const int64_t tiles = ntx * nty;
-    if (kchunk <= 0) {
-        // Short chunks keep many CTAs in flight (no wave tail) while consecutive
-        // CTAs - neighbouring tiles of one chunk - share their halo planes in L2;
-        // each chunk pays two extra planes.  Measured (sweeps at 256^3 and 512^3):
-        // FP32 is fastest at 8 planes; FP64 at 8 planes on small grids and flat from
-        // 24 to 40 planes at 512^3, so about 64 CTAs per SM between 8 and 32 planes.
-        const int64_t target = 64LL * sm_count();
-        const int64_t kmax = sizeof(E) == 8 ? 32 : 8;
-        int64_t kc = (g.nz - 2) * tiles / target;
-        kchunk = (int)(kc < 8 ? 8 : (kc > kmax ? kmax : kc));
-    }
+    if (kchunk <= 0) kchunk = step_kchunk(sizeof(E), g, tiles);
     const int64_t gz = (g.nz - 2 + kchunk - 1) / kchunk;
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
     p.nx = g.nx;
@@ -162,6 +245,10 @@ bool tma_encoder_available() { return encode_fn() != nullptr; }
 
 bool f64_scaled_wide(Grid3 g, const void *T2, const void *T, const void *Ci) {
     if (launch_override(PS_OVERRIDE_F64_PX2) == 1) return false;
+    // 128-node tiles, unless 64-node ones leave fewer lanes past the row's end (us a step, four
+    // / two per thread: 192^3 41 / 34, 320^3 150 / 132, 448^3 357 / 330; equal widths 256^3 71 /
+    // 71, 384^3 212 / 216).  Below a million nodes the launch counts, not the lanes.
+    if (64 * ((g.nx + 63) / 64) < 128 * ((g.nx + 127) / 128) && (double)g.n() >= 1e6) return false;
     return g.nx % 4 == 0 && ((((uintptr_t)T2 | (uintptr_t)T | (uintptr_t)Ci) & 31u) == 0);
 }
 
@@ -182,6 +269,58 @@ static cudaError_t launch_zmarch_b(void *T2, const void *T, void *E2, const void
     if (MODE != Z_F32_COMP && write_bnd)
         return launch_zmarch_t<MODE, BY, NST, MODE != Z_F32_COMP>(T2, T, E2, Ein, Ci, g, p, kchunk, s);
     return launch_zmarch_t<MODE, BY, NST, false>(T2, T, E2, Ein, Ci, g, p, kchunk, s);
+}
+
+template <int MODE, int PX, int BY, int MINB, bool kBnd>
+static cudaError_t launch_rag_t(void *T2, const void *T, const void *Ci, Grid3 g, ZParams p, cudaStream_t s) {
+    constexpr int NST = 4;
+    using R = ZRag<MODE, PX, BY>;
+    using E = typename R::E;
+    constexpr size_t smem = NST * R::SB + NST * 8;
+    static unsigned attr_gen[64] = {0};
+    cudaError_t ae;
+    if (!set_smem_attr_once((const void *)k_zmarch_rag<MODE, PX, BY, NST, MINB, kBnd>, (int)smem, attr_gen, &ae))
+        return ae;
+    CUtensorMap mT, mC;
+    if (!make_tensor_map_rows(&mT, T, sizeof(E), g.n(), 2 * g.nx, R::W, R::kPairs ? R::H / 2 : 0) ||
+        !make_tensor_map_rows(&mC, Ci, sizeof(E), g.n(), 2 * g.nx, R::W, R::kPairs ? BY / 2 : 0))
+        return cudaErrorInvalidValue;
+    const int64_t ntx = (g.nx - 2 + R::BX - 1) / R::BX, nty = (g.ny - 2 + BY - 1) / BY, tiles = ntx * nty;
+    int kchunk = launch_override(PS_OVERRIDE_KCHUNK);
+    if (kchunk <= 0) kchunk = step_kchunk(sizeof(E), g, tiles);
+    const int64_t gz = (g.nz - 2 + kchunk - 1) / kchunk;
+    if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
+    p.nx = g.nx;
+    p.ny = g.ny;
+    p.nz = g.nz;
+    p.pitch = g.nx;
+    p.ntx = (int)ntx;
+    p.kchunk = kchunk;
+    return launch_pdl(k_zmarch_rag<MODE, PX, BY, NST, MINB, kBnd>, dim3((unsigned)tiles, (unsigned)gz, 1),
+                      dim3(32 * BY), smem, s, mT, mC, T2, p);
+}
+
+template <int MODE, int PX, int BY, int MINB>
+static cudaError_t launch_rag_b(void *T2, const void *T, const void *Ci, Grid3 g, ZParams p, cudaStream_t s,
+                                bool write_bnd) {
+    if (write_bnd) return launch_rag_t<MODE, PX, BY, MINB, true>(T2, T, Ci, g, p, s);
+    return launch_rag_t<MODE, PX, BY, MINB, false>(T2, T, Ci, g, p, s);
+}
+
+cudaError_t launch_zmarch_ragged(int mode, void *T2, const void *T, const void *Ci, StepCoef c, Grid3 g,
+                                 cudaStream_t s, bool write_bnd) {
+    const ZParams p = make_params(c);
+    switch (mode) {
+        case Z_F64_EMU_ISO_DMUL:
+            return launch_rag_b<Z_F64_EMU_ISO_DMUL, 2, 8, 3>(T2, T, Ci, g, p, s, write_bnd);
+        case Z_F64_EMU_ANISO:
+            return launch_rag_b<Z_F64_EMU_ANISO, 2, 8, 3>(T2, T, Ci, g, p, s, write_bnd);
+        case Z_F64_SCALED:
+            return launch_rag_b<Z_F64_SCALED, 2, 8, 3>(T2, T, Ci, g, p, s, write_bnd);
+        case Z_F32:
+            return launch_rag_b<Z_F32, 4, 8, 4>(T2, T, Ci, g, p, s, write_bnd);
+    }
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_zmarch(int mode, void *T2, const void *T, void *E2, const void *Ein, const void *Ci,
@@ -208,7 +347,7 @@ cudaError_t launch_zmarch(int mode, void *T2, const void *T, void *E2, const voi
             return launch_zmarch_b<Z_F64_NATIVE, 8, 4>(T2, T, E2, Ein, Ci, g, p, kchunk, s, wb);
         case Z_F64_SCALED:
             // four nodes per thread (4-row tiles, 128 threads) where rows allow 32-byte
-            // accesses: measured 2-3% faster at 512^3 and 768^3 than two per thread
+            // accesses and fill its tiles (f64_scaled_wide): measured 2-3% faster at 512^3 and 768^3 than two per thread
             // (8-row tiles of four per thread, at two CTAs per SM, were 15% slower)
             if (f64_scaled_wide(g, T2, T, Ci))
                 return launch_zmarch_b<Z_F64_SCALED4, 4, 4>(T2, T, E2, Ein, Ci, g, p, kchunk, s, wb);

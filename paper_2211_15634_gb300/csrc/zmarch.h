@@ -32,6 +32,17 @@ struct ZParams {
 bool zmarch_supported(Grid3 g, int esz, const void *a, const void *b, const void *c);
 // The same for one forward step, unless PS_OVERRIDE_STEP_PLAIN asks for the plain kernel.
 bool step_tma_ok(Grid3 g, int esz, const void *a, const void *b, const void *c);
+// The same for rows that are no multiple of 16 bytes, staged row by row (zrag_tile.cuh): any
+// nx, fewer than 2^31 elements.
+bool ragged_supported(Grid3 g, const void *a, const void *b, const void *c);
+bool step_ragged_ok(Grid3 g, int esz, const void *a, const void *b, const void *c);
+// Map over n consecutive elements: rows of rowlen (a multiple of 16 bytes; a last part of a
+// row is left out) with a box of bx x by, or with by = 0 one line with a box of bx.
+bool make_tensor_map_rows(CUtensorMap *m, const void *ptr, int esz, int64_t n, int64_t rowlen, unsigned bx,
+                          unsigned by);
+// Grids whose steps inside a time loop take the column kernels (stencil_basic.cuh); mode:
+// Z_F32, Z_F32_COMP, Z_F64_SCALED or Z_F64_EMU_ANISO (any unequal spacings).
+bool step_small(Grid3 g, int mode);
 // 3-D tiled tensor map over a (nz, ny, nx) field with a bx x by x 1 box.
 bool make_tensor_map_3d(CUtensorMap *m, const void *ptr, int esz, Grid3 g, unsigned bx, unsigned by);
 // The same over a grid whose rows are `pitch` elements apart (pitch*esz a multiple of 16).
@@ -39,8 +50,8 @@ bool make_tensor_map_3d_pitch(CUtensorMap *m, const void *ptr, int esz, Grid3 g,
                               unsigned bx, unsigned by);
 // True when the driver's tensor-map encoder could be loaded (a GPU driver is present).
 bool tma_encoder_available();
-// Whether the pre-scaled FP64 step takes the four-nodes-per-thread kernel (rows of a
-// multiple of 32 bytes, 32-byte aligned fields; PS_F64_VARIANT=px2 turns it off).
+// Whether the pre-scaled FP64 step takes the four-nodes-per-thread kernel (rows of a multiple
+// of 32 bytes whose length suits its 128-node tiles, 32-byte aligned fields).
 bool f64_scaled_wide(Grid3 g, const void *T2, const void *T, const void *Ci);
 // Step parameters of the z-march kernels for coefficients c on grid g with row pitch `pitch`.
 ZParams zparams_for(StepCoef c, Grid3 g, int64_t pitch);
@@ -65,6 +76,10 @@ bool emu_ok(StepCoef c);
 // boundary nodes of planes 1 .. nz-2 as copies of T's (not with Z_F32_COMP).
 cudaError_t launch_zmarch(int mode, void *T2, const void *T, void *E2, const void *Ein, const void *Ci,
                           StepCoef c, Grid3 g, cudaStream_t s, bool write_bnd = false);
+// The same on ragged rows (mode: Z_F64_EMU_ISO_DMUL, Z_F64_EMU_ANISO, Z_F64_SCALED or Z_F32;
+// the caller has checked step_ragged_ok).
+cudaError_t launch_zmarch_ragged(int mode, void *T2, const void *T, const void *Ci, StepCoef c, Grid3 g,
+                                 cudaStream_t s, bool write_bnd = false);
 unsigned zmarch_device_error(bool clear);
 
 }  // namespace psd
