@@ -113,6 +113,12 @@ k_adjoint_basic_scaled(double *__restrict__ Tbar, double *__restrict__ Csbar,
     }
 }
 
+// Odd nx on the kernel of adjoint_scaled.cu (its row-pair form).
+static bool use_ragged_f64(Grid3 g, const void *a, const void *b, const void *c, const void *d, const void *e) {
+    return launch_override(PS_OVERRIDE_ADJ_PLAIN) != 1 && g.nx % 2 == 1 && ragged_supported(g, a, b, c) &&
+           ragged_supported(g, c, d, e);
+}
+
 static bool use_tma(Grid3 g, int esz, const void *a, const void *b, const void *c, const void *d,
                     const void *e) {
     const void *ptrs[5] = {c, d, e, a, b};  // the three TMA-read fields first
@@ -124,13 +130,17 @@ cudaError_t launch_adjoint_f64(double *Tbar, double *Cibar, const double *ybar, 
                                const double *Ci, StepCoef c, Grid3 g, cudaStream_t s) {
     if (use_tma(g, 8, Tbar, Cibar, ybar, T, Ci))
         return launch_adjoint_zmarch<double>(Tbar, Cibar, ybar, T, Ci, c, g, s);
+    if (emu_ok(c) && use_ragged_f64(g, Tbar, Cibar, ybar, T, Ci)) {
+        const EmuCoef ek = emu_coef(c.dtlam, c.ax, c.ay, c.az);
+        if (ek.common) return launch_adjoint_given(Tbar, Cibar, ybar, T, Ci, ek, g, s);
+    }
     return launch_adjoint_basic<double>(Tbar, Cibar, ybar, T, Ci,
                                         CoefT<double>{c.dtlam, c.ax, c.ay, c.az}, g, s);
 }
 
 cudaError_t launch_adjoint_f64_scaled(double *Tbar, double *Csbar, const double *ybar,
                                       const double *T, const double *Cs, Grid3 g, cudaStream_t s) {
-    if (use_tma(g, 8, Tbar, Csbar, ybar, T, Cs))
+    if (use_tma(g, 8, Tbar, Csbar, ybar, T, Cs) || use_ragged_f64(g, Tbar, Csbar, ybar, T, Cs))
         return launch_adjoint_scaled(Tbar, Csbar, ybar, T, Cs, g, s);
     const dim3 block(32, 8, 1);
     const int64_t gx = (g.nx + block.x - 1) / block.x, gy = (g.ny + block.y - 1) / block.y;

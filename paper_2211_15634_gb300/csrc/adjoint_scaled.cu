@@ -91,20 +91,28 @@ static __device__ __noinline__ double adjs_lap_general(unsigned long long c, uns
 // replaces the DADD, Cibar by one more DMUL); AX_COMMON, Ci as given on unequal spacings: w =
 // Ci*ybar, Tbar = ybar + L(w) and Cibar += ybar*L(T) with L = sum_d dt*lam*_d^2 * (second
 // difference along d), the axes' exact sums combined as integers (emu_L_common).
-template <int BY, int NST, int kAx, bool kGiven>
+// kRag: odd nx.  A plane of a field arrives as two boxes, its even and its odd tile rows, over
+// the field mapped as rows of 2*nx (zrag_tile.cuh); a row's data then starts at its slot's
+// first or second element, and lanes own nodes lane and lane + 32 of their row.  Measured
+// against the plain column kernel: 161 x 128 x 96 unequal 49 against 204 us, 257^3 pre-scaled
+// 248 against 735 (a fifth of that in the tiles of the one column past 256).
+template <int BY, int NST, int kAx, bool kGiven, bool kRag>
 __global__ void __launch_bounds__(32 * BY, 3)
 k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmY,
                  const __grid_constant__ CUtensorMap tmC, double *__restrict__ Tbar,
-                 double *__restrict__ Csbar, const AdjSParams p) {
+                 double *__restrict__ Csbar, const double *__restrict__ ybar, const AdjSParams p) {
     constexpr int PX = 2, HX = 2, BX = 64, W = BX + 2 * HX, H = BY + 2;
     constexpr int NHALO = 2 * BX + 2 * BY;  // y-halo rows and x-halo columns (no corners)
     static_assert(NHALO <= 32 * BY, "one halo value per thread at most");
     constexpr unsigned TB = W * H * 8;
-    constexpr unsigned TBA = (TB + 127) / 128 * 128, SS = TBA / 8;  // box stride in elements
+    constexpr unsigned WBA = (TB + 127) / 128 * 128, WS = WBA / 8;  // w tile stride
+    constexpr unsigned HBX = (TB / 2 + 127) / 128 * 128;             // box of even or odd rows
+    constexpr unsigned TBA = kRag ? 2 * HBX : WBA, SS = TBA / 8;     // field stride in elements
+    constexpr int XS = kRag ? 32 : 1;                                // between a lane's two nodes
     extern __shared__ __align__(128) unsigned char smem[];
     double *ring = (double *)smem;                       // NST stages x {T, ybar, Cs}
     long long *wtile = (long long *)(smem + 3 * NST * TBA);  // 3 rotating w tiles
-    uint64_t *bar = (uint64_t *)(smem + 3 * NST * TBA + 3 * TBA);
+    uint64_t *bar = (uint64_t *)(smem + 3 * NST * TBA + 3 * WBA);
     __shared__ int s_abort, s_E;
     grid_dep_wait();  // the previous launch's writes (and its reads of Tbar) are complete
     grid_dep_launch();
@@ -117,6 +125,21 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
 
     auto issue = [&](int s, int q) {
         mbar_expect_tx(&bar[s], 3 * TB);
+        if constexpr (kRag) {
+            // tile row h is field row r + h; o: the residue of row r, boxes of rows h = 0, 2, ..
+            // and h = 1, 3, ..; x from column -1 rounded down to an even element
+            const int64_t r = (int64_t)q * ny + Y0 - 1;
+            const int o = (int)(r & 1), g0 = (int)(r >> 1), g1 = (int)((r + 1) >> 1);
+            const int x0 = (o * nx + X0 - 1) & ~1, x1 = ((o ^ 1) * nx + X0 - 1) & ~1;
+            const CUtensorMap *tm[3] = {&tmT, &tmY, &tmC};
+#pragma unroll
+            for (int f = 0; f < 3; ++f) {
+                unsigned char *dst = (unsigned char *)(ring + (3 * s + f) * SS);
+                tma_load_2d(dst, tm[f], &bar[s], x0, g0);
+                tma_load_2d(dst + HBX, tm[f], &bar[s], x1, g1);
+            }
+            return;
+        }
         tma_load_3d(ring + (3 * s + 0) * SS, &tmT, &bar[s], X0 - HX, Y0 - 1, q);
         tma_load_3d(ring + (3 * s + 1) * SS, &tmY, &bar[s], X0 - HX, Y0 - 1, q);
         tma_load_3d(ring + (3 * s + 2) * SS, &tmC, &bar[s], X0 - HX, Y0 - 1, q);
@@ -148,12 +171,27 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
         return mbar_wait(&bar[s], ph);
     };
 
-    // this thread's own nodes (row, col .. col+1 of the tile) and halo node
-    const int row = ty + 1, col = HX + lane * PX;
-    const int gy = Y0 + ty, gx0 = X0 + lane * PX;
+    // this thread's own nodes (row, col and col + XS of the tile) and halo node
+    const int row = ty + 1, col = HX + (kRag ? lane : lane * PX);
+    const int gy = Y0 + ty, gx0 = X0 + (kRag ? lane : lane * PX);
     const bool iny = gy >= 1 && gy <= ny - 2;
     const bool m0 = iny && gx0 >= 1 && gx0 <= nx - 2;
-    const bool m1 = iny && gx0 + 1 >= 1 && gx0 + 1 <= nx - 2;
+    const bool m1 = iny && gx0 + XS >= 1 && gx0 + XS <= nx - 2;
+    // position of tile row r, column c (the w tile's columns, node x = X0 - HX + c) in a field
+    // of plane q.  kRag: row r of the field's even or odd box, shifted by the row's offset
+    // d = (row * nx + X0 - 1) mod 2 = (row + 1) mod 2 (odd nx, even X0)
+    auto at = [&](int r, int c, int q) -> int {
+        if (!kRag) return r * W + c;
+        const int d = (q * ny + Y0 + r) & 1;
+        return (r & 1) * (int)(HBX / 8) + (r >> 1) * W + c - 1 + d;
+    };
+    // values at the lane's two nodes of a field row at position o (and of a w tile row)
+    auto two = [&](const double *f, int o) -> double2 {
+        return kRag ? make_double2(f[o], f[o + XS]) : *(const double2 *)(f + o);
+    };
+    // a last single row is outside the row-pair map (N rows, N odd): its ybar, which Tbar
+    // copies there, is read from the field itself
+    const bool lone = kRag && gy == ny - 1 && (((int64_t)ny * nz) & 1);
     const int t = threadIdx.x;
     const bool has_h = t < NHALO;
     int hr, hc;
@@ -166,26 +204,42 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
         hc = (u & 1) ? HX + BX : HX - 1;
     }
     const int hidx = has_h ? hr * W + hc : 0;
+    if (!has_h) hr = 0, hc = 1;
     const int hx = X0 - HX + hc, hy = Y0 - 1 + hr;
     const bool hm = has_h && hx >= 1 && hx <= nx - 2 && hy >= 1 && hy <= ny - 2;
 
+    auto put2 = [&](long long *o, long long a, long long b) {
+        if (kRag) {
+            o[0] = a;
+            o[XS] = b;
+        } else {
+            *(longlong2 *)o = make_longlong2(a, b);
+        }
+    };
     // w of plane q from a stage: own two nodes and the halo node, as doubles
     double w0, w1, wh;
     double2 ynext;  // ybar at the own nodes of plane q (the next iteration's centre)
     auto w_compute = [&](int s, int q) -> int {
         const double *Ys = ring + (3 * s + 1) * SS, *Cs = ring + (3 * s + 2) * SS;
         const bool zin = q >= 1 && q <= nz - 2;
-        ynext = *(const double2 *)(Ys + row * W + col);
-        const double2 c2 = *(const double2 *)(Cs + row * W + col);
+        const int o = at(row, col, q);
+        ynext = two(Ys, o);
+        const double2 c2 = two(Cs, o);
+        if (lone && q == nz - 1) {
+            const double *yl = ybar + (int64_t)nx * ((int64_t)ny * nz - 1) + gx0;
+            if (gx0 <= nx - 1) ynext.x = yl[0];
+            if (gx0 + XS <= nx - 1) ynext.y = yl[XS];
+        }
         w0 = (zin && m0) ? c2.x * ynext.x : 0.0;
         w1 = (zin && m1) ? c2.y * ynext.y : 0.0;
-        wh = (zin && hm) ? Cs[hidx] * Ys[hidx] : 0.0;
+        const int oh = at(hr, hc, q);
+        wh = (zin && hm) ? Cs[oh] * Ys[oh] : 0.0;
         return max(max(emu_exp(dbits(w0)), emu_exp(dbits(w1))), emu_exp(dbits(wh)));
     };
     auto w_store = [&](long long *wt, int E, long long &f0, long long &f1) {
         f0 = adjs_fixed(dbits(w0), E);
         f1 = adjs_fixed(dbits(w1), E);
-        *(longlong2 *)(wt + row * W + col) = make_longlong2(f0, f1);
+        put2(wt + row * W + col, f0, f1);
         if (has_h) wt[hidx] = adjs_fixed(dbits(wh), E);
     };
 
@@ -193,8 +247,8 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
     int s_m = 0, s_c = 1 % NST;
     bool ok = acquire(s_m);
     ok = acquire(s_c) && ok;
-    double2 tm = *(const double2 *)(ring + (3 * s_m) * SS + row * W + col);
-    double2 tc = *(const double2 *)(ring + (3 * s_c) * SS + row * W + col);
+    double2 tm = two(ring + (3 * s_m) * SS, at(row, col, k0 - 1));
+    double2 tc = two(ring + (3 * s_c) * SS, at(row, col, k0));
     int em = w_compute(s_m, k0 - 1);  // includes both own w of plane k0-1
     const double wm0d = w0, wm1d = w1;  // (its halo value is not needed)
     em = max(em, w_compute(s_c, k0));
@@ -217,8 +271,9 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
     long long wm0 = adjs_fixed(dbits(wm0d), Esc), wm1 = adjs_fixed(dbits(wm1d), Esc);
 
     const bool row_out = gy <= ny - 1;
-    const bool all_x = gx0 + PX - 1 <= nx - 1;
+    const bool all_x = !kRag && gx0 + PX - 1 <= nx - 1;
     const bool all_in = m0 && m1;
+    const bool vec = !kRag && all_in;  // 16-byte accesses to Csbar
 
     for (int k = k0; k < k1; ++k) {
         const int s_n = nexts(s_c);  // stage of plane k+1
@@ -228,18 +283,18 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
         // Csbar of plane k: issued early, used at the end of the iteration
         double2 cb = make_double2(0.0, 0.0);
         if (do_ci) {
-            if (all_in) {
+            if (vec) {
                 cb = *(const double2 *)(Csbar + base);
             } else {
                 if (m0) cb.x = Csbar[base];
-                if (m1) cb.y = Csbar[base + 1];
+                if (m1) cb.y = Csbar[base + XS];
             }
         }
         ok = acquire(s_n);
         const int wnxt = wcur == 2 ? 0 : wcur + 1;
         const int emn = w_compute(s_n, k + 1);
         long long wp0, wp1;
-        w_store(wtile + wnxt * SS, Esc, wp0, wp1);
+        w_store(wtile + wnxt * WS, Esc, wp0, wp1);
         if (!ok) {
             s_abort = 1;
             atomicOr(&g_adjs_error, 1u);
@@ -256,37 +311,46 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
             __syncthreads();
             const int E2 = s_E;
             const int d = E2 - Esc;  // > 0
-            long long *wk = wtile + wcur * SS;
+            long long *wk = wtile + wcur * WS;
             auto shr = [d](long long v) { return d >= 64 ? 0ll : (v >> d); };
             wc0 = shr(wc0);
             wc1 = shr(wc1);
             wm0 = shr(wm0);
             wm1 = shr(wm1);
-            *(longlong2 *)(wk + row * W + col) = make_longlong2(wc0, wc1);
+            put2(wk + row * W + col, wc0, wc1);
             if (has_h) wk[hidx] = shr(wk[hidx]);
             Esc = E2;
-            w_store(wtile + wnxt * SS, Esc, wp0, wp1);
+            w_store(wtile + wnxt * WS, Esc, wp0, wp1);
             __syncthreads();
         }
         if (threadIdx.x == 0 && k - 1 + NST <= k1) issue(s_m, k - 1 + NST);  // plane k-1's stage
 
         if (row_out) {
             // ---- Tbar = ybar + L(w), exact integer sums, one DADD per node
-            const long long *wk = wtile + wcur * SS;
-            const long long wl = wk[row * W + col - 1], wr = wk[row * W + col + PX];
-            const longlong2 wu = *(const longlong2 *)(wk + (row - 1) * W + col);
-            const longlong2 wd = *(const longlong2 *)(wk + (row + 1) * W + col);
+            const long long *wk = wtile + wcur * WS + row * W + col;
+            // x-neighbours: of node 0 (wl, wr0) and of node 1 (wl1, wr); side by side where the
+            // lane's nodes are neighbours
+            const long long wl = wk[-1], wr = wk[kRag ? XS + 1 : PX];
+            const long long wr0 = kRag ? wk[1] : wc1, wl1 = kRag ? wk[XS - 1] : wc0;
+            longlong2 wu, wd;
+            if constexpr (kRag) {
+                wu = make_longlong2(wk[-W], wk[XS - W]);
+                wd = make_longlong2(wk[W], wk[XS + W]);
+            } else {
+                wu = *(const longlong2 *)(wk - W);
+                wd = *(const longlong2 *)(wk + W);
+            }
             const int sc = Esc - 1079;
             double2 tb;
-            const long long S0 = ((wl + wc1) + (wu.x + wd.x)) + (wm0 + wp0) - 6 * wc0;
-            const long long S1 = ((wc0 + wr) + (wu.y + wd.y)) + (wm1 + wp1) - 6 * wc1;
+            const long long S0 = ((wl + wr0) + (wu.x + wd.x)) + (wm0 + wp0) - 6 * wc0;
+            const long long S1 = ((wl1 + wr) + (wu.y + wd.y)) + (wm1 + wp1) - 6 * wc1;
             if constexpr (kAx == AX_COMMON) {
                 if (Esc == 0x7ff) {  // a non-finite w in this CTA's march: report NaN
                     tb.x = tb.y = __longlong_as_double(0x7ff8000000000000ll);
                 } else {
                     const long long a2 = 2 * wc0, b2 = 2 * wc1;
-                    tb.x = yc.x + emu_L_common<3>(wl + wc1 - a2, wu.x + wd.x - a2, wm0 + wp0 - a2, sc, 0ull, p.ek);
-                    tb.y = yc.y + emu_L_common<3>(wc0 + wr - b2, wu.y + wd.y - b2, wm1 + wp1 - b2, sc, 0ull, p.ek);
+                    tb.x = yc.x + emu_L_common<3>(wl + wr0 - a2, wu.x + wd.x - a2, wm0 + wp0 - a2, sc, 0ull, p.ek);
+                    tb.y = yc.y + emu_L_common<3>(wl1 + wr - b2, wu.y + wd.y - b2, wm1 + wp1 - b2, sc, 0ull, p.ek);
                 }
             } else if (Esc >= 57 && Esc <= 2042) {  // CTA-uniform: the packed sums are normal
                 tb.x = kGiven ? fma(p.ek.Kx, adjs_pack_normal(S0, sc), yc.x) : yc.x + adjs_pack_normal(S0, sc);
@@ -301,71 +365,81 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
                 *(double2 *)(Tbar + base) = tb;
             } else {
                 if (gx0 <= nx - 1) Tbar[base] = tb.x;
-                if (gx0 + 1 <= nx - 1) Tbar[base + 1] = tb.y;
+                if (gx0 + XS <= nx - 1) Tbar[base + XS] = tb.y;
             }
 
             // ---- Csbar += ybar * L(T), bit-pattern sums on the same-binade fast path
             if (do_ci) {
                 const double *Tk = ring + (3 * s_c) * SS;
-                const double2 tp = *(const double2 *)(ring + (3 * s_n) * SS + row * W + col);
-                const double2 tu = *(const double2 *)(Tk + (row - 1) * W + col);
-                const double2 td = *(const double2 *)(Tk + (row + 1) * W + col);
-                const double tl = Tk[row * W + col - 1], tr = Tk[row * W + col + PX];
+                const double2 tp = two(ring + (3 * s_n) * SS, at(row, col, k + 1));
+                const double2 tu = two(Tk, at(row - 1, col, k));
+                const double2 td = two(Tk, at(row + 1, col, k));
+                const double *To = Tk + at(row, col, k);
+                const double tl = To[-1], tr = To[kRag ? XS + 1 : PX];
                 const unsigned long long c0 = dbits(tc.x), c1 = dbits(tc.y);
                 const unsigned long long xl = dbits(tl), xr = dbits(tr);
+                const unsigned long long xr0 = kRag ? dbits(To[1]) : c1, xl1 = kRag ? dbits(To[XS - 1]) : c0;
                 const unsigned long long u0 = dbits(tu.x), u1 = dbits(tu.y), d0 = dbits(td.x),
                                          d1 = dbits(td.y), m0b = dbits(tm.x), m1b = dbits(tm.y),
                                          p0 = dbits(tp.x), p1 = dbits(tp.y);
                 unsigned hc0 = (unsigned)(c0 >> 32);
-                unsigned hw[11] = {(unsigned)(xl >> 32), (unsigned)(xr >> 32), (unsigned)(u0 >> 32),
+                unsigned hw[kRag ? 13 : 11] = {(unsigned)(xl >> 32), (unsigned)(xr >> 32), (unsigned)(u0 >> 32),
                                    (unsigned)(d0 >> 32), (unsigned)(m0b >> 32), (unsigned)(p0 >> 32),
                                    (unsigned)(u1 >> 32), (unsigned)(d1 >> 32), (unsigned)(m1b >> 32),
                                    (unsigned)(p1 >> 32), (unsigned)(c1 >> 32)};
+                if constexpr (kRag) {
+                    hw[11] = (unsigned)(xr0 >> 32);
+                    hw[12] = (unsigned)(xl1 >> 32);
+                }
                 if (!all_in) {  // values of unstored nodes must not force the general path
                     // a lane that stores neither node (past the grid: zeros) votes for the fast
                     // path: its reference is 1.0's word (its outputs are never stored)
                     if (!m0 && !m1) hc0 = 0x3ff00000u;
                     if (!m0) hw[0] = hw[2] = hw[3] = hw[4] = hw[5] = hc0;
                     if (!m1) hw[1] = hw[6] = hw[7] = hw[8] = hw[9] = hc0;
+                    if constexpr (kRag) {  // the nodes are no neighbours: each has its own six
+                        if (!m0) hc0 = m1 ? (unsigned)(c1 >> 32) : 0x3ff00000u;
+                        if (!m0) hw[0] = hw[2] = hw[3] = hw[4] = hw[5] = hw[11] = hc0;
+                        if (!m1) hw[1] = hw[6] = hw[7] = hw[8] = hw[9] = hw[10] = hw[12] = hc0;
+                    }
                     if (!m0 && !m1) hw[10] = hc0;
                 }
                 const bool fast = emu_same_binade_hi(hw, hc0);
                 double L0, L1;
                 if (kAx == AX_COMMON && __all_sync(0xffffffffu, fast)) {
                     const unsigned long long a2 = 2ull * c0, b2 = 2ull * c1;
-                    const int sct = emu_exp(c0) - 1075;
-                    const unsigned long long flip = c0 & 0x8000000000000000ull;  // negative: minus
-                    L0 = emu_L_common<3>((long long)(xl + c1 - a2), (long long)(u0 + d0 - a2),
+                    const int sct = (int)((hc0 >> 20) & 0x7ffu) - 1075;
+                    const unsigned long long flip = (unsigned long long)(hc0 & 0x80000000u) << 32;  // negative: minus
+                    L0 = emu_L_common<3>((long long)(xl + xr0 - a2), (long long)(u0 + d0 - a2),
                                          (long long)(m0b + p0 - a2), sct, flip, p.ek);
-                    L1 = emu_L_common<3>((long long)(c0 + xr - b2), (long long)(u1 + d1 - b2),
+                    L1 = emu_L_common<3>((long long)(xl1 + xr - b2), (long long)(u1 + d1 - b2),
                                          (long long)(m1b + p1 - b2), sct, flip, p.ek);
                 } else if (kAx != AX_COMMON && __all_sync(0xffffffffu, fast)) {
-                    const long long S0t = (long long)(((xl + c1) + (u0 + d0)) + (m0b + p0) - 6ull * c0);
-                    const long long S1t = (long long)(((c0 + xr) + (u1 + d1)) + (m1b + p1) - 6ull * c1);
-                    const int e = emu_exp(c0);
-                    const int sct = (e ? e : 1) - 1075;
-                    const unsigned long long flip = c0 & 0x8000000000000000ull;  // negative: minus
+                    const long long S0t = (long long)(((xl + xr0) + (u0 + d0)) + (m0b + p0) - 6ull * c0);
+                    const long long S1t = (long long)(((xl1 + xr) + (u1 + d1)) + (m1b + p1) - 6ull * c1);
+                    const int sct = (int)((hc0 >> 20) & 0x7ffu) - 1075;
+                    const unsigned long long flip = (unsigned long long)(hc0 & 0x80000000u) << 32;  // negative: minus
                     unsigned long long g0, g1;
                     const unsigned long long a0 = emu_abs(S0t, &g0), a1 = emu_abs(S1t, &g1);
                     L0 = bitsd(emu_pack_mag_normal(a0, sct) | (g0 ^ flip));
                     L1 = bitsd(emu_pack_mag_normal(a1, sct) | (g1 ^ flip));
                 } else {
-                    L0 = m0 ? adjs_lap_general<kAx>(c0, xl, c1, u0, d0, m0b, p0, p.ek) : 0.0;
-                    L1 = m1 ? adjs_lap_general<kAx>(c1, c0, xr, u1, d1, m1b, p1, p.ek) : 0.0;
+                    L0 = m0 ? adjs_lap_general<kAx>(c0, xl, xr0, u0, d0, m0b, p0, p.ek) : 0.0;
+                    L1 = m1 ? adjs_lap_general<kAx>(c1, xl1, xr, u1, d1, m1b, p1, p.ek) : 0.0;
                 }
                 cb.x = fma(kAx == AX_ISO && kGiven ? p.ek.Kx * yc.x : yc.x, L0, cb.x);
                 cb.y = fma(kAx == AX_ISO && kGiven ? p.ek.Kx * yc.y : yc.y, L1, cb.y);
-                if (all_in) {
+                if (vec) {
                     *(double2 *)(Csbar + base) = cb;
                 } else {
                     if (m0) Csbar[base] = cb.x;
-                    if (m1) Csbar[base + 1] = cb.y;
+                    if (m1) Csbar[base + XS] = cb.y;
                 }
             }
         }
         // rotate: plane k becomes the minus neighbour, plane k+1 the centre
         tm = tc;
-        tc = *(const double2 *)(ring + (3 * s_n) * SS + row * W + col);
+        tc = two(ring + (3 * s_n) * SS, at(row, col, k + 1));
         yc = ynext;
         wm0 = wc0;
         wm1 = wc1;
@@ -377,19 +451,21 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
     }
 }
 
-template <int kAx, bool kGiven>
-static cudaError_t launch_adjs(double *Tbar, double *Csbar, const double *ybar, const double *T,
+template <int kAx, bool kGiven, bool kRag>
+static cudaError_t launch_adjs_t(double *Tbar, double *Csbar, const double *ybar, const double *T,
                                const double *Cs, const EmuCoef &ek, Grid3 g, cudaStream_t s) {
     constexpr int BY = 8, NST = 3, PX = 2, BX = 32 * PX, W = BX + 2 * PX, H = BY + 2;
-    constexpr unsigned TBA = (W * H * 8 + 127) / 128 * 128;
-    constexpr size_t smem = 3 * NST * TBA + 3 * TBA + NST * 8;
+    constexpr unsigned WBA = (W * H * 8 + 127) / 128 * 128;
+    constexpr unsigned TBA = kRag ? 2 * ((W * H / 2 * 8 + 127) / 128 * 128) : WBA;
+    constexpr size_t smem = 3 * NST * TBA + 3 * WBA + NST * 8;
     static unsigned attr_gen[64] = {0};
     cudaError_t ae;
-    if (!set_smem_attr_once((const void *)k_adjoint_scaled<BY, NST, kAx, kGiven>, (int)smem, attr_gen, &ae)) return ae;
+    if (!set_smem_attr_once((const void *)k_adjoint_scaled<BY, NST, kAx, kGiven, kRag>, (int)smem, attr_gen, &ae)) return ae;
     CUtensorMap mT, mY, mC;
-    if (!make_tensor_map_3d(&mT, T, 8, g, W, H) || !make_tensor_map_3d(&mY, ybar, 8, g, W, H) ||
-        !make_tensor_map_3d(&mC, Cs, 8, g, W, H))
-        return cudaErrorInvalidValue;
+    auto map = [&](CUtensorMap *m, const double *f) {
+        return kRag ? make_tensor_map_rows(m, f, 8, g.n(), 2 * g.nx, W, H / 2) : make_tensor_map_3d(m, f, 8, g, W, H);
+    };
+    if (!map(&mT, T) || !map(&mY, ybar) || !map(&mC, Cs)) return cudaErrorInvalidValue;
     const int64_t ntx = (g.nx + BX - 1) / BX, nty = (g.ny + BY - 1) / BY, tiles = ntx * nty;
     int kchunk = launch_override(PS_OVERRIDE_ADJ_KCHUNK);
     if (kchunk <= 0) {
@@ -422,8 +498,15 @@ static cudaError_t launch_adjs(double *Tbar, double *Csbar, const double *ybar, 
     const int64_t gz = (g.nz + kchunk - 1) / kchunk;
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
     AdjSParams p{g.nx, g.ny, g.nz, kchunk, (int)ntx, ek};
-    return launch_pdl(k_adjoint_scaled<BY, NST, kAx, kGiven>, dim3((unsigned)tiles, (unsigned)gz, 1), dim3(32 * BY), smem, s,
-                      mT, mY, mC, Tbar, Csbar, p);
+    return launch_pdl(k_adjoint_scaled<BY, NST, kAx, kGiven, kRag>, dim3((unsigned)tiles, (unsigned)gz, 1), dim3(32 * BY), smem, s,
+                      mT, mY, mC, Tbar, Csbar, ybar, p);
+}
+
+template <int kAx, bool kGiven>
+static cudaError_t launch_adjs(double *Tbar, double *Csbar, const double *ybar, const double *T,
+                               const double *Cs, const EmuCoef &ek, Grid3 g, cudaStream_t s) {
+    if (g.nx % 2) return launch_adjs_t<kAx, kGiven, true>(Tbar, Csbar, ybar, T, Cs, ek, g, s);
+    return launch_adjs_t<kAx, kGiven, false>(Tbar, Csbar, ybar, T, Cs, ek, g, s);
 }
 
 cudaError_t launch_adjoint_scaled(double *Tbar, double *Csbar, const double *ybar, const double *T,
