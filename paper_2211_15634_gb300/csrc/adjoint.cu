@@ -159,6 +159,8 @@ cudaError_t launch_adjoint_f32(float *Tbar, float *Cibar, const float *ybar, con
     const void *ptrs[5] = {T, ybar, Ci, Cibar, Tbar};
     if (launch_override(PS_OVERRIDE_ADJ_PLAIN) != 1 && adjoint_f32_supported(g, ptrs, 5))
         return launch_adjoint_f32_tma(Tbar, Cibar, ybar, T, Ci, c, g, s);
+    if (launch_override(PS_OVERRIDE_ADJ_PLAIN) != 1 && adjoint_f32_ragged(g, ptrs, 5))
+        return launch_adjoint_f32_rag(Tbar, Cibar, ybar, T, Ci, c, g, s);
     return launch_adjoint_basic<float>(
         Tbar, Cibar, ybar, T, Ci,
         CoefT<float>{(float)c.dtlam, (float)c.ax, (float)c.ay, (float)c.az}, g, s);

@@ -36,6 +36,10 @@ struct Adj32Params {
     float Kx, Ky, Kz;
 };
 
+// row slot of the ragged form: 130 elements from a 16-byte boundary, on 128 bytes
+constexpr int kRag32W = 136;
+constexpr unsigned kRag32Slot = 640;
+
 template <int BY, int NST, int MINB>
 __global__ void __launch_bounds__(32 * BY, MINB)
 k_adjoint_f32(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmY,
@@ -222,6 +226,209 @@ k_adjoint_f32(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ C
         wm = wc;
         wc = wp;
         s_c = s_n;
+    }
+}
+
+// The FP32 transposed step on ragged rows (nx % 4 != 0): the march above with every plane of
+// T, ybar and Ci staged row by row (zrag_tile.cuh: one copy per row, issued by the warp that
+// owns the row, its data 0 .. 3 elements into its slot) and lanes on nodes lane + 32*i of
+// their row.  The x-neighbours of w come from the neighbouring lanes, so that only their y
+// and z copies are formed twice; Cibar is read by plain loads issued at the top of a plane.
+// 8-row tiles and three stages (58 KB): 24 warps per SM.  Measured against the plain column
+// kernel: 161 x 128 x 96 14 against 19 us, 255^3 70 against 234, 511^3 543 against 1577.
+template <int BY, int NST>
+__global__ void __launch_bounds__(32 * BY, 3)
+k_adjoint_f32_rag(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmY,
+                  const __grid_constant__ CUtensorMap tmC, float *__restrict__ Tbar,
+                  float *__restrict__ Cibar, const Adj32Params p) {
+    constexpr int PX = 4, BX = 128, W = kRag32W, H = BY + 2;
+    constexpr unsigned RB = W * 4, SLOT = kRag32Slot, SB = 3 * H * SLOT;
+    constexpr int SL = SLOT / 4;
+    extern __shared__ __align__(128) unsigned char smem[];
+    uint64_t *bar = (uint64_t *)(smem + NST * SB);
+    __shared__ int s_abort;
+    grid_dep_wait();  // the previous launch's writes (and its reads of Tbar) are complete
+    grid_dep_launch();
+
+    const int lane = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int X0 = (int)(blockIdx.x % p.ntx) * BX, Y0 = (int)(blockIdx.x / p.ntx) * BY;
+    const int k0 = (int)blockIdx.y * p.kchunk;
+    const int k1 = min(k0 + p.kchunk, p.nz);  // output planes [k0, k1)
+    const int nx = p.nx, ny = p.ny, nz = p.nz, nplane = nx * ny;
+
+    auto issue = [&](int s, int q) {  // the warp's rows of plane q (q = -1 and q = nz read zeros
+        if (lane != 0) return;        // or rows that no interior node uses)
+        const bool edge = ty == 0 || ty == BY - 1;
+        const int hrow = ty == 0 ? 0 : H - 1;
+        mbar_expect_tx(&bar[s], 3 * RB * (edge ? 2u : 1u));
+        unsigned char *st = smem + s * SB;
+        const int e0 = q * nplane + (Y0 - 1) * nx + X0 - 1;  // tile row 0, column -1
+        const int xo = (e0 + (ty + 1) * nx) & ~3, xh = (e0 + hrow * nx) & ~3;
+        const CUtensorMap *tm[3] = {&tmT, &tmY, &tmC};
+#pragma unroll
+        for (int f = 0; f < 3; ++f) {
+            tma_load_1d(st + (f * H + ty + 1) * SLOT, tm[f], &bar[s], xo);
+            if (edge) tma_load_1d(st + (f * H + hrow) * SLOT, tm[f], &bar[s], xh);
+        }
+    };
+    if (threadIdx.x == 0) {
+        s_abort = 0;
+        for (int s = 0; s < NST; ++s) mbar_init(&bar[s], BY);  // one arrival per warp
+        fence_mbar_init();
+    }
+    __syncthreads();
+    // plane q = k0-1+i lives in stage i % NST
+    for (int s = 0; s < NST; ++s)
+        if (k0 - 1 + s <= k1) issue(s, k0 - 1 + s);
+
+    unsigned par = 0u;  // bit s: parity of the next completion of stage s
+    auto nexts = [](int s) { return s + 1 == NST ? 0 : s + 1; };
+    auto acquire = [&](int s) -> bool {
+        const unsigned ph = (par >> s) & 1u;
+        par ^= 1u << s;
+        return mbar_wait(&bar[s], ph);
+    };
+    // After a timed-out wait: bounded waits for the copies of the last NST planes issued
+    // (up to plane q_iss), so that no TMA write lands after the CTA exits.
+    auto drain = [&](int q_iss) {
+        for (int q = max(k0 - 1, q_iss - NST + 1); q <= q_iss; ++q) {
+            const int i = q - (k0 - 1);
+            mbar_wait(&bar[i % NST], (unsigned)(i / NST) & 1u);
+        }
+    };
+    // the lane's first node in tile row h of field f (0 T, 1 ybar, 2 Ci) in stage s; d: the
+    // row's offset in its slot, (row * nx + X0 - 1) mod 4
+    auto at = [&](int f, int s, int h, int d) {
+        return (const float *)(smem + s * SB) + (f * H + h) * SL + d + 1 + lane;
+    };
+
+    const int gy = Y0 + ty, gx0 = X0 + lane;
+    const bool iy = gy >= 1 && gy <= ny - 2, iyu = gy - 1 >= 1 && gy - 1 <= ny - 2,
+               iyd = gy + 1 >= 1 && gy + 1 <= ny - 2;
+    bool ix[PX];
+#pragma unroll
+    for (int i = 0; i < PX; ++i) ix[i] = gx0 + 32 * i >= 1 && gx0 + 32 * i <= nx - 2;
+    const bool ixl = X0 - 1 >= 1 && X0 - 1 <= nx - 2, ixr = X0 + BX <= nx - 2;  // the tile's x halo
+    const bool row_out = gy <= ny - 1;
+    const int dplane = nplane & 3, drow = nx & 3;
+    int dk = ((k0 - 1) * nplane + gy * nx + X0 - 1) & 3;  // own row of plane k0-1
+
+    // ---- prologue: planes k0-1 and k0
+    auto own_w = [&](int s, int d, int q, const float (&y)[PX], float (&w)[PX]) {
+        const float *c = at(2, s, ty + 1, d);
+        const bool in = q >= 1 && q <= nz - 2 && iy;
+#pragma unroll
+        for (int i = 0; i < PX; ++i) w[i] = a32_w(c[32 * i], y[i], in && ix[i]);
+    };
+    int s_m = 0, s_c = 1 % NST;
+    bool ok = acquire(s_m);
+    ok = acquire(s_c) && ok;
+    float tm_[PX], wm[PX], tc[PX], yc[PX], wc[PX];
+    {
+        float ym[PX];
+#pragma unroll
+        for (int i = 0; i < PX; ++i) {
+            tm_[i] = at(0, s_m, ty + 1, dk)[32 * i];
+            ym[i] = at(1, s_m, ty + 1, dk)[32 * i];
+        }
+        own_w(s_m, dk, k0 - 1, ym, wm);
+    }
+    dk = (dk + dplane) & 3;
+#pragma unroll
+    for (int i = 0; i < PX; ++i) {
+        tc[i] = at(0, s_c, ty + 1, dk)[32 * i];
+        yc[i] = at(1, s_c, ty + 1, dk)[32 * i];
+    }
+    own_w(s_c, dk, k0, yc, wc);
+    if (!ok) {
+        s_abort = 1;
+        atomicOr(&g_adj32_error, 1u);
+    }
+    __syncthreads();  // every thread is done with plane k0-1's stage
+    if (s_abort) {
+        drain(min(k0 - 2 + NST, k1));
+        return;
+    }
+    if (k0 - 1 + NST <= k1) issue(s_m, k0 - 1 + NST);
+
+    const float Kx = p.Kx, Ky = p.Ky, Kz = p.Kz;
+    int64_t base = (int64_t)gx0 + (int64_t)nx * ((int64_t)gy + (int64_t)ny * k0);
+    for (int k = k0; k < k1; ++k, base += nplane) {
+        const bool iz = k >= 1 && k <= nz - 2;
+        float cb[PX];
+#pragma unroll
+        for (int i = 0; i < PX; ++i) cb[i] = (iz && iy && ix[i]) ? Cibar[base + 32 * i] : 0.f;
+        const int s_n = nexts(s_c), dn = (dk + dplane) & 3;
+        ok = acquire(s_n);
+        float tp[PX], yp[PX], wp[PX];
+#pragma unroll
+        for (int i = 0; i < PX; ++i) {
+            tp[i] = at(0, s_n, ty + 1, dn)[32 * i];
+            yp[i] = at(1, s_n, ty + 1, dn)[32 * i];
+        }
+        own_w(s_n, dn, k + 1, yp, wp);
+        // x-neighbours of w in plane k (every lane of the warp takes part)
+        float wl[PX], wr[PX];
+        {
+            const float *Yo = at(1, s_c, ty + 1, dk) - lane, *Co = at(2, s_c, ty + 1, dk) - lane;
+            float pl = lane == 0 ? a32_w(Co[-1], Yo[-1], iz && iy && ixl) : 0.f;   // column -1
+            float pr = lane == 31 ? a32_w(Co[BX], Yo[BX], iz && iy && ixr) : 0.f;  // column BX
+#pragma unroll
+            for (int i = 0; i < PX; ++i) {
+                const float v = __shfl_sync(0xffffffffu, wc[i], (lane + 31) & 31);
+                wl[i] = lane == 0 ? pl : v;
+                pl = v;  // lane 0: node 31 of this group is the left neighbour of the next group's node 0
+            }
+#pragma unroll
+            for (int i = PX - 1; i >= 0; --i) {
+                const float v = __shfl_sync(0xffffffffu, wc[i], (lane + 1) & 31);
+                wr[i] = lane == 31 ? pr : v;
+                pr = v;
+            }
+        }
+        if (row_out) {
+            const int du = (dk - drow) & 3, dd = (dk + drow) & 3;
+            const float *Yu = at(1, s_c, ty, du), *Cu = at(2, s_c, ty, du);
+            const float *Yd = at(1, s_c, ty + 2, dd), *Cd = at(2, s_c, ty + 2, dd);
+            const bool mu = iz && iyu, md = iz && iyd;
+#pragma unroll
+            for (int i = 0; i < PX; ++i) {
+                const float wu = a32_w(Cu[32 * i], Yu[32 * i], mu && ix[i]);
+                const float wd = a32_w(Cd[32 * i], Yd[32 * i], md && ix[i]);
+                const float tb = a32_tbar(yc[i], a32_lap(wc[i], wl[i], wr[i], wu, wd, wm[i], wp[i], Kx, Ky, Kz));
+                if (gx0 + 32 * i <= nx - 1) Tbar[base + 32 * i] = tb;
+            }
+            if (iz && iy) {
+                const float *To = at(0, s_c, ty + 1, dk), *Tu = at(0, s_c, ty, du), *Td = at(0, s_c, ty + 2, dd);
+#pragma unroll
+                for (int i = 0; i < PX; ++i) {
+                    const float c = a32_cibar(cb[i], yc[i],
+                                              a32_lap(tc[i], To[32 * i - 1], To[32 * i + 1], Tu[32 * i], Td[32 * i],
+                                                      tm_[i], tp[i], Kx, Ky, Kz));
+                    if (ix[i]) Cibar[base + 32 * i] = c;
+                }
+            }
+        }
+        if (!ok) {
+            s_abort = 1;
+            atomicOr(&g_adj32_error, 1u);
+        }
+        __syncthreads();  // every thread is done with plane k's stage
+        if (s_abort) {
+            drain(min(k - 1 + NST, k1));
+            return;
+        }
+        if (k + NST <= k1) issue(s_c, k + NST);
+#pragma unroll
+        for (int i = 0; i < PX; ++i) {
+            tm_[i] = tc[i];
+            tc[i] = tp[i];
+            yc[i] = yp[i];
+            wm[i] = wc[i];
+            wc[i] = wp[i];
+        }
+        s_c = s_n;
+        dk = dn;
     }
 }
 
@@ -571,6 +778,24 @@ cudaError_t launch_adjoint2_f32(float *Tbar, float *Cibar, const float *ybar, co
     return launch_adj2_t<4, 3>(Tbar, Cibar, ybar, S1, S0, Ci, g, p, kchunk, s);
 }
 
+// Planes per CTA of the one-step kernels; slots: CTAs resident at once.
+static int adj32_kchunk(int64_t slots, int64_t nz, int64_t tiles) {
+    // One wave when it takes chunks of at most 12 or of 32-96 planes: every tile's
+    // z-range split into as many chunks as there are CTA slots per tile, all CTAs
+    // resident at once (no tail).  Else 16-plane chunks (each chunk re-reads two planes);
+    // 32 where 16 would leave fewer than four waves of CTAs and 32 still gives one and
+    // a half.  Measured: 256^3 at 64 (one wave; 4.5% ahead of 32, 8% of 16), 512^3 and
+    // 768^3 at 16-24 (within 1%); small grids against the 16 planes they had: 32^3 2.8 /
+    // 10.3 us, 64^3 4.7 / 10.4, 96^3 6.2 / 10.5, 128^3 10 / 12.2, 160 x 128 x 96 13.2 / 16.6.
+    const int64_t cols = nz * tiles;
+    const int64_t per_tile = tiles > 0 ? slots / tiles : 0;
+    const int64_t one_wave = per_tile > 0 ? (nz + per_tile - 1) / per_tile : 0;
+    if (one_wave > 0 && one_wave <= 12)
+        return (int)(one_wave < 2 ? 2 : one_wave);
+    if (one_wave >= 32 && one_wave <= 96) return (int)one_wave;
+    return (cols < 4 * 16 * slots && 2 * cols >= 3 * 32 * slots) ? 32 : 16;
+}
+
 template <int BY, int NST, int MINB>
 static cudaError_t launch_adj32_t(float *Tbar, float *Cibar, const float *ybar, const float *T,
                                   const float *Ci, Grid3 g, Adj32Params p, int kchunk, cudaStream_t s) {
@@ -585,24 +810,7 @@ static cudaError_t launch_adj32_t(float *Tbar, float *Cibar, const float *ybar, 
         !make_tensor_map_3d(&mC, Ci, 4, g, W, H) || !make_tensor_map_3d(&mB, Cibar, 4, g, BX, BY))
         return cudaErrorInvalidValue;
     const int64_t ntx = (g.nx + BX - 1) / BX, nty = (g.ny + BY - 1) / BY, tiles = ntx * nty;
-    if (kchunk <= 0) {
-        // One wave when it takes chunks of at most 12 or of 32-96 planes: every tile's
-        // z-range split into as many chunks as there are CTA slots per tile, all CTAs
-        // resident at once (no tail).  Else 16-plane chunks (each chunk re-reads two planes);
-        // 32 where 16 would leave fewer than four waves of CTAs and 32 still gives one and
-        // a half.  Measured: 256^3 at 64 (one wave; 4.5% ahead of 32, 8% of 16), 512^3 and
-        // 768^3 at 16-24 (within 1%); small grids against the 16 planes they had: 32^3 2.8 /
-        // 10.3 us, 64^3 4.7 / 10.4, 96^3 6.2 / 10.5, 128^3 10 / 12.2, 160 x 128 x 96 13.2 / 16.6.
-        const int64_t slots = (int64_t)MINB * sm_count(), cols = g.nz * tiles;
-        const int64_t per_tile = tiles > 0 ? slots / tiles : 0;
-        const int64_t one_wave = per_tile > 0 ? (g.nz + per_tile - 1) / per_tile : 0;
-        if (one_wave > 0 && one_wave <= 12)
-            kchunk = (int)(one_wave < 2 ? 2 : one_wave);
-        else if (one_wave >= 32 && one_wave <= 96)
-            kchunk = (int)one_wave;
-        else
-            kchunk = (cols < 4 * 16 * slots && 2 * cols >= 3 * 32 * slots) ? 32 : 16;
-    }
+    if (kchunk <= 0) kchunk = adj32_kchunk((int64_t)MINB * sm_count(), g.nz, tiles);
     const int64_t gz = (g.nz + kchunk - 1) / kchunk;
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
     p.nx = (int)g.nx;
@@ -622,6 +830,54 @@ bool adjoint_f32_supported(Grid3 g, const void *const *ptrs, int nptr) {
     // 32-bit plane and row indices in the kernel; TMA coordinates are 32-bit as well
     if (g.nx > (1LL << 31) - 256 || g.ny > (1LL << 31) - 64 || g.nz > (1LL << 31) - 64) return false;
     return zmarch_supported(g, 4, ptrs[0], ptrs[0], ptrs[0]);
+}
+
+bool adjoint_f32_ragged(Grid3 g, const void *const *ptrs, int nptr) {
+    if (g.nx % 4 == 0) return false;
+    for (int i = 0; i < nptr; ++i)
+        if (!ragged_supported(g, ptrs[i], ptrs[i], ptrs[i])) return false;
+    return true;
+}
+
+cudaError_t launch_adjoint_f32_rag(float *Tbar, float *Cibar, const float *ybar, const float *T,
+                                   const float *Ci, StepCoef c, Grid3 g, cudaStream_t s) {
+    constexpr int BY = 8, NST = 3, BX = 128;
+    constexpr size_t smem = NST * 3 * (BY + 2) * kRag32Slot + NST * 8;
+    static unsigned attr_gen[64] = {0};
+    cudaError_t ae;
+    if (!set_smem_attr_once((const void *)k_adjoint_f32_rag<BY, NST>, (int)smem, attr_gen, &ae)) return ae;
+    CUtensorMap mT, mY, mC;
+    if (!make_tensor_map_rows(&mT, T, 4, g.n(), 0, kRag32W, 0) ||
+        !make_tensor_map_rows(&mY, ybar, 4, g.n(), 0, kRag32W, 0) ||
+        !make_tensor_map_rows(&mC, Ci, 4, g.n(), 0, kRag32W, 0))
+        return cudaErrorInvalidValue;
+    const int64_t ntx = (g.nx + BX - 1) / BX, nty = (g.ny + BY - 1) / BY, tiles = ntx * nty;
+    int kchunk = launch_override(PS_OVERRIDE_ADJ_KCHUNK);
+    if (kchunk <= 0) {
+        // one wave where it fills the chip (255^3: 37 planes 70 us, 8 planes 76), else 16
+        // planes, 8 where those would be less than two waves (191^3 41 us, 47 at 16; 257^3
+        // 100 at 16, 110 in one wave of 0.87)
+        const int64_t slots = 3LL * sm_count(), per_tile = slots / tiles;
+        const int64_t one_wave = per_tile > 0 ? (g.nz + per_tile - 1) / per_tile : 0;
+        const int64_t used = one_wave > 0 ? tiles * ((g.nz + one_wave - 1) / one_wave) : 0;
+        if (one_wave > 0 && one_wave <= 96 && (one_wave <= 12 || 100 * used >= 95 * slots))
+            kchunk = (int)(one_wave < 2 ? 2 : one_wave);
+        else
+            kchunk = tiles * ((g.nz + 15) / 16) < 2 * slots ? 8 : 16;
+    }
+    const int64_t gz = (g.nz + kchunk - 1) / kchunk;
+    if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
+    Adj32Params p{};
+    p.Kx = (float)(c.dtlam * c.ax);
+    p.Ky = (float)(c.dtlam * c.ay);
+    p.Kz = (float)(c.dtlam * c.az);
+    p.nx = (int)g.nx;
+    p.ny = (int)g.ny;
+    p.nz = (int)g.nz;
+    p.ntx = (int)ntx;
+    p.kchunk = kchunk;
+    return launch_pdl(k_adjoint_f32_rag<BY, NST>, dim3((unsigned)tiles, (unsigned)gz, 1), dim3(32 * BY), smem, s,
+                      mT, mY, mC, Tbar, Cibar, p);
 }
 
 cudaError_t launch_adjoint_f32_tma(float *Tbar, float *Cibar, const float *ybar, const float *T,

@@ -81,6 +81,10 @@ unsigned adjoint_scaled_device_error(bool clear);
 bool adjoint_f32_supported(Grid3 g, const void *const *ptrs, int nptr);
 cudaError_t launch_adjoint_f32_tma(float *Tbar, float *Cibar, const float *ybar, const float *T,
                                    const float *Ci, StepCoef c, Grid3 g, cudaStream_t s);
+// The same on ragged rows (nx % 4 != 0, fewer than 2^31 elements).
+bool adjoint_f32_ragged(Grid3 g, const void *const *ptrs, int nptr);
+cudaError_t launch_adjoint_f32_rag(float *Tbar, float *Cibar, const float *ybar, const float *T,
+                                   const float *Ci, StepCoef c, Grid3 g, cudaStream_t s);
 unsigned adjoint_f32_device_error(bool clear);
 // 2-D form of the step (diffusion2d.cu); mode is a ZMode: Z_F32, Z_F64_SCALED,
 // Z_F64_EMU_ISO_DMUL or Z_F64_NATIVE

@@ -111,7 +111,7 @@ bool make_tensor_map_rows(CUtensorMap *m, const void *ptr, int esz, int64_t n, i
     auto fn = encode_fn();
     if (!fn) return false;
     const bool line = by == 0;  // one line of n elements
-    const cuuint64_t dims[2] = {(cuuint64_t)(line ? n : rowlen), (cuuint64_t)(line ? 1 : n / rowlen)};
+    const cuuint64_t dims[2] = {(cuuint64_t)(line ? n : rowlen), (cuuint64_t)(line ? 1 : n / (rowlen > 0 ? rowlen : 1))};
     const cuuint64_t strides[1] = {line ? 0 : (cuuint64_t)(rowlen * esz)};
     const cuuint32_t box[2] = {bx, line ? 1u : by}, estr[2] = {1, 1};
     const CUresult r = fn(m, esz == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
