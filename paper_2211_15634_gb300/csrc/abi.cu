@@ -178,8 +178,7 @@ static int check_step_args(const void *T2, const void *T, const void *Ci, double
 }
 
 // One step; E2 / E: correction fields of the two-float state (PS_RUN_COMPENSATED).
-// in_loop: one of a time loop's steps (internal.h).  write_bnd: the step also stores T's x
-// and y boundary nodes of planes 1 .. nz-2 into T2 (not with PS_RUN_COMPENSATED).
+// in_loop, write_bnd: internal.h (the latter not with PS_RUN_COMPENSATED).
 static cudaError_t enqueue_step(void *T2, const void *T, void *E2, const void *E, const void *Ci,
                                 StepCoef c, Grid3 g, int dtype, unsigned flags, cudaStream_t s,
                                 bool in_loop = false, bool write_bnd = false) {
@@ -188,7 +187,7 @@ static cudaError_t enqueue_step(void *T2, const void *T, void *E2, const void *E
             return launch_step_f64_scaled((double *)T2, (const double *)T, (const double *)Ci, g, s,
                                           write_bnd, in_loop);
         if (flags & PS_RUN_NATIVE_F64)
-            return launch_step_f64_native((double *)T2, (const double *)T, (const double *)Ci, c, g, s, write_bnd);
+            return launch_step_f64_native((double *)T2, (const double *)T, (const double *)Ci, c, g, s);
         return launch_step_f64_fast((double *)T2, (const double *)T, (const double *)Ci, c, g, s, write_bnd, in_loop);
     }
     if (flags & PS_RUN_COMPENSATED)
@@ -197,13 +196,11 @@ static cudaError_t enqueue_step(void *T2, const void *T, void *E2, const void *E
     return launch_step_f32((float *)T2, (const float *)T, (const float *)Ci, c, g, s, write_bnd, in_loop);
 }
 
-// True when PS_RUN_TEMPORAL2 fuses step pairs for these arguments (the mode is checked by the
-// caller: FP32 plain, or FP64 on the pre-scaled coefficient).  FP32 pairs leave small grids
-// to the single steps' column kernel, which is faster there (us a step, pairs against single
-// steps: 64^3 4.6 / 2.2, 192^3 17 / 14), unless a z-chunk is set for them.  states: pairs that
-// keep both states, see states_column.
-static bool temporal2_ok(Grid3 g, int dtype, const void *T, const void *T2, const void *Ci, bool states = false) {
-    if (dtype == PS_F32 && (!states || (double)g.n() <= 2.2e6) && step_small(g, Z_F32) && launch_override(PS_OVERRIDE_KCHUNK2) <= 0) return false;
+// True when the pair kernels can serve these arguments (FP32 plain, or FP64 on the pre-scaled
+// coefficient: the caller checks the mode) and, in FP32, are faster than single steps.  A
+// z-chunk set for the pairs asks for them.
+static bool pairs_ok(Grid3 g, int dtype, const void *T, const void *T2, const void *Ci, bool states = false) {
+    if (dtype == PS_F32 && !pairs_pay(g, states) && launch_override(PS_OVERRIDE_KCHUNK2) <= 0) return false;
     return zmarch2_supported(g, elem_bytes(dtype), T, T2, Ci) &&
            zmarch2_supported(g, elem_bytes(dtype), T2, T, Ci);
 }
@@ -214,10 +211,11 @@ static cudaError_t enqueue_step2(void *T2, const void *T, const void *Ci, StepCo
     return launch_step2_f32((float *)T2, (const float *)T, (const float *)Ci, c, g, s);
 }
 
-// Boundary copy followed by nt steps with alternating buffers.  With
-// PS_RUN_TEMPORAL2 the steps go in fused pairs; when the number of passes would
-// leave the result in the other buffer than nt's parity says, one pair is run
-// as two single steps.
+// Boundary copy followed by nt steps with alternating buffers.  The steps go in fused pairs
+// with PS_RUN_TEMPORAL2, and in FP32 wherever pairs are faster; as many as leave T(nt) in the
+// buffer that nt's parity says (an even number), the rest as single steps.  Without the flag
+// the last step is a single one, so that the other buffer ends with T(nt-1) as it does when
+// every step is.
 // `comp` (PS_RUN_COMPENSATED): two correction fields, comp[0, n) paired with T and
 // comp[n, 2n) with T2; their boundaries are copied like T's.
 static cudaError_t enqueue_run(void *T, void *T2, void *comp, const void *Ci, StepCoef c, Grid3 g,
@@ -225,15 +223,13 @@ static cudaError_t enqueue_run(void *T, void *T2, void *comp, const void *Ci, St
     cudaError_t e = launch_copy_boundary(T2, T, g, elem_bytes(dtype), s);
     float *EA = (float *)comp, *EB = comp ? (float *)comp + g.n() : nullptr;
     if (comp && e == cudaSuccess) e = launch_copy_boundary(EB, EA, g, 4, s);
-    int pairs = 0, singles = nt;
-    if ((flags & PS_RUN_TEMPORAL2) && temporal2_ok(g, dtype, T, T2, Ci)) {
-        pairs = nt / 2;
-        singles = nt & 1;
-        if (((pairs + singles) & 1) != (nt & 1)) {
-            pairs -= 1;
-            singles += 2;
-        }
-    }
+    const bool asked = (flags & PS_RUN_TEMPORAL2) != 0;
+    const bool may = asked || (dtype == PS_F32 && !(flags & PS_RUN_COMPENSATED) &&
+                               launch_override(PS_OVERRIDE_KCHUNK) <= 0 &&
+                               launch_override(PS_OVERRIDE_STEP_PLAIN) != 1);
+    int pairs = 0;
+    if (may && pairs_ok(g, dtype, T, T2, Ci)) pairs = (asked ? nt : nt - 1) / 4 * 2;
+    const int singles = nt - 2 * pairs;
     for (int it = 0; it < pairs + singles && e == cudaSuccess; ++it) {
         void *src = (it & 1) ? T2 : T;
         void *dst = (it & 1) ? T : T2;
@@ -350,7 +346,8 @@ int ps_device_error(unsigned *out_host, int clear) {
     *out_host = zmarch_device_error(clear != 0) | adjoint_device_error(clear != 0) |
                 adjoint_scaled_device_error(clear != 0) | zmarch2_device_error(clear != 0) |
                 adjoint_f32_device_error(clear != 0) | batch_device_error(clear != 0) |
-                batch_zmarch_device_error(clear != 0);
+                batch_zmarch_device_error(clear != 0) |
+                zpair_device_error(clear != 0);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "ps_device_error");
     return PS_OK;
@@ -369,8 +366,8 @@ const char *ps_diffusion3d_step_kernel(const void *T2, const void *T, const void
                                        double dt, double _dx, double _dy, double _dz, int64_t nx,
                                        int64_t ny, int64_t nz, int dtype, unsigned flags) {
     const Grid3 g{nx, ny, nz};
-    if ((flags & PS_RUN_TEMPORAL2) && temporal2_ok(g, dtype, T, T2, Ci)) {
-        if (dtype == PS_F32 && !(flags & PS_RUN_COMPENSATED)) return "k_zmarch2<F32>";
+    if ((flags & PS_RUN_TEMPORAL2) && pairs_ok(g, dtype, T, T2, Ci)) {
+        if (dtype == PS_F32 && !(flags & PS_RUN_COMPENSATED)) return "k_zpair<F32>";
         if (dtype == PS_F64 && (flags & PS_RUN_CI_SCALED)) return "k_zmarch2<F64_SCALED>";
     }
     if (dtype == PS_F64)
@@ -515,11 +512,11 @@ static int plan_states(int nt, int every, bool pairs, std::vector<StatesOp> *ops
 }
 
 // Whether a state-keeping loop's single steps may take the column kernel on a small grid.
-// FP32 only up to 2.2 million nodes: beyond, pairs that write both states are faster, and
+// Aligned FP32 rows only up to 2.2 million nodes: beyond, pairs that write both states are faster, and
 // beside a reverse sweep the march's few CTAs leave the transposed steps more of each SM
 // (192^3, nt = 64, checkpoints every 8: the gradient 3.87 ms, 4.28 with the column kernel).
 static bool states_column(int dtype, Grid3 g) {
-    return dtype == PS_F64 || (double)g.n() <= 2.2e6;
+    return dtype == PS_F64 || g.nx % 4 != 0 || (double)g.n() <= 2.2e6;
 }
 
 // Whether PS_RUN_TEMPORAL2 runs fused pairs for this state-keeping loop (at least two
@@ -527,8 +524,8 @@ static bool states_column(int dtype, Grid3 g) {
 // stride, so T0 and the first two grids decide).
 static bool states_pairs(unsigned flags, int dtype, int nt, Grid3 g, const void *T0, const void *grid0,
                          const void *grid1, const void *Ci) {
-    return (flags & PS_RUN_TEMPORAL2) && dtype == PS_F32 && nt >= 2 && temporal2_ok(g, dtype, T0, grid0, Ci, true) &&
-           temporal2_ok(g, dtype, grid0, grid1, Ci, true);
+    return (flags & PS_RUN_TEMPORAL2) && dtype == PS_F32 && nt >= 2 && pairs_ok(g, dtype, T0, grid0, Ci, true) &&
+           pairs_ok(g, dtype, grid0, grid1, Ci, true);
 }
 
 static cudaError_t enqueue_run_states(const void *T0, char *base, int64_t grid_stride, size_t esz, int every,
@@ -537,20 +534,25 @@ static cudaError_t enqueue_run_states(const void *T0, char *base, int64_t grid_s
     const int nslots = nt / every, nwork = (every > 1 && nt > 0) ? 2 : 0;
     auto grid = [&](int slot) { return (void *)(base + (size_t)slot * (size_t)grid_stride * esz); };
     auto slot_grid = [&](int slot) { return slot >= 0 ? grid(slot) : grid(nslots + (-1 - slot)); };
-    // The boundary of every grid this call writes is T0's.  The steps store the x and y faces
-    // themselves (beside their own row stores), so only the two z faces of each grid are
-    // copied here.
+    // The boundary of every grid this call writes is T0's.  Where the march serves the steps
+    // they store the x and y faces themselves (in their own row stores), so only the two z
+    // faces of each grid are copied here; else the whole boundary is.
+    const bool scaled = (flags & PS_RUN_CI_SCALED) != 0, native = (flags & PS_RUN_NATIVE_F64) != 0;
+    const bool in_loop = states_column(dtype, g);
     const int ngrids = nslots + nwork;
+    bool steps_bnd = true;
+    for (int k = 0; k < ngrids && steps_bnd; ++k)
+        steps_bnd = step_takes_march(dtype, scaled, native, in_loop, c, g, grid(k), T0, Ci) &&
+                    step_takes_march(dtype, scaled, native, in_loop, c, g, grid(k), grid(k), Ci);
     // PS_RUN_TEMPORAL2 (FP32): fused pairs.  With every = 1 they keep both states and
     // store both states' x and y faces; with every > 1 they keep only their second state
     // and write interior nodes only, so the whole boundary is copied then.
     const bool pairs = ngrids >= 2 && states_pairs(flags, dtype, nt, g, T0, grid(0), grid(1), Ci);
-    const bool faces_by_steps = !(pairs && every > 1);
+    const bool faces_by_steps = steps_bnd && !(pairs && every > 1);
     if (nt > 0 && ngrids > 0) {
         cudaError_t e = launch_copy_boundary_many(base, ngrids, grid_stride, T0, g, (int)esz, s, faces_by_steps);
         if (e != cudaSuccess) return e;
     }
-    const bool in_loop = states_column(dtype, g);
     std::vector<StatesOp> ops;
     plan_states(nt, every, pairs, &ops);
     const void *cur = T0;

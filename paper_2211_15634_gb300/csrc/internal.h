@@ -43,22 +43,26 @@ int api_fail(int status, const char *msg);
 int api_cuda_fail(cudaError_t e, const char *where);
 
 // ---- forward step kernels (step_f64.cu, step_f32.cu) ----
-// write_bnd: the step also stores the x and y boundary nodes of planes 1 .. nz-2 as copies
-// of T's.  in_loop: one step of a time loop, which may take the column kernel on a small grid
-// (bit for bit the same).
+// in_loop: one step of a time loop, which may take the column kernel on a small grid (bit for
+// bit the same).  write_bnd: where the TMA march serves the step (step_takes_march) it also
+// stores the x and y boundary nodes of planes 1 .. nz-2 as copies of T's.
 cudaError_t launch_step_f64_native(double *T2, const double *T, const double *Ci, StepCoef c,
-                                   Grid3 g, cudaStream_t s, bool write_bnd = false);
+                                   Grid3 g, cudaStream_t s);
 cudaError_t launch_step_f64_fast(double *T2, const double *T, const double *Ci, StepCoef c,
                                  Grid3 g, cudaStream_t s, bool write_bnd = false, bool in_loop = false);
 cudaError_t launch_step_f32(float *T2, const float *T, const float *Ci, StepCoef c, Grid3 g,
                             cudaStream_t s, bool write_bnd = false, bool in_loop = false);
+// True when the one-step launcher for these arguments takes the TMA march (aligned or ragged
+// rows), so that write_bnd is honoured; scaled = PS_RUN_CI_SCALED, native = PS_RUN_NATIVE_F64.
+bool step_takes_march(int dtype, bool scaled, bool native, bool in_loop, StepCoef c, Grid3 g, const void *T2,
+                      const void *T, const void *Ci);
 // compensated FP32 step on the two-float state (T, E) -> (T2, E2)
 cudaError_t launch_step_f32_comp(float *T2, const float *T, float *E2, const float *E, const float *Ci,
                                  StepCoef c, Grid3 g, cudaStream_t s, bool in_loop = false);
 cudaError_t launch_step_f64_scaled(double *T2, const double *T, const double *Cs, Grid3 g,
                                    cudaStream_t s, bool write_bnd = false, bool in_loop = false);
 cudaError_t launch_scale_ci(double *Cs, const double *Ci, double K, int64_t n, cudaStream_t s);
-// two steps per pass (zmarch2.cu): T2 = step(step(T)); the caller checks zmarch2_supported
+// two steps per pass (FP32 zpair.cu, FP64 zmarch2.cu): T2 = step(step(T)); the caller checks zmarch2_supported
 // (the same preconditions as the one-step TMA kernel)
 bool zmarch2_supported(Grid3 g, int esz, const void *a, const void *b, const void *c);
 cudaError_t launch_step2_f32(float *T2, const float *T, const float *Ci, StepCoef c, Grid3 g,
@@ -70,6 +74,7 @@ cudaError_t launch_step2_f64_scaled(double *T2, const double *T, const double *C
 cudaError_t launch_step2_states_f32(float *T1o, float *T2, const float *T, const float *Ci, StepCoef c,
                                     Grid3 g, cudaStream_t s);
 unsigned zmarch2_device_error(bool clear);
+unsigned zpair_device_error(bool clear);
 const char *step_f64_kernel_name(Grid3 g, const void *T2, const void *T, const void *Ci, StepCoef c,
                                  bool scaled);
 const char *step_f32_kernel_name(Grid3 g, const void *T2, const void *T, const void *Ci);

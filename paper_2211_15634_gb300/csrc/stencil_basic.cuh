@@ -10,6 +10,8 @@
 // 4.3 / 2.2, 96^3 4.4 / 3.6, 160^3 10.9 / 8.8, 192^3 14.3 / 13.7, 208^3 19 / 22.  And grids
 // that the march cannot take (2^31 nodes and more on ragged rows, spacings more than 16
 // apart on odd nx, plain FP64, the two-float step on ragged rows).
+// They never store boundary nodes: x faces stored beside the interior cost more than the
+// boundary copy they save (127^3 FP32 states: 10.1 us a step against 8.3).
 // The next step's CTAs are let in at the end of the march, not at its start: with one wave of
 // CTAs or less they would fill whatever slots are free and leave the SMs unevenly loaded
 // (FP32 160 x 63 x 311: 9.0 us against 7.5).
@@ -30,33 +32,8 @@ struct CoefT {
     F dtlam, ax, ay, az;
 };
 
-// kBnd: the columns beside the x and y faces store T's boundary values of the planes [k0, k1)
-// they have marched (the corners by the column in the corner).  A loop of its own: inside the
-// march it held registers the arithmetic needs (spills at 64).
-template <typename F>
-__device__ __forceinline__ void column_boundary(F *__restrict__ T2, const F *__restrict__ T, int64_t i, int64_t j,
-                                                int64_t k0, int64_t k1, int64_t nx, int64_t ny) {
-    const bool l = i == 1, r = i == nx - 2, d = j == 1, u = j == ny - 2;
-    if (!(l || r || d || u)) return;
-#pragma unroll 1
-    for (int64_t k = k0; k < k1; ++k) {
-        const int64_t p = i + nx * (j + ny * k);
-        auto put = [&](bool on, int64_t q) {
-            if (on) T2[q] = T[q];
-        };
-        put(l, p - 1);
-        put(r, p + 1);
-        put(d, p - nx);
-        put(u, p + nx);
-        put(l && d, p - nx - 1);
-        put(r && d, p - nx + 1);
-        put(l && u, p + nx - 1);
-        put(r && u, p + nx + 1);
-    }
-}
-
 // FP64 data with the one-DFMA emulated arithmetic of emu64.cuh.
-template <int kAx, bool kScaled, bool kBnd>
+template <int kAx, bool kScaled>
 __global__ void __launch_bounds__(256)
 k_step_basic_emu(double *__restrict__ T2, const double *__restrict__ T,
                  const double *__restrict__ Ci, EmuCoef c, int64_t nx, int64_t ny, int64_t nz,
@@ -73,24 +50,22 @@ k_step_basic_emu(double *__restrict__ T2, const double *__restrict__ T,
     int64_t p = i + sy * (j + ny * k0);
     unsigned long long tm = Tb[p - sz], tc = Tb[p];
     for (int64_t k = k0; k < k1; ++k, p += sz) {
-        const unsigned long long tp = Tb[p + sz];
+        const unsigned long long tp = Tb[p + sz], xm = Tb[p - 1], xp = Tb[p + 1], ym = Tb[p - sy], yp = Tb[p + sy];
         if (kScaled)  // Ci holds dt*lam*_d^2*Ci (isotropic grid)
-            T2[p] = emu_step_node_scaled(tc, Tb[p - 1], Tb[p + 1], Tb[p - sy], Tb[p + sy], tm, tp, Ci[p]);
+            T2[p] = emu_step_node_scaled(tc, xm, xp, ym, yp, tm, tp, Ci[p]);
         else
-            T2[p] = emu_step_node<kAx, false>(tc, Tb[p - 1], Tb[p + 1], Tb[p - sy], Tb[p + sy], tm,
-                                               tp, Ci[p], c);
+            T2[p] = emu_step_node<kAx, false>(tc, xm, xp, ym, yp, tm, tp, Ci[p], c);
         tm = tc;
         tc = tp;
     }
     grid_dep_launch();
-    if constexpr (kBnd) column_boundary(T2, T, i, j, k0, k1, nx, ny);
 }
 
 // Fig. 1 step!: T2 = T + dt*lam*Ci*((d2x*_dx^2 + d2y*_dy^2) + d2z*_dz^2) at
 // interior nodes; the z-range of this block is [k0, k1).  FP32: f32_node's roundings.
 // kComp (FP32): the state is the two-float pair (T, E) and (T2, E2) receives the
 // compensated step (comp32_node, node.cuh).
-template <typename F, bool kComp, bool kBnd>
+template <typename F, bool kComp>
 __global__ void __launch_bounds__(256)
 k_step_basic(F *__restrict__ T2, const F *__restrict__ T, F *__restrict__ E2,
              const F *__restrict__ E, const F *__restrict__ Ci, CoefT<F> c, int64_t nx, int64_t ny,
@@ -113,21 +88,22 @@ k_step_basic(F *__restrict__ T2, const F *__restrict__ T, F *__restrict__ E2,
                                 E[p + 1], E[p - sy], E[p + sy], E[p - sz], E[p + sz], Ci[p], c.dtlam,
                                 c.ax, c.ay, c.az, &e2);
             E2[p] = e2;
-        } else if constexpr (sizeof(F) == 4) {
-            T2[p] = f32_node(tc, T[p - 1], T[p + 1], T[p - sy], T[p + sy], tm, tp, Ci[p], c.dtlam, c.ax, c.ay,
-                             c.az);
         } else {
-            const F d2x = (T[p + 1] - tc) - (tc - T[p - 1]);
-            const F d2y = (T[p + sy] - tc) - (tc - T[p - sy]);
-            const F d2z = (tp - tc) - (tc - tm);
-            const F lap = (d2x * c.ax + d2y * c.ay) + d2z * c.az;
-            T2[p] = tc + c.dtlam * (Ci[p] * lap);
+            const F xm = T[p - 1], xp = T[p + 1], ym = T[p - sy], yp = T[p + sy];
+            if constexpr (sizeof(F) == 4) {
+                T2[p] = f32_node(tc, xm, xp, ym, yp, tm, tp, Ci[p], c.dtlam, c.ax, c.ay, c.az);
+            } else {
+                const F d2x = (xp - tc) - (tc - xm);
+                const F d2y = (yp - tc) - (tc - ym);
+                const F d2z = (tp - tc) - (tc - tm);
+                const F lap = (d2x * c.ax + d2y * c.ay) + d2z * c.az;
+                T2[p] = tc + c.dtlam * (Ci[p] * lap);
+            }
         }
         tm = tc;
         tc = tp;
     }
     grid_dep_launch();
-    if constexpr (kBnd) column_boundary(T2, T, i, j, k0, k1, nx, ny);
 }
 
 // Launch shape of the column kernels: 32 x 8 columns per CTA and kchunk planes.  false: the
@@ -161,36 +137,28 @@ inline bool column_shape(int64_t nx, int64_t ny, int64_t nz, bool f32, bool smal
 
 template <int kAx, bool kScaled>
 inline cudaError_t launch_basic_emu_t(double *T2, const double *T, const double *Ci, const EmuCoef &c, Grid3 g,
-                                      cudaStream_t s, bool write_bnd, bool small) {
+                                      cudaStream_t s, bool small) {
     dim3 grid;
     int kc;
     if (!column_shape(g.nx, g.ny, g.nz, false, small, &grid, &kc)) return cudaErrorInvalidConfiguration;
-    if (write_bnd)
-        return launch_pdl(k_step_basic_emu<kAx, kScaled, true>, grid, dim3(32, 8), 0, s, T2, T, Ci, c, g.nx, g.ny,
-                          g.nz, kc);
-    return launch_pdl(k_step_basic_emu<kAx, kScaled, false>, grid, dim3(32, 8), 0, s, T2, T, Ci, c, g.nx, g.ny,
-                      g.nz, kc);
+    return launch_pdl(k_step_basic_emu<kAx, kScaled>, grid, dim3(32, 8), 0, s, T2, T, Ci, c, g.nx, g.ny, g.nz, kc);
 }
 
 inline cudaError_t launch_step_basic_emu(double *T2, const double *T, const double *Ci, const EmuCoef &c, bool iso,
-                                         Grid3 g, cudaStream_t s, bool scaled, bool write_bnd, bool small) {
-    if (scaled) return launch_basic_emu_t<AX_ISO, true>(T2, T, Ci, c, g, s, write_bnd, small);
-    if (iso) return launch_basic_emu_t<AX_ISO, false>(T2, T, Ci, c, g, s, write_bnd, small);
-    if (c.common) return launch_basic_emu_t<AX_COMMON, false>(T2, T, Ci, c, g, s, write_bnd, small);
-    return launch_basic_emu_t<AX_FAR, false>(T2, T, Ci, c, g, s, write_bnd, small);
+                                         Grid3 g, cudaStream_t s, bool scaled, bool small) {
+    if (scaled) return launch_basic_emu_t<AX_ISO, true>(T2, T, Ci, c, g, s, small);
+    if (iso) return launch_basic_emu_t<AX_ISO, false>(T2, T, Ci, c, g, s, small);
+    if (c.common) return launch_basic_emu_t<AX_COMMON, false>(T2, T, Ci, c, g, s, small);
+    return launch_basic_emu_t<AX_FAR, false>(T2, T, Ci, c, g, s, small);
 }
 
 template <typename F, bool kComp>
 cudaError_t launch_step_basic(F *T2, const F *T, F *E2, const F *E, const F *Ci, CoefT<F> c, Grid3 g,
-                              cudaStream_t s, bool write_bnd, bool small) {
+                              cudaStream_t s, bool small) {
     dim3 grid;
     int kc;
     if (!column_shape(g.nx, g.ny, g.nz, sizeof(F) == 4 && !kComp, small, &grid, &kc)) return cudaErrorInvalidConfiguration;
-    if (!kComp && write_bnd)
-        return launch_pdl(k_step_basic<F, kComp, !kComp>, grid, dim3(32, 8), 0, s, T2, T, E2, E, Ci, c, g.nx, g.ny,
-                          g.nz, kc);
-    return launch_pdl(k_step_basic<F, kComp, false>, grid, dim3(32, 8), 0, s, T2, T, E2, E, Ci, c, g.nx, g.ny, g.nz,
-                      kc);
+    return launch_pdl(k_step_basic<F, kComp>, grid, dim3(32, 8), 0, s, T2, T, E2, E, Ci, c, g.nx, g.ny, g.nz, kc);
 }
 
 }  // namespace psd

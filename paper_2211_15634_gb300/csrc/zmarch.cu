@@ -150,9 +150,10 @@ bool step_small(Grid3 g, int mode) {
         case Z_F32:  // full rows 5e5 nodes 3.0 / 2.9, 1e6 4.1 / 3.7; 192^3 13.1 / 14.3, 200^3 16 / 16;
                      // ragged 205^3 20.8 / 21.7, 211^3 25.5 / 23.8
             return n <= (aligned ? (full ? 6e5 : 7.5e6) : 8.8e6);
-        case Z_F32_COMP:  // 160^3 14 / 19, 176^3 25 / 25; ragged rows have no march: only the
-                          // column kernel's chunks differ (343 x 96 x 95: 12.0 us, long ones 11.6)
-            return n <= (aligned ? 4.3e6 : 2.5e6);
+        case Z_F32_COMP:  // 160^3 14 / 19, 176^3 25 / 25; full rows 128^3 9.4 / 10.9, 368 x 112 x 72
+                          // 12.0 / 10.8; ragged rows have no march: only the column
+                          // kernel's chunks differ (343 x 96 x 95: 12.0 us, long ones 11.6)
+            return n <= (aligned ? (full ? 2.2e6 : 4.3e6) : 2.5e6);
         case Z_F64_EMU_ANISO:  // 192^3 37 / 41, 200^3 53 / 49; ragged 219^3 61 / 64, 227^3 71 / 69
             return n <= (aligned ? 7.5e6 : 1.05e7);
         default: {

@@ -43,6 +43,9 @@ bool make_tensor_map_rows(CUtensorMap *m, const void *ptr, int esz, int64_t n, i
 // Grids whose steps inside a time loop take the column kernels (stencil_basic.cuh); mode:
 // Z_F32, Z_F32_COMP, Z_F64_SCALED or Z_F64_EMU_ANISO (any unequal spacings).
 bool step_small(Grid3 g, int mode);
+// Whether fused FP32 pairs (zpair.cu) beat single steps in a loop on this grid; states: a
+// loop that keeps every state.
+bool pairs_pay(Grid3 g, bool states);
 // 3-D tiled tensor map over a (nz, ny, nx) field with a bx x by x 1 box.
 bool make_tensor_map_3d(CUtensorMap *m, const void *ptr, int esz, Grid3 g, unsigned bx, unsigned by);
 // The same over a grid whose rows are `pitch` elements apart (pitch*esz a multiple of 16).

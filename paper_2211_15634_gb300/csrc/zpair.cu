@@ -1,0 +1,413 @@
+// FP32 steps fused in pairs over a single grid: T2 = step(step(T)) in one pass, one read of T
+// and Ci and one write of T2 (temporal blocking of depth 2).
+//
+// What binds.  One step at a time moves 12 bytes per node (228 us at 512^3, the copy rate).
+// A pair moves the same for two steps, so it must not cost more than about 60 instructions
+// per node to stay with the memory.  A thread therefore steps eight nodes (four along x in each
+// of two rows) with packed FP32 arithmetic (f32x2, the same roundings as f32_node), shares the
+// first differences along x between neighbours and along z between planes, and its loop's own
+// instructions count for eight nodes.  Measured (us a step): 512^3 134.5, 384^3 59.9, 256^3
+// 19.5, where the four-node form with a scalar ring around the tile (zmarch2_tile.cuh, 83
+// instructions per node and pass against 53) took 179, 82.8 and 27.6.  Four nodes per thread
+// with halo rows and columns in whole warps and lanes took 188 at 512^3 (the 120 columns that
+// leaves waste a seventh of the lanes), and passes of three and four steps in that form 215
+// and 372 per step's share: more levels cost more instructions than the memory they save.
+//
+// Layout.  A CTA owns 128 x BY output nodes and a chunk of planes [k0, k1).  Warp w steps rows
+// 2w and 2w+1 of the BY + 2 rows from Y0-1; level 1 (the state after one step) is formed on all
+// of them, level 2 stored from the inner BY.  Iteration z steps level 1 at plane z+1 and level 2
+// at plane z: a node itself and its z-neighbours are the thread's registers, the x-neighbours
+// the thread's or its neighbour lanes' (shuffles), the y-neighbours the thread's other row or
+// shared memory - T's plane in its stage, level 1's tile of plane z, written one iteration
+// earlier (two slots).  Level 1 in the columns beside the tile (X0-1 and X0+128) is formed
+// by one more warp, a row per lane.  One barrier per iteration.  T plane q (BY + 4 rows) and
+// Ci plane q-1 (BY + 2 rows) arrive by TMA in one stage on one mbarrier, used in iterations
+// q-2 and (T's x- and y-neighbours) q-1; Ci moves to level 2 in registers.
+// Nodes that are not interior have their Ci replaced by zero, which keeps their value: they are
+// never stored, and a non-finite value of theirs can only come from, and only reaches, the one
+// interior node beside them.  (kStates stores them, so there they are selected.)
+#include <cudaTypedefs.h>
+
+#include "internal.h"
+#include "node.cuh"
+#include "pdl.cuh"
+#include "tma.cuh"
+#include "zmarch.h"
+
+namespace psd {
+
+__device__ unsigned g_zpair_error;  // set when an mbarrier wait times out
+
+struct ZPairParams {
+    int nx, ny, nz, kchunk, ntx;
+    float dtlam, ax, ay, az;
+};
+
+// Two FP32 values in one 64-bit register pair, one instruction for both.
+using f2 = unsigned long long;
+__device__ __forceinline__ f2 f2_make(float a, float b) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float f2_lo(f2 v) { return __uint_as_float((unsigned)v); }
+__device__ __forceinline__ float f2_hi(f2 v) { return __uint_as_float((unsigned)(v >> 32)); }
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// a - b as a fused multiply-add by -1: one rounding, the difference's (sub.f32x2 was slower)
+__device__ __forceinline__ f2 f2_sub(f2 a, f2 b) { return f2_fma(b, 0xbf800000bf800000ull, a); }
+
+struct V4 {  // four nodes of a row
+    f2 a, b;
+};
+__device__ __forceinline__ V4 v4_load(const float *p) {
+    const ulonglong2 v = *(const ulonglong2 *)p;
+    return V4{v.x, v.y};
+}
+__device__ __forceinline__ void v4_store(float *p, V4 v) { *(ulonglong2 *)p = make_ulonglong2(v.a, v.b); }
+__device__ __forceinline__ V4 v4_sub(V4 x, V4 y) { return V4{f2_sub(x.a, y.a), f2_sub(x.b, y.b)}; }
+__device__ __forceinline__ V4 v4_select(const bool (&m)[4], V4 x, V4 y) {
+    return V4{f2_make(m[0] ? f2_lo(x.a) : f2_lo(y.a), m[1] ? f2_hi(x.a) : f2_hi(y.a)),
+              f2_make(m[2] ? f2_lo(x.b) : f2_lo(y.b), m[3] ? f2_hi(x.b) : f2_hi(y.b))};
+}
+
+struct ZCoef2 {
+    f2 dtlam, ax, ay, az;
+};
+
+// f32_node of four neighbouring nodes: c the centres, left / right the values beside them, up /
+// dn the rows above and below, en = zp - c and eo = c - zm the differences along z.
+__device__ __forceinline__ V4 v4_step(V4 c, float left, float right, V4 up, V4 dn, V4 en, V4 eo, V4 ci,
+                                      const ZCoef2 &k) {
+    const float c0 = f2_lo(c.a), c1 = f2_hi(c.a), c2 = f2_lo(c.b), c3 = f2_hi(c.b);
+    const float d0 = __fsub_rn(c0, left), d1 = __fsub_rn(c1, c0), d2 = __fsub_rn(c2, c1), d3 = __fsub_rn(c3, c2),
+                d4 = __fsub_rn(right, c3);
+    const f2 xa = f2_make(__fsub_rn(d1, d0), __fsub_rn(d2, d1)), xb = f2_make(__fsub_rn(d3, d2), __fsub_rn(d4, d3));
+    const V4 y = v4_sub(v4_sub(dn, c), v4_sub(c, up)), z = v4_sub(en, eo);
+    const f2 la = f2_fma(z.a, k.az, f2_fma(y.a, k.ay, f2_mul(xa, k.ax)));
+    const f2 lb = f2_fma(z.b, k.az, f2_fma(y.b, k.ay, f2_mul(xb, k.ax)));
+    return V4{f2_fma(k.dtlam, f2_mul(ci.a, la), c.a), f2_fma(k.dtlam, f2_mul(ci.b, lb), c.b)};
+}
+
+template <int BY>
+struct ZPair {
+    static constexpr int BX = 128, W = BX + 8, ROWS = BY + 2, TROWS = BY + 4, NW = ROWS / 2;
+    static_assert(BY % 2 == 0 && ROWS <= 16, "two rows per warp, a halo row per lane of half a warp");
+    static constexpr unsigned TB = (TROWS * W * 4 + 127) / 128 * 128, CB = (ROWS * W * 4 + 127) / 128 * 128;
+    static constexpr unsigned SB = TB + CB, LB = CB;  // stage, level-1 tile slot
+    static constexpr int NTH = 32 * (NW + 1);
+};
+
+// kStates: level 1 goes to T1o too, and T1o and T2 are written at every node of the output
+// rows, boundary nodes as T's.
+template <int BY, int NST, int MINB, bool kStates>
+__global__ void __launch_bounds__(ZPair<BY>::NTH, MINB)
+k_zpair(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmC, float *__restrict__ T2,
+        const ZPairParams p, float *__restrict__ T1o) {
+    using Z = ZPair<BY>;
+    constexpr int W = Z::W, ROWS = Z::ROWS, NW = Z::NW;
+    constexpr int LBF = Z::LB / 4, CF = Z::TB / 4;
+    extern __shared__ __align__(128) unsigned char smem[];
+    float *tiles = (float *)(smem + NST * Z::SB);  // level 1 of plane q in slot q % 2
+    uint64_t *bar = (uint64_t *)(smem + NST * Z::SB + 2 * Z::LB);
+    __shared__ int s_abort;
+    grid_dep_wait();  // the previous launch's writes (and its reads of T2) are complete
+    grid_dep_launch();
+
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int nx = p.nx, ny = p.ny, nz = p.nz;
+    const int X0 = (int)(blockIdx.x % p.ntx) * Z::BX, Y0 = (int)(blockIdx.x / p.ntx) * BY;
+    const int k0 = 1 + (int)blockIdx.y * p.kchunk, k1 = min(k0 + p.kchunk, nz - 1);  // output planes
+
+    // stage j % NST: T plane k0 - 2 + j, and for j >= 2 Ci plane k0 - 3 + j
+    const int jmax = k1 - k0 + 3;
+    auto issue = [&](int j) {
+        const int s = j % NST, q = k0 - 2 + j;
+        unsigned char *st = smem + s * Z::SB;
+        mbar_expect_tx(&bar[s], Z::TROWS * W * 4 + (j >= 2 ? ROWS * W * 4 : 0));
+        tma_load_3d(st, &tmT, &bar[s], X0 - 4, Y0 - 2, q);
+        if (j >= 2) tma_load_3d(st + Z::TB, &tmC, &bar[s], X0 - 4, Y0 - 1, q - 1);
+    };
+    if (threadIdx.x == 0) {
+        s_abort = 0;
+        for (int s = 0; s < NST; ++s) mbar_init(&bar[s], 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int j = 0; j < NST && j <= jmax; ++j) issue(j);
+    // After a timed-out wait: bounded waits for the copies still in flight (stages up to j),
+    // so that no TMA write lands after the CTA exits.
+    auto drain = [&](int j) {
+        for (int i = max(0, j - NST + 1); i <= j; ++i) mbar_wait(&bar[i % NST], (unsigned)(i / NST) & 1u);
+    };
+    bool ok = mbar_wait(&bar[0], 0u);
+    ok = mbar_wait(&bar[1], 0u) && ok;
+    int s1 = 1 % NST, s0 = 2 % NST;  // stages of T planes z+1 and z+2 (and Ci plane z+1)
+    unsigned par = 3u;               // parity of each stage's next completion
+    const int zfirst = k0 - 2;       // level 1 from plane k0 - 1 on
+
+    if (w == NW) {
+        // ---- the halo warp: level 1 at column X0-1 (lanes 0-15) and X0+128 (lanes 16-31),
+        // tile row lane % 16
+        const int r = min(lane & 15, ROWS - 1), hc = lane < 16 ? 3 : 4 + Z::BX;  // box column
+        const int x = X0 - 4 + hc, y = Y0 - 1 + r;
+        const bool in = x >= 1 && x <= nx - 2 && y >= 1 && y <= ny - 2;
+        const bool put = (lane & 15) < ROWS;
+        const int o = (r + 1) * W + hc;  // the node in a T box
+        float c = ((const float *)(smem + Z::SB))[o], e = __fsub_rn(c, ((const float *)smem)[o]);
+        __syncthreads();  // stage 0 is read
+        int j = 2;
+        for (int z = zfirst; z < k1; ++z, ++j) {
+            ok = mbar_wait(&bar[s0], (par >> s0) & 1u) && ok;
+            par ^= 1u << s0;
+            const float *t0 = (const float *)(smem + s0 * Z::SB), *t1 = (const float *)(smem + s1 * Z::SB);
+            const float zp = t0[o], en = __fsub_rn(zp, c), ci = t0[CF + r * W + hc];
+            const float d2x = __fsub_rn(__fsub_rn(t1[o + 1], c), __fsub_rn(c, t1[o - 1]));
+            const float d2y = __fsub_rn(__fsub_rn(t1[o + W], c), __fsub_rn(c, t1[o - W]));
+            const float lap = __fmaf_rn(__fsub_rn(en, e), p.az, __fmaf_rn(d2y, p.ay, __fmul_rn(d2x, p.ax)));
+            const float v = __fmaf_rn(p.dtlam, __fmul_rn(ci, lap), c);
+            if (put) tiles[((z + 1) & 1) * LBF + r * W + hc] = in && z + 1 >= 1 && z + 1 <= nz - 2 ? v : c;
+            e = en;
+            c = zp;
+            if (!ok) {
+                s_abort = 1;
+                atomicOr(&g_zpair_error, 1u);
+            }
+            __syncthreads();
+            if (s_abort) return;  // warp 0 waits for the copies in flight
+            s1 = s0;
+            s0 = s0 + 1 == NST ? 0 : s0 + 1;
+        }
+        return;
+    }
+
+    // ---- rows ra = 2w and ra + 1 of the stepped rows (T box rows one more)
+    const int ra = 2 * w, gya = Y0 - 1 + ra, gx0 = X0 + 4 * lane;
+    const bool ina = gya >= 1 && gya <= ny - 2, inb = gya + 1 >= 1 && gya + 1 <= ny - 2;
+    const bool xedge = X0 == 0 || X0 + Z::BX > nx - 1;  // CTA-uniform: x boundary nodes in the tile
+    bool in[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) in[i] = gx0 + i >= 1 && gx0 + i <= nx - 2;
+    const bool outa = w > 0 && (kStates ? gya <= ny - 1 : ina);
+    const bool outb = w < NW - 1 && (kStates ? gya + 1 <= ny - 1 : inb);
+    const ZCoef2 k{f2_make(p.dtlam, p.dtlam), f2_make(p.ax, p.ax), f2_make(p.ay, p.ay), f2_make(p.az, p.az)};
+    const int oT = (ra + 1) * W + 4 + 4 * lane, oC = ra * W + 4 + 4 * lane;  // own nodes in a T box, in a Ci box or tile
+    const int up1 = max(ra - 1, 0) * W + 4 + 4 * lane, dn1 = min(ra + 2, ROWS - 1) * W + 4 + 4 * lane;
+    const bool eL = lane == 0, eR = lane == 31;
+    const int oE = eR ? 4 : -1;  // from the own nodes to the value beside the tile (lanes 0, 31)
+
+    V4 ca, cb, ea, eb;  // level 0 of plane z+1, and its difference to plane z
+    {
+        const float *t0 = (const float *)smem, *t1 = (const float *)(smem + Z::SB);
+        ca = v4_load(t1 + oT);
+        cb = v4_load(t1 + oT + W);
+        ea = v4_sub(ca, v4_load(t0 + oT));
+        eb = v4_sub(cb, v4_load(t0 + oT + W));
+    }
+    V4 c1a{0ull, 0ull}, c1b = c1a, e1a = c1a, e1b = c1a;  // level 1 of plane z, difference to z-1
+    V4 cia = c1a, cib = c1a;                               // Ci of plane z
+    __syncthreads();  // stage 0 (own rows only) is read
+    if (threadIdx.x == 0 && NST <= jmax) issue(NST);
+
+    // x-neighbours of a row held in registers; f: the row's own nodes in shared memory, whose
+    // columns beside the tile lanes 0 and 31 read
+    auto beside = [&](V4 v, const float *f, float &left, float &right) {
+        float h = 0.f;
+        if (eL || eR) h = f[oE];
+        left = __shfl_up_sync(0xffffffffu, f2_hi(v.b), 1);
+        right = __shfl_down_sync(0xffffffffu, f2_lo(v.a), 1);
+        left = eL ? h : left;
+        right = eR ? h : right;
+    };
+    int64_t base = (int64_t)gx0 + (int64_t)nx * ((int64_t)gya + (int64_t)ny * zfirst);
+    const int64_t plane = (int64_t)nx * ny;
+    int j = 2;
+#pragma unroll 2
+    for (int z = zfirst; z < k1; ++z, ++j, base += plane) {
+        ok = mbar_wait(&bar[s0], (par >> s0) & 1u) && ok;
+        par ^= 1u << s0;
+        const float *t0 = (const float *)(smem + s0 * Z::SB), *t1 = (const float *)(smem + s1 * Z::SB);
+        float *const w1 = tiles + ((z + 1) & 1) * LBF;     // level 1 of plane z+1
+        const float *const w0 = tiles + (z & 1) * LBF;     // and of plane z
+        // level 1 of plane z+1
+        const V4 za = v4_load(t0 + oT), zb = v4_load(t0 + oT + W);
+        V4 na = v4_load(t0 + CF + oC), nb = v4_load(t0 + CF + oC + W);  // Ci of plane z+1
+        const bool zin = z + 1 >= 1 && z + 1 <= nz - 2;
+        if (!kStates) {
+            if (!(ina && zin)) na = V4{0ull, 0ull};
+            if (!(inb && zin)) nb = V4{0ull, 0ull};
+            if (xedge) {
+                na = v4_select(in, na, V4{0ull, 0ull});
+                nb = v4_select(in, nb, V4{0ull, 0ull});
+            }
+        }
+        const V4 ena = v4_sub(za, ca), enb = v4_sub(zb, cb);
+        float la, ra_, lb, rb_;
+        beside(ca, t1 + oT, la, ra_);
+        beside(cb, t1 + oT + W, lb, rb_);
+        V4 oa = v4_step(ca, la, ra_, v4_load(t1 + oT - W), cb, ena, ea, na, k);
+        V4 ob = v4_step(cb, lb, rb_, ca, v4_load(t1 + oT + 2 * W), enb, eb, nb, k);
+        if constexpr (kStates) {
+            if (!(ina && zin)) oa = ca;
+            if (!(inb && zin)) ob = cb;
+            if (xedge) {
+                oa = v4_select(in, oa, ca);
+                ob = v4_select(in, ob, cb);
+            }
+        }
+        v4_store(w1 + oC, oa);
+        v4_store(w1 + oC + W, ob);
+        ca = za;
+        cb = zb;
+        ea = ena;
+        eb = enb;
+        // level 2 of plane z
+        const V4 fna = v4_sub(oa, c1a), fnb = v4_sub(ob, c1b);
+        if (z >= k0) {
+            beside(c1a, w0 + oC, la, ra_);
+            beside(c1b, w0 + oC + W, lb, rb_);
+            V4 ya = v4_step(c1a, la, ra_, v4_load(w0 + up1), c1b, fna, e1a, cia, k);
+            V4 yb = v4_step(c1b, lb, rb_, c1a, v4_load(w0 + dn1), fnb, e1b, cib, k);
+            if constexpr (kStates) {
+                if (!ina) ya = c1a;
+                if (!inb) yb = c1b;
+                if (xedge) {
+                    ya = v4_select(in, ya, c1a);
+                    yb = v4_select(in, yb, c1b);
+                }
+                auto put = [&](float *t, V4 v) {
+                    if (gx0 + 3 <= nx - 1) {
+                        v4_store(t, v);
+                    } else {
+                        const float o4[4] = {f2_lo(v.a), f2_hi(v.a), f2_lo(v.b), f2_hi(v.b)};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if (gx0 + i <= nx - 1) t[i] = o4[i];
+                    }
+                };
+                if (outa) {
+                    put(T1o + base, c1a);
+                    put(T2 + base, ya);
+                }
+                if (outb) {
+                    put(T1o + base + nx, c1b);
+                    put(T2 + base + nx, yb);
+                }
+            } else {
+                auto put = [&](float *t, V4 v) {
+                    if (!xedge || (in[0] && in[3])) {
+                        v4_store(t, v);
+                    } else {
+                        const float o4[4] = {f2_lo(v.a), f2_hi(v.a), f2_lo(v.b), f2_hi(v.b)};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if (in[i]) t[i] = o4[i];
+                    }
+                };
+                if (outa) put(T2 + base, ya);
+                if (outb) put(T2 + base + nx, yb);
+            }
+        }
+        c1a = oa;
+        c1b = ob;
+        e1a = fna;
+        e1b = fnb;
+        cia = na;
+        cib = nb;
+        if (!ok) {
+            s_abort = 1;
+            atomicOr(&g_zpair_error, 1u);
+        }
+        // level 1 of plane z+1 is complete, T plane z+1's stage no longer read
+        __syncthreads();
+        if (s_abort) {
+            drain(min(j - 2 + NST, jmax));
+            return;
+        }
+        if (threadIdx.x == 0 && j - 1 + NST <= jmax) issue(j - 1 + NST);
+        s1 = s0;
+        s0 = s0 + 1 == NST ? 0 : s0 + 1;
+    }
+}
+
+template <int BY, int NST, int MINB, bool kStates>
+static cudaError_t launch_pair_t(float *T1o, float *T2, const float *T, const float *Ci, StepCoef c, Grid3 g,
+                                 cudaStream_t s) {
+    using Z = ZPair<BY>;
+    constexpr size_t smem = NST * Z::SB + 2 * Z::LB + NST * 8;
+    static unsigned attr_gen[64] = {0};
+    cudaError_t ae;
+    if (!set_smem_attr_once((const void *)k_zpair<BY, NST, MINB, kStates>, (int)smem, attr_gen, &ae)) return ae;
+    CUtensorMap mT, mC;
+    if (!make_tensor_map_3d(&mT, T, 4, g, Z::W, Z::TROWS) || !make_tensor_map_3d(&mC, Ci, 4, g, Z::W, Z::ROWS))
+        return cudaErrorInvalidValue;
+    const int64_t ntx = (g.nx + Z::BX - 1) / Z::BX, nty = (g.ny + BY - 1) / BY, tiles = ntx * nty;
+    int kchunk = launch_override(PS_OVERRIDE_KCHUNK2);
+    if (kchunk <= 0) {
+        const int64_t slots = (int64_t)MINB * sm_count();
+        const int64_t per_tile = tiles > 0 ? slots / tiles : 0;
+        const int64_t one_wave = per_tile > 0 ? (g.nz - 2 + per_tile - 1) / per_tile : 0;
+        if (one_wave <= 96 && one_wave > 0) {
+            // all CTAs resident at once
+            kchunk = (int)(one_wave < 8 ? 8 : one_wave);
+        } else {
+            // the chunk whose waves march the fewest planes in all (each chunk two and a half
+            // more than it stores): 384^3 61 us a step at 40 planes, 67 at 35
+            double best = 0.0;
+            for (int c = 16; c <= 96; ++c) {
+                const int64_t ctas = tiles * ((g.nz - 2 + c - 1) / c), waves = (ctas + slots - 1) / slots;
+                const double cost = (double)waves * (c + 2.5);
+                if (kchunk <= 0 || cost < best) {
+                    best = cost;
+                    kchunk = c;
+                }
+            }
+        }
+    }
+    const int64_t gz = (g.nz - 2 + kchunk - 1) / kchunk;
+    if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
+    const ZPairParams p{(int)g.nx, (int)g.ny, (int)g.nz, kchunk, (int)ntx, (float)c.dtlam, (float)c.ax, (float)c.ay,
+                        (float)c.az};
+    return launch_pdl(k_zpair<BY, NST, MINB, kStates>, dim3((unsigned)tiles, (unsigned)gz, 1), dim3(Z::NTH), smem,
+                      s, mT, mC, T2, p, T1o);
+}
+
+// 14-row tiles, four stages (91 KB), two CTAs per SM (96 registers).
+cudaError_t launch_step2_f32(float *T2, const float *T, const float *Ci, StepCoef c, Grid3 g, cudaStream_t s) {
+    return launch_pair_t<14, 4, 2, false>(nullptr, T2, T, Ci, c, g, s);
+}
+
+cudaError_t launch_step2_states_f32(float *T1o, float *T2, const float *T, const float *Ci, StepCoef c, Grid3 g,
+                                    cudaStream_t s) {
+    return launch_pair_t<14, 4, 2, true>(T1o, T2, T, Ci, c, g, s);
+}
+
+bool pairs_pay(Grid3 g, bool states) {
+    // by nodes and the share of useful lanes (us a step, single steps / pairs): 128^3 5.1 / 6.2,
+    // 160^3 (0.63) 8.5 / 9.3, 192^3 (0.75) 12.8 / 12.1, 112 x 480 x 64 (0.88) 9.5 / 6.4, 256 x
+    // 128 x 128 9.5 / 6.7; loops that keep every state 128^3 6.0 / 7.1, 160^3 13.1 / 11.0,
+    // 256^3 33.8 / 27.1
+    const double lanes = (double)g.nx / (128.0 * (double)((g.nx + 127) / 128));
+    return (double)g.n() * lanes > (states ? 2.2e6 : 2.8e6);
+}
+
+unsigned zpair_device_error(bool clear) {
+    unsigned v = 0;
+    cudaMemcpyFromSymbol(&v, g_zpair_error, sizeof(v));
+    if (clear) {
+        const unsigned z = 0;
+        cudaMemcpyToSymbol(g_zpair_error, &z, sizeof(z));
+    }
+    return v;
+}
+
+}  // namespace psd
