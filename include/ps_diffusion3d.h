@@ -311,6 +311,21 @@ int ps_diffusion3d_adjoint2_ex(void *Tbar, void *Cibar, const void *ybar, const 
                                double _dy, double _dz, int64_t nx, int64_t ny, int64_t nz, int dtype,
                                unsigned flags, void *stream);
 
+/* nsteps transposed steps in a row, as a reverse sweep takes them: step i reads the
+ * state states[i] (a host array of nsteps device pointers, the last step's state
+ * first) and the cotangent the step before left; the cotangent alternates between
+ * ybar (which holds dL/dT of the last state on entry and is overwritten) and Tbar,
+ * and Cibar accumulates every step's term.  Bit for bit nsteps
+ * ps_diffusion3d_adjoint_ex calls with the buffers swapped, in one call: on small
+ * grids a step takes less time than a call from an interpreted language.
+ * *result_in_Tbar (may be NULL) is nsteps & 1: the buffer that holds the result.
+ * Flags and aliasing rules as for ps_diffusion3d_adjoint_ex, ybar being an output
+ * too; nsteps >= 0. */
+int ps_diffusion3d_adjoint_sweep(void *Tbar, void *Cibar, void *ybar, const void *const *states,
+                                 int nsteps, const void *Ci, double lam, double dt, double _dx,
+                                 double _dy, double _dz, int64_t nx, int64_t ny, int64_t nz,
+                                 int dtype, unsigned flags, void *stream, int *result_in_Tbar);
+
 /* ---------------------------------------------------------------------
  * Reductions in FP64 (deterministic: a fixed partition and a fixed
  * summation order, independent of timing).  A, B are device arrays of n

@@ -169,6 +169,12 @@ class _GridViews:
     def __len__(self) -> int:
         return self.count
 
+    def ptr(self, i: int) -> int:
+        """Device address of grid i (no view is made)."""
+        if not 0 <= i < self.count:
+            raise IndexError("state grid index out of range")
+        return self.flat.data_ptr() + i * self.stride * self.flat.element_size()
+
     def __getitem__(self, i):
         if isinstance(i, slice):
             return [self[j] for j in range(*i.indices(self.count))]
@@ -265,6 +271,31 @@ def adjoint(Tbar, Cibar, ybar, T, Ci, lam: float, dt: float, inv_spacing, *,
         _field(Tbar, "Tbar", code), _field(Cibar, "Cibar", code), _field(ybar, "ybar", code),
         _field(T, "T", code), _field(Ci, "Ci", code), lam, dt, *inv_spacing, nx, ny, nz, code,
         _lib.PS_RUN_CI_SCALED if ci_scaled else 0, _stream(T)))
+
+
+def adjoint_sweep(Tbar, Cibar, ybar, states, Ci, lam: float, dt: float, inv_spacing, *,
+                  ci_scaled: bool = False):
+    """The transposed steps of the given states (the last step's state first) in one library
+    call: bit for bit :func:`adjoint` for each with ``ybar`` and ``Tbar`` swapped after every
+    step, so both are overwritten.  Returns (result, other): the buffer that holds the last
+    step's cotangent and the other one.  ``states``: tensors like ``ybar``, or device
+    addresses (ints) of such fields that the caller keeps alive until the call returns."""
+    code = _code(ybar)
+    _same(ybar, Tbar, Cibar, Ci)
+    nx, ny, nz = _grid(ybar)
+    ptrs = (ctypes.c_void_p * max(len(states), 1))()
+    for i, s in enumerate(states):
+        if isinstance(s, int):
+            ptrs[i] = s
+        else:
+            _same(ybar, s)
+            ptrs[i] = _field(s, "state", code)
+    odd = ctypes.c_int(0)
+    check(_lib.load().ps_diffusion3d_adjoint_sweep(
+        _field(Tbar, "Tbar", code), _field(Cibar, "Cibar", code), _field(ybar, "ybar", code), ptrs, len(states),
+        _field(Ci, "Ci", code), lam, dt, *inv_spacing, nx, ny, nz, code,
+        _lib.PS_RUN_CI_SCALED if ci_scaled else 0, _stream(ybar), ctypes.byref(odd)))
+    return (Tbar, ybar) if odd.value else (ybar, Tbar)
 
 
 def _grid2d(t: torch.Tensor):

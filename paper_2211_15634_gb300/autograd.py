@@ -76,6 +76,28 @@ def state_pairs_default(T0) -> bool:
     return T0.dtype == torch.float32
 
 
+class _EveryState:
+    """The checkpoints of ``every = 1``: T0 and the first nt - 1 grids of a block, as tensors
+    made on access (a sweep needs only their addresses)."""
+
+    def __init__(self, T0, block, nt: int):
+        self.T0, self.block, self.nt = T0, block, nt
+
+    def __len__(self) -> int:
+        return self.nt
+
+    def __getitem__(self, i: int):
+        if i < 0:
+            i += self.nt
+        if not 0 <= i < self.nt:
+            raise IndexError("checkpoint index out of range")
+        return self.T0 if i == 0 else self.block.grids[i - 1]
+
+    def addresses(self):
+        """Device addresses of the states, the last one first."""
+        return [self.block.grids.ptr(i - 1) for i in range(self.nt - 1, 0, -1)] + [self.T0.data_ptr()]
+
+
 def forward_checkpointed(T0, Ci, lam, dt, inv, nt, every, coef=None, graph=True, state_pairs=None):
     """Run nt steps; return (final state, [checkpoint at step 0, every, 2*every, ...], kept).
 
@@ -95,6 +117,8 @@ def forward_checkpointed(T0, Ci, lam, dt, inv, nt, every, coef=None, graph=True,
         # every state in one block; the steps write straight into it (one library call)
         block = api.StateBlock(T0, nt, boundary=False)  # run_states sets the boundaries
         cur = api.run_states(T0, block, 1, C, lam, dt, inv, nt, ci_scaled=scaled, graph=graph, temporal2=pairs)
+        if T0.is_cuda:
+            return cur, _EveryState(T0, block, nt), None
         return cur, [T0] + block.grids[:nt - 1], None
     nseg = (nt - 1) // every + 1
     first_kept = max(0, nseg - 2)
@@ -136,6 +160,13 @@ def backward_checkpointed(ybar_nt, Ci, lam, dt, inv, nt, every, ckpts, coef=None
     ybar = ybar_nt.contiguous().clone()
     tbar = torch.empty_like(ybar)
     cibar = torch.zeros_like(Ci)  # dL/dCs when scaled
+    # on the GPU a segment's transposed steps are one library call
+    native = ybar.is_cuda and not pairs
+    if native and isinstance(ckpts, _EveryState):
+        ybar, _ = api.adjoint_sweep(tbar, cibar, ybar, ckpts.addresses(), C, lam, dt, inv, ci_scaled=scaled)
+        if scaled:  # dL/dCi = dt*lam*_dx^2 * dL/dCs
+            api.scale_ci(cibar, lam, dt, inv, out=cibar)
+        return ybar, cibar
     nseg = len(ckpts)
     seg_len = max(0, min(every, nt) - 1)  # recomputed states per segment
     seg_buf = dict(kept) if kept else {}  # segment -> block holding its states
@@ -184,9 +215,14 @@ def backward_checkpointed(ybar_nt, Ci, lam, dt, inv, nt, every, ckpts, coef=None
                 recompute(s)
             t0 = s * every
             t1 = min(t0 + every, nt)
-            states = [ckpts[s]] + (seg_buf[s].grids[:t1 - t0 - 1] if t1 - t0 > 1 else [])
+            if native and t1 > t0:
+                grids = seg_buf[s].grids if t1 - t0 > 1 else None
+                states = [grids.ptr(i) for i in range(t1 - t0 - 2, -1, -1)] + [ckpts[s]]
+                ybar, tbar = api.adjoint_sweep(tbar, cibar, ybar, states, C, lam, dt, inv, ci_scaled=scaled)
+            elif not native:
+                states = [ckpts[s]] + (seg_buf[s].grids[:t1 - t0 - 1] if t1 - t0 > 1 else [])
             t = t1 - 1
-            while t >= t0:
+            while t >= t0 and not native:
                 if pairs and t - 1 >= t0:  # steps t and t-1 in one pass
                     api.adjoint2(tbar, cibar, ybar, states[t - t0], states[t - 1 - t0], C, lam, dt, inv)
                     t -= 2

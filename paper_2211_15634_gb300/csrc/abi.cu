@@ -710,10 +710,11 @@ int ps_diffusion3d_adjoint(void *Tbar, void *Cibar, const void *ybar, const void
                                      dtype, 0u, stream);
 }
 
-int ps_diffusion3d_adjoint_ex(void *Tbar, void *Cibar, const void *ybar, const void *T,
-                              const void *Ci, double lam, double dt, double _dx, double _dy,
-                              double _dz, int64_t nx, int64_t ny, int64_t nz, int dtype,
-                              unsigned flags, void *stream) {
+namespace psd {
+// Everything a transposed step checks; ybar_out: ybar is written too (a sweep).
+static int check_adjoint_args(const void *Tbar, const void *Cibar, const void *ybar, const void *T, const void *Ci,
+                              double lam, double dt, double _dx, double _dy, double _dz, int64_t nx, int64_t ny,
+                              int64_t nz, int dtype, unsigned flags, bool ybar_out) {
     if (flags & ~PS_RUN_CI_SCALED) return fail(PS_ERR_ARG, "unknown flags 0x%x", flags);
     PS_TRY(check_dtype(dtype));
     PS_TRY(check_grid(nx, ny, nz));
@@ -733,20 +734,52 @@ int ps_diffusion3d_adjoint_ex(void *Tbar, void *Cibar, const void *ybar, const v
         return fail(PS_ERR_ALIAS, "Tbar overlaps an input");
     if (overlap(Cibar, ybar, bytes) || overlap(Cibar, T, bytes) || overlap(Cibar, Ci, bytes))
         return fail(PS_ERR_ALIAS, "Cibar overlaps an input");
-    PS_TRY(check_scaled(flags, dtype, _dx, _dy, _dz));
+    if (ybar_out && (overlap(ybar, T, bytes) || overlap(ybar, Ci, bytes)))
+        return fail(PS_ERR_ALIAS, "ybar overlaps a state or Ci");
+    return check_scaled(flags, dtype, _dx, _dy, _dz);
+}
+
+static cudaError_t enqueue_adjoint(void *Tbar, void *Cibar, const void *ybar, const void *T, const void *Ci,
+                                   StepCoef c, Grid3 g, int dtype, unsigned flags, cudaStream_t s) {
+    if (flags & PS_RUN_CI_SCALED)
+        return launch_adjoint_f64_scaled((double *)Tbar, (double *)Cibar, (const double *)ybar, (const double *)T,
+                                         (const double *)Ci, g, s);
+    if (dtype == PS_F64)
+        return launch_adjoint_f64((double *)Tbar, (double *)Cibar, (const double *)ybar, (const double *)T,
+                                  (const double *)Ci, c, g, s);
+    return launch_adjoint_f32((float *)Tbar, (float *)Cibar, (const float *)ybar, (const float *)T,
+                              (const float *)Ci, c, g, s);
+}
+}  // namespace psd
+
+int ps_diffusion3d_adjoint_ex(void *Tbar, void *Cibar, const void *ybar, const void *T,
+                              const void *Ci, double lam, double dt, double _dx, double _dy,
+                              double _dz, int64_t nx, int64_t ny, int64_t nz, int dtype,
+                              unsigned flags, void *stream) {
+    PS_TRY(check_adjoint_args(Tbar, Cibar, ybar, T, Ci, lam, dt, _dx, _dy, _dz, nx, ny, nz, dtype, flags, false));
+    const cudaError_t e = enqueue_adjoint(Tbar, Cibar, ybar, T, Ci, make_coef(lam, dt, _dx, _dy, _dz),
+                                          Grid3{nx, ny, nz}, dtype, flags, (cudaStream_t)stream);
+    if (e != cudaSuccess) return cuda_fail(e, "ps_diffusion3d_adjoint");
+    return PS_OK;
+}
+
+int ps_diffusion3d_adjoint_sweep(void *Tbar, void *Cibar, void *ybar, const void *const *states,
+                                 int nsteps, const void *Ci, double lam, double dt, double _dx,
+                                 double _dy, double _dz, int64_t nx, int64_t ny, int64_t nz,
+                                 int dtype, unsigned flags, void *stream, int *result_in_Tbar) {
+    if (nsteps < 0) return fail(PS_ERR_ARG, "nsteps = %d < 0", nsteps);
+    if (nsteps > 0 && !states) return fail(PS_ERR_ARG, "states is NULL");
+    for (int i = 0; i < nsteps; ++i)  // all of them before the first launch
+        PS_TRY(check_adjoint_args(Tbar, Cibar, ybar, states[i], Ci, lam, dt, _dx, _dy, _dz, nx, ny, nz, dtype, flags,
+                                  true));
     const StepCoef c = make_coef(lam, dt, _dx, _dy, _dz);
     const Grid3 g{nx, ny, nz};
-    cudaError_t e;
-    if (flags & PS_RUN_CI_SCALED)
-        e = launch_adjoint_f64_scaled((double *)Tbar, (double *)Cibar, (const double *)ybar,
-                                      (const double *)T, (const double *)Ci, g, (cudaStream_t)stream);
-    else if (dtype == PS_F64)
-        e = launch_adjoint_f64((double *)Tbar, (double *)Cibar, (const double *)ybar,
-                               (const double *)T, (const double *)Ci, c, g, (cudaStream_t)stream);
-    else
-        e = launch_adjoint_f32((float *)Tbar, (float *)Cibar, (const float *)ybar, (const float *)T,
-                               (const float *)Ci, c, g, (cudaStream_t)stream);
-    if (e != cudaSuccess) return cuda_fail(e, "ps_diffusion3d_adjoint");
+    for (int i = 0; i < nsteps; ++i) {
+        void *src = (i & 1) ? Tbar : ybar, *dst = (i & 1) ? ybar : Tbar;
+        const cudaError_t e = enqueue_adjoint(dst, Cibar, src, states[i], Ci, c, g, dtype, flags, (cudaStream_t)stream);
+        if (e != cudaSuccess) return cuda_fail(e, "ps_diffusion3d_adjoint_sweep");
+    }
+    if (result_in_Tbar) *result_in_Tbar = nsteps & 1;
     return PS_OK;
 }
 
