@@ -2,7 +2,7 @@
 // y-march.
 //
 // Warp w owns a strip of 32*PX columns (PX nodes per lane: two 16-byte accesses when
-// the rows allow them - eight FP32 or four FP64 nodes - else PX = 1) and a chunk of
+// the rows allow them - eight FP32 or four FP64 nodes - else PX nodes 32 apart) and a chunk of
 // interior rows [j0, j1).  Each
 // lane keeps its own values of rows j-1, j, j+1 and Ci of row j in registers and
 // loads row j+2 and Ci of row j+1 while it computes row j: plain coalesced loads,
@@ -17,6 +17,7 @@
 #include "emu64.cuh"
 #include "internal.h"
 #include "node.cuh"
+#include "pdl.cuh"
 #include "zmarch.h"
 
 namespace psd {
@@ -116,48 +117,89 @@ __device__ __forceinline__ void load_row(E (&v)[PX], const E *__restrict__ A, in
     for (int i = 0; i < PX; ++i) v[i] = x + i < nx ? __ldg(q + i) : E(0);
 }
 
+// The same for a lane's strided nodes x, x + 32, ..
+template <typename E, int PX>
+__device__ __forceinline__ void load_strided(E (&v)[PX], const E *__restrict__ A, int64_t r, int64_t nx, int64_t x) {
+    const E *q = A + r * nx + x;
+#pragma unroll
+    for (int i = 0; i < PX; ++i) v[i] = x + 32 * i < nx ? __ldg(q + 32 * i) : E(0);
+}
+
 // MINB CTAs of 8 warps per SM: 3 for two FP64 / eight FP32 nodes per lane and the
 // scalar forms (the FP64 emulated modes spill at 4, measured 4% slower there); 2 for four
 // FP64 nodes per lane (111 registers, no spill)
-template <int MODE, int PX, int MINB = 3>
+// XS: distance between a lane's nodes - 1, neighbours (16-byte accesses), or 32, for rows at
+// any element: consecutive lanes on consecutive elements, so that scalar accesses still fill
+// whole sectors, and the loop's own instructions count for PX nodes.
+template <int MODE, int PX, int MINB, int XS>
 __global__ void __launch_bounds__(256, MINB)
 k_ymarch2d(typename M2D<MODE>::E *__restrict__ T2, const typename M2D<MODE>::E *__restrict__ T,
            const typename M2D<MODE>::E *__restrict__ Ci, const P2D p) {
     using E = typename M2D<MODE>::E;
+    grid_dep_wait();  // the previous step's writes (and its reads of T2) are complete
     const int lane = threadIdx.x & 31;
     const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int64_t strip = warp % p.nstrips, chunk = warp / p.nstrips;
     const int64_t nx = p.nx, ny = p.ny;
     const int64_t j0 = 1 + chunk * p.chunk, j1 = min(j0 + p.chunk, ny - 1);  // rows [j0, j1)
     if (j0 >= j1) return;  // warp-uniform
-    const int64_t x0 = strip * 32 * PX, gx0 = x0 + lane * PX;
+    const int64_t x0 = strip * 32 * PX, gx0 = x0 + lane * (XS == 1 ? PX : 1);
     const bool has_l = lane == 0 && x0 >= 1, has_r = lane == 31 && x0 + 32 * PX < nx;
     bool wr[PX];
 #pragma unroll
-    for (int i = 0; i < PX; ++i) wr[i] = gx0 + i >= 1 && gx0 + i <= nx - 2;
-    const bool all_w = gx0 >= 1 && gx0 + PX - 1 <= nx - 2;
+    for (int i = 0; i < PX; ++i) wr[i] = gx0 + XS * i >= 1 && gx0 + XS * i <= nx - 2;
+    const bool all_w = gx0 >= 1 && gx0 + XS * (PX - 1) <= nx - 2;
+    auto load = [&](E (&v)[PX], const E *__restrict__ A, int64_t r) {
+        if constexpr (XS == 1)
+            load_row<E, PX>(v, A, r, nx, gx0);
+        else
+            load_strided<E, PX>(v, A, r, nx, gx0);
+    };
 
     E up[PX], c[PX], dn[PX], ci[PX], nxt[PX], cin[PX];
-    load_row<E, PX>(up, T, j0 - 1, nx, gx0);
-    load_row<E, PX>(c, T, j0, nx, gx0);
-    load_row<E, PX>(dn, T, j0 + 1, nx, gx0);
-    load_row<E, PX>(ci, Ci, j0, nx, gx0);
+    load(up, T, j0 - 1);
+    load(c, T, j0);
+    load(dn, T, j0 + 1);
+    load(ci, Ci, j0);
     E hl = has_l ? __ldg(T + j0 * nx + x0 - 1) : E(0), hr = has_r ? __ldg(T + j0 * nx + x0 + 32 * PX) : E(0);
     for (int64_t j = j0; j < j1; ++j) {
         // row j+2 (the next "down" row) and Ci of row j+1, and the strip-edge values of
         // row j+1, are in flight while row j is computed
         const bool more = j + 1 < j1;
         if (more) {
-            load_row<E, PX>(nxt, T, j + 2, nx, gx0);
-            load_row<E, PX>(cin, Ci, j + 1, nx, gx0);
+            load(nxt, T, j + 2);
+            load(cin, Ci, j + 1);
         }
         const E hl1 = (more && has_l) ? __ldg(T + (j + 1) * nx + x0 - 1) : E(0);
         const E hr1 = (more && has_r) ? __ldg(T + (j + 1) * nx + x0 + 32 * PX) : E(0);
-        // x-neighbours across lanes
-        E left = __shfl_up_sync(0xffffffffu, c[PX - 1], 1);
-        E right = __shfl_down_sync(0xffffffffu, c[0], 1);
-        if (lane == 0) left = hl;
-        if (lane == 31) right = hr;
+        // x-neighbours: a lane's own or the neighbouring lanes' (strided: the neighbouring lane's
+        // node of the same group of 32, at its ends of the group beside it)
+        E xl[PX], xr[PX];
+        if constexpr (XS == 1) {
+            xl[0] = __shfl_up_sync(0xffffffffu, c[PX - 1], 1);
+            xr[PX - 1] = __shfl_down_sync(0xffffffffu, c[0], 1);
+            if (lane == 0) xl[0] = hl;
+            if (lane == 31) xr[PX - 1] = hr;
+#pragma unroll
+            for (int i = 1; i < PX; ++i) {
+                xl[i] = c[i - 1];
+                xr[i - 1] = c[i];
+            }
+        } else {
+            E pl = hl, pr = hr;
+#pragma unroll
+            for (int i = 0; i < PX; ++i) {
+                const E v = __shfl_sync(0xffffffffu, c[i], (lane + 31) & 31);
+                xl[i] = lane == 0 ? pl : v;
+                pl = v;
+            }
+#pragma unroll
+            for (int i = PX - 1; i >= 0; --i) {
+                const E v = __shfl_sync(0xffffffffu, c[i], (lane + 1) & 31);
+                xr[i] = lane == 31 ? pr : v;
+                pr = v;
+            }
+        }
         E out[PX];
         bool warp_fast = false;
         if constexpr (MODE == Z_F64_SCALED || MODE == Z_F64_EMU_ISO_DMUL || MODE == Z_F64_EMU_ANISO) {
@@ -169,10 +211,13 @@ k_ymarch2d(typename M2D<MODE>::E *__restrict__ T2, const typename M2D<MODE>::E *
             for (int i = 0; i < PX; ++i) any_wr = any_wr || wr[i];
             // a lane that writes none of its nodes (past the grid) votes for the fast path:
             // its reference is 1.0's word (its outputs are never stored)
-            const unsigned hc = any_wr ? (unsigned)(dbits(c[0]) >> 32) : 0x3ff00000u;
-            unsigned hw[3 * PX + 1];
-            hw[0] = wr[0] ? (unsigned)(dbits(left) >> 32) : hc;
-            hw[1] = wr[PX - 1] ? (unsigned)(dbits(right) >> 32) : hc;
+            // (strided lanes: the first node they write; node i's centre is no neighbour of theirs)
+            unsigned hc = any_wr ? (unsigned)(dbits(c[0]) >> 32) : 0x3ff00000u;
+            if constexpr (XS != 1 && PX > 1)
+                if (any_wr && !wr[0]) hc = (unsigned)(dbits(c[1]) >> 32);
+            unsigned hw[XS == 1 ? 3 * PX + 1 : 5 * PX];
+            hw[0] = wr[0] ? (unsigned)(dbits(xl[0]) >> 32) : hc;
+            hw[1] = wr[PX - 1] ? (unsigned)(dbits(xr[PX - 1]) >> 32) : hc;
 #pragma unroll
             for (int i = 0; i < PX; ++i) {
                 hw[2 + 2 * i] = wr[i] ? (unsigned)(dbits(up[i]) >> 32) : hc;
@@ -180,14 +225,22 @@ k_ymarch2d(typename M2D<MODE>::E *__restrict__ T2, const typename M2D<MODE>::E *
             }
 #pragma unroll
             for (int i = 1; i < PX; ++i) {
-                const bool need = wr[i] || wr[i - 1] || (i + 1 < PX && wr[i + 1]);
+                const bool need = wr[i] || (XS == 1 && (wr[i - 1] || (i + 1 < PX && wr[i + 1])));
                 hw[1 + 2 * PX + i] = need ? (unsigned)(dbits(c[i]) >> 32) : hc;
+            }
+            if constexpr (XS != 1) {  // hw[3*PX + 1 ..]: the x-neighbours not among the words yet
+#pragma unroll
+                for (int i = 1; i < PX; ++i) {
+                    hw[3 * PX + i] = wr[i] ? (unsigned)(dbits(xl[i]) >> 32) : hc;
+                    hw[4 * PX + i - 1] = wr[i - 1] ? (unsigned)(dbits(xr[i - 1]) >> 32) : hc;
+                }
+                hw[5 * PX - 1] = hc;
             }
             warp_fast = __all_sync(0xffffffffu, emu_same_binade_hi(hw, hc));
         }
 #pragma unroll
         for (int i = 0; i < PX; ++i) {
-            const E xm = i == 0 ? left : c[i - 1], xp = i == PX - 1 ? right : c[i + 1];
+            const E xm = xl[i], xp = xr[i];
             if constexpr (MODE == Z_F64_SCALED) {
                 if (warp_fast) {
                     out[i] = emu_fast_node_scaled(dbits(c[i]), dbits(xm), dbits(xp), dbits(up[i]), dbits(dn[i]),
@@ -211,7 +264,7 @@ k_ymarch2d(typename M2D<MODE>::E *__restrict__ T2, const typename M2D<MODE>::E *
             out[i] = node2d<MODE, E>(c[i], xm, xp, up[i], dn[i], ci[i], p);
         }
         E *q = T2 + j * nx + gx0;
-        if constexpr (PX * sizeof(E) == 32) {
+        if constexpr (XS == 1 && PX * sizeof(E) == 32) {
             if (all_w) {
                 if constexpr (sizeof(E) == 8) {
                     ((double2 *)q)[0] = make_double2(out[0], out[1]);
@@ -225,7 +278,7 @@ k_ymarch2d(typename M2D<MODE>::E *__restrict__ T2, const typename M2D<MODE>::E *
                 for (int i = 0; i < PX; ++i)
                     if (wr[i]) q[i] = out[i];
             }
-        } else if constexpr (PX * sizeof(E) == 16) {
+        } else if constexpr (XS == 1 && PX * sizeof(E) == 16) {
             if (all_w) {
                 if constexpr (sizeof(E) == 8)
                     *(double2 *)q = make_double2(out[0], out[1]);
@@ -239,7 +292,7 @@ k_ymarch2d(typename M2D<MODE>::E *__restrict__ T2, const typename M2D<MODE>::E *
         } else {
 #pragma unroll
             for (int i = 0; i < PX; ++i)
-                if (wr[i]) q[i] = out[i];
+                if (wr[i]) q[XS * i] = out[i];
         }
 #pragma unroll
         for (int i = 0; i < PX; ++i) {
@@ -251,6 +304,7 @@ k_ymarch2d(typename M2D<MODE>::E *__restrict__ T2, const typename M2D<MODE>::E *
         hl = hl1;
         hr = hr1;
     }
+    grid_dep_launch();  // at the end: less than a wave of CTAs would else fill up unevenly
 }
 
 // Edges of a 2-D field: T2 = T on rows 0, ny-1 and columns 0, nx-1 (Fig. 1's
@@ -271,25 +325,30 @@ __global__ void k_copy_edges2d(E *__restrict__ T2, const E *__restrict__ T, int6
     }
 }
 
-template <int MODE, int PX, int MINB = 3>
+template <int MODE, int PX, int MINB = 3, int XS = 1>
 static cudaError_t launch_2d_t(void *T2, const void *T, const void *Ci, P2D p, int64_t nx, int64_t ny,
                                cudaStream_t s) {
     using E = typename M2D<MODE>::E;
     p.nx = nx;
     p.ny = ny;
     p.nstrips = (int)((nx + 32 * PX - 1) / (32 * PX));
-    // chunks of 16-256 rows, about eight waves of resident warps (48 per SM)
     int chunk = launch_override(PS_OVERRIDE_CHUNK2D);
     if (chunk <= 0) {
-        const int64_t target = 8LL * 48 * sm_count();
-        const int64_t c = (ny - 2) * (int64_t)p.nstrips / target;
-        chunk = (int)(c < 16 ? 16 : (c > 256 ? 256 : c));
+        // A row's loads come one row ahead, so a chunk is a chain of round trips: on small grids
+        // one or two rows per warp, a few where the warps make some waves, and about eight
+        // waves of long chunks (which re-read two rows each) only on large ones.  us a step
+        // against the 16 rows small grids had: FP64 512^2 3.1 / 14, 1024^2 6.5 / 14, 2048^2
+        // 19.8 / 20.2; FP32 512^2 2.2 / 8.4, 1024^2 3.3 / 8.3, 4096^2 34 / 39.
+        const int64_t rows = (ny - 2) * (int64_t)p.nstrips;  // warps at one row each
+        const double waves = (double)rows / (8.0 * MINB * sm_count());
+        const int64_t c = rows / (8LL * 48 * sm_count());
+        chunk = waves <= 1.0 ? 1 : (waves <= 2.0 ? 2 : (waves <= 32.0 ? 4 : (int)(c < 8 ? 8 : (c > 256 ? 256 : c))));
     }
     p.chunk = chunk;
     const int64_t nch = (ny - 2 + chunk - 1) / chunk, warps = nch * p.nstrips, blocks = (warps + 7) / 8;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    k_ymarch2d<MODE, PX, MINB><<<(unsigned)blocks, 256, 0, s>>>((E *)T2, (const E *)T, (const E *)Ci, p);
-    return cudaGetLastError();
+    return launch_pdl(k_ymarch2d<MODE, PX, MINB, XS>, dim3((unsigned)blocks), dim3(256), 0, s, (E *)T2, (const E *)T,
+                      (const E *)Ci, p);
 }
 
 // mode: Z_F32, Z_F64_SCALED (Ci holds dt*lam*_dx^2*Ci, equal spacings), Z_F64_EMU_ISO_DMUL
@@ -305,26 +364,33 @@ cudaError_t launch_step2d(int mode, void *T2, const void *T, const void *Ci, Ste
     p.ek.az = 0.0;                               // (and vanishes in the general path's plain form)
     const int esz = mode == Z_F32 ? 4 : 8;
     const bool vec = ((nx * esz) % 16 == 0) && ((((uintptr_t)T2 | (uintptr_t)T | (uintptr_t)Ci) & 15u) == 0);
+    // Rows at any element take strided lanes (us a step at 6000 x 8191 against one node per lane:
+    // FP64 pre-scaled 265 / 323, unequal spacings 313 / 359, FP32 106 / 227).
     switch (mode) {
         case Z_F32:
             // eight nodes per lane (two 16-byte accesses): measured 7-9% faster than four at
-            // 16384^2 and 32768^2
-            return vec ? launch_2d_t<Z_F32, 8>(T2, T, Ci, p, nx, ny, s) : launch_2d_t<Z_F32, 1>(T2, T, Ci, p, nx, ny, s);
+            // 16384^2 and 32768^2; strided four at four CTAs per SM (eight at three spill: 128 us)
+            return vec ? launch_2d_t<Z_F32, 8>(T2, T, Ci, p, nx, ny, s)
+                       : launch_2d_t<Z_F32, 4, 4, 32>(T2, T, Ci, p, nx, ny, s);
         // FP64: four nodes per lane (two 16-byte accesses) at two CTAs per SM, measured 8%
         // faster than two per lane at three CTAs per SM at 16384^2 (6% at 8192^2); four per
-        // lane at three CTAs per SM spilled and ran 25% slower
+        // lane at three CTAs per SM spilled and ran 25% slower.  Strided: two at four CTAs (four
+        // at two: 273 us)
         case Z_F64_SCALED:
             return vec ? launch_2d_t<Z_F64_SCALED, 4, 2>(T2, T, Ci, p, nx, ny, s)
-                       : launch_2d_t<Z_F64_SCALED, 1>(T2, T, Ci, p, nx, ny, s);
+                       : launch_2d_t<Z_F64_SCALED, 2, 4, 32>(T2, T, Ci, p, nx, ny, s);
         case Z_F64_EMU_ISO_DMUL:
             return vec ? launch_2d_t<Z_F64_EMU_ISO_DMUL, 4, 2>(T2, T, Ci, p, nx, ny, s)
-                       : launch_2d_t<Z_F64_EMU_ISO_DMUL, 1>(T2, T, Ci, p, nx, ny, s);
+                       : launch_2d_t<Z_F64_EMU_ISO_DMUL, 2, 4, 32>(T2, T, Ci, p, nx, ny, s);
         // spacings within a factor of 16 of each other; beyond that plain FP64, whose products
         // lose nothing at any ratio
         case Z_F64_EMU_ANISO:
             if (!p.ek.common) break;
-            return vec ? launch_2d_t<Z_F64_EMU_ANISO, 4, 2>(T2, T, Ci, p, nx, ny, s)
-                       : launch_2d_t<Z_F64_EMU_ANISO, 1>(T2, T, Ci, p, nx, ny, s);
+            if (!vec) return launch_2d_t<Z_F64_EMU_ANISO, 2, 4, 32>(T2, T, Ci, p, nx, ny, s);
+            // bound by issue, so more warps with fewer nodes each once there are many rows:
+            // 6000 x 8192 245 us, 255 with four per lane; 2048^2 29 and 28
+            if (nx * ny >= (1LL << 24)) return launch_2d_t<Z_F64_EMU_ANISO, 2, 4>(T2, T, Ci, p, nx, ny, s);
+            return launch_2d_t<Z_F64_EMU_ANISO, 4, 2>(T2, T, Ci, p, nx, ny, s);
         default:
             break;
     }
