@@ -771,8 +771,10 @@ KERNEL_SOURCES = {
                   "paper_2211_15634_gb300/csrc/emu64.cuh",
                   "paper_2211_15634_gb300/csrc/node.cuh", "paper_2211_15634_gb300/csrc/tma.cuh",
                   "paper_2211_15634_gb300/csrc/pdl.cuh"],
-    "k_zpair": ["paper_2211_15634_gb300/csrc/zpair.cu", "paper_2211_15634_gb300/csrc/tma.cuh",
-                "paper_2211_15634_gb300/csrc/pdl.cuh"],
+    "k_zpair": ["paper_2211_15634_gb300/csrc/zpair.cu", "paper_2211_15634_gb300/csrc/f32x2.cuh",
+                "paper_2211_15634_gb300/csrc/tma.cuh", "paper_2211_15634_gb300/csrc/pdl.cuh"],
+    "k_zpair_rag": ["paper_2211_15634_gb300/csrc/zpair_rag.cu", "paper_2211_15634_gb300/csrc/f32x2.cuh",
+                    "paper_2211_15634_gb300/csrc/tma.cuh", "paper_2211_15634_gb300/csrc/pdl.cuh"],
     "k_zmarch_rag": ["paper_2211_15634_gb300/csrc/zmarch.cu", "paper_2211_15634_gb300/csrc/zrag_tile.cuh",
                      "paper_2211_15634_gb300/csrc/zmarch_tile.cuh", "paper_2211_15634_gb300/csrc/zmarch.h",
                      "paper_2211_15634_gb300/csrc/emu64.cuh", "paper_2211_15634_gb300/csrc/node.cuh",

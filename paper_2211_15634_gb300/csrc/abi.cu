@@ -205,9 +205,17 @@ static bool pairs_ok(Grid3 g, int dtype, const void *T, const void *T2, const vo
            zmarch2_supported(g, elem_bytes(dtype), T2, T, Ci);
 }
 
+// The same for the FP32 pairs on rows that are no multiple of 16 bytes (loops only).
+static bool pairs_ragged_ok(Grid3 g, int dtype, const void *T, const void *T2, const void *Ci) {
+    if (dtype != PS_F32 || g.nx % 4 == 0) return false;
+    if (!pairs_pay_ragged(g) && launch_override(PS_OVERRIDE_KCHUNK2) <= 0) return false;
+    return ragged_supported(g, T, T2, Ci);
+}
+
 static cudaError_t enqueue_step2(void *T2, const void *T, const void *Ci, StepCoef c, Grid3 g,
                                  int dtype, cudaStream_t s) {
     if (dtype == PS_F64) return launch_step2_f64_scaled((double *)T2, (const double *)T, (const double *)Ci, g, s);
+    if (g.nx % 4) return launch_step2_ragged_f32((float *)T2, (const float *)T, (const float *)Ci, c, g, s);
     return launch_step2_f32((float *)T2, (const float *)T, (const float *)Ci, c, g, s);
 }
 
@@ -228,7 +236,8 @@ static cudaError_t enqueue_run(void *T, void *T2, void *comp, const void *Ci, St
                                launch_override(PS_OVERRIDE_KCHUNK) <= 0 &&
                                launch_override(PS_OVERRIDE_STEP_PLAIN) != 1);
     int pairs = 0;
-    if (may && pairs_ok(g, dtype, T, T2, Ci)) pairs = (asked ? nt : nt - 1) / 4 * 2;
+    if (may && (pairs_ok(g, dtype, T, T2, Ci) || pairs_ragged_ok(g, dtype, T, T2, Ci)))
+        pairs = (asked ? nt : nt - 1) / 4 * 2;
     const int singles = nt - 2 * pairs;
     for (int it = 0; it < pairs + singles && e == cudaSuccess; ++it) {
         void *src = (it & 1) ? T2 : T;
@@ -347,7 +356,7 @@ int ps_device_error(unsigned *out_host, int clear) {
                 adjoint_scaled_device_error(clear != 0) | zmarch2_device_error(clear != 0) |
                 adjoint_f32_device_error(clear != 0) | batch_device_error(clear != 0) |
                 batch_zmarch_device_error(clear != 0) |
-                zpair_device_error(clear != 0);
+                zpair_device_error(clear != 0) | zpair_rag_device_error(clear != 0);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "ps_device_error");
     return PS_OK;
@@ -370,6 +379,8 @@ const char *ps_diffusion3d_step_kernel(const void *T2, const void *T, const void
         if (dtype == PS_F32 && !(flags & PS_RUN_COMPENSATED)) return "k_zpair<F32>";
         if (dtype == PS_F64 && (flags & PS_RUN_CI_SCALED)) return "k_zmarch2<F64_SCALED>";
     }
+    if ((flags & PS_RUN_TEMPORAL2) && !(flags & PS_RUN_COMPENSATED) && pairs_ragged_ok(g, dtype, T, T2, Ci))
+        return "k_zpair_rag<F32>";
     if (dtype == PS_F64)
         return step_f64_kernel_name(g, T2, T, Ci, make_coef(lam, dt, _dx, _dy, _dz),
                                     (flags & PS_RUN_CI_SCALED) != 0);

@@ -67,6 +67,8 @@ cudaError_t launch_scale_ci(double *Cs, const double *Ci, double K, int64_t n, c
 bool zmarch2_supported(Grid3 g, int esz, const void *a, const void *b, const void *c);
 cudaError_t launch_step2_f32(float *T2, const float *T, const float *Ci, StepCoef c, Grid3 g,
                              cudaStream_t s);
+// the same on rows that are no multiple of 16 bytes (ragged_supported)
+cudaError_t launch_step2_ragged_f32(float *T2, const float *T, const float *Ci, StepCoef c, Grid3 g, cudaStream_t s);
 cudaError_t launch_step2_f64_scaled(double *T2, const double *T, const double *Cs, Grid3 g,
                                     cudaStream_t s);
 // A fused FP32 pair that keeps both states: T1 = step(T) to T1o, T2 = step(T1), both
@@ -75,6 +77,7 @@ cudaError_t launch_step2_states_f32(float *T1o, float *T2, const float *T, const
                                     Grid3 g, cudaStream_t s);
 unsigned zmarch2_device_error(bool clear);
 unsigned zpair_device_error(bool clear);
+unsigned zpair_rag_device_error(bool clear);
 const char *step_f64_kernel_name(Grid3 g, const void *T2, const void *T, const void *Ci, StepCoef c,
                                  bool scaled);
 const char *step_f32_kernel_name(Grid3 g, const void *T2, const void *T, const void *Ci);

@@ -121,6 +121,17 @@ bool make_tensor_map_rows(CUtensorMap *m, const void *ptr, int esz, int64_t n, i
     return r == CUDA_SUCCESS;
 }
 
+bool make_tensor_map_quarter(CUtensorMap *m, const float *ptr, Grid3 g, int64_t r, unsigned bx, unsigned by) {
+    auto fn = encode_fn();
+    if (!fn) return false;
+    const int64_t shift = r * g.nx & 3;
+    const cuuint64_t dims[2] = {(cuuint64_t)(g.nx + shift), (cuuint64_t)((g.ny * g.nz - r + 3) / 4)};
+    const cuuint64_t strides[1] = {(cuuint64_t)(16 * g.nx)};
+    const cuuint32_t box[2] = {bx, by}, estr[2] = {1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(ptr + (r * g.nx - shift)), dims, strides, box,
+              estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 bool ragged_supported(Grid3 g, const void *a, const void *b, const void *c) {
     if (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c) & 15u) return false;
     // element coordinates of planes -1 .. nz, tiles past the grid included, fit 32 bits

@@ -40,12 +40,18 @@ bool step_ragged_ok(Grid3 g, int esz, const void *a, const void *b, const void *
 // row is left out) with a box of bx x by, or with by = 0 one line with a box of bx.
 bool make_tensor_map_rows(CUtensorMap *m, const void *ptr, int esz, int64_t n, int64_t rowlen, unsigned bx,
                           unsigned by);
+// Map over the FP32 grid's rows r, r+4, ... (flat rows y + ny*z, r < 4) with a box of bx x by; row r
+// starts at element r*nx mod 4 of the map's first row.
+bool make_tensor_map_quarter(CUtensorMap *m, const float *ptr, Grid3 g, int64_t r, unsigned bx, unsigned by);
+// Planes per chunk of the FP32 pair kernels for `tiles` tiles on `slots` resident CTAs.
+int pair_kchunk(Grid3 g, int64_t tiles, int64_t slots);
 // Grids whose steps inside a time loop take the column kernels (stencil_basic.cuh); mode:
 // Z_F32, Z_F32_COMP, Z_F64_SCALED or Z_F64_EMU_ANISO (any unequal spacings).
 bool step_small(Grid3 g, int mode);
 // Whether fused FP32 pairs (zpair.cu) beat single steps in a loop on this grid; states: a
 // loop that keeps every state.
 bool pairs_pay(Grid3 g, bool states);
+bool pairs_pay_ragged(Grid3 g);  // on rows that are no multiple of 16 bytes
 // 3-D tiled tensor map over a (nz, ny, nx) field with a bx x by x 1 box.
 bool make_tensor_map_3d(CUtensorMap *m, const void *ptr, int esz, Grid3 g, unsigned bx, unsigned by);
 // The same over a grid whose rows are `pitch` elements apart (pitch*esz a multiple of 16).

@@ -28,6 +28,7 @@
 // interior node beside them.  (kStates stores them, so there they are selected.)
 #include <cudaTypedefs.h>
 
+#include "f32x2.cuh"
 #include "internal.h"
 #include "node.cuh"
 #include "pdl.cuh"
@@ -43,45 +44,15 @@ struct ZPairParams {
     float dtlam, ax, ay, az;
 };
 
-// Two FP32 values in one 64-bit register pair, one instruction for both.
-using f2 = unsigned long long;
-__device__ __forceinline__ f2 f2_make(float a, float b) {
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float f2_lo(f2 v) { return __uint_as_float((unsigned)v); }
-__device__ __forceinline__ float f2_hi(f2 v) { return __uint_as_float((unsigned)(v >> 32)); }
-__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
-    f2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
-    f2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-// a - b as a fused multiply-add by -1: one rounding, the difference's (sub.f32x2 was slower)
-__device__ __forceinline__ f2 f2_sub(f2 a, f2 b) { return f2_fma(b, 0xbf800000bf800000ull, a); }
-
-struct V4 {  // four nodes of a row
-    f2 a, b;
-};
 __device__ __forceinline__ V4 v4_load(const float *p) {
     const ulonglong2 v = *(const ulonglong2 *)p;
     return V4{v.x, v.y};
 }
 __device__ __forceinline__ void v4_store(float *p, V4 v) { *(ulonglong2 *)p = make_ulonglong2(v.a, v.b); }
-__device__ __forceinline__ V4 v4_sub(V4 x, V4 y) { return V4{f2_sub(x.a, y.a), f2_sub(x.b, y.b)}; }
 __device__ __forceinline__ V4 v4_select(const bool (&m)[4], V4 x, V4 y) {
     return V4{f2_make(m[0] ? f2_lo(x.a) : f2_lo(y.a), m[1] ? f2_hi(x.a) : f2_hi(y.a)),
               f2_make(m[2] ? f2_lo(x.b) : f2_lo(y.b), m[3] ? f2_hi(x.b) : f2_hi(y.b))};
 }
-
-struct ZCoef2 {
-    f2 dtlam, ax, ay, az;
-};
 
 // f32_node of four neighbouring nodes: c the centres, left / right the values beside them, up /
 // dn the rows above and below, en = zp - c and eo = c - zm the differences along z.
@@ -339,26 +310,16 @@ k_zpair(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtenso
     }
 }
 
-template <int BY, int NST, int MINB, bool kStates>
-static cudaError_t launch_pair_t(float *T1o, float *T2, const float *T, const float *Ci, StepCoef c, Grid3 g,
-                                 cudaStream_t s) {
-    using Z = ZPair<BY>;
-    constexpr size_t smem = NST * Z::SB + 2 * Z::LB + NST * 8;
-    static unsigned attr_gen[64] = {0};
-    cudaError_t ae;
-    if (!set_smem_attr_once((const void *)k_zpair<BY, NST, MINB, kStates>, (int)smem, attr_gen, &ae)) return ae;
-    CUtensorMap mT, mC;
-    if (!make_tensor_map_3d(&mT, T, 4, g, Z::W, Z::TROWS) || !make_tensor_map_3d(&mC, Ci, 4, g, Z::W, Z::ROWS))
-        return cudaErrorInvalidValue;
-    const int64_t ntx = (g.nx + Z::BX - 1) / Z::BX, nty = (g.ny + BY - 1) / BY, tiles = ntx * nty;
+// Planes per chunk for `tiles` tiles on `slots` resident CTAs.
+int pair_kchunk(Grid3 g, int64_t tiles, int64_t slots) {
     int kchunk = launch_override(PS_OVERRIDE_KCHUNK2);
     if (kchunk <= 0) {
-        const int64_t slots = (int64_t)MINB * sm_count();
         const int64_t per_tile = tiles > 0 ? slots / tiles : 0;
         const int64_t one_wave = per_tile > 0 ? (g.nz - 2 + per_tile - 1) / per_tile : 0;
         if (one_wave <= 96 && one_wave > 0) {
-            // all CTAs resident at once
-            kchunk = (int)(one_wave < 8 ? 8 : one_wave);
+            // all CTAs resident at once; chunks of fewer than six planes lose more than they
+            // spread (odd rows, 129^3: 7.6 us a step at 4 planes, 6.4 at 6, 7.5 at 8)
+            kchunk = (int)(one_wave < 6 ? 6 : one_wave);
         } else {
             // the chunk whose waves march the fewest planes in all (each chunk two and a half
             // more than it stores): 384^3 61 us a step at 40 planes, 67 at 35
@@ -373,6 +334,22 @@ static cudaError_t launch_pair_t(float *T1o, float *T2, const float *T, const fl
             }
         }
     }
+    return kchunk;
+}
+
+template <int BY, int NST, int MINB, bool kStates>
+static cudaError_t launch_pair_t(float *T1o, float *T2, const float *T, const float *Ci, StepCoef c, Grid3 g,
+                                 cudaStream_t s) {
+    using Z = ZPair<BY>;
+    constexpr size_t smem = NST * Z::SB + 2 * Z::LB + NST * 8;
+    static unsigned attr_gen[64] = {0};
+    cudaError_t ae;
+    if (!set_smem_attr_once((const void *)k_zpair<BY, NST, MINB, kStates>, (int)smem, attr_gen, &ae)) return ae;
+    CUtensorMap mT, mC;
+    if (!make_tensor_map_3d(&mT, T, 4, g, Z::W, Z::TROWS) || !make_tensor_map_3d(&mC, Ci, 4, g, Z::W, Z::ROWS))
+        return cudaErrorInvalidValue;
+    const int64_t ntx = (g.nx + Z::BX - 1) / Z::BX, nty = (g.ny + BY - 1) / BY, tiles = ntx * nty;
+    const int kchunk = pair_kchunk(g, tiles, (int64_t)MINB * sm_count());
     const int64_t gz = (g.nz - 2 + kchunk - 1) / kchunk;
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
     const ZPairParams p{(int)g.nx, (int)g.ny, (int)g.nz, kchunk, (int)ntx, (float)c.dtlam, (float)c.ax, (float)c.ay,
