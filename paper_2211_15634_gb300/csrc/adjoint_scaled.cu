@@ -451,6 +451,35 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
     }
 }
 
+// Planes per chunk where there are only a few waves of CTAs: the one that ends soonest, counting
+// planes and 1.2 more per chunk for whole waves, a last wave with one or two CTAs per SM for
+// 0.5 and 0.86 of a full one (fitted to sweeps of 25 shapes), and the tiles' shorter last
+// chunks in the slots that are left.  us against chunks that give three waves of
+// whatever filling: 100^3 21.1 / 23.7, 128^3 29.7 / 32.1, 160^3 58.4 / 62.3, 128 x 150 x 200
+// 45.5 / 53.2, 161 x 128 x 96 (unequal) 49.8 / 51.6; none of the 25 slower.
+static int adjs_chunk(int64_t nz, int64_t tiles, int64_t slots) {
+    auto wave = [slots](int64_t ctas) { return ctas == 0 ? 0.0 : ctas * 3 <= slots ? 0.5 : ctas * 3 <= 2 * slots ? 0.86 : 1.0; };
+    int kc = 4;
+    double best = 0.0;
+    for (int c = 4; c <= 40 && c <= nz; ++c) {
+        const int64_t full = tiles * (nz / c), waves = full / slots, r = full % slots;
+        const int rem = (int)(nz % c);
+        double last = wave(r) * (c + 1.2);
+        if (rem) {
+            const int64_t over = tiles - (r ? slots - r : 0);  // last chunks beyond the wave's free slots
+            const double l2 = over > 0 ? (r ? c + 1.2 : 0.0) + wave(over < slots ? over : slots) * (rem + 1.2)
+                                       : wave(r + tiles) * (rem + 1.2);
+            last = over > 0 || l2 > last ? l2 : last;
+        }
+        const double cost = (waves * (c + 1.2) + last) * (waves ? 0.98 : 1.0);
+        if (c == 4 || cost < best) {
+            best = cost;
+            kc = c;
+        }
+    }
+    return kc;
+}
+
 template <int kAx, bool kGiven, bool kRag>
 static cudaError_t launch_adjs_t(double *Tbar, double *Csbar, const double *ybar, const double *T,
                                const double *Cs, const EmuCoef &ek, Grid3 g, cudaStream_t s) {
@@ -475,13 +504,11 @@ static cudaError_t launch_adjs_t(double *Tbar, double *Csbar, const double *ybar
         // (3.93 waves) 0.1734 ms against 0.1777 at 16 (4.49 waves); 512^3 at 22-24
         // planes 1.5% ahead of 16.
         const int64_t slots = 3LL * sm_count();
-        const int64_t kc = g.nz * tiles / (3 * slots);
-        if (kc < 16) {
+        if (g.nz * tiles / (3 * slots) < 16) {
             // (chunks below 4 planes only where 4 leave most of the chip idle: 32^3 4.1 us at
             // 1 plane against 7.6, 48^3 5.2 at 2 against 7.7, 64^3 7.6 at 4 against 8.4 at 2)
             const int64_t at4 = tiles * ((g.nz + 3) / 4);
-            const int least = at4 * 8 < slots ? 1 : (at4 * 4 < slots ? 2 : 4);
-            kchunk = (int)(kc < least ? least : kc);
+            kchunk = at4 * 8 < slots ? 1 : (at4 * 4 < slots ? 2 : adjs_chunk(g.nz, tiles, slots));
         } else {
             kchunk = 16;
             int64_t best = -1;
