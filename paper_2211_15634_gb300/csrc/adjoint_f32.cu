@@ -24,6 +24,7 @@
 #include "internal.h"
 #include "pdl.cuh"
 #include "tma.cuh"
+#include "waves.h"
 #include "zmarch.h"
 
 namespace psd {
@@ -778,24 +779,6 @@ cudaError_t launch_adjoint2_f32(float *Tbar, float *Cibar, const float *ybar, co
     return launch_adj2_t<4, 3>(Tbar, Cibar, ybar, S1, S0, Ci, g, p, kchunk, s);
 }
 
-// Planes per CTA of the one-step kernels; slots: CTAs resident at once.
-static int adj32_kchunk(int64_t slots, int64_t nz, int64_t tiles) {
-    // One wave when it takes chunks of at most 12 or of 32-96 planes: every tile's
-    // z-range split into as many chunks as there are CTA slots per tile, all CTAs
-    // resident at once (no tail).  Else 16-plane chunks (each chunk re-reads two planes);
-    // 32 where 16 would leave fewer than four waves of CTAs and 32 still gives one and
-    // a half.  Measured: 256^3 at 64 (one wave; 4.5% ahead of 32, 8% of 16), 512^3 and
-    // 768^3 at 16-24 (within 1%); small grids against the 16 planes they had: 32^3 2.8 /
-    // 10.3 us, 64^3 4.7 / 10.4, 96^3 6.2 / 10.5, 128^3 10 / 12.2, 160 x 128 x 96 13.2 / 16.6.
-    const int64_t cols = nz * tiles;
-    const int64_t per_tile = tiles > 0 ? slots / tiles : 0;
-    const int64_t one_wave = per_tile > 0 ? (nz + per_tile - 1) / per_tile : 0;
-    if (one_wave > 0 && one_wave <= 12)
-        return (int)(one_wave < 2 ? 2 : one_wave);
-    if (one_wave >= 32 && one_wave <= 96) return (int)one_wave;
-    return (cols < 4 * 16 * slots && 2 * cols >= 3 * 32 * slots) ? 32 : 16;
-}
-
 template <int BY, int NST, int MINB>
 static cudaError_t launch_adj32_t(float *Tbar, float *Cibar, const float *ybar, const float *T,
                                   const float *Ci, Grid3 g, Adj32Params p, int kchunk, cudaStream_t s) {
@@ -810,7 +793,13 @@ static cudaError_t launch_adj32_t(float *Tbar, float *Cibar, const float *ybar, 
         !make_tensor_map_3d(&mC, Ci, 4, g, W, H) || !make_tensor_map_3d(&mB, Cibar, 4, g, BX, BY))
         return cudaErrorInvalidValue;
     const int64_t ntx = (g.nx + BX - 1) / BX, nty = (g.ny + BY - 1) / BY, tiles = ntx * nty;
-    if (kchunk <= 0) kchunk = adj32_kchunk((int64_t)MINB * sm_count(), g.nz, tiles);
+    // A few waves: fitted to sweeps of 27 shapes (us against one wave or 16 planes: 144^3 22.6 / 29.8,
+    // 160^3 26.0 / 32.8, 200 x 150 x 128 18.3 / 21.2, 320^3 125 / 131); many: 16 planes (each
+    // chunk re-reads two)
+    if (kchunk <= 0)
+        kchunk = g.nz * tiles < 160LL * MINB * sm_count()
+                     ? wave_chunk(g.nz, tiles, sm_count(), MINB, WaveCost{2.0, 0.6, 0.0, 2, 64})
+                     : 16;
     const int64_t gz = (g.nz + kchunk - 1) / kchunk;
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
     p.nx = (int)g.nx;
@@ -853,18 +842,10 @@ cudaError_t launch_adjoint_f32_rag(float *Tbar, float *Cibar, const float *ybar,
         return cudaErrorInvalidValue;
     const int64_t ntx = (g.nx + BX - 1) / BX, nty = (g.ny + BY - 1) / BY, tiles = ntx * nty;
     int kchunk = launch_override(PS_OVERRIDE_ADJ_KCHUNK);
-    if (kchunk <= 0) {
-        // one wave where it fills the chip (255^3: 37 planes 70 us, 8 planes 76), else 16
-        // planes, 8 where those would be less than two waves (191^3 41 us, 47 at 16; 257^3
-        // 100 at 16, 110 in one wave of 0.87)
-        const int64_t slots = 3LL * sm_count(), per_tile = slots / tiles;
-        const int64_t one_wave = per_tile > 0 ? (g.nz + per_tile - 1) / per_tile : 0;
-        const int64_t used = one_wave > 0 ? tiles * ((g.nz + one_wave - 1) / one_wave) : 0;
-        if (one_wave > 0 && one_wave <= 96 && (one_wave <= 12 || 100 * used >= 95 * slots))
-            kchunk = (int)(one_wave < 2 ? 2 : one_wave);
-        else
-            kchunk = tiles * ((g.nz + 15) / 16) < 2 * slots ? 8 : 16;
-    }
+    // fitted to sweeps of 25 shapes (us against one wave, 8 or 16 planes: 161^3 32.1 / 33.4, 191^3
+    // 42.9 / 45.1, 225^3 59.9 / 63.2, 321^3 157 / 163)
+    if (kchunk <= 0)
+        kchunk = wave_chunk(g.nz, tiles, sm_count(), 3, WaveCost{1.0, 0.5, 0.0, 2, 40});
     const int64_t gz = (g.nz + kchunk - 1) / kchunk;
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
     Adj32Params p{};

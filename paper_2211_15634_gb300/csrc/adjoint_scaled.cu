@@ -36,6 +36,7 @@
 #include "internal.h"
 #include "pdl.cuh"
 #include "tma.cuh"
+#include "waves.h"
 #include "zmarch.h"
 
 namespace psd {
@@ -451,35 +452,6 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
     }
 }
 
-// Planes per chunk where there are only a few waves of CTAs: the one that ends soonest, counting
-// planes and 1.2 more per chunk for whole waves, a last wave with one or two CTAs per SM for
-// 0.5 and 0.86 of a full one (fitted to sweeps of 25 shapes), and the tiles' shorter last
-// chunks in the slots that are left.  us against chunks that give three waves of
-// whatever filling: 100^3 21.1 / 23.7, 128^3 29.7 / 32.1, 160^3 58.4 / 62.3, 128 x 150 x 200
-// 45.5 / 53.2, 161 x 128 x 96 (unequal) 49.8 / 51.6; none of the 25 slower.
-static int adjs_chunk(int64_t nz, int64_t tiles, int64_t slots) {
-    auto wave = [slots](int64_t ctas) { return ctas == 0 ? 0.0 : ctas * 3 <= slots ? 0.5 : ctas * 3 <= 2 * slots ? 0.86 : 1.0; };
-    int kc = 4;
-    double best = 0.0;
-    for (int c = 4; c <= 40 && c <= nz; ++c) {
-        const int64_t full = tiles * (nz / c), waves = full / slots, r = full % slots;
-        const int rem = (int)(nz % c);
-        double last = wave(r) * (c + 1.2);
-        if (rem) {
-            const int64_t over = tiles - (r ? slots - r : 0);  // last chunks beyond the wave's free slots
-            const double l2 = over > 0 ? (r ? c + 1.2 : 0.0) + wave(over < slots ? over : slots) * (rem + 1.2)
-                                       : wave(r + tiles) * (rem + 1.2);
-            last = over > 0 || l2 > last ? l2 : last;
-        }
-        const double cost = (waves * (c + 1.2) + last) * (waves ? 0.98 : 1.0);
-        if (c == 4 || cost < best) {
-            best = cost;
-            kc = c;
-        }
-    }
-    return kc;
-}
-
 template <int kAx, bool kGiven, bool kRag>
 static cudaError_t launch_adjs_t(double *Tbar, double *Csbar, const double *ybar, const double *T,
                                const double *Cs, const EmuCoef &ek, Grid3 g, cudaStream_t s) {
@@ -506,9 +478,17 @@ static cudaError_t launch_adjs_t(double *Tbar, double *Csbar, const double *ybar
         const int64_t slots = 3LL * sm_count();
         if (g.nz * tiles / (3 * slots) < 16) {
             // (chunks below 4 planes only where 4 leave most of the chip idle: 32^3 4.1 us at
-            // 1 plane against 7.6, 48^3 5.2 at 2 against 7.7, 64^3 7.6 at 4 against 8.4 at 2)
-            const int64_t at4 = tiles * ((g.nz + 3) / 4);
-            kchunk = at4 * 8 < slots ? 1 : (at4 * 4 < slots ? 2 : adjs_chunk(g.nz, tiles, slots));
+            // 1 plane against 7.6, 48^3 5.2 at 2 against 7.7, 64^3 7.6 at 4 against 8.4 at 2).
+            // A few waves: fitted to sweeps of 40 shapes (us against chunks for about three waves:
+            // 100^3 21.1 / 23.7, 160^3 58.4 / 62.3, 161^3 69.9 / 77.6, 128 x 150 x 200 45.5 / 53.2), but
+            // not where the last tile of a row is nearly empty: its CTAs end early, and what
+            // the others gain by long chunks is lost (129 x 400 x 96 139 us, 130 in short ones)
+            const int64_t at4 = tiles * ((g.nz + 3) / 4), kc = g.nz * tiles / (3 * slots);
+            const bool thin = g.nx % BX >= 1 && g.nx % BX <= BX / 4;
+            kchunk = at4 * 8 < slots ? 1
+                     : at4 * 4 < slots ? 2
+                     : thin            ? (int)(kc < 4 ? 4 : kc)
+                                       : wave_chunk(g.nz, tiles, sm_count(), 3, WaveCost{0.5, 0.6, 0.05, 3, 40});
         } else {
             kchunk = 16;
             int64_t best = -1;

@@ -16,6 +16,7 @@
 #include "node.cuh"
 #include "pdl.cuh"
 #include "tma.cuh"
+#include "waves.h"
 #include "zmarch.h"
 #include "zmarch_tile.cuh"
 #include "zrag_tile.cuh"
@@ -193,17 +194,23 @@ bool step_tma_ok(Grid3 g, int esz, const void *a, const void *b, const void *c) 
 }
 
 // Planes per CTA of the one-step march.
-static int step_kchunk(int esz, Grid3 g, int64_t tiles) {
+// per_sm: CTAs that an SM holds; waves: their cost, or null.
+static int step_kchunk(int esz, Grid3 g, int64_t tiles, int per_sm, const WaveCost *waves) {
     // Short chunks keep many CTAs in flight (no wave tail) while consecutive
     // CTAs - neighbouring tiles of one chunk - share their halo planes in L2;
     // each chunk pays two extra planes.  Measured (sweeps at 256^3 and 512^3):
-    // FP32 is fastest at 8 planes; FP64 at 8 planes on small grids and flat from
-    // 24 to 40 planes at 512^3, so about 64 CTAs per SM between 8 and 32 planes.
+    // FP32 is fastest at 8 planes; FP64 at 8 planes on small grids, at 13-18 at 320^3 and flat
+    // from 24 to 40 planes at 512^3, so about 32 CTAs per SM between 8 and 32 planes (with 64:
+    // 320^3 134 us a step / 130, 321^3 150 / 144, 384^3 216 / 212).
     // FP32 grids up to 3 million nodes (a few CTAs per SM): 3 planes (128^3 5.1 against 5.6 us).
     if (esz == 4 && (double)g.nx * (double)g.ny * (double)g.nz <= 3e6) return 3;
-    const int64_t target = 64LL * sm_count();
+    const int64_t target = 32LL * sm_count();
     const int64_t kmax = esz == 8 ? 32 : 8;
     const int64_t kc = (g.nz - 2) * tiles / target;
+    // FP64 grids of a few waves: the chunk whose waves end soonest, fitted to sweeps of 13 to 18
+    // shapes each (us a step against 8 planes: 128 x 150 x 200 20.8 / 23.9, 400 x 100 x 60 15.2 /
+    // 16.8, 128^3 12.9 / 16.2, 256 x 40 x 400 22.4 / 24.2)
+    if (waves && kc <= 8) return wave_chunk(g.nz - 2, tiles, sm_count(), per_sm, *waves);
     return (int)(kc < 8 ? 8 : (kc > kmax ? kmax : kc));
 }
 
@@ -230,7 +237,15 @@ static cudaError_t launch_zmarch_t(void *T2, const void *T, void *E2, const void
     }
     const int64_t ntx = (g.nx + BX - 1) / BX, nty = (g.ny + BY - 1) / BY;
     const int64_t tiles = ntx * nty;
-    if (kchunk <= 0) kchunk = step_kchunk(sizeof(E), g, tiles);
+    if (kchunk <= 0) {
+        constexpr WaveCost wide{2.0, 0.6, 0.2, 3, 12}, narrow{1.0, 0.4, 0.2, 3, 8};
+        constexpr bool kWide = MODE == Z_F64_SCALED4;
+        // (from 2.5 waves of 8 planes on, 8 stay as fast or faster: 128 x 144 x 496 45 us a step, 46 at 12)
+        const bool few = 2 * tiles * ((g.nz + 5) / 8) < 5 * 5LL * sm_count();
+        kchunk = step_kchunk(sizeof(E), g, tiles, kWide ? 5 : 4,
+                             kWide ? (few ? &wide : nullptr)
+                             : MODE == Z_F64_SCALED || MODE == Z_F64_EMU_ISO_DMUL ? &narrow : nullptr);
+    }
     const int64_t gz = (g.nz - 2 + kchunk - 1) / kchunk;
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
     p.nx = g.nx;
@@ -299,7 +314,11 @@ static cudaError_t launch_rag_t(void *T2, const void *T, const void *Ci, Grid3 g
         return cudaErrorInvalidValue;
     const int64_t ntx = (g.nx - 2 + R::BX - 1) / R::BX, nty = (g.ny - 2 + BY - 1) / BY, tiles = ntx * nty;
     int kchunk = launch_override(PS_OVERRIDE_KCHUNK);
-    if (kchunk <= 0) kchunk = step_kchunk(sizeof(E), g, tiles);
+    if (kchunk <= 0) {
+        constexpr WaveCost ragged{0.5, 0.4, 0.1, 3, 12};
+        kchunk = step_kchunk(sizeof(E), g, tiles, 3,
+                             MODE == Z_F64_SCALED || MODE == Z_F64_EMU_ISO_DMUL ? &ragged : nullptr);
+    }
     const int64_t gz = (g.nz - 2 + kchunk - 1) / kchunk;
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
     p.nx = g.nx;

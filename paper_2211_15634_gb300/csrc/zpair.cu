@@ -317,9 +317,9 @@ int pair_kchunk(Grid3 g, int64_t tiles, int64_t slots) {
         const int64_t per_tile = tiles > 0 ? slots / tiles : 0;
         const int64_t one_wave = per_tile > 0 ? (g.nz - 2 + per_tile - 1) / per_tile : 0;
         if (one_wave <= 96 && one_wave > 0) {
-            // all CTAs resident at once; chunks of fewer than six planes lose more than they
-            // spread (odd rows, 129^3: 7.6 us a step at 4 planes, 6.4 at 6, 7.5 at 8)
-            kchunk = (int)(one_wave < 6 ? 6 : one_wave);
+            // all CTAs resident at once (112^3 5.4 us a step at 3 planes, 6.6 at 6; odd rows, 129^3 7.6
+            // at 4, 7.1 at 5, 7.6 at 6)
+            kchunk = (int)(one_wave < 3 ? 3 : one_wave);
         } else {
             // the chunk whose waves march the fewest planes in all (each chunk two and a half
             // more than it stores): 384^3 61 us a step at 40 planes, 67 at 35
