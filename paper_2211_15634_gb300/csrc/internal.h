@@ -173,7 +173,7 @@ unsigned batch_device_error(bool clear);
 int64_t batch_zmarch_xy_tiles(int dtype, int64_t nx, int64_t ny, BatchItem *out);
 // fused-pair tiles (one width, 8 rows), kind 2; returns their number
 int64_t batch_zmarch2_xy_tiles(int dtype, int64_t nx, int64_t ny, BatchItem *out);
-constexpr int kBatchZmarchMaps = 9;  // tensor maps per problem (wide, narrow, fused pair)
+constexpr int kBatchZmarchMaps = 12;  // tensor maps per problem (wide, narrow, quarter, fused pair)
 bool batch_zmarch_fill(void *zparams_dst, void *z2params_dst, void *maps_dst, const BatchProblem &r,
                        StepCoef c, int dtype);
 size_t batch_z2params_bytes();

@@ -81,7 +81,7 @@ __device__ __forceinline__ void zmarch_tile(const CUtensorMap *tmT, const CUtens
     using Tr = ZTraits<MODE>;
     using E = typename Tr::E;
     using V = typename Tr::V;
-    static_assert(LPR == 32 || LPR == 16, "a tile row is one warp or half a warp");
+    static_assert(LPR == 32 || LPR == 16 || LPR == 8, "a tile row is a warp, half or a quarter of one");
     constexpr int PX = Tr::PX, HX = PX, BX = LPR * PX, W = BX + 2 * HX, H = BY + 2;
     constexpr unsigned TB = W * H * sizeof(E), CB = BX * BY * sizeof(E);
     constexpr unsigned TBA = (TB + 127) / 128 * 128, CBA = (CB + 127) / 128 * 128;
@@ -155,7 +155,7 @@ __device__ __forceinline__ void zmarch_tile(const CUtensorMap *tmT, const CUtens
     const int gx0 = X0 + lane * PX;
     const bool row_ok = gy >= 1 && gy <= p.ny - 2;
     // lanes of this warp that compute (the fast-path vote below runs inside row_ok;
-    // with two tile rows per warp, row_ok can differ between the halves)
+    // with several tile rows per warp, row_ok can differ between them)
     const unsigned rmask = LPR == 32 ? 0xffffffffu : __ballot_sync(0xffffffffu, row_ok);
     bool all_x = gx0 >= 1 && gx0 + PX - 1 <= p.nx - 2;
     E *__restrict__ T2 = (E *)T2v;
