@@ -1085,12 +1085,13 @@ int ps_from_deviation_pair(double *T, const float *D, const float *E, double t_r
 // ------------------------------------------------------------------ batch
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// kernel 1 (z-march): the x-y tile is the kernel's own; default chunks of 64 planes
-// (measured on the 256-problem workload: 64 >= 32 > 16 > 8 planes, FP32 and FP64)
+// kernel 1 (z-march): the x-y tile is the kernel's own; the caller has set tz (batch_zchunk), fused
+// pairs take chunks of kPairZ planes (measured on the 256-problem workload: 64 >= 32 > 16 > 8)
+constexpr int kPairZ = 64;
 static int resolve_tiles(int dtype, int *tx, int *ty, int *tz, int kernel = 0) {
     int dx, dy, dz;
     batch_default_tile(dtype, &dx, &dy, &dz);
-    if (kernel == 1) dz = 64;
+    if (kernel == 1) dz = kPairZ;
     if (*tx == 0) *tx = dx;
     if (*ty == 0) *ty = dy;
     if (*tz == 0) *tz = dz;
@@ -1185,6 +1186,23 @@ static int64_t items_of(const ps_problem &p, int kernel, int dtype, int tx, int 
     return ((p.nx - 2 + tx - 1) / tx) * ((p.ny - 2 + ty - 1) / ty) * ((p.nz - 2 + tz - 1) / tz);
 }
 
+// Default planes per z-march item.  With P planes for each of the chip's CTA slots, an item of c
+// planes reads two and a half more (P * 2.5 / c in all) and leaves up to c planes of tail: c
+// about 2 sqrt(P).  FP32 items are bound by latency rather than issue and want half as many again,
+// and where whole grids fill most of one wave they stay whole.  Measured, 10 steps (us, 64 planes /
+// this rule): FP64 16 grids of 32^3 to 64^3 460 / 195, 64 of 40^3 to 70^3 932 / 775, 64 of 60^3 to
+// 110^3 2500 / 2250, 128 of 32^3 to 160^3 7488 / 7480; FP32 267 / 98, 435 / 370, 1164 / 1060, 3374 /
+// 3375; 128 of 40^3 to 60^3 479 whole, 525 in 16 planes.
+static int batch_zchunk(const ps_problem *probs, int nprob, int dtype) {
+    double planes = 0.0;
+    for (int q = 0; q < nprob; ++q)
+        planes += (double)batch_zmarch_xy_tiles(dtype, probs[q].nx, probs[q].ny, nullptr) * (double)(probs[q].nz - 2);
+    const double P = planes / (4.0 * sm_count());
+    if (dtype == PS_F32 && P >= 34.0 && P <= 64.0) return 64;
+    const double c = (dtype == PS_F64 ? 2.0 : 3.0) * std::sqrt(P);
+    return c < 4.0 ? 4 : (c > 64.0 ? 64 : (int)c);
+}
+
 struct TableLayout {
     size_t problems, zparams, z2params, maps, items, items2, bytes;
 };
@@ -1224,6 +1242,8 @@ static int plan_table(const ps_problem *probs, int nprob, int dtype, int tile_x,
     }
     const int k = choose_kernel(probs, nprob, dtype, flags);
     if (k < 0) return k;
+    const int tile_z2 = tile_z ? tile_z : kPairZ;
+    if (k == 1 && tile_z == 0) tile_z = batch_zchunk(probs, nprob, dtype);
     PS_TRY(resolve_tiles(dtype, &tile_x, &tile_y, &tile_z, k));
     int64_t n = 0, n2 = 0;
     for (int q = 0; q < nprob; ++q) {
@@ -1231,8 +1251,10 @@ static int plan_table(const ps_problem *probs, int nprob, int dtype, int tile_x,
         const int st = problem_tiles(probs[q], dtype, tile_x, tile_y, tile_z, &tx, &ty, &tz, k);
         if (st != PS_OK) return fail(st, "problem %d: %s", q, g_err.c_str());
         n += items_of(probs[q], k, dtype, tx, ty, tz);
-        if (flags & PS_BATCH_TEMPORAL2)
-            n2 += batch_zmarch2_xy_tiles(dtype, probs[q].nx, probs[q].ny, nullptr) * ((probs[q].nz - 2 + tz - 1) / tz);
+        if (flags & PS_BATCH_TEMPORAL2) {
+            const int tz2 = probs[q].tile_z ? probs[q].tile_z : tile_z2;
+            n2 += batch_zmarch2_xy_tiles(dtype, probs[q].nx, probs[q].ny, nullptr) * ((probs[q].nz - 2 + tz2 - 1) / tz2);
+        }
     }
     if (k == 1 && (n > 0x7fffffffLL || n2 > 0x7fffffffLL))
         return fail(PS_ERR_ARG, "%lld work items: at most 2^31-1", (long long)std::max(n, n2));
@@ -1262,6 +1284,8 @@ int ps_batch_table_fill_ex(void *host_buf, size_t bytes, const ps_problem *probs
     int64_t nitems = 0, nitems2 = 0;
     int kernel = 0;
     PS_TRY(plan_table(probs, nprob, dtype, tile_x, tile_y, tile_z, flags, &nitems, &nitems2, &kernel));
+    const int tile_z2 = tile_z ? tile_z : kPairZ;
+    if (kernel == 1 && tile_z == 0) tile_z = batch_zchunk(probs, nprob, dtype);
     PS_TRY(resolve_tiles(dtype, &tile_x, &tile_y, &tile_z, kernel));
     const TableLayout L = table_layout(nprob, nitems, nitems2, kernel);
     if (bytes < L.bytes) return fail(PS_ERR_ARG, "table buffer has %zu bytes, needs %zu", bytes, L.bytes);
@@ -1342,16 +1366,17 @@ int ps_batch_table_fill_ex(void *host_buf, size_t bytes, const ps_problem *probs
                     it.nk = (int16_t)std::min<int64_t>(tz, p.nz - 1 - k0);
                     work.push_back({0, it});
                 }
-            if (nitems2) {  // the fused-pair list: wide tiles only, the same z-chunks
+            if (nitems2) {  // the fused-pair list: wide tiles only
                 std::vector<BatchItem> xy2((size_t)batch_zmarch2_xy_tiles(dtype, p.nx, p.ny, nullptr));
                 batch_zmarch2_xy_tiles(dtype, p.nx, p.ny, xy2.data());
-                for (int64_t k0 = 1; k0 < p.nz - 1; k0 += tz)
+                const int tz2 = p.tile_z ? p.tile_z : tile_z2;
+                for (int64_t k0 = 1; k0 < p.nz - 1; k0 += tz2)
                     for (const BatchItem &t : xy2) {
                         BatchItem it = t;
                         it.prob = q;
                         it.k0 = (int32_t)k0;
                         it.ni = it.nj = 0;
-                        it.nk = (int16_t)std::min<int64_t>(tz, p.nz - 1 - k0);
+                        it.nk = (int16_t)std::min<int64_t>(tz2, p.nz - 1 - k0);
                         work2.push_back({0, it});
                     }
             }
