@@ -70,12 +70,12 @@ def coefficient(Ci, lam, dt, inv):
 
 
 def state_pairs_default(T0) -> bool:
-    """Whether the forward pass's state-keeping loops run fused step pairs that write both
-    states (``api.run_states(temporal2=True)``: FP32 only; bit for bit the same states).
-    Measured at 256^3, nt = 200: 200 states in 5.74 against 6.71 ms, the gradient with every
-    state kept 18.52 against 19.52 ms.  The reverse sweep's recomputes stay single steps by
-    default: there they run beside the transposed steps, and in pairs the sqrt(nt)
-    gradient measured slower (22.00 against 21.80 ms)."""
+    """Whether the loops that keep states run fused step pairs that write both states
+    (``api.run_states(temporal2=True)``: FP32 only; bit for bit the same states; single
+    steps where pairs would not be faster).  Measured at 256^3, nt = 200: 200 states in
+    5.39 against 6.84 ms, the gradient with every state kept 18.1 against 19.5 ms.  The
+    recomputes run beside the transposed steps: 192^3, nt = 60, a checkpoint every 8 steps
+    3.28 ms against 3.40, 256^3, 49, every 7 5.07 against 5.16, 160^3, 64, 8 2.51 and 2.49."""
     return T0.dtype == torch.float32
 
 
@@ -156,9 +156,9 @@ def backward_checkpointed(ybar_nt, Ci, lam, dt, inv, nt, every, ckpts, coef=None
     :func:`forward_checkpointed`.  ``kept``: segments whose states the forward kept
     (:func:`forward_checkpointed`); they are not recomputed, and their blocks then serve
     as the recomputes' buffers.  ``state_pairs``: the recomputes run fused step pairs, as
-    in :func:`forward_checkpointed` (default off, see :func:`state_pairs_default`)."""
+    in :func:`forward_checkpointed` (default :func:`state_pairs_default`)."""
     C, scaled = coefficient(Ci, lam, dt, inv) if coef is None else coef
-    spairs = bool(state_pairs)
+    spairs = state_pairs_default(ybar_nt) if state_pairs is None else bool(state_pairs)
     pairs = bool(pairs) and not scaled and api.adjoint2_supported(ybar_nt)
     ybar = ybar_nt.contiguous().clone()
     tbar = torch.empty_like(ybar)
