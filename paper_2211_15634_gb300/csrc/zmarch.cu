@@ -373,6 +373,10 @@ cudaError_t launch_zmarch(int mode, void *T2, const void *T, void *E2, const voi
             // axis keeps its own rounded product (512 x 384 x 256: 443 against 280 us)
             if (!p.ek.common)
                 return launch_zmarch_b<Z_F64_EMU_ANISO_FAR, 8, 4>(T2, T, E2, Ein, Ci, g, p, kchunk, s, wb);
+            // four nodes per thread on large grids (us a step, two / four: 512 x 384 x 256 280 / 273, 512^3
+            // 731 / 711, 256^3 103 / 103, 240 x 200 x 300 100 / 103)
+            if ((double)g.n() >= 3e7 && f64_scaled_wide(g, T2, T, Ci))
+                return launch_zmarch_b<Z_F64_EMU_ANISO4, 4, 4>(T2, T, E2, Ein, Ci, g, p, kchunk, s, wb);
             return launch_zmarch_b<Z_F64_EMU_ANISO, 8, 4>(T2, T, E2, Ein, Ci, g, p, kchunk, s, wb);
         case Z_F64_NATIVE:
             return launch_zmarch_b<Z_F64_NATIVE, 8, 4>(T2, T, E2, Ein, Ci, g, p, kchunk, s, wb);

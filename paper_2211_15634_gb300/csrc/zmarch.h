@@ -17,6 +17,7 @@ enum ZMode {
     Z_F64_EMU_ISO_DMUL = 5,  // two FP64 ops per node: fma(Ci*K, S, T)
     Z_F64_SCALED = 6,        // Ci already holds dt*lam*_d^2*Ci: fma(Cs, S, T)
     Z_F64_SCALED4 = 7,       // as Z_F64_SCALED, four nodes per thread (32-byte accesses)
+    Z_F64_EMU_ANISO4 = 9,    // as Z_F64_EMU_ANISO, four nodes per thread
     Z_F64_EMU_ANISO_FAR = 8,  // spacings more than 16 apart: one rounded product per axis
 };
 

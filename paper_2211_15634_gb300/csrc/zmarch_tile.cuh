@@ -52,6 +52,8 @@ struct ZTraits<Z_F64_SCALED4> {
     static constexpr int PX = 4;
 };
 template <>
+struct ZTraits<Z_F64_EMU_ANISO4> : ZTraits<Z_F64_SCALED4> {};
+template <>
 struct ZTraits<Z_F32> {
     using E = float;
     using V = float4;
@@ -188,8 +190,9 @@ __device__ __forceinline__ void zmarch_tile(const CUtensorMap *tmT, const CUtens
             V cv{};  // E2 at the own nodes (two-float state)
             V out;
             if constexpr (MODE == Z_F64_EMU_ISO || MODE == Z_F64_EMU_ANISO || MODE == Z_F64_EMU_ANISO_FAR ||
-                          MODE == Z_F64_EMU_ISO_DMUL || MODE == Z_F64_SCALED || MODE == Z_F64_SCALED4) {
-                constexpr int kAx = MODE == Z_F64_EMU_ANISO ? AX_COMMON
+                          MODE == Z_F64_EMU_ISO_DMUL || MODE == Z_F64_SCALED || MODE == Z_F64_SCALED4 ||
+                          MODE == Z_F64_EMU_ANISO4) {
+                constexpr int kAx = MODE == Z_F64_EMU_ANISO || MODE == Z_F64_EMU_ANISO4 ? AX_COMMON
                                     : MODE == Z_F64_EMU_ANISO_FAR ? AX_FAR : AX_ISO;
                 constexpr bool kDmul = MODE == Z_F64_EMU_ISO_DMUL;
                 constexpr bool kScaled = MODE == Z_F64_SCALED || MODE == Z_F64_SCALED4;
