@@ -356,7 +356,8 @@ int ps_device_error(unsigned *out_host, int clear) {
                 adjoint_scaled_device_error(clear != 0) | zmarch2_device_error(clear != 0) |
                 adjoint_f32_device_error(clear != 0) | batch_device_error(clear != 0) |
                 batch_zmarch_device_error(clear != 0) |
-                zpair_device_error(clear != 0) | zpair_rag_device_error(clear != 0);
+                zpair_device_error(clear != 0) | zpair_rag_device_error(clear != 0) |
+                comp_rag_device_error(clear != 0);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "ps_device_error");
     return PS_OK;

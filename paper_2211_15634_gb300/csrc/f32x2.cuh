@@ -26,6 +26,7 @@ __device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
 }
 // a - b as a fused multiply-add by -1: one rounding, the difference's (sub.f32x2 was slower)
 __device__ __forceinline__ f2 f2_sub(f2 a, f2 b) { return f2_fma(b, 0xbf800000bf800000ull, a); }
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b) { return f2_fma(a, 0x3f8000003f800000ull, b); }
 
 struct V4 {  // four nodes of a row
     f2 a, b;
@@ -34,5 +35,10 @@ __device__ __forceinline__ V4 v4_sub(V4 x, V4 y) { return V4{f2_sub(x.a, y.a), f
 struct ZCoef2 {
     f2 dtlam, ax, ay, az;
 };
+
+// Four nodes of a row 32 apart, from f.
+__device__ __forceinline__ V4 v4_load32(const float *f) {
+    return V4{f2_make(f[0], f[32]), f2_make(f[64], f[96])};
+}
 
 }  // namespace psd

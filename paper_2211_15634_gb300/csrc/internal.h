@@ -78,6 +78,7 @@ cudaError_t launch_step2_states_f32(float *T1o, float *T2, const float *T, const
 unsigned zmarch2_device_error(bool clear);
 unsigned zpair_device_error(bool clear);
 unsigned zpair_rag_device_error(bool clear);
+unsigned comp_rag_device_error(bool clear);
 const char *step_f64_kernel_name(Grid3 g, const void *T2, const void *T, const void *Ci, StepCoef c,
                                  bool scaled);
 const char *step_f32_kernel_name(Grid3 g, const void *T2, const void *T, const void *Ci);

@@ -22,13 +22,15 @@ cudaError_t launch_step_f32(float *T2, const float *T, const float *Ci, StepCoef
     return launch_step_basic<float, false>(T2, T, nullptr, nullptr, Ci, coef_f32(c), g, s, false);
 }
 
-// Two-float state (D, E) -> (D2, E2): the TMA z-march stages E like T.
+// Two-float state (D, E) -> (D2, E2): the TMA z-march stages E like T (odd rows: zcomp_rag.cu).
 cudaError_t launch_step_f32_comp(float *T2, const float *T, float *E2, const float *E, const float *Ci,
                                  StepCoef c, Grid3 g, cudaStream_t s, bool in_loop) {
     if (in_loop && step_small(g, Z_F32_COMP))
         return launch_step_basic<float, true>(T2, T, E2, E, Ci, coef_f32(c), g, s, true);
     if (step_tma_ok(g, 4, T2, T, Ci) && step_tma_ok(g, 4, E2, E, Ci))
         return launch_zmarch(Z_F32_COMP, T2, T, E2, E, Ci, c, g, s);
+    if (comp_ragged_ok(g, T2, T, Ci))
+        return launch_comp_ragged(T2, T, E2, E, Ci, c, g, s);
     return launch_step_basic<float, true>(T2, T, E2, E, Ci, coef_f32(c), g, s, false);
 }
 

@@ -125,7 +125,7 @@ bool make_tensor_map_rows(CUtensorMap *m, const void *ptr, int esz, int64_t n, i
 bool make_tensor_map_quarter(CUtensorMap *m, const float *ptr, Grid3 g, int64_t r, unsigned bx, unsigned by) {
     auto fn = encode_fn();
     if (!fn) return false;
-    const int64_t shift = r * g.nx & 3;
+    const int64_t shift = (r * g.nx + (int64_t)((uintptr_t)ptr >> 2)) & 3;
     const cuuint64_t dims[2] = {(cuuint64_t)(g.nx + shift), (cuuint64_t)((g.ny * g.nz - r + 3) / 4)};
     const cuuint64_t strides[1] = {(cuuint64_t)(16 * g.nx)};
     const cuuint32_t box[2] = {bx, by}, estr[2] = {1, 1};
@@ -163,9 +163,10 @@ bool step_small(Grid3 g, int mode) {
                      // ragged 205^3 20.8 / 21.7, 211^3 25.5 / 23.8
             return n <= (aligned ? (full ? 6e5 : 7.5e6) : 8.8e6);
         case Z_F32_COMP:  // 160^3 14 / 19, 176^3 25 / 25; full rows 128^3 9.4 / 10.9, 368 x 112 x 72
-                          // 12.0 / 10.8; ragged rows have no march: only the column
-                          // kernel's chunks differ (343 x 96 x 95: 12.0 us, long ones 11.6)
-            return n <= (aligned ? (full ? 2.2e6 : 4.3e6) : 2.5e6);
+                          // 12.0 / 10.8; odd rows (zcomp_rag.cu) 2.1e6 nodes 11.3 / 9.9, rows that
+                          // leave lanes idle 173^3 24 / 25, 177^3 30 / 26, 163 x 150 x 200 26 / 25
+            if (!aligned) return n <= ((double)(g.nx - 2) >= 0.85 * 128.0 * (double)((g.nx - 2 + 127) / 128) ? 2e6 : 5.2e6);
+            return n <= (full ? 2.2e6 : 4.3e6);
         case Z_F64_EMU_ANISO:  // 192^3 37 / 41, 200^3 53 / 49; ragged 219^3 61 / 64, 227^3 71 / 69
             return n <= (aligned ? 7.5e6 : 1.05e7);
         default: {
@@ -186,6 +187,14 @@ bool step_ragged_ok(Grid3 g, int esz, const void *a, const void *b, const void *
     if (esz == 4 && (double)(g.nx - 2) < 0.6 * 128.0 * (double)((g.nx - 2 + 127) / 128) &&
         launch_override(PS_OVERRIDE_KCHUNK) <= 0)
         return false;
+    return ragged_supported(g, a, b, c);
+}
+
+bool comp_ragged_ok(Grid3 g, const void *a, const void *b, const void *c) {
+    if (launch_override(PS_OVERRIDE_STEP_PLAIN) == 1 || g.nx % 4 == 0) return false;
+    // rows that leave more than half of the 128-node tiles idle: the column kernel (us a step, column
+    // / here: 67 x 400 x 400, 0.51 in use, 86 / 55; 131 x 300 x 300, 0.50, 85 / 60)
+    if ((double)(g.nx - 2) < 0.5 * 128.0 * (double)((g.nx - 2 + 127) / 128)) return false;
     return ragged_supported(g, a, b, c);
 }
 

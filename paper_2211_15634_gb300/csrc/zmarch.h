@@ -37,13 +37,19 @@ bool step_tma_ok(Grid3 g, int esz, const void *a, const void *b, const void *c);
 // nx, fewer than 2^31 elements.
 bool ragged_supported(Grid3 g, const void *a, const void *b, const void *c);
 bool step_ragged_ok(Grid3 g, int esz, const void *a, const void *b, const void *c);
+bool comp_ragged_ok(Grid3 g, const void *a, const void *b, const void *c);  // the two-float step
 // Map over n consecutive elements: rows of rowlen (a multiple of 16 bytes; a last part of a
 // row is left out) with a box of bx x by, or with by = 0 one line with a box of bx.
 bool make_tensor_map_rows(CUtensorMap *m, const void *ptr, int esz, int64_t n, int64_t rowlen, unsigned bx,
                           unsigned by);
 // Map over the FP32 grid's rows r, r+4, ... (flat rows y + ny*z, r < 4) with a box of bx x by; row r
-// starts at element r*nx mod 4 of the map's first row.
+// starts at element (r*nx + the field's first element in its 16 bytes) mod 4 of the map's rows.
 bool make_tensor_map_quarter(CUtensorMap *m, const float *ptr, Grid3 g, int64_t r, unsigned bx, unsigned by);
+// The four such maps (by flat row mod 4) of N fields.
+template <int N>
+struct RagMaps {
+    CUtensorMap f[N][4];
+};
 // Planes per chunk of the FP32 pair kernels for `tiles` tiles on `slots` resident CTAs.
 int pair_kchunk(Grid3 g, int64_t tiles, int64_t slots);
 // Grids whose steps inside a time loop take the column kernels (stencil_basic.cuh); mode:
@@ -91,5 +97,9 @@ cudaError_t launch_zmarch(int mode, void *T2, const void *T, void *E2, const voi
 cudaError_t launch_zmarch_ragged(int mode, void *T2, const void *T, const void *Ci, StepCoef c, Grid3 g,
                                  cudaStream_t s, bool write_bnd = false);
 unsigned zmarch_device_error(bool clear);
+// One step of the two-float state on ragged rows (zcomp_rag.cu); the caller has checked comp_ragged_ok
+// of T2, T and Ci.  E and E2 may start at any element.
+cudaError_t launch_comp_ragged(float *T2, const float *T, float *E2, const float *E, const float *Ci, StepCoef c,
+                               Grid3 g, cudaStream_t s);
 
 }  // namespace psd

@@ -25,10 +25,6 @@ namespace psd {
 
 __device__ unsigned g_zpair_rag_error;  // set when an mbarrier wait times out
 
-struct RagMaps {
-    CUtensorMap T[4], C[4];  // by flat row mod 4
-};
-
 struct ZPairRagParams {
     int nx, ny, nz, kchunk, ntx;
     float dtlam, ax, ay, az;
@@ -49,10 +45,6 @@ struct ZPairRag {
     static __device__ __forceinline__ int crow(int q) { return 4 * TGF + (q & 3) * CGF + (q >> 2) * W; }
 };
 
-// Four nodes of a row 32 apart, from f.
-__device__ __forceinline__ V4 v4_load32(const float *f) {
-    return V4{f2_make(f[0], f[32]), f2_make(f[64], f[96])};
-}
 // f32_node of four nodes: l / r the x-neighbours, up / dn the rows above and below, en = zp - c and
 // eo = c - zm the differences along z.
 __device__ __forceinline__ V4 v4_step32(V4 c, V4 l, V4 r, V4 up, V4 dn, V4 en, V4 eo, V4 ci, const ZCoef2 &k) {
@@ -68,7 +60,7 @@ __device__ __forceinline__ V4 v4_pick(const bool (&m)[4], V4 x, V4 y) {
 
 template <int BY, int NST, int MINB>
 __global__ void __launch_bounds__(ZPairRag<BY>::NTH, MINB)
-k_zpair_rag(const __grid_constant__ RagMaps maps, float *__restrict__ T2, const ZPairRagParams p) {
+k_zpair_rag(const __grid_constant__ RagMaps<2> maps, float *__restrict__ T2, const ZPairRagParams p) {
     using Z = ZPairRag<BY>;
     constexpr int W1 = Z::W1, ROWS = Z::ROWS, NW = Z::NW, LBF = Z::LB / 4;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -94,11 +86,11 @@ k_zpair_rag(const __grid_constant__ RagMaps maps, float *__restrict__ T2, const 
         const int r = q * ny + Y0 - 2, rc = r - ny + 1;
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-            tma_load_2d(st + i * Z::TGF, &maps.T[(r + i) & 3], &bar[s], xt - 4, (r + i) >> 2);
+            tma_load_2d(st + i * Z::TGF, &maps.f[0][(r + i) & 3], &bar[s], xt - 4, (r + i) >> 2);
         if (j >= 2)
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-                tma_load_2d(st + 4 * Z::TGF + i * Z::CGF, &maps.C[(rc + i) & 3], &bar[s], xt - 4, (rc + i) >> 2);
+                tma_load_2d(st + 4 * Z::TGF + i * Z::CGF, &maps.f[1][(rc + i) & 3], &bar[s], xt - 4, (rc + i) >> 2);
     };
     if (threadIdx.x == 0) {
         s_abort = 0;
@@ -282,10 +274,10 @@ static cudaError_t launch_pair_rag_t(float *T2, const float *T, const float *Ci,
     static unsigned attr_gen[64] = {0};
     cudaError_t ae;
     if (!set_smem_attr_once((const void *)k_zpair_rag<BY, NST, MINB>, (int)smem, attr_gen, &ae)) return ae;
-    RagMaps maps;
+    RagMaps<2> maps;
     for (int m = 0; m < 4; ++m)
-        if (!make_tensor_map_quarter(&maps.T[m], T, g, m, Z::W, Z::TG) ||
-            !make_tensor_map_quarter(&maps.C[m], Ci, g, m, Z::W, Z::CG))
+        if (!make_tensor_map_quarter(&maps.f[0][m], T, g, m, Z::W, Z::TG) ||
+            !make_tensor_map_quarter(&maps.f[1][m], Ci, g, m, Z::W, Z::CG))
             return cudaErrorInvalidValue;
     const int64_t ntx = (g.nx - 2 + Z::BX - 1) / Z::BX, nty = (g.ny - 2 + BY - 1) / BY, tiles = ntx * nty;
     const int kchunk = pair_kchunk(g, tiles, (int64_t)MINB * sm_count());
