@@ -83,8 +83,10 @@ typedef enum {
 #define PS_RUN_TEMPORAL2 16u  /* run only: two steps per pass (temporal blocking of depth
                                  2), bit for bit the same result; needs PS_F32 without
                                  PS_RUN_COMPENSATED, or PS_F64 with PS_RUN_CI_SCALED (else
-                                 PS_ERR_UNSUPPORTED); grids the TMA kernels cannot serve
-                                 (nx*sizeof not a multiple of 16) run single steps */
+                                 PS_ERR_UNSUPPORTED).  FP64: rows that are no multiple of
+                                 16 bytes run single steps.  FP32: pairs wherever they are
+                                 faster, and a loop without the flag takes them too, but for
+                                 its last step (the other buffer then holds T(nt-1)) */
 
 /* Library version (major*10000 + minor*100 + patch). */
 int ps_version(void);
@@ -220,7 +222,8 @@ int ps_diffusion3d_run_ex(void *T, void *T2, void *comp, const void *Ci, double 
  * states - with every = 1 pairs that write both states (one pass over HBM per
  * two states: read the state and Ci, write two states); with every > 1 pairs
  * that never step over a kept state (a single step where one would).  Grids
- * the fused-pair kernel cannot serve run single steps.  Which work grid holds
+ * where pairs would not be faster, and rows that are no multiple of 16 bytes,
+ * run single steps.  Which work grid holds
  * T(nt) can differ from the single-step loop's (*final_slot says). */
 int ps_diffusion3d_run_states(const void *T0, void *states, int64_t grid_stride, int every,
                               const void *Ci, double lam, double dt, double _dx, double _dy,
@@ -438,7 +441,8 @@ int ps_diffusion2d_run(void *T, void *T2, const void *Ci, double lam, double dt,
  *    caches; any sizes and pitches;
  *  - the TMA z-march (PS_BATCH_ZMARCH): one CTA per item, the x-y tile of
  *    the single-grid step kernel (64 x 8 nodes FP64, 128 x 8 FP32, boundary
- *    included) and tile_z planes, staged by TMA, with the single-grid step's
+ *    included; the last columns in tiles of half or a quarter of that width)
+ *    and tile_z planes, staged by TMA, with the single-grid step's
  *    arithmetic (a problem's result equals its single run's bit for bit).
  *    Needs rows that start on 16-byte boundaries (pitch * element size a
  *    multiple of 16; see `pitch`), the CUDA driver's tensor-map encoder, and
@@ -467,14 +471,14 @@ typedef struct {
 #define PS_BATCH_TEMPORAL2 8u  /* z-march, PS_F32 or PS_F64 with PS_BATCH_CI_SCALED: the table
                                   also lists two-steps-per-pass items (temporal blocking of
                                   depth 2, the single-grid fused-pair kernel's tiles: 64 x 8
-                                  FP64, 128 x 8 FP32, the problem's tile_z planes) for
+                                  FP64, 128 x 8 FP32, tile_z or else 64 planes) for
                                   ps_diffusion3d_batch_run_ex with PS_RUN_TEMPORAL2 */
 
 /* Bytes of the table for these problems, tile shape and flags (tile_x,
  * tile_y: interior nodes per column-march item in x and y, tile_x*tile_y
  * <= 4096; tile_z: planes per item; 0 picks the library default for the
- * dtype and kernel (z-march: 64 planes); a problem's own nonzero tile
- * fields override these).  0 when an
+ * dtype and kernel (z-march: 4 to 64 planes, by the work of the whole batch);
+ * a problem's own nonzero tile fields override these).  0 when an
  * argument is invalid (ps_batch_table_fill_ex reports why). */
 size_t ps_batch_table_bytes_ex(const ps_problem *probs, int nprob, int dtype, int tile_x, int tile_y,
                                int tile_z, unsigned flags);

@@ -163,12 +163,12 @@ struct BatchItem {
     int32_t prob;
     int32_t i0, j0, k0;      // first interior node of the work item
     int16_t ni, nj, nk;       // extents (clipped to the interior; z-march: ni = nj = 0)
-    int16_t kind;             // z-march: 0 a wide tile (one warp per row), 1 a narrow one
+    int16_t kind;             // z-march: 0 a wide tile (one warp per row), 1 half, 2 a quarter as wide
 };
 cudaError_t launch_batch_step(const void *dev_table, int parity, int dtype, cudaStream_t s);
 unsigned batch_device_error(bool clear);
 // TMA z-march batch (batch_tma.cu): tile width per dtype, tile height, the per-problem
-// records (ZParams and three tensor maps), the launch (grid = one CTA per item)
+// records (ZParams and twelve tensor maps), the launch (grid = one CTA per item)
 // x-y tiles of the z-march over an nx x ny plane: (x0, y0, kind) into out[i].i0/.j0/.kind
 // when out is not null; returns their number
 int64_t batch_zmarch_xy_tiles(int dtype, int64_t nx, int64_t ny, BatchItem *out);

@@ -1,6 +1,6 @@
 // FP32 forward step dispatch (deviation storage D = T - T_ref): TMA z-march when nx is a
-// multiple of 4, else its row-by-row form (zrag_tile.cuh) below 2^31 nodes, else the plain
-// column march.  Small grids inside a time loop take the column march (stencil_basic.cuh).
+// multiple of 4, else its row-by-row form (zrag_tile.cuh; the two-float state zcomp_rag.cu) below
+// 2^31 nodes, else the plain column march.  Small grids inside a time loop take the column march (stencil_basic.cuh).
 #include "internal.h"
 #include "stencil_basic.cuh"
 #include "zmarch.h"

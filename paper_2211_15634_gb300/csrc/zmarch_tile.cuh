@@ -4,7 +4,7 @@
 // very same arithmetic as a single grid.
 //
 // A CTA owns one x-y tile of BX x BY nodes (BX = LPR threads * PX nodes per
-// thread, LPR = 32: one warp per tile row; LPR = 16: two rows per warp, for
+// thread, LPR = 32: one warp per tile row; LPR = 16, 8: two, four rows per warp, for
 // narrow grids) and a chunk of z-planes.  For every plane a
 // single thread issues one TMA box load of the tile plus a one-node halo in
 // y and a 16-byte halo in x (so every box starts on a 16-byte boundary) into
