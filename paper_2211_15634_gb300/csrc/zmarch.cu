@@ -208,13 +208,13 @@ static int step_kchunk(int esz, Grid3 g, int64_t tiles, int per_sm, const WaveCo
     // Short chunks keep many CTAs in flight (no wave tail) while consecutive
     // CTAs - neighbouring tiles of one chunk - share their halo planes in L2;
     // each chunk pays two extra planes.  Measured (sweeps at 256^3 and 512^3):
-    // FP32 is fastest at 8 planes; FP64 at 8 planes on small grids, at 13-18 at 320^3 and flat
-    // from 24 to 40 planes at 512^3, so about 32 CTAs per SM between 8 and 32 planes (with 64:
-    // 320^3 134 us a step / 130, 321^3 150 / 144, 384^3 216 / 212).
+    // FP32 is fastest at 8 planes; FP64 at 8 planes on small grids, at 13-18 at 320^3 and at 24
+    // at 448^3 to 640^3 (1% ahead of 32), so about 32 CTAs per SM between 8 and 24 planes (with
+    // 64: 320^3 134 us a step / 130, 321^3 150 / 144, 384^3 216 / 212).
     // FP32 grids up to 3 million nodes (a few CTAs per SM): 3 planes (128^3 5.1 against 5.6 us).
     if (esz == 4 && (double)g.nx * (double)g.ny * (double)g.nz <= 3e6) return 3;
     const int64_t target = 32LL * sm_count();
-    const int64_t kmax = esz == 8 ? 32 : 8;
+    const int64_t kmax = esz == 8 ? 24 : 8;
     const int64_t kc = (g.nz - 2) * tiles / target;
     // FP64 grids of a few waves: the chunk whose waves end soonest, fitted to sweeps of 13 to 18
     // shapes each (us a step against 8 planes: 128 x 150 x 200 20.8 / 23.9, 400 x 100 x 60 15.2 /
