@@ -122,7 +122,7 @@ inline bool column_shape(int64_t nx, int64_t ny, int64_t nz, bool f32, bool smal
         const int64_t planes = gx * gy * (nz - 2);  // CTAs at one plane each
         if (f32) {
             const double r = (double)planes / (2.0 * sm_count());
-            if (r < 17.0) kc = r < 1.0 ? 1 : (r < 6.0 ? 4 : 8);
+            if (r < 16.0) kc = r < 1.0 ? 1 : (r < 6.0 ? 4 : 8);
         } else {
             kc = planes / (8LL * sm_count());
             kc = kc < 1 ? 1 : (kc > 8 ? 8 : kc);

@@ -249,8 +249,9 @@ static cudaError_t launch_zmarch_t(void *T2, const void *T, void *E2, const void
     if (kchunk <= 0) {
         constexpr WaveCost wide{2.0, 0.6, 0.2, 3, 12}, narrow{1.0, 0.4, 0.2, 3, 8};
         constexpr bool kWide = MODE == Z_F64_SCALED4;
-        // (from 2.5 waves of 8 planes on, 8 stay as fast or faster: 128 x 144 x 496 45 us a step, 46 at 12)
-        const bool few = 2 * tiles * ((g.nz + 5) / 8) < 5 * 5LL * sm_count();
+        // (from two waves of 8 planes on, 8 stay as fast or faster: 128 x 144 x 496 45 us a step, 46 at
+        // 12; 208 x 361 x 79, a field of both signs, 61 and 62.5)
+        const bool few = tiles * ((g.nz + 5) / 8) < 2 * 5LL * sm_count();
         kchunk = step_kchunk(sizeof(E), g, tiles, kWide ? 5 : 4,
                              kWide ? (few ? &wide : nullptr)
                              : MODE == Z_F64_SCALED || MODE == Z_F64_EMU_ISO_DMUL ? &narrow : nullptr);

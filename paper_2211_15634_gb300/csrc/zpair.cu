@@ -369,12 +369,17 @@ cudaError_t launch_step2_states_f32(float *T1o, float *T2, const float *T, const
 }
 
 bool pairs_pay(Grid3 g, bool states) {
-    // by nodes and the share of useful lanes (us a step, single steps / pairs): 128^3 5.1 / 6.2,
-    // 160^3 (0.63) 8.5 / 9.3, 192^3 (0.75) 12.8 / 12.1, 112 x 480 x 64 (0.88) 9.5 / 6.4, 256 x
-    // 128 x 128 9.5 / 6.7; loops that keep every state 128^3 6.0 / 7.1, 160^3 13.1 / 11.0,
-    // 256^3 33.8 / 27.1
-    const double lanes = (double)g.nx / (128.0 * (double)((g.nx + 127) / 128));
-    return (double)g.n() * lanes > (states ? 2.2e6 : 2.8e6);
+    const double n = (double)g.n(), lanes = (double)g.nx / (128.0 * (double)((g.nx + 127) / 128));
+    // loops that keep every state (us a step, single steps / pairs): 128^3 6.0 / 7.1, 160^3 (0.63) 13.1
+    // / 11.0, 256^3 33.8 / 27.1
+    if (states) return n * lanes > 2.2e6;
+    // By nodes and the share of useful lanes against the column kernel's, which steps small grids
+    // and wastes at most 31 columns (us a step, single steps / pairs): 108 x 48 x 128 (0.84 of the
+    // lanes) 3.8 / 4.1, 104^3 5.5 / 4.3, 128^3 5.6 / 5.2, 72 x 300 x 200 (0.56, the column kernel's
+    // 0.75) 12.3 / 11.0, 160^3 (0.63, 1.0) 8.9 / 9.7, 192^3 13.0 / 12.4, 144 x 250 x 250 24.3 / 18.7,
+    // 372 x 96 x 96 9.6 / 6.3
+    const double column = (double)g.nx / (32.0 * (double)((g.nx + 31) / 32));
+    return lanes < 0.65 * column ? n > 7.5e6 && n * lanes > 2.8e6 : n * lanes > 7.5e5;
 }
 
 unsigned zpair_device_error(bool clear) {

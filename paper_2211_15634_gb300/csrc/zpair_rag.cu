@@ -295,12 +295,14 @@ cudaError_t launch_step2_ragged_f32(float *T2, const float *T, const float *Ci, 
 }
 
 bool pairs_pay_ragged(Grid3 g) {
-    // by nodes and the share of useful lanes, whose loss a pair pays twice (us a step, single
-    // steps - column kernels on these sizes - / pairs): 129^3 (0.99) 6.8 / 6.4, 60 x 100 x 511
-    // 7.4 / 6.4, 64 x 480 x 111 (0.85) 9.0 / 7.7, 161^3 (0.62) 9.2 / 12.1, 181^3 (0.70) 12.1 /
-    // 12.3, 193^3 (0.75) 18.5 / 14.7, 255^3 33.4 / 22.5
-    const double lanes = (double)(g.nx - 2) / (128.0 * (double)((g.nx - 2 + 127) / 128));
-    return (double)g.n() * lanes * lanes * lanes > 2.05e6;
+    // Up to 8.8 million nodes single steps are the column kernel's, whose fields stay in L2, so pairs need
+    // well-filled tiles; from there on both read HBM (us a step, single steps / pairs, share of
+    // useful lanes): 231 x 48 x 48 (0.89) 3.5 / 3.7, 103^3 (0.79) 5.4 / 4.7, 127 x 128 x 128 6.3 / 5.3, 98 x
+    // 200 x 80 (0.75) 5.8 / 5.2, 159^3 (0.61) 8.9 / 10.9, 191^3 (0.74) 13.2 / 14.0, 299 x 256 x 64 (0.77) 10.8 /
+    // 10.3, 143 x 250 x 250 (0.55) 24.7 / 21.3, 255^3 33.4 / 22.5
+    const double n = (double)g.n(), lanes = (double)(g.nx - 2) / (128.0 * (double)((g.nx - 2 + 127) / 128));
+    if (n > 8.8e6) return lanes >= 0.5 || n * lanes * lanes * lanes > 2.05e6;
+    return n * lanes * lanes > 6e5 && lanes >= (n < 3.5e6 ? 0.75 : 0.76);
 }
 
 unsigned zpair_rag_device_error(bool clear) {
