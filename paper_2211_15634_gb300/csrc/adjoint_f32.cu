@@ -800,6 +800,7 @@ static cudaError_t launch_adj32_t(float *Tbar, float *Cibar, const float *ybar, 
         kchunk = g.nz * tiles < 160LL * MINB * sm_count()
                      ? wave_chunk(g.nz, tiles, sm_count(), MINB, WaveCost{2.0, 0.6, 0.0, 2, 64})
                      : 16;
+    kchunk = grid_chunk(g.nz, kchunk);
     const int64_t gz = (g.nz + kchunk - 1) / kchunk;
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
     p.nx = (int)g.nx;
@@ -846,6 +847,7 @@ cudaError_t launch_adjoint_f32_rag(float *Tbar, float *Cibar, const float *ybar,
     // 42.9 / 45.1, 225^3 59.9 / 63.2, 321^3 157 / 163)
     if (kchunk <= 0)
         kchunk = wave_chunk(g.nz, tiles, sm_count(), 3, WaveCost{1.0, 0.5, 0.0, 2, 40});
+    kchunk = grid_chunk(g.nz, kchunk);
     const int64_t gz = (g.nz + kchunk - 1) / kchunk;
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
     Adj32Params p{};

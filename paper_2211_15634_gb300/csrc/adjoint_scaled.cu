@@ -502,6 +502,7 @@ static cudaError_t launch_adjs_t(double *Tbar, double *Csbar, const double *ybar
             }
         }
     }
+    kchunk = grid_chunk(g.nz, kchunk);
     const int64_t gz = (g.nz + kchunk - 1) / kchunk;
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
     AdjSParams p{g.nx, g.ny, g.nz, kchunk, (int)ntx, ek};

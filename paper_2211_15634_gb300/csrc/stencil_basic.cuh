@@ -24,6 +24,7 @@
 #include "internal.h"
 #include "node.cuh"
 #include "pdl.cuh"
+#include "waves.h"
 
 namespace psd {
 
@@ -128,6 +129,7 @@ inline bool column_shape(int64_t nx, int64_t ny, int64_t nz, bool f32, bool smal
             kc = kc < 1 ? 1 : (kc > 8 ? 8 : kc);
         }
     }
+    kc = grid_chunk(nz, (int)kc);
     const int64_t gz = (nz - 2 + kc - 1) / kc;
     if (gx > 0x7fffffff || gy > 65535 || gz > 65535) return false;
     *grid = dim3((unsigned)gx, (unsigned)gy, (unsigned)gz);

@@ -68,4 +68,11 @@ inline int wave_chunk(int64_t nz, int64_t tiles, int sms, int per_sm, const Wave
     return e.chunk;
 }
 
+// A chunk long enough for the planes to fit the 65535 CTAs that a grid has along z (a few nodes
+// in x and y, over half a million in z).
+inline int grid_chunk(int64_t nz, int chunk) {
+    const int64_t least = (nz + 65534) / 65535;
+    return chunk < least ? (int)least : chunk;
+}
+
 }  // namespace psd

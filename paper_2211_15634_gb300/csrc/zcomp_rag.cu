@@ -243,6 +243,7 @@ cudaError_t launch_comp_ragged(float *T2, const float *T, float *E2, const float
     const int64_t ntx = (g.nx - 2 + Z::BX - 1) / Z::BX, nty = (g.ny - 2 + Z::BY - 1) / Z::BY, tiles = ntx * nty;
     int kchunk = launch_override(PS_OVERRIDE_KCHUNK);
     if (kchunk <= 0) kchunk = wave_chunk(g.nz - 2, tiles, sm_count(), Z::MINB, WaveCost{1.5, 0.6, 0.0, 3, 48});
+    kchunk = grid_chunk(g.nz, kchunk);
     const int64_t gz = (g.nz - 2 + kchunk - 1) / kchunk;
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
     const CompRagParams p{(int)g.nx, (int)g.ny, (int)g.nz, kchunk, (int)ntx, (int)(((uintptr_t)E >> 2) & 3), (float)c.dtlam, (float)c.ax, (float)c.ay,

@@ -256,6 +256,7 @@ static cudaError_t launch_zmarch_t(void *T2, const void *T, void *E2, const void
                              kWide ? (few ? &wide : nullptr)
                              : MODE == Z_F64_SCALED || MODE == Z_F64_EMU_ISO_DMUL ? &narrow : nullptr);
     }
+    kchunk = grid_chunk(g.nz, kchunk);
     const int64_t gz = (g.nz - 2 + kchunk - 1) / kchunk;
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
     p.nx = g.nx;
@@ -329,6 +330,7 @@ static cudaError_t launch_rag_t(void *T2, const void *T, const void *Ci, Grid3 g
         kchunk = step_kchunk(sizeof(E), g, tiles, 3,
                              MODE == Z_F64_SCALED || MODE == Z_F64_EMU_ISO_DMUL ? &ragged : nullptr);
     }
+    kchunk = grid_chunk(g.nz, kchunk);
     const int64_t gz = (g.nz - 2 + kchunk - 1) / kchunk;
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
     p.nx = g.nx;

@@ -33,6 +33,7 @@
 #include "node.cuh"
 #include "pdl.cuh"
 #include "tma.cuh"
+#include "waves.h"
 #include "zmarch.h"
 
 namespace psd {
@@ -334,7 +335,7 @@ int pair_kchunk(Grid3 g, int64_t tiles, int64_t slots) {
             }
         }
     }
-    return kchunk;
+    return grid_chunk(g.nz, kchunk);
 }
 
 template <int BY, int NST, int MINB, bool kStates>
