@@ -109,7 +109,8 @@ k_step_basic(F *__restrict__ T2, const F *__restrict__ T, F *__restrict__ E2,
 
 // Launch shape of the column kernels: 32 x 8 columns per CTA and kchunk planes.  false: the
 // grid does not fit a launch.
-inline bool column_shape(int64_t nx, int64_t ny, int64_t nz, bool f32, bool small, dim3 *grid, int *kchunk) {
+enum ColumnKind { COL_F64, COL_F32, COL_COMP };
+inline bool column_shape(int64_t nx, int64_t ny, int64_t nz, ColumnKind kind, bool small, dim3 *grid, int *kchunk) {
     const int64_t gx = (nx - 2 + 31) / 32, gy = (ny - 2 + 7) / 8;
     // about 8 blocks per SM, each chunk at least 16 planes
     const int64_t want = (8LL * sm_count() + gx * gy - 1) / (gx * gy);
@@ -121,12 +122,18 @@ inline bool column_shape(int64_t nx, int64_t ny, int64_t nz, bool f32, bool smal
         // the long chunks, and 1 where even that leaves SMs idle.  Sweeps at 32^3 .. 192^3:
         // within 10% of the best chunk at each.
         const int64_t planes = gx * gy * (nz - 2);  // CTAs at one plane each
-        if (f32) {
+        if (kind == COL_F32) {
             const double r = (double)planes / (2.0 * sm_count());
             if (r < 16.0) kc = r < 1.0 ? 1 : (r < 6.0 ? 4 : 8);
         } else {
             kc = planes / (8LL * sm_count());
-            kc = kc < 1 ? 1 : (kc > 8 ? 8 : kc);
+            if (kind == COL_COMP && kc > 8) {
+                // long chunks that just fit eight CTAs per SM: 145 x 200 x 160 18.3 us a step, 19.4 in 8
+                // planes, 193 x 100 x 250 18.7 and 19.8, 190 x 100 x 150 12.0 and 12.8
+                while (gx * gy * ((nz - 2 + kc - 1) / kc) > 8LL * sm_count() && kc < nz) ++kc;
+            } else {
+                kc = kc < 1 ? 1 : (kc > 8 ? 8 : kc);
+            }
         }
     }
     kc = grid_chunk(nz, (int)kc);
@@ -142,7 +149,7 @@ inline cudaError_t launch_basic_emu_t(double *T2, const double *T, const double 
                                       cudaStream_t s, bool small) {
     dim3 grid;
     int kc;
-    if (!column_shape(g.nx, g.ny, g.nz, false, small, &grid, &kc)) return cudaErrorInvalidConfiguration;
+    if (!column_shape(g.nx, g.ny, g.nz, COL_F64, small, &grid, &kc)) return cudaErrorInvalidConfiguration;
     return launch_pdl(k_step_basic_emu<kAx, kScaled>, grid, dim3(32, 8), 0, s, T2, T, Ci, c, g.nx, g.ny, g.nz, kc);
 }
 
@@ -159,7 +166,7 @@ cudaError_t launch_step_basic(F *T2, const F *T, F *E2, const F *E, const F *Ci,
                               cudaStream_t s, bool small) {
     dim3 grid;
     int kc;
-    if (!column_shape(g.nx, g.ny, g.nz, sizeof(F) == 4 && !kComp, small, &grid, &kc)) return cudaErrorInvalidConfiguration;
+    if (!column_shape(g.nx, g.ny, g.nz, sizeof(F) == 8 ? COL_F64 : kComp ? COL_COMP : COL_F32, small, &grid, &kc)) return cudaErrorInvalidConfiguration;
     return launch_pdl(k_step_basic<F, kComp>, grid, dim3(32, 8), 0, s, T2, T, E2, E, Ci, c, g.nx, g.ny, g.nz, kc);
 }
 

@@ -204,15 +204,16 @@ bool step_tma_ok(Grid3 g, int esz, const void *a, const void *b, const void *c) 
 
 // Planes per CTA of the one-step march.
 // per_sm: CTAs that an SM holds; waves: their cost, or null.
-static int step_kchunk(int esz, Grid3 g, int64_t tiles, int per_sm, const WaveCost *waves) {
+static int step_kchunk(int esz, Grid3 g, int64_t tiles, int per_sm, const WaveCost *waves, bool comp = false) {
     // Short chunks keep many CTAs in flight (no wave tail) while consecutive
     // CTAs - neighbouring tiles of one chunk - share their halo planes in L2;
     // each chunk pays two extra planes.  Measured (sweeps at 256^3 and 512^3):
     // FP32 is fastest at 8 planes; FP64 at 8 planes on small grids, at 13-18 at 320^3 and at 24
     // at 448^3 to 640^3 (1% ahead of 32), so about 32 CTAs per SM between 8 and 24 planes (with
     // 64: 320^3 134 us a step / 130, 321^3 150 / 144, 384^3 216 / 212).
-    // FP32 grids up to 3 million nodes (a few CTAs per SM): 3 planes (128^3 5.1 against 5.6 us).
-    if (esz == 4 && (double)g.nx * (double)g.ny * (double)g.nz <= 3e6) return 3;
+    // FP32 grids up to 3 million nodes (a few CTAs per SM): 3 planes (128^3 5.1 against 5.6 us), the
+    // two-float state up to 2.5 (384 x 96 x 64 10.4 against 11.5, but 400 x 140 x 52 13.7 against 11.5).
+    if (esz == 4 && (double)g.nx * (double)g.ny * (double)g.nz <= (comp ? 2.5e6 : 3e6)) return 3;
     const int64_t target = 32LL * sm_count();
     const int64_t kmax = esz == 8 ? 24 : 8;
     const int64_t kc = (g.nz - 2) * tiles / target;
@@ -254,7 +255,8 @@ static cudaError_t launch_zmarch_t(void *T2, const void *T, void *E2, const void
         const bool few = tiles * ((g.nz + 5) / 8) < 2 * 5LL * sm_count();
         kchunk = step_kchunk(sizeof(E), g, tiles, kWide ? 5 : 4,
                              kWide ? (few ? &wide : nullptr)
-                             : MODE == Z_F64_SCALED || MODE == Z_F64_EMU_ISO_DMUL ? &narrow : nullptr);
+                             : MODE == Z_F64_SCALED || MODE == Z_F64_EMU_ISO_DMUL ? &narrow : nullptr,
+                             MODE == Z_F32_COMP);
     }
     kchunk = grid_chunk(g.nz, kchunk);
     const int64_t gz = (g.nz - 2 + kchunk - 1) / kchunk;
