@@ -165,7 +165,11 @@ bool step_small(Grid3 g, int mode) {
         case Z_F32_COMP:  // 160^3 14 / 19, 176^3 25 / 25; full rows 128^3 9.4 / 10.9, 368 x 112 x 72
                           // 12.0 / 10.8; odd rows (zcomp_rag.cu) 2.1e6 nodes 11.3 / 9.9, rows that
                           // leave lanes idle 173^3 24 / 25, 177^3 30 / 26, 163 x 150 x 200 26 / 25
-            if (!aligned) return n <= ((double)(g.nx - 2) >= 0.85 * 128.0 * (double)((g.nx - 2 + 127) / 128) ? 2e6 : 5.2e6);
+            // (also where the column kernel's 32-column CTAs leave as many idle: 99 x 150 x 200 15.3 / 13.3)
+            if (!aligned) {
+                const int64_t x = g.nx - 2, tiled = (x + 127) / 128 * 128, columns = (x + 31) / 32 * 32;
+                return n <= (tiled == columns || (double)x >= 0.85 * (double)tiled ? 2e6 : 5.2e6);
+            }
             return n <= (full ? 2.2e6 : 4.3e6);
         case Z_F64_EMU_ANISO:  // 192^3 37 / 41, 200^3 53 / 49; ragged 219^3 61 / 64, 227^3 71 / 69
             return n <= (aligned ? 7.5e6 : 1.05e7);
