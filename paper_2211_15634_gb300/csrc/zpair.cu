@@ -6,8 +6,8 @@
 // per node to stay with the memory.  A thread therefore steps eight nodes (four along x in each
 // of two rows) with packed FP32 arithmetic (f32x2, the same roundings as f32_node), shares the
 // first differences along x between neighbours and along z between planes, and its loop's own
-// instructions count for eight nodes.  Measured (us a step): 512^3 134.5, 384^3 59.9, 256^3
-// 19.5, where the four-node form with a scalar ring around the tile (zmarch2_tile.cuh, 83
+// instructions count for eight nodes.  Measured (us a step): 512^3 130.9, 384^3 57.4, 256^3
+// 18.8, where the four-node form with a scalar ring around the tile (zmarch2_tile.cuh, 83
 // instructions per node and pass against 53) took 179, 82.8 and 27.6.  Four nodes per thread
 // with halo rows and columns in whole warps and lanes took 188 at 512^3 (the 120 columns that
 // leaves waste a seventh of the lanes), and passes of three and four steps in that form 215
@@ -23,9 +23,12 @@
 // by one more warp, a row per lane.  One barrier per iteration.  T plane q (BY + 4 rows) and
 // Ci plane q-1 (BY + 2 rows) arrive by TMA in one stage on one mbarrier, used in iterations
 // q-2 and (T's x- and y-neighbours) q-1; Ci moves to level 2 in registers.
-// Nodes that are not interior have their Ci replaced by zero, which keeps their value: they are
-// never stored, and a non-finite value of theirs can only come from, and only reaches, the one
-// interior node beside them.  (kStates stores them, so there they are selected.)
+// Level 1 of a node that is not interior is its level 0: its rate of change (Ci times the bracket of
+// f32_node) is replaced by the zero that leaves every value as it is.  Not its Ci: the bracket reads
+// the zeros outside the grid and the nodes beside it in the face, so it may be infinite or NaN
+// where every value that an interior stencil reads is finite.  Replacing the rate rather than
+// selecting between the old and the new value keeps the old one from being held longer (us a step,
+// on one GPU: 512^3 130.9 with the rate, 137.2 with Ci, 142.7 with the value; 256^3 18.8, 19.7, 20.4).
 #include <cudaTypedefs.h>
 
 #include "f32x2.cuh"
@@ -50,14 +53,15 @@ __device__ __forceinline__ V4 v4_load(const float *p) {
     return V4{v.x, v.y};
 }
 __device__ __forceinline__ void v4_store(float *p, V4 v) { *(ulonglong2 *)p = make_ulonglong2(v.a, v.b); }
-__device__ __forceinline__ V4 v4_select(const bool (&m)[4], V4 x, V4 y) {
-    return V4{f2_make(m[0] ? f2_lo(x.a) : f2_lo(y.a), m[1] ? f2_hi(x.a) : f2_hi(y.a)),
-              f2_make(m[2] ? f2_lo(x.b) : f2_lo(y.b), m[3] ? f2_hi(x.b) : f2_hi(y.b))};
+// x, with y's first node where f0 and its last where f3.
+__device__ __forceinline__ V4 v4_faces(V4 x, V4 y, bool f0, bool f3) {
+    return V4{f2_make(f0 ? f2_lo(y.a) : f2_lo(x.a), f2_hi(x.a)), f2_make(f2_lo(x.b), f3 ? f2_hi(y.b) : f2_hi(x.b))};
 }
 
-// f32_node of four neighbouring nodes: c the centres, left / right the values beside them, up /
-// dn the rows above and below, en = zp - c and eo = c - zm the differences along z.
-__device__ __forceinline__ V4 v4_step(V4 c, float left, float right, V4 up, V4 dn, V4 en, V4 eo, V4 ci,
+// Ci times the bracket of f32_node, of four neighbouring nodes: c the centres, left / right the
+// values beside them, up / dn the rows above and below, en = zp - c and eo = c - zm the differences
+// along z.
+__device__ __forceinline__ V4 v4_rate(V4 c, float left, float right, V4 up, V4 dn, V4 en, V4 eo, V4 ci,
                                       const ZCoef2 &k) {
     const float c0 = f2_lo(c.a), c1 = f2_hi(c.a), c2 = f2_lo(c.b), c3 = f2_hi(c.b);
     const float d0 = __fsub_rn(c0, left), d1 = __fsub_rn(c1, c0), d2 = __fsub_rn(c2, c1), d3 = __fsub_rn(c3, c2),
@@ -66,7 +70,10 @@ __device__ __forceinline__ V4 v4_step(V4 c, float left, float right, V4 up, V4 d
     const V4 y = v4_sub(v4_sub(dn, c), v4_sub(c, up)), z = v4_sub(en, eo);
     const f2 la = f2_fma(z.a, k.az, f2_fma(y.a, k.ay, f2_mul(xa, k.ax)));
     const f2 lb = f2_fma(z.b, k.az, f2_fma(y.b, k.ay, f2_mul(xb, k.ax)));
-    return V4{f2_fma(k.dtlam, f2_mul(ci.a, la), c.a), f2_fma(k.dtlam, f2_mul(ci.b, lb), c.b)};
+    return V4{f2_mul(ci.a, la), f2_mul(ci.b, lb)};
+}
+__device__ __forceinline__ V4 v4_add(V4 c, V4 rate, const ZCoef2 &k) {
+    return V4{f2_fma(k.dtlam, rate.a, c.a), f2_fma(k.dtlam, rate.b, c.b)};
 }
 
 template <int BY>
@@ -165,13 +172,15 @@ k_zpair(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtenso
     // ---- rows ra = 2w and ra + 1 of the stepped rows (T box rows one more)
     const int ra = 2 * w, gya = Y0 - 1 + ra, gx0 = X0 + 4 * lane;
     const bool ina = gya >= 1 && gya <= ny - 2, inb = gya + 1 >= 1 && gya + 1 <= ny - 2;
-    const bool xedge = X0 == 0 || X0 + Z::BX > nx - 1;  // CTA-uniform: x boundary nodes in the tile
-    bool in[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) in[i] = gx0 + i >= 1 && gx0 + i <= nx - 2;
+    // rows are whole groups of four: only a lane's first and last node can be on an x face, and
+    // a lane past the row's end has no node at all (what it forms is read by no interior node)
+    const bool row = gx0 < nx, f0 = gx0 == 0, f3 = gx0 + 4 >= nx;
     const bool outa = w > 0 && (kStates ? gya <= ny - 1 : ina);
     const bool outb = w < NW - 1 && (kStates ? gya + 1 <= ny - 1 : inb);
     const ZCoef2 k{f2_make(p.dtlam, p.dtlam), f2_make(p.ax, p.ax), f2_make(p.ay, p.ay), f2_make(p.az, p.az)};
+    // a rate that leaves every value as it is (its product with dtlam is -0)
+    const f2 z2 = f2_make(copysignf(0.f, -p.dtlam), copysignf(0.f, -p.dtlam));
+    const V4 still{z2, z2};
     const int oT = (ra + 1) * W + 4 + 4 * lane, oC = ra * W + 4 + 4 * lane;  // own nodes in a T box, in a Ci box or tile
     const int up1 = max(ra - 1, 0) * W + 4 + 4 * lane, dn1 = min(ra + 2, ROWS - 1) * W + 4 + 4 * lane;
     const bool eL = lane == 0, eR = lane == 31;
@@ -212,30 +221,19 @@ k_zpair(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtenso
         const float *const w0 = tiles + (z & 1) * LBF;     // and of plane z
         // level 1 of plane z+1
         const V4 za = v4_load(t0 + oT), zb = v4_load(t0 + oT + W);
-        V4 na = v4_load(t0 + CF + oC), nb = v4_load(t0 + CF + oC + W);  // Ci of plane z+1
+        const V4 na = v4_load(t0 + CF + oC), nb = v4_load(t0 + CF + oC + W);  // Ci of plane z+1
         const bool zin = z + 1 >= 1 && z + 1 <= nz - 2;
-        if (!kStates) {
-            if (!(ina && zin)) na = V4{0ull, 0ull};
-            if (!(inb && zin)) nb = V4{0ull, 0ull};
-            if (xedge) {
-                na = v4_select(in, na, V4{0ull, 0ull});
-                nb = v4_select(in, nb, V4{0ull, 0ull});
-            }
-        }
         const V4 ena = v4_sub(za, ca), enb = v4_sub(zb, cb);
         float la, ra_, lb, rb_;
         beside(ca, t1 + oT, la, ra_);
         beside(cb, t1 + oT + W, lb, rb_);
-        V4 oa = v4_step(ca, la, ra_, v4_load(t1 + oT - W), cb, ena, ea, na, k);
-        V4 ob = v4_step(cb, lb, rb_, ca, v4_load(t1 + oT + 2 * W), enb, eb, nb, k);
-        if constexpr (kStates) {
-            if (!(ina && zin)) oa = ca;
-            if (!(inb && zin)) ob = cb;
-            if (xedge) {
-                oa = v4_select(in, oa, ca);
-                ob = v4_select(in, ob, cb);
-            }
-        }
+        V4 qa = v4_rate(ca, la, ra_, v4_load(t1 + oT - W), cb, ena, ea, na, k);
+        V4 qb = v4_rate(cb, lb, rb_, ca, v4_load(t1 + oT + 2 * W), enb, eb, nb, k);
+        if (!(ina && zin)) qa = still;
+        if (!(inb && zin)) qb = still;
+        qa = v4_faces(qa, still, f0, f3);
+        qb = v4_faces(qb, still, f0, f3);
+        const V4 oa = v4_add(ca, qa, k), ob = v4_add(cb, qb, k);
         v4_store(w1 + oC, oa);
         v4_store(w1 + oC + W, ob);
         ca = za;
@@ -247,42 +245,32 @@ k_zpair(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtenso
         if (z >= k0) {
             beside(c1a, w0 + oC, la, ra_);
             beside(c1b, w0 + oC + W, lb, rb_);
-            V4 ya = v4_step(c1a, la, ra_, v4_load(w0 + up1), c1b, fna, e1a, cia, k);
-            V4 yb = v4_step(c1b, lb, rb_, c1a, v4_load(w0 + dn1), fnb, e1b, cib, k);
+            V4 ya = v4_add(c1a, v4_rate(c1a, la, ra_, v4_load(w0 + up1), c1b, fna, e1a, cia, k), k);
+            V4 yb = v4_add(c1b, v4_rate(c1b, lb, rb_, c1a, v4_load(w0 + dn1), fnb, e1b, cib, k), k);
             if constexpr (kStates) {
                 if (!ina) ya = c1a;
                 if (!inb) yb = c1b;
-                if (xedge) {
-                    ya = v4_select(in, ya, c1a);
-                    yb = v4_select(in, yb, c1b);
+                if (X0 == 0 || X0 + Z::BX > nx - 1) {  // CTA-uniform: x faces in the tile
+                    ya = v4_faces(ya, c1a, f0, f3);
+                    yb = v4_faces(yb, c1b, f0, f3);
                 }
-                auto put = [&](float *t, V4 v) {
-                    if (gx0 + 3 <= nx - 1) {
-                        v4_store(t, v);
-                    } else {
-                        const float o4[4] = {f2_lo(v.a), f2_hi(v.a), f2_lo(v.b), f2_hi(v.b)};
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            if (gx0 + i <= nx - 1) t[i] = o4[i];
-                    }
-                };
-                if (outa) {
-                    put(T1o + base, c1a);
-                    put(T2 + base, ya);
+                if (outa && row) {
+                    v4_store(T1o + base, c1a);
+                    v4_store(T2 + base, ya);
                 }
-                if (outb) {
-                    put(T1o + base + nx, c1b);
-                    put(T2 + base + nx, yb);
+                if (outb && row) {
+                    v4_store(T1o + base + nx, c1b);
+                    v4_store(T2 + base + nx, yb);
                 }
             } else {
                 auto put = [&](float *t, V4 v) {
-                    if (!xedge || (in[0] && in[3])) {
+                    if (!(f0 || f3)) {
                         v4_store(t, v);
-                    } else {
-                        const float o4[4] = {f2_lo(v.a), f2_hi(v.a), f2_lo(v.b), f2_hi(v.b)};
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            if (in[i]) t[i] = o4[i];
+                    } else if (row) {
+                        if (!f0) t[0] = f2_lo(v.a);
+                        t[1] = f2_hi(v.a);
+                        t[2] = f2_lo(v.b);
+                        if (!f3) t[3] = f2_hi(v.b);
                     }
                 };
                 if (outa) put(T2 + base, ya);
