@@ -9,7 +9,7 @@ import pytest
 import torch
 
 from gpu_helpers import to_dev, to_host
-from paper_2211_15634_gb300 import api, inputs
+from paper_2211_15634_gb300 import api, autograd, inputs
 
 pytestmark = [pytest.mark.gpu,
               pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
@@ -95,4 +95,65 @@ def test_kept_states_equal_single_steps(launch_override, shape, nt, every, field
         launch_override(kchunk2=chunk)
         for x, y in zip(run(True), want):
             assert same(x, y)
+    assert api.device_error() == 0
+
+
+# (nt, every) with one pair and one single, pairs only, singles between kept states, no kept state
+PLANS = [(1, 1), (2, 1), (3, 1), (8, 1), (7, 2), (9, 3), (10, 5), (4, 7)]
+
+
+@pytest.mark.parametrize("nt,every", PLANS)
+@pytest.mark.parametrize("shape", [(13, 21, 68), (19, 37, 132), (7, 9, 36)])
+def test_kept_states_plans_from_the_graph_cache(launch_override, shape, nt, every):
+    """Replayed and with unset grids: every kept state, its boundary, and T(nt)."""
+    T0, C, inv, dt = setup(shape, "random")
+    launch_override(kchunk=16, kchunk2=0)
+    cur, want = T0.clone(), []
+    nxt = cur.clone()
+    for t in range(1, nt + 1):
+        api.step(nxt, cur, C, 0.9, dt, inv)
+        cur, nxt = nxt, cur
+        if t % every == 0:
+            want.append(cur.clone())
+    launch_override(kchunk=0, kchunk2=4)
+    block = api.StateBlock(T0, nt // every + (2 if every > 1 else 0), boundary=False)
+    for _ in range(3):  # captured, then replayed
+        block.flat.fill_(float("nan"))
+        out = api.run_states(T0, block, every, C, 0.9, dt, inv, nt, graph=True, temporal2=True)
+        for g, w in zip(block.grids, want):
+            assert torch.equal(g, w)
+        assert torch.equal(out, cur)
+    api.clear_graph_cache()
+    assert api.device_error() == 0
+
+
+@pytest.mark.parametrize("every", [1, 3, 20])
+def test_gradient_with_forced_pairs(launch_override, every):
+    """Forward pass and recomputes in pairs: the gradient of single steps, bit for bit."""
+    D0, C, inv, dt = setup((13, 21, 68), "random")
+    Tobs, got = D0 * 0.98, []
+    for pairs in (False, True):
+        launch_override(kchunk2=4 if pairs else 0)
+        got.append(autograd.loss_and_grad(D0, C, Tobs, 0.9, dt, inv, 10, every=every, state_pairs=pairs))
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
+    assert torch.count_nonzero(got[0][2]) > 0
+
+
+@pytest.mark.parametrize("n,nt", [(1296, 5), (196, 9)])
+def test_default_loop_takes_pairs(launch_override, n, nt):
+    """Without flag or override, past 2^31 elements and on a size that no tile divides."""
+    T0 = inputs.uniform_field_torch(3, n, n, n, "cuda").float()
+    C = (0.5 + 0.25 * inputs.uniform_field_torch(4, n, n, n, "cuda")).float()
+    assert api.step_kernel_name(T0.clone(), T0, C, 1.0, 1e-7, (n - 1.0,) * 3, temporal2=True) == "k_zpair<F32>"
+
+    def run():
+        T, T2 = T0.clone(), torch.empty_like(T0)
+        return api.run(T, T2, C, 1.0, 0.1 / n ** 2, (n - 1.0,) * 3, nt), T, T2
+
+    launch_override(kchunk=16)
+    want = run()
+    launch_override(kchunk=0)
+    for a, b in zip(run(), want):
+        assert torch.equal(a, b)
     assert api.device_error() == 0
