@@ -208,6 +208,18 @@ __device__ __forceinline__ bool emu_same_binade(unsigned long long c, unsigned l
     return ((d & 0xfff00000u) == 0u) && emu_fast_exponent(hc);
 }
 
+// FP64 bit pattern nearest to a * 2^t (a < 2^63; sign bit not set): Inf from 2^1024 up, below the
+// normal range the nearest subnormal.
+__device__ __forceinline__ unsigned long long emu_pack_any(unsigned long long a, int t) {
+    const int be = 63 - __clzll((long long)a) + t + 1022;
+    if (a != 0ull && be <= 0) {  // units of 2^-1074: a * 2^(t + 1074), below 2^53
+        const int s = -(t + 1074);
+        if (s <= 0) return a << -s;
+        return s >= 64 ? 0ull : (a + (1ull << (s - 1))) >> s;
+    }
+    return a == 0ull ? 0ull : emu_pack_mag(a, t);
+}
+
 // (sum_d r_d * S_d) * 2^(sc + re) for exact per-axis sums |S_d| <= 2^61: the sums are shifted
 // left together until the largest fills 62 bits, biased by 2^62 to be unsigned, multiplied by
 // the 63-bit r_d keeping the top 64 bits of each product (three 32 x 32-bit multiplies with
@@ -249,7 +261,7 @@ __device__ __forceinline__ double emu_L_common(long long sx, long long sy, long 
     }
     unsigned long long sg;
     const unsigned long long a = emu_abs(v, &sg);
-    return bitsd((a == 0ull ? 0ull : emu_pack_mag(a, t)) | (sg ^ flip));
+    return bitsd(emu_pack_any(a, t) | (sg ^ flip));
 }
 
 // L (as FP64 bits, with sign) from exact per-axis sums at scale 2^sc.
