@@ -132,7 +132,7 @@ cudaError_t launch_adjoint_f64(double *Tbar, double *Cibar, const double *ybar, 
         return launch_adjoint_zmarch<double>(Tbar, Cibar, ybar, T, Ci, c, g, s);
     if (emu_ok(c) && use_ragged_f64(g, Tbar, Cibar, ybar, T, Ci)) {
         const EmuCoef ek = emu_coef(c.dtlam, c.ax, c.ay, c.az);
-        if (ek.common) return launch_adjoint_given(Tbar, Cibar, ybar, T, Ci, ek, g, s);
+        if (ek.axes != AX_FAR) return launch_adjoint_given(Tbar, Cibar, ybar, T, Ci, ek, g, s);
     }
     return launch_adjoint_basic<double>(Tbar, Cibar, ybar, T, Ci,
                                         CoefT<double>{c.dtlam, c.ax, c.ay, c.az}, g, s);

@@ -46,7 +46,7 @@ __device__ unsigned g_adjs_error;  // set when an mbarrier wait times out
 struct AdjSParams {
     int64_t nx, ny, nz;
     int kchunk, ntx;
-    EmuCoef ek;  // AX_COMMON: dt*lam*_d^2 of the axes at one exponent
+    EmuCoef ek;  // AX_COMMON, AX_SPREAD: dt*lam*_d^2 of the axes at one exponent
 };
 
 // Fixed-point value of FP64 bits v at scale 2^(E-1079) (E >= the exponent of v).
@@ -75,11 +75,11 @@ static __device__ __noinline__ double adjs_lap_general(unsigned long long c, uns
     int sc;
     const double cc = bitsd(c);
     if (emu_sums_general(c, xm, xp, ym, yp, zm, zp, sx, sy, sz, sc)) {
-        if constexpr (kAx == AX_COMMON) return emu_L_signed<AX_COMMON>(sx, sy, sz, sc, c, k);
+        if constexpr (kAx != AX_ISO) return emu_L_signed<kAx>(sx, sy, sz, sc, c, k);
         return emu_pack(sx + sy + sz, sc);
     }
     // Inf / NaN: plain FP64 propagates it
-    if constexpr (kAx == AX_COMMON) {
+    if constexpr (kAx != AX_ISO) {
         const double d2x = (bitsd(xp) - cc) - (cc - bitsd(xm)), d2y = (bitsd(yp) - cc) - (cc - bitsd(ym)),
                      d2z = (bitsd(zp) - cc) - (cc - bitsd(zm));
         return k.dtlam * ((d2x * k.ax + d2y * k.ay) + d2z * k.az);
@@ -89,7 +89,7 @@ static __device__ __noinline__ double adjs_lap_general(unsigned long long c, uns
 
 // kAx, kGiven: AX_ISO on the pre-scaled coefficient; AX_ISO and kGiven, Ci as given on equal
 // spacings: w = Ci*ybar, the one dt*lam*_d^2 multiplied in last (Tbar by the DFMA that
-// replaces the DADD, Cibar by one more DMUL); AX_COMMON, Ci as given on unequal spacings: w =
+// replaces the DADD, Cibar by one more DMUL); AX_COMMON and AX_SPREAD, Ci as given on unequal spacings: w =
 // Ci*ybar, Tbar = ybar + L(w) and Cibar += ybar*L(T) with L = sum_d dt*lam*_d^2 * (second
 // difference along d), the axes' exact sums combined as integers (emu_L_common).
 // kRag: odd nx.  A plane of a field arrives as two boxes, its even and its odd tile rows, over
@@ -345,13 +345,13 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
             double2 tb;
             const long long S0 = ((wl + wr0) + (wu.x + wd.x)) + (wm0 + wp0) - 6 * wc0;
             const long long S1 = ((wl1 + wr) + (wu.y + wd.y)) + (wm1 + wp1) - 6 * wc1;
-            if constexpr (kAx == AX_COMMON) {
+            if constexpr (kAx != AX_ISO) {
                 if (Esc == 0x7ff) {  // a non-finite w in this CTA's march: report NaN
                     tb.x = tb.y = __longlong_as_double(0x7ff8000000000000ll);
                 } else {
                     const long long a2 = 2 * wc0, b2 = 2 * wc1;
-                    tb.x = yc.x + emu_L_common<3>(wl + wr0 - a2, wu.x + wd.x - a2, wm0 + wp0 - a2, sc, 0ull, p.ek);
-                    tb.y = yc.y + emu_L_common<3>(wl1 + wr - b2, wu.y + wd.y - b2, wm1 + wp1 - b2, sc, 0ull, p.ek);
+                    tb.x = yc.x + emu_L_common<3, kAx == AX_SPREAD, false>(wl + wr0 - a2, wu.x + wd.x - a2, wm0 + wp0 - a2, sc, 0ull, p.ek);
+                    tb.y = yc.y + emu_L_common<3, kAx == AX_SPREAD, false>(wl1 + wr - b2, wu.y + wd.y - b2, wm1 + wp1 - b2, sc, 0ull, p.ek);
                 }
             } else if (Esc >= 57 && Esc <= 2042) {  // CTA-uniform: the packed sums are normal
                 tb.x = kGiven ? fma(p.ek.Kx, adjs_pack_normal(S0, sc), yc.x) : yc.x + adjs_pack_normal(S0, sc);
@@ -407,15 +407,15 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
                 }
                 const bool fast = emu_same_binade_hi(hw, hc0);
                 double L0, L1;
-                if (kAx == AX_COMMON && __all_sync(0xffffffffu, fast)) {
+                if (kAx != AX_ISO && __all_sync(0xffffffffu, fast)) {
                     const unsigned long long a2 = 2ull * c0, b2 = 2ull * c1;
                     const int sct = (int)((hc0 >> 20) & 0x7ffu) - 1075;
                     const unsigned long long flip = (unsigned long long)(hc0 & 0x80000000u) << 32;  // negative: minus
-                    L0 = emu_L_common<3>((long long)(xl + xr0 - a2), (long long)(u0 + d0 - a2),
+                    L0 = emu_L_common<3, kAx == AX_SPREAD, true>((long long)(xl + xr0 - a2), (long long)(u0 + d0 - a2),
                                          (long long)(m0b + p0 - a2), sct, flip, p.ek);
-                    L1 = emu_L_common<3>((long long)(xl1 + xr - b2), (long long)(u1 + d1 - b2),
+                    L1 = emu_L_common<3, kAx == AX_SPREAD, true>((long long)(xl1 + xr - b2), (long long)(u1 + d1 - b2),
                                          (long long)(m1b + p1 - b2), sct, flip, p.ek);
-                } else if (kAx != AX_COMMON && __all_sync(0xffffffffu, fast)) {
+                } else if (kAx == AX_ISO && __all_sync(0xffffffffu, fast)) {
                     const long long S0t = (long long)(((xl + xr0) + (u0 + d0)) + (m0b + p0) - 6ull * c0);
                     const long long S1t = (long long)(((xl1 + xr) + (u1 + d1)) + (m1b + p1) - 6ull * c1);
                     const int sct = (int)((hc0 >> 20) & 0x7ffu) - 1075;
@@ -526,7 +526,8 @@ cudaError_t launch_adjoint_given(double *Tbar, double *Cibar, const double *ybar
                                  const double *Ci, const EmuCoef &ek, Grid3 g, cudaStream_t s) {
     if (ek.ax == ek.ay && ek.ay == ek.az)
         return launch_adjs<AX_ISO, true>(Tbar, Cibar, ybar, T, Ci, ek, g, s);
-    return launch_adjs<AX_COMMON, true>(Tbar, Cibar, ybar, T, Ci, ek, g, s);
+    if (ek.axes == AX_COMMON) return launch_adjs<AX_COMMON, true>(Tbar, Cibar, ybar, T, Ci, ek, g, s);
+    return launch_adjs<AX_SPREAD, true>(Tbar, Cibar, ybar, T, Ci, ek, g, s);
 }
 
 unsigned adjoint_scaled_device_error(bool clear) {

@@ -432,7 +432,7 @@ cudaError_t launch_adjoint_zmarch(E *Tbar, E *Cibar, const E *ybar, const E *T, 
     const int kchunk = launch_override(PS_OVERRIDE_ADJ_KCHUNK);
     if (emu_ok(c)) {
         const EmuCoef ek = emu_coef(c.dtlam, c.ax, c.ay, c.az);
-        if (ek.common) return launch_adjoint_given(Tbar, Cibar, ybar, T, Ci, ek, g, s);
+        if (ek.axes != AX_FAR) return launch_adjoint_given(Tbar, Cibar, ybar, T, Ci, ek, g, s);
     }
     return launch_adj_t<E, 8, 3>(Tbar, Cibar, ybar, T, Ci, g, p, kchunk, s);
 }

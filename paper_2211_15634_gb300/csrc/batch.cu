@@ -20,11 +20,12 @@ constexpr int kBatchThreads = 256;
 __device__ unsigned g_batch_error;  // bit 1: a table built for the z-march kernel was given
 
 // Not inlined, so that spacings this far apart cost the other problems no registers.
+template <int kAx>
 static __device__ __noinline__ double emu_step_node_far(unsigned long long c, unsigned long long xm,
                                                         unsigned long long xp, unsigned long long ym,
                                                         unsigned long long yp, unsigned long long zm,
                                                         unsigned long long zp, double ci, const EmuCoef k) {
-    return emu_step_node<AX_FAR, false>(c, xm, xp, ym, yp, zm, zp, ci, k);
+    return emu_step_node<kAx, false>(c, xm, xp, ym, yp, zm, zp, ci, k);
 }
 
 template <typename F>
@@ -55,7 +56,7 @@ __device__ __forceinline__ void batch_item(const BatchItem &item, const BatchPro
         } else if constexpr (sizeof(F) == 8) {
             const unsigned long long *__restrict__ Tb = (const unsigned long long *)T;
             EmuCoef k{EmuK{P.kxm, P.kxe}, EmuK{P.kym, P.kye}, EmuK{P.kzm, P.kze},
-                            P.dtlam, P.ax, P.ay, P.az, 0.0, 0ull, 0ull, 0ull, 0, 0};
+                            P.dtlam, P.ax, P.ay, P.az, 0.0, 0ull, 0ull, 0ull, 0, 0, 0, 0, 0};
             unsigned long long tm = Tb[p - sz], tc = Tb[p];
             if (P.iso) {
                 for (int kk = k0; kk < k1; ++kk, p += sz) {
@@ -65,7 +66,7 @@ __device__ __forceinline__ void batch_item(const BatchItem &item, const BatchPro
                     tm = tc;
                     tc = tp;
                 }
-            } else if (emu_set_common(k); k.common) {
+            } else if (emu_set_common(k); k.axes == AX_COMMON) {
                 for (int kk = k0; kk < k1; ++kk, p += sz) {
                     const unsigned long long tp = Tb[p + sz];
                     T2[p] = emu_step_node<AX_COMMON, false>(tc, Tb[p - 1], Tb[p + 1], Tb[p - sy],
@@ -76,8 +77,11 @@ __device__ __forceinline__ void batch_item(const BatchItem &item, const BatchPro
             } else {
                 for (int kk = k0; kk < k1; ++kk, p += sz) {
                     const unsigned long long tp = Tb[p + sz];
-                    T2[p] = emu_step_node_far(tc, Tb[p - 1], Tb[p + 1], Tb[p - sy], Tb[p + sy], tm, tp,
-                                              Ci[p], k);
+                    T2[p] = k.axes == AX_SPREAD
+                                ? emu_step_node_far<AX_SPREAD>(tc, Tb[p - 1], Tb[p + 1], Tb[p - sy], Tb[p + sy], tm,
+                                                               tp, Ci[p], k)
+                                : emu_step_node_far<AX_FAR>(tc, Tb[p - 1], Tb[p + 1], Tb[p - sy], Tb[p + sy], tm, tp,
+                                                            Ci[p], k);
                     tm = tc;
                     tc = tp;
                 }

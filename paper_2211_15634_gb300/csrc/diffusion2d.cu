@@ -48,6 +48,8 @@ struct M2D<Z_F64_EMU_ANISO> {
     using E = double;
 };
 template <>
+struct M2D<Z_F64_EMU_ANISO_SPREAD> : M2D<Z_F64_EMU_ANISO> {};
+template <>
 struct M2D<Z_F64_NATIVE> {
     using E = double;
 };
@@ -61,9 +63,10 @@ __device__ __forceinline__ E node2d(E c, E xm, E xp, E ym, E yp, E ci, const P2D
     } else if constexpr (MODE == Z_F64_EMU_ISO_DMUL) {
         return emu_step_node<AX_ISO, true>(dbits(c), dbits(xm), dbits(xp), dbits(ym), dbits(yp), dbits(c),
                                            dbits(c), ci, p.ek);
-    } else if constexpr (MODE == Z_F64_EMU_ANISO) {
-        return emu_step_node<AX_COMMON, false, 2>(dbits(c), dbits(xm), dbits(xp), dbits(ym), dbits(yp), dbits(c),
-                                                  dbits(c), ci, p.ek);
+    } else if constexpr (MODE == Z_F64_EMU_ANISO || MODE == Z_F64_EMU_ANISO_SPREAD) {
+        constexpr int kAx = MODE == Z_F64_EMU_ANISO ? AX_COMMON : AX_SPREAD;
+        return emu_step_node<kAx, false, 2>(dbits(c), dbits(xm), dbits(xp), dbits(ym), dbits(yp), dbits(c),
+                                            dbits(c), ci, p.ek);
     } else {
         const double d2x = (xp - c) - (c - xm), d2y = (yp - c) - (c - ym);
         return c + p.ek.dtlam * (ci * (d2x * p.ek.ax + d2y * p.ek.ay));
@@ -202,7 +205,8 @@ k_ymarch2d(typename M2D<MODE>::E *__restrict__ T2, const typename M2D<MODE>::E *
         }
         E out[PX];
         bool warp_fast = false;
-        if constexpr (MODE == Z_F64_SCALED || MODE == Z_F64_EMU_ISO_DMUL || MODE == Z_F64_EMU_ANISO) {
+        if constexpr (MODE == Z_F64_SCALED || MODE == Z_F64_EMU_ISO_DMUL || MODE == Z_F64_EMU_ANISO ||
+                      MODE == Z_F64_EMU_ANISO_SPREAD) {
             // one same-binade check over this lane's distinct values (words of nodes that
             // are not written replaced by the reference, so they cannot force the general
             // path); the whole warp takes the short path together when all lanes pass
@@ -253,11 +257,11 @@ k_ymarch2d(typename M2D<MODE>::E *__restrict__ T2, const typename M2D<MODE>::E *
                                                          dbits(dn[i]), dbits(c[i]), dbits(c[i]), ci[i], p.ek);
                     continue;
                 }
-            } else if constexpr (MODE == Z_F64_EMU_ANISO) {
+            } else if constexpr (MODE == Z_F64_EMU_ANISO || MODE == Z_F64_EMU_ANISO_SPREAD) {
                 if (warp_fast) {
-                    out[i] = emu_fast_node<AX_COMMON, false, 2>(dbits(c[i]), dbits(xm), dbits(xp), dbits(up[i]),
-                                                                dbits(dn[i]), dbits(c[i]), dbits(c[i]), ci[i],
-                                                                p.ek);
+                    constexpr int kAx = MODE == Z_F64_EMU_ANISO ? AX_COMMON : AX_SPREAD;
+                    out[i] = emu_fast_node<kAx, false, 2>(dbits(c[i]), dbits(xm), dbits(xp), dbits(up[i]),
+                                                          dbits(dn[i]), dbits(c[i]), dbits(c[i]), ci[i], p.ek);
                     continue;
                 }
             }
@@ -351,6 +355,16 @@ static cudaError_t launch_2d_t(void *T2, const void *T, const void *Ci, P2D p, i
                       (const E *)Ci, p);
 }
 
+template <int MODE>
+static cudaError_t launch_aniso2d(bool vec, void *T2, const void *T, const void *Ci, P2D p, int64_t nx, int64_t ny,
+                                  cudaStream_t s) {
+    if (!vec) return launch_2d_t<MODE, 2, 4, 32>(T2, T, Ci, p, nx, ny, s);
+    // bound by issue, so more warps with fewer nodes each once there are many rows:
+    // 6000 x 8192 245 us, 255 with four per lane; 2048^2 29 and 28
+    if (nx * ny >= (1LL << 24)) return launch_2d_t<MODE, 2, 4>(T2, T, Ci, p, nx, ny, s);
+    return launch_2d_t<MODE, 4, 2>(T2, T, Ci, p, nx, ny, s);
+}
+
 // mode: Z_F32, Z_F64_SCALED (Ci holds dt*lam*_dx^2*Ci, equal spacings), Z_F64_EMU_ISO_DMUL
 // (equal spacings, positive coefficient), Z_F64_EMU_ANISO (unequal ones within a factor of
 // 16) or Z_F64_NATIVE (anything else in FP64)
@@ -385,12 +399,9 @@ cudaError_t launch_step2d(int mode, void *T2, const void *T, const void *Ci, Ste
         // spacings within a factor of 16 of each other; beyond that plain FP64, whose products
         // lose nothing at any ratio
         case Z_F64_EMU_ANISO:
-            if (!p.ek.common) break;
-            if (!vec) return launch_2d_t<Z_F64_EMU_ANISO, 2, 4, 32>(T2, T, Ci, p, nx, ny, s);
-            // bound by issue, so more warps with fewer nodes each once there are many rows:
-            // 6000 x 8192 245 us, 255 with four per lane; 2048^2 29 and 28
-            if (nx * ny >= (1LL << 24)) return launch_2d_t<Z_F64_EMU_ANISO, 2, 4>(T2, T, Ci, p, nx, ny, s);
-            return launch_2d_t<Z_F64_EMU_ANISO, 4, 2>(T2, T, Ci, p, nx, ny, s);
+            if (p.ek.axes == AX_COMMON) return launch_aniso2d<Z_F64_EMU_ANISO>(vec, T2, T, Ci, p, nx, ny, s);
+            if (p.ek.axes == AX_SPREAD) return launch_aniso2d<Z_F64_EMU_ANISO_SPREAD>(vec, T2, T, Ci, p, nx, ny, s);
+            break;
         default:
             break;
     }

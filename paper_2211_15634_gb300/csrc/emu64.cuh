@@ -62,33 +62,43 @@ struct EmuCoef {
     EmuK kx, ky, kz;  // dt*lam*_d^2 per axis as integer mantissa and exponent
     double dtlam, ax, ay, az;
     double Kx;        // dt*lam*_dx^2 (the kDmul variant, iso grids)
-    // the three K as integers at one exponent, K_d = r_d * 2^re (emu_set_common); common: whether
-    // that is exact, i.e. the K lie within a factor of 2^8 (spacings within 16)
+    // the K as integers at one exponent (emu_set_common): K_d = r_d * 2^(re + h_d), h_d = 0 but with
+    // AX_SPREAD; axes: which of AX_COMMON, AX_SPREAD, AX_FAR serves them
+    // (bytes: a node's general path takes the record by value, and a longer one cost 2-D fields of
+    // both signs a third of their time)
     unsigned long long rx, ry, rz;
-    int re, common;
+    int re;
+    signed char hx, hy, hz, axes;
 };
 
-// How a node's Laplacian combines its axes: one K (equal spacings), one K per axis as
-// integers at a common exponent, or one K per axis at its own exponent (spacings so unequal
-// that the small K would lose bits at the large one's exponent).
-enum EmuAxes { AX_COMMON = 0, AX_ISO = 1, AX_FAR = 2 };
+// How a node's Laplacian combines its axes: one K (equal spacings); one K per axis as integers at the
+// highest exponent (AX_COMMON: the K within a factor of 2^2, to the bit of their exponents, i.e.
+// spacings within 2 to 2.8 of each other); the sums at the lowest exponent instead (AX_SPREAD: within 2^8,
+// spacings within 16), for which AX_COMMON's K would keep too few bits; or a rounded product for each
+// (AX_FAR), beyond which the shifted sums would not fit 64 bits.
+enum EmuAxes { AX_COMMON = 0, AX_ISO = 1, AX_FAR = 2, AX_SPREAD = 3 };
 
-// Sets common, re and r_d from the three K.
+// Sets axes, re, r_d and h_d from the three K.
 __host__ __device__ inline void emu_set_common(EmuCoef &c) {
     const int exy = c.kx.e > c.ky.e ? c.kx.e : c.ky.e, e = exy > c.kz.e ? exy : c.kz.e;
-    // mantissas are multiples of 2^10: after a shift by at most 8 still of 4 (emu_L_common)
-    c.common = e - c.kx.e <= 8 && e - c.ky.e <= 8 && e - c.kz.e <= 8;
-    if (!c.common) return;
-    c.re = e;
-    c.rx = c.kx.m >> (e - c.kx.e);
-    c.ry = c.ky.m >> (e - c.ky.e);
-    c.rz = c.kz.m >> (e - c.kz.e);
+    const int lxy = c.kx.e < c.ky.e ? c.kx.e : c.ky.e, l = lxy < c.kz.e ? lxy : c.kz.e;
+    const int gap = e - l;
+    c.axes = (signed char)(gap <= 2 ? AX_COMMON : (gap <= 8 ? AX_SPREAD : AX_FAR));
+    const bool up = c.axes == AX_COMMON;
+    c.re = up ? e : l;
+    // mantissas are multiples of 2^10: after a shift by at most 2 still of 4 (emu_L_common)
+    c.rx = up ? c.kx.m >> (e - c.kx.e) : c.kx.m;
+    c.ry = up ? c.ky.m >> (e - c.ky.e) : c.ky.m;
+    c.rz = up ? c.kz.m >> (e - c.kz.e) : c.kz.m;
+    c.hx = (signed char)(up ? 0 : c.kx.e - l);
+    c.hy = (signed char)(up ? 0 : c.ky.e - l);
+    c.hz = (signed char)(up ? 0 : c.kz.e - l);
 }
 
 // K_d = dtlam * a_d (positive normal, or the emulated forms are not run).
 inline EmuCoef emu_coef(double dtlam, double ax, double ay, double az) {
     EmuCoef c{emu_const(dtlam * ax), emu_const(dtlam * ay), emu_const(dtlam * az), dtlam, ax, ay, az,
-              dtlam * ax, 0ull, 0ull, 0ull, 0, 0};
+              dtlam * ax, 0ull, 0ull, 0ull, 0, 0, 0, 0, 0};
     emu_set_common(c);
     return c;
 }
@@ -220,25 +230,49 @@ __device__ __forceinline__ unsigned long long emu_pack_any(unsigned long long a,
     return a == 0ull ? 0ull : emu_pack_mag(a, t);
 }
 
-// (sum_d r_d * S_d) * 2^(sc + re) for exact per-axis sums |S_d| <= 2^61: the sums are shifted
-// left together until the largest fills 62 bits, biased by 2^62 to be unsigned, multiplied by
-// the 63-bit r_d keeping the top 64 bits of each product (three 32 x 32-bit multiplies with
+// sum_d K_d * S_d * 2^sc for exact per-axis sums, with one rounding.  kSmall: |S_d| < 2^53 (differences of
+// one binade's bit patterns), else |S_d| <= 2^59.
+//
+// The sums are shifted left together until the largest fills 62 bits, biased by 2^62 to be unsigned,
+// multiplied by the 63-bit r_d keeping the top 64 bits of each product (three 32 x 32-bit multiplies with
 // the accumulation inside; the dropped low product is below one unit), added, unbiased
 // (sum r_d / 4, exact as r_d % 4 == 0) and converted once: one rounding to 53 bits of a value
-// known to about 2^-59 of its largest term.  A node then needs two FP64-pipe instructions
-// (the conversion and the final DFMA), which the pipe serves in about the time HBM needs, and
-// about 110 integer ones, which bind.  Measured, us a step: 512 x 384 x 256 nodes 280 (443
+// known to six units of 2^-59 (three axes, two each) of the product of the largest sum and the largest
+// r.  With AX_COMMON that is up to 2^2 times the largest term there is, so the value is known to 2^-54.4 of
+// its largest term, or 2^-56 where one axis alone varies (a rounding for each axis: 2^-53 for each).
+// AX_SPREAD first brings the sums to the lowest exponent (S_d * 2^h_d, the largest of which then
+// belongs to the largest term, to within a factor of two): 2^-56.4 of the largest term at any ratio
+// (0.07 units of 2^-53 found), at three more 64-bit shifts where the sums are small and some 25
+// instructions where their length has to be looked at (larger ones may not fit: bits below 2^-60 of the
+// largest are dropped).  A node needs two FP64-pipe instructions (the
+// conversion and the final DFMA), which the pipe serves in about the time HBM needs, and
+// about 110 integer ones, which bind.  Measured, us a step: 512 x 384 x 256 nodes 271 (443
 // with one product, pack and FP64 sum per axis, three FP64 instructions and less exact; 307
-// with the integer pack in place of the conversion); 2-D 8192 x 6000 255 (878 in plain FP64,
-// ten FP64 instructions per node; 274 with the integer pack).
-// kDim = 2: the z sum is not there.
-template <int kDim>
+// with the integer pack in place of the conversion; 285 as AX_SPREAD); 2-D 8192 x 6000 247 (878 in plain
+// FP64, ten FP64 instructions per node; 253 as AX_SPREAD).
+// The same real sums at another scale 2^sc give the same result, bit for bit, and so does every path of
+// a node.  kDim = 2: the z sum is not there.
+template <int kDim, bool kSpread, bool kSmall>
 __device__ __forceinline__ double emu_L_common(long long sx, long long sy, long long sz, int sc,
                                                unsigned long long flip, const EmuCoef &k) {
+    if (kSpread && kSmall) {
+        sx <<= k.hx;
+        sy <<= k.hy;
+        if (kDim == 3) sz <<= k.hz;
+    } else if (kSpread) {  // to 61 bits
+        auto bits = [](long long s) { return 64 - __clzll(s ^ (s >> 63)); };
+        int b = max(bits(sx) + k.hx, bits(sy) + k.hy);
+        if (kDim == 3) b = max(b, bits(sz) + k.hz);
+        const int q = max(b - 61, 0);
+        auto shift = [](long long s, int h) { return h >= 0 ? s << h : s >> -h; };
+        sx = shift(sx, k.hx - q);
+        sy = shift(sy, k.hy - q);
+        if (kDim == 3) sz = shift(sz, k.hz - q);
+        sc += q;
+    }
     unsigned long long m = (unsigned long long)(sx ^ (sx >> 63)) | (unsigned long long)(sy ^ (sy >> 63));
     if (kDim == 3) m |= (unsigned long long)(sz ^ (sz >> 63));
-    // 2m + 1 scales with the sums bit for bit (also where one is -1), so the same real sums
-    // at another scale 2^sc give the same result
+    // 2m + 1 scales with the sums bit for bit (also where one is -1)
     const int n = __clzll((long long)(2ull * m + 1ull)) - 1;
     auto term = [n](long long s, unsigned long long r) -> unsigned long long {
         const unsigned long long u = ((unsigned long long)s << n) + (1ull << 62);  // [0, 2^63)
@@ -265,15 +299,15 @@ __device__ __forceinline__ double emu_L_common(long long sx, long long sy, long 
 }
 
 // L (as FP64 bits, with sign) from exact per-axis sums at scale 2^sc.
-template <int kAx, int kDim = 3>
+template <int kAx, int kDim = 3, bool kSmall = false>
 __device__ __forceinline__ double emu_L(long long sx, long long sy, long long sz, int sc,
                                         unsigned long long flip, const EmuCoef &k) {
     unsigned long long sg;
     if (kAx == AX_ISO) {
         const unsigned long long a = emu_abs(sx + sy + sz, &sg);
         return bitsd(emu_scaled_mag(a, sc, k.kx) | (sg ^ flip));
-    } else if (kAx == AX_COMMON) {
-        return emu_L_common<kDim>(sx, sy, sz, sc, flip, k);
+    } else if (kAx == AX_COMMON || kAx == AX_SPREAD) {
+        return emu_L_common<kDim, kAx == AX_SPREAD, kSmall>(sx, sy, sz, sc, flip, k);
     } else {
         unsigned long long s1, s2, s3;
         const unsigned long long ax = emu_abs(sx, &s1), ay = emu_abs(sy, &s2), az = emu_abs(sz, &s3);
@@ -284,13 +318,13 @@ __device__ __forceinline__ double emu_L(long long sx, long long sy, long long sz
     }
 }
 
-// emu_L of signed sums (the general path).  AX_COMMON truncates its products, so the sums
+// emu_L of signed sums (the general path).  emu_L_common truncates its products, so the sums
 // are first taken with the centre's sign, as the fast and window paths have them: every path
 // of a node then gives the same bits, and a field of the other sign exactly the other sign.
 template <int kAx, int kDim = 3>
 __device__ __forceinline__ double emu_L_signed(long long sx, long long sy, long long sz, int sc,
                                                unsigned long long c, const EmuCoef &k) {
-    if (kAx != AX_COMMON) return emu_L<kAx, kDim>(sx, sy, sz, sc, 0ull, k);
+    if (kAx != AX_COMMON && kAx != AX_SPREAD) return emu_L<kAx, kDim>(sx, sy, sz, sc, 0ull, k);
     const long long neg = (long long)c >> 63;  // conditional negation: (s ^ neg) - neg
     return emu_L<kAx, kDim>((sx ^ neg) - neg, (sy ^ neg) - neg, (sz ^ neg) - neg, sc,
                             c & 0x8000000000000000ull, k);
@@ -317,7 +351,7 @@ __device__ __forceinline__ double emu_fast_node(unsigned long long c, unsigned l
         const double Sd = bitsd(emu_pack_mag_normal(a, sc) | (sg ^ flip));
         return fma(ci * k.Kx, Sd, bitsd(c));
     }
-    return fma(ci, emu_L<kAx, kDim>(sx, sy, sz, sc, flip, k), bitsd(c));
+    return fma(ci, emu_L<kAx, kDim, true>(sx, sy, sz, sc, flip, k), bitsd(c));
 }
 
 // Signed fixed-point value of FP64 bits v at scale 2^(Emax' - 1079), where

@@ -157,7 +157,8 @@ inline cudaError_t launch_step_basic_emu(double *T2, const double *T, const doub
                                          Grid3 g, cudaStream_t s, bool scaled, bool small) {
     if (scaled) return launch_basic_emu_t<AX_ISO, true>(T2, T, Ci, c, g, s, small);
     if (iso) return launch_basic_emu_t<AX_ISO, false>(T2, T, Ci, c, g, s, small);
-    if (c.common) return launch_basic_emu_t<AX_COMMON, false>(T2, T, Ci, c, g, s, small);
+    if (c.axes == AX_COMMON) return launch_basic_emu_t<AX_COMMON, false>(T2, T, Ci, c, g, s, small);
+    if (c.axes == AX_SPREAD) return launch_basic_emu_t<AX_SPREAD, false>(T2, T, Ci, c, g, s, small);
     return launch_basic_emu_t<AX_FAR, false>(T2, T, Ci, c, g, s, small);
 }
 

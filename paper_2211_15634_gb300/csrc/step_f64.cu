@@ -35,7 +35,7 @@ cudaError_t launch_step_f64_fast(double *T2, const double *T, const double *Ci, 
     if (step_tma_ok(g, 8, T2, T, Ci))
         return launch_zmarch(iso ? Z_F64_EMU_ISO : Z_F64_EMU_ANISO, T2, T, nullptr, nullptr, Ci, c, g, s,
                              write_bnd);
-    if (ek.common && step_ragged_ok(g, 8, T2, T, Ci))
+    if (ek.axes != AX_FAR && step_ragged_ok(g, 8, T2, T, Ci))
         return launch_zmarch_ragged(iso ? Z_F64_EMU_ISO_DMUL : Z_F64_EMU_ANISO, T2, T, Ci, c, g, s, write_bnd);
     return launch_step_basic_emu(T2, T, Ci, ek, iso, g, s, false, false);
 }
@@ -62,7 +62,7 @@ bool step_takes_march(int dtype, bool scaled, bool native, bool in_loop, StepCoe
     const bool iso = c.ax == c.ay && c.ay == c.az;                                // launch_step_f64_fast
     if (in_loop && !iso && step_small(g, Z_F64_EMU_ANISO)) return false;
     return step_tma_ok(g, 8, T2, T, Ci) ||
-           (emu_coef(c.dtlam, c.ax, c.ay, c.az).common && step_ragged_ok(g, 8, T2, T, Ci));
+           (emu_coef(c.dtlam, c.ax, c.ay, c.az).axes != AX_FAR && step_ragged_ok(g, 8, T2, T, Ci));
 }
 
 const char *step_f64_kernel_name(Grid3 g, const void *T2, const void *T, const void *Ci, StepCoef c,
@@ -75,7 +75,7 @@ const char *step_f64_kernel_name(Grid3 g, const void *T2, const void *T, const v
     if (!emu_ok(c)) return "k_step_basic<double>";
     const bool iso = c.ax == c.ay && c.ay == c.az;
     if (step_tma_ok(g, 8, T2, T, Ci)) return iso ? "k_zmarch<F64_EMU_ISO>" : "k_zmarch<F64_EMU_ANISO>";
-    if (emu_coef(c.dtlam, c.ax, c.ay, c.az).common && step_ragged_ok(g, 8, T2, T, Ci))
+    if (emu_coef(c.dtlam, c.ax, c.ay, c.az).axes != AX_FAR && step_ragged_ok(g, 8, T2, T, Ci))
         return iso ? "k_zmarch_rag<F64_EMU_ISO>" : "k_zmarch_rag<F64_EMU_ANISO>";
     return "k_step_basic_emu";
 }

@@ -363,6 +363,8 @@ cudaError_t launch_zmarch_ragged(int mode, void *T2, const void *T, const void *
         case Z_F64_EMU_ISO_DMUL:
             return launch_rag_b<Z_F64_EMU_ISO_DMUL, 2, 8, 3>(T2, T, Ci, g, p, s, write_bnd);
         case Z_F64_EMU_ANISO:
+            if (p.ek.axes == AX_SPREAD)
+                return launch_rag_b<Z_F64_EMU_ANISO_SPREAD, 2, 8, 3>(T2, T, Ci, g, p, s, write_bnd);
             return launch_rag_b<Z_F64_EMU_ANISO, 2, 8, 3>(T2, T, Ci, g, p, s, write_bnd);
         case Z_F64_SCALED:
             return launch_rag_b<Z_F64_SCALED, 2, 8, 3>(T2, T, Ci, g, p, s, write_bnd);
@@ -386,10 +388,13 @@ cudaError_t launch_zmarch(int mode, void *T2, const void *T, void *E2, const voi
             // (measured faster than one DFMA after a 64 x 64-bit high multiply by K)
             if (mode == Z_F64_EMU_ISO)
                 return launch_zmarch_b<Z_F64_EMU_ISO_DMUL, 8, 4>(T2, T, E2, Ein, Ci, g, p, kchunk, s, wb);
-            // spacings more than 16 apart: the small K would lose bits at the large one's
-            // exponent (and a field that varies along that axis alone its accuracy), so each
-            // axis keeps its own rounded product (512 x 384 x 256: 443 against 280 us)
-            if (!p.ek.common)
+            // spacings 2 to 16 apart: the sums at the lowest exponent instead of the K at the highest (285 us a
+            // step against 271 at 512 x 384 x 256, but every axis keeps its bits)
+            if (p.ek.axes == AX_SPREAD)
+                return launch_zmarch_b<Z_F64_EMU_ANISO_SPREAD, 8, 4>(T2, T, E2, Ein, Ci, g, p, kchunk, s, wb);
+            // more than 16 apart: the shifted sums would not fit 64 bits, so each axis has its own
+            // rounded product (443 us)
+            if (p.ek.axes == AX_FAR)
                 return launch_zmarch_b<Z_F64_EMU_ANISO_FAR, 8, 4>(T2, T, E2, Ein, Ci, g, p, kchunk, s, wb);
             // four nodes per thread on large grids (us a step, two / four: 512 x 384 x 256 280 / 273, 512^3
             // 731 / 711, 256^3 103 / 103, 240 x 200 x 300 100 / 103)

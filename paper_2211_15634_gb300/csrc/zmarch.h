@@ -18,6 +18,7 @@ enum ZMode {
     Z_F64_SCALED = 6,        // Ci already holds dt*lam*_d^2*Ci: fma(Cs, S, T)
     Z_F64_SCALED4 = 7,       // as Z_F64_SCALED, four nodes per thread (32-byte accesses)
     Z_F64_EMU_ANISO4 = 9,    // as Z_F64_EMU_ANISO, four nodes per thread
+    Z_F64_EMU_ANISO_SPREAD = 10,  // spacings up to 16 apart (AX_SPREAD)
     Z_F64_EMU_ANISO_FAR = 8,  // spacings more than 16 apart: one rounded product per axis
 };
 
@@ -82,7 +83,7 @@ unsigned adjoint_device_error(bool clear);
 cudaError_t launch_adjoint_scaled(double *Tbar, double *Csbar, const double *ybar, const double *T,
                                   const double *Cs, Grid3 g, cudaStream_t s);
 // The same kernel on Ci as given: equal spacings, or the axes' coefficients at one exponent
-// (ek.common).
+// (ek.axes other than AX_FAR).
 cudaError_t launch_adjoint_given(double *Tbar, double *Cibar, const double *ybar, const double *T,
                                  const double *Ci, const EmuCoef &ek, Grid3 g, cudaStream_t s);
 // True when dt*lam*_d^2 is positive and normal on every axis (the emulated FP64 forms).

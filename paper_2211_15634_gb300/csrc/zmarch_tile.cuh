@@ -38,6 +38,8 @@ struct ZTraits<Z_F64_EMU_ISO> {
 template <>
 struct ZTraits<Z_F64_EMU_ANISO> : ZTraits<Z_F64_EMU_ISO> {};
 template <>
+struct ZTraits<Z_F64_EMU_ANISO_SPREAD> : ZTraits<Z_F64_EMU_ISO> {};
+template <>
 struct ZTraits<Z_F64_EMU_ANISO_FAR> : ZTraits<Z_F64_EMU_ISO> {};
 template <>
 struct ZTraits<Z_F64_NATIVE> : ZTraits<Z_F64_EMU_ISO> {};
@@ -191,8 +193,9 @@ __device__ __forceinline__ void zmarch_tile(const CUtensorMap *tmT, const CUtens
             V out;
             if constexpr (MODE == Z_F64_EMU_ISO || MODE == Z_F64_EMU_ANISO || MODE == Z_F64_EMU_ANISO_FAR ||
                           MODE == Z_F64_EMU_ISO_DMUL || MODE == Z_F64_SCALED || MODE == Z_F64_SCALED4 ||
-                          MODE == Z_F64_EMU_ANISO4) {
+                          MODE == Z_F64_EMU_ANISO4 || MODE == Z_F64_EMU_ANISO_SPREAD) {
                 constexpr int kAx = MODE == Z_F64_EMU_ANISO || MODE == Z_F64_EMU_ANISO4 ? AX_COMMON
+                                    : MODE == Z_F64_EMU_ANISO_SPREAD ? AX_SPREAD
                                     : MODE == Z_F64_EMU_ANISO_FAR ? AX_FAR : AX_ISO;
                 constexpr bool kDmul = MODE == Z_F64_EMU_ISO_DMUL;
                 constexpr bool kScaled = MODE == Z_F64_SCALED || MODE == Z_F64_SCALED4;

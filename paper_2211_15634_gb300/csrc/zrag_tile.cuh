@@ -182,7 +182,8 @@ __device__ __forceinline__ void zrag_tile(const CUtensorMap *tmT, const CUtensor
             const E *Cc = stage(sk) + R::crow(ty) + dk + 1 + lane;
             E out[PX];
             if constexpr (kF64) {
-                constexpr int kAx = MODE == Z_F64_EMU_ANISO ? AX_COMMON : AX_ISO;
+                constexpr int kAx = MODE == Z_F64_EMU_ANISO ? AX_COMMON
+                                    : MODE == Z_F64_EMU_ANISO_SPREAD ? AX_SPREAD : AX_ISO;
                 constexpr bool kDmul = MODE == Z_F64_EMU_ISO_DMUL, kScaled = MODE == Z_F64_SCALED;
                 unsigned long long c[PX], xm[PX], xp[PX], ym[PX], yp[PX], zm[PX], zp[PX];
                 double ci[PX];
