@@ -758,6 +758,7 @@ static cudaError_t launch_adj2_t(float *Tbar, float *Cibar, const float *ybar, c
         return cudaErrorInvalidValue;
     const int64_t ntx = (g.nx + BX - 1) / BX, nty = (g.ny + BY - 1) / BY, tiles = ntx * nty;
     if (kchunk <= 0) kchunk = 32;  // each chunk re-reads four planes and recomputes two of y1
+    kchunk = grid_chunk(g.nz, kchunk);
     const int64_t gz = (g.nz + kchunk - 1) / kchunk;
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
     p.nx = (int)g.nx;

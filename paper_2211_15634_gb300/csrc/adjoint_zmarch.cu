@@ -28,6 +28,7 @@
 #include "internal.h"
 #include "pdl.cuh"
 #include "tma.cuh"
+#include "waves.h"
 #include "zmarch.h"
 
 namespace psd {
@@ -402,6 +403,7 @@ static cudaError_t launch_adj_t(E *Tbar, E *Cibar, const E *ybar, const E *T, co
         const int64_t kc = g.nz * tiles / waves;
         kchunk = (int)(kc < 4 ? 4 : (kc > 16 ? 16 : kc));
     }
+    kchunk = grid_chunk(g.nz, kchunk);
     const int64_t gz = (g.nz + kchunk - 1) / kchunk;
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
     p.nx = g.nx;

@@ -8,6 +8,7 @@
 #include "node.cuh"
 #include "pdl.cuh"
 #include "tma.cuh"
+#include "waves.h"
 #include "zmarch.h"
 #include "zmarch2_tile.cuh"
 
@@ -53,6 +54,7 @@ static cudaError_t launch_z2(E *T2, const E *T, const E *Ci, Z2Params p, Grid3 g
         const int64_t kc = (g.nz - 2) * tiles / waves;
         kchunk = (int)(kc < 8 ? 8 : (kc > 32 ? 32 : kc));
     }
+    kchunk = grid_chunk(g.nz, kchunk);
     const int64_t gz = (g.nz - 2 + kchunk - 1) / kchunk;
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
     p.nx = g.nx;
