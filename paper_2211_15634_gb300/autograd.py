@@ -24,6 +24,7 @@ single steps; measured no faster than single steps on GB300, so off by default).
 from __future__ import annotations
 
 import math
+from collections.abc import Sequence
 
 import torch
 
@@ -79,7 +80,15 @@ def state_pairs_default(T0) -> bool:
     return T0.dtype == torch.float32
 
 
-class _EveryState:
+def _block_addresses(block, count: int, like):
+    """Device addresses of the block's first ``count`` grids, the last one first, for calls that
+    take them as fields like ``like``."""
+    if block.flat.dtype != like.dtype or block.flat.device != like.device or block.grids.shape != tuple(like.shape):
+        raise ValueError("the kept states must have the cotangent's shape, dtype and device")
+    return [block.grids.ptr(i) for i in range(count - 1, -1, -1)]
+
+
+class _EveryState(Sequence):
     """The checkpoints of ``every = 1``: T0 and the first nt - 1 grids of a block, as tensors
     made on access (a sweep needs only their addresses)."""
 
@@ -89,16 +98,25 @@ class _EveryState:
     def __len__(self) -> int:
         return self.nt
 
-    def __getitem__(self, i: int):
+    def __getitem__(self, i):
+        if isinstance(i, slice):
+            return [self[j] for j in range(*i.indices(self.nt))]
         if i < 0:
             i += self.nt
         if not 0 <= i < self.nt:
             raise IndexError("checkpoint index out of range")
         return self.T0 if i == 0 else self.block.grids[i - 1]
 
-    def addresses(self):
-        """Device addresses of the states, the last one first."""
-        return [self.block.grids.ptr(i - 1) for i in range(self.nt - 1, 0, -1)] + [self.T0.data_ptr()]
+    def __add__(self, other):
+        return self[:] + list(other)
+
+    def __radd__(self, other):
+        return list(other) + self[:]
+
+    def states(self, nt: int, like):
+        """The states before the first nt steps for :func:`api.adjoint_sweep`, the last one first."""
+        n = min(nt, self.nt)
+        return _block_addresses(self.block, n - 1, like) + [self.T0] if n > 0 else []
 
 
 def forward_checkpointed(T0, Ci, lam, dt, inv, nt, every, coef=None, graph=True, state_pairs=None):
@@ -165,8 +183,8 @@ def backward_checkpointed(ybar_nt, Ci, lam, dt, inv, nt, every, ckpts, coef=None
     cibar = torch.zeros_like(Ci)  # dL/dCs when scaled
     # on the GPU a segment's transposed steps are one library call
     native = ybar.is_cuda and not pairs
-    if native and isinstance(ckpts, _EveryState):
-        ybar, _ = api.adjoint_sweep(tbar, cibar, ybar, ckpts.addresses(), C, lam, dt, inv, ci_scaled=scaled)
+    if native and every == 1 and isinstance(ckpts, _EveryState):
+        ybar, _ = api.adjoint_sweep(tbar, cibar, ybar, ckpts.states(nt, ybar), C, lam, dt, inv, ci_scaled=scaled)
         if scaled:  # dL/dCi = dt*lam*_dx^2 * dL/dCs
             api.scale_ci(cibar, lam, dt, inv, out=cibar)
         return ybar, cibar
@@ -219,8 +237,7 @@ def backward_checkpointed(ybar_nt, Ci, lam, dt, inv, nt, every, ckpts, coef=None
             t0 = s * every
             t1 = min(t0 + every, nt)
             if native and t1 > t0:
-                grids = seg_buf[s].grids if t1 - t0 > 1 else None
-                states = [grids.ptr(i) for i in range(t1 - t0 - 2, -1, -1)] + [ckpts[s]]
+                states = (_block_addresses(seg_buf[s], t1 - t0 - 1, ybar) if t1 - t0 > 1 else []) + [ckpts[s]]
                 ybar, tbar = api.adjoint_sweep(tbar, cibar, ybar, states, C, lam, dt, inv, ci_scaled=scaled)
             elif not native:
                 states = [ckpts[s]] + (seg_buf[s].grids[:t1 - t0 - 1] if t1 - t0 > 1 else [])
