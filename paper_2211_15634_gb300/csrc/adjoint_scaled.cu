@@ -87,6 +87,49 @@ static __device__ __noinline__ double adjs_lap_general(unsigned long long c, uns
     return (((bitsd(xm) + bitsd(xp)) + (bitsd(ym) + bitsd(yp))) + (bitsd(zm) + bitsd(zp))) - 6.0 * cc;
 }
 
+// Odd rows whose march meets an infinite or NaN w, which no fixed point holds: plain FP64 from the fields
+// themselves (the plain column kernels' arithmetic, adjoint.cu).  kGiven: Ci as given, else the pre-scaled
+// coefficient.
+struct AdjsFields {
+    const double *ybar, *Ci;
+    int nx, ny, nz;
+    double dtlam, ax, ay, az;
+};
+template <bool kGiven>
+__device__ __forceinline__ double adjs_plain_lap(const AdjsFields &f, double c, double xm, double xp, double ym,
+                                                 double yp, double zm, double zp) {
+    if (!kGiven) return ((xm + xp) + (ym + yp)) + (zm + zp) - 6.0 * c;
+    const double d2x = (xp - c) - (c - xm), d2y = (yp - c) - (c - ym), d2z = (zp - c) - (c - zm);
+    return (d2x * f.ax + d2y * f.ay) + d2z * f.az;
+}
+// Tbar of one node.
+template <bool kGiven>
+__device__ __noinline__ double adjs_plain(const AdjsFields f, int x, int y, int z) {
+    auto w = [&](int i, int j, int k) -> double {
+        if (i < 1 || i > f.nx - 2 || j < 1 || j > f.ny - 2 || k < 1 || k > f.nz - 2) return 0.0;
+        const int64_t q = i + (int64_t)f.nx * (j + (int64_t)f.ny * k);
+        return kGiven ? f.dtlam * (f.Ci[q] * f.ybar[q]) : f.Ci[q] * f.ybar[q];
+    };
+    return f.ybar[x + (int64_t)f.nx * (y + (int64_t)f.ny * z)] +
+           adjs_plain_lap<kGiven>(f, w(x, y, z), w(x - 1, y, z), w(x + 1, y, z), w(x, y - 1, z), w(x, y + 1, z),
+                                  w(x, y, z - 1), w(x, y, z + 1));
+}
+// Planes [k0, k1) at nodes x0 and x1 of row y: the rest of a march.
+template <bool kGiven>
+__device__ __noinline__ void adjs_plain_march(const AdjsFields f, double *Tbar, double *Cbar, const double *T, int x0,
+                                              int x1, int y, int k0, int k1) {
+    if (y > f.ny - 1) return;
+    const int64_t sy = f.nx, sz = sy * f.ny;
+    for (int k = k0; k < k1; ++k)
+        for (int x = x0; x <= x1 && x <= f.nx - 1; x += x1 - x0) {
+            const int64_t q = x + sy * y + sz * k;
+            Tbar[q] = adjs_plain<kGiven>(f, x, y, k);
+            if (x < 1 || x > f.nx - 2 || y < 1 || y > f.ny - 2 || k < 1 || k > f.nz - 2) continue;
+            const double L = adjs_plain_lap<kGiven>(f, T[q], T[q - 1], T[q + 1], T[q - sy], T[q + sy], T[q - sz], T[q + sz]);
+            Cbar[q] = kGiven ? Cbar[q] + f.dtlam * (f.ybar[q] * L) : fma(f.ybar[q], L, Cbar[q]);
+        }
+}
+
 // kAx, kGiven: AX_ISO on the pre-scaled coefficient; AX_ISO and kGiven, Ci as given on equal
 // spacings: w = Ci*ybar, the one dt*lam*_d^2 multiplied in last (Tbar by the DFMA that
 // replaces the DADD, Cibar by one more DMUL); AX_COMMON and AX_SPREAD, Ci as given on unequal spacings: w =
@@ -101,7 +144,8 @@ template <int BY, int NST, int kAx, bool kGiven, bool kRag>
 __global__ void __launch_bounds__(32 * BY, 3)
 k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmY,
                  const __grid_constant__ CUtensorMap tmC, double *__restrict__ Tbar,
-                 double *__restrict__ Csbar, const double *__restrict__ ybar, const AdjSParams p) {
+                 double *__restrict__ Csbar, const double *__restrict__ ybar, const double *__restrict__ T,
+                 const double *__restrict__ Ci, const AdjSParams p) {
     constexpr int PX = 2, HX = 2, BX = 64, W = BX + 2 * HX, H = BY + 2;
     constexpr int NHALO = 2 * BX + 2 * BY;  // y-halo rows and x-halo columns (no corners)
     static_assert(NHALO <= 32 * BY, "one halo value per thread at most");
@@ -266,6 +310,22 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
         return;
     }
     int Esc = s_E;  // CTA-uniform
+    // A non-finite w (Esc 0x7ff) makes the CTA's Tbar NaN from there on; on odd rows it stays with the nodes
+    // that meet it: with equal spacings the march ends and plain FP64 takes its rest, else the march goes on
+    // and forms every Tbar so (either form costs the other kernel 3 to 5% in registers; this way 257^3
+    // pre-scaled 251 us, 249.5 without, 257 x 200 x 180 unequal 212 and 212).
+    auto fields = [&]() {
+        return AdjsFields{ybar, Ci, nx, ny, nz, p.ek.dtlam, p.ek.ax, p.ek.ay, p.ek.az};
+    };
+    constexpr bool kEnds = kRag && kAx == AX_ISO;
+    auto plain_rest = [&](int k) {
+        drain(min(k + 1, k1));
+        adjs_plain_march<kGiven>(fields(), Tbar, Csbar, T, gx0, gx0 + XS, gy, k, k1);
+    };
+    if (kEnds && Esc == 0x7ff) {
+        plain_rest(k0);
+        return;
+    }
     int wcur = 0;
     long long wc0, wc1;
     w_store(wtile, Esc, wc0, wc1);
@@ -311,6 +371,10 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
             if (lane == 0) atomicMax(&s_E, e);
             __syncthreads();
             const int E2 = s_E;
+            if (kEnds && E2 == 0x7ff) {
+                plain_rest(k);
+                return;
+            }
             const int d = E2 - Esc;  // > 0
             long long *wk = wtile + wcur * WS;
             auto shr = [d](long long v) { return d >= 64 ? 0ll : (v >> d); };
@@ -346,8 +410,12 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
             const long long S0 = ((wl + wr0) + (wu.x + wd.x)) + (wm0 + wp0) - 6 * wc0;
             const long long S1 = ((wl1 + wr) + (wu.y + wd.y)) + (wm1 + wp1) - 6 * wc1;
             if constexpr (kAx != AX_ISO) {
-                if (Esc == 0x7ff) {  // a non-finite w in this CTA's march: report NaN
+                if (Esc == 0x7ff) {  // a non-finite w in this CTA's march
                     tb.x = tb.y = __longlong_as_double(0x7ff8000000000000ll);
+                    if constexpr (kRag) {
+                        if (gx0 <= nx - 1) tb.x = adjs_plain<kGiven>(fields(), gx0, gy, k);
+                        if (gx0 + XS <= nx - 1) tb.y = adjs_plain<kGiven>(fields(), gx0 + XS, gy, k);
+                    }
                 } else {
                     const long long a2 = 2 * wc0, b2 = 2 * wc1;
                     tb.x = yc.x + emu_L_common<3, kAx == AX_SPREAD, false>(wl + wr0 - a2, wu.x + wd.x - a2, wm0 + wp0 - a2, sc, 0ull, p.ek);
@@ -356,7 +424,7 @@ k_adjoint_scaled(const __grid_constant__ CUtensorMap tmT, const __grid_constant_
             } else if (Esc >= 57 && Esc <= 2042) {  // CTA-uniform: the packed sums are normal
                 tb.x = kGiven ? fma(p.ek.Kx, adjs_pack_normal(S0, sc), yc.x) : yc.x + adjs_pack_normal(S0, sc);
                 tb.y = kGiven ? fma(p.ek.Kx, adjs_pack_normal(S1, sc), yc.y) : yc.y + adjs_pack_normal(S1, sc);
-            } else if (Esc == 0x7ff) {  // a non-finite w in this CTA's march: report NaN
+            } else if (!kRag && Esc == 0x7ff) {  // a non-finite w in this CTA's march
                 tb.x = tb.y = __longlong_as_double(0x7ff8000000000000ll);
             } else {
                 tb.x = kGiven ? fma(p.ek.Kx, adjs_pack(S0, sc), yc.x) : yc.x + adjs_pack(S0, sc);
@@ -507,7 +575,7 @@ static cudaError_t launch_adjs_t(double *Tbar, double *Csbar, const double *ybar
     if (tiles > 0x7fffffffLL || gz > 65535) return cudaErrorInvalidConfiguration;
     AdjSParams p{g.nx, g.ny, g.nz, kchunk, (int)ntx, ek};
     return launch_pdl(k_adjoint_scaled<BY, NST, kAx, kGiven, kRag>, dim3((unsigned)tiles, (unsigned)gz, 1), dim3(32 * BY), smem, s,
-                      mT, mY, mC, Tbar, Csbar, ybar, p);
+                      mT, mY, mC, Tbar, Csbar, ybar, T, Cs, p);
 }
 
 template <int kAx, bool kGiven>
