@@ -34,8 +34,12 @@ static inline int wave_chunk_of(int64_t nz64, int64_t tiles, int sms, int per_sm
         double last = wave(r) * (c + w.extra);
         if (rem) {
             const double over = t - (r > 0.0 ? slots - r : 0.0);  // short chunks past the free slots
-            last = over > 0.0 ? (r > 0.0 ? c + w.extra : 0.0) + wave(over < slots ? over : slots) * (rem + w.extra)
-                              : wave(r + t) * (rem + w.extra) + wave(r) * (c - rem);
+            if (over > 0.0) {  // waves of their own, as many as it takes
+                const double more = (double)(int64_t)((over - 0.5) * inv_slots);
+                last = (r > 0.0 ? c + w.extra : 0.0) + (more + wave(over - more * slots)) * (rem + w.extra);
+            } else {
+                last = wave(r + t) * (rem + w.extra) + wave(r) * (c - rem);
+            }
         }
         const double cost = (waves * (c + w.extra) + last) * (waves > 0.0 ? 1.0 - w.later : 1.0);
         if (best < 0.0 || cost < best) {
