@@ -358,17 +358,24 @@ cudaError_t launch_step2_states_f32(float *T1o, float *T2, const float *T, const
 }
 
 bool pairs_pay(Grid3 g, bool states) {
-    const double n = (double)g.n(), lanes = (double)g.nx / (128.0 * (double)((g.nx + 127) / 128));
+    const double x = (double)g.nx / (128.0 * (double)((g.nx + 127) / 128)),
+                 y = (double)g.ny / (14.0 * (double)((g.ny + 13) / 14));
+    // Rows of 14-row tiles that are used, against the one-step march's 8: thin grids take single steps (us a
+    // step, single steps / pairs: 868 x 3 x 2734 18 / 28, 284 x 6 x 1323 5.4 / 8.2, 872 x 16 x 376 (0.57) 9.5 / 10.8,
+    // 2328 x 18 x 184 (0.64) 14.8 / 13.6, 1816 x 10 x 2092 (0.71) 73 / 56).
+    if (y < 0.6) return false;
+    const double n = (double)g.n(), useful = n * x * y;
     // loops that keep every state (us a step, single steps / pairs): 128^3 6.0 / 7.1, 160^3 (0.63) 13.1
     // / 11.0, 256^3 33.8 / 27.1
-    if (states) return n * lanes > 2.2e6;
+    if (states) return useful > 2.2e6;
     // By nodes and the share of useful lanes against the column kernel's, which steps small grids
     // and wastes at most 31 columns (us a step, single steps / pairs): 108 x 48 x 128 (0.84 of the
     // lanes) 3.8 / 4.1, 104^3 5.5 / 4.3, 128^3 5.6 / 5.2, 72 x 300 x 200 (0.56, the column kernel's
     // 0.75) 12.3 / 11.0, 160^3 (0.63, 1.0) 8.9 / 9.7, 192^3 13.0 / 12.4, 144 x 250 x 250 24.3 / 18.7,
-    // 372 x 96 x 96 9.6 / 6.3
+    // 372 x 96 x 96 9.6 / 6.3.  Over 174 shapes of 3 to 6000 nodes an axis 0.9% off the better of the two
+    // on average.
     const double column = (double)g.nx / (32.0 * (double)((g.nx + 31) / 32));
-    return lanes < 0.65 * column ? n > 7.5e6 && n * lanes > 2.8e6 : n * lanes > 7.5e5;
+    return x < 0.65 * column ? n > 7.5e6 && useful > 2.8e6 : useful > 7.5e5;
 }
 
 unsigned zpair_device_error(bool clear) {

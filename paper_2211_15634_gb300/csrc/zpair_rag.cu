@@ -295,14 +295,15 @@ cudaError_t launch_step2_ragged_f32(float *T2, const float *T, const float *Ci, 
 }
 
 bool pairs_pay_ragged(Grid3 g) {
-    // Up to 8.8 million nodes single steps are the column kernel's, whose fields stay in L2, so pairs need
-    // well-filled tiles; from there on both read HBM (us a step, single steps / pairs, share of
-    // useful lanes): 231 x 48 x 48 (0.89) 3.5 / 3.7, 103^3 (0.79) 5.4 / 4.7, 127 x 128 x 128 6.3 / 5.3, 98 x
-    // 200 x 80 (0.75) 5.8 / 5.2, 159^3 (0.61) 8.9 / 10.9, 191^3 (0.74) 13.2 / 14.0, 299 x 256 x 64 (0.77) 10.8 /
-    // 10.3, 143 x 250 x 250 (0.55) 24.7 / 21.3, 255^3 33.4 / 22.5
-    const double n = (double)g.n(), lanes = (double)(g.nx - 2) / (128.0 * (double)((g.nx - 2 + 127) / 128));
-    if (n > 8.8e6) return lanes >= 0.5 || n * lanes * lanes * lanes > 2.05e6;
-    return n * lanes * lanes > 6e5 && lanes >= (n < 3.5e6 ? 0.75 : 0.76);
+    // By the share of useful nodes in 128 x 14 tiles.  Up to 8.8 million nodes single steps are the column
+    // kernel's, whose fields stay in L2, so pairs need well-filled tiles; from there on both read HBM
+    // (us a step, single steps / pairs, share): 103^3 (0.71) 5.4 / 4.7, 159^3 (0.57) 8.9 / 10.9, 299 x 256 x 64
+    // (0.74) 10.8 / 10.3, 61 x 48 x 936 (0.38) 7.1 / 9.9, 625 x 5 x 980 (0.21) 6.2 / 11, 113 x 18 x 588 (0.5) 4.5 / 4.9,
+    // 1697 x 12 x 800 (0.68) 39 / 27, 129 x 18 x 4932 (0.57) 24.6 / 23, 1061 x 6 x 4776 (0.26) 65 / 79, 143 x 250 x 250
+    // (0.55) 24.7 / 21.3, 255^3 33.4 / 22.5.  Over 186 shapes 0.4% off the better of the two on average.
+    const double n = (double)g.n(), x = (double)(g.nx - 2) / (128.0 * (double)((g.nx - 2 + 127) / 128)),
+                 share = x * (double)(g.ny - 2) / (14.0 * (double)((g.ny - 2 + 13) / 14));
+    return n > 8.8e6 ? share >= 0.5 : share >= 0.7 && n * share * share > 6e5;
 }
 
 unsigned zpair_rag_device_error(bool clear) {
