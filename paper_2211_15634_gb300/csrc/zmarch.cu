@@ -150,55 +150,75 @@ bool zmarch_supported(Grid3 g, int esz, const void *a, const void *b, const void
     return encode_fn() != nullptr;
 }
 
-bool step_small(Grid3 g, int mode) {
+// Share of n items' tiles of t that is used.
+static double fill(int64_t n, int64_t t) { return (double)n / (double)((n + t - 1) / t * t); }
+
+bool step_small(Grid3 g, int mode, bool in_loop) {
     // a set z-chunk or nodes-per-thread override asks for the march
     if (launch_override(PS_OVERRIDE_KCHUNK) > 0 || launch_override(PS_OVERRIDE_F64_PX2) == 1) return false;
+    const bool fp32 = mode == Z_F32 || mode == Z_F32_COMP;
+    const bool aligned = (g.nx * (fp32 ? 4 : 8)) % 16 == 0;
+    // on aligned rows a single step keeps the march, and so does Ci as given on equal spacings, whose one-binade
+    // form multiplies Ci by K first, which rounds another way than the column kernel's K*S
+    if (aligned && (!in_loop || mode == Z_F64_EMU_ISO)) return false;
     const double n = (double)g.nx * (double)g.ny * (double)g.nz;
     // The line lies where the march catches up (us a step, column / march).
-    const bool aligned = (g.nx * (mode == Z_F32 || mode == Z_F32_COMP ? 4 : 8)) % 16 == 0;
     // rows that fill the march's 128-node tiles by 77% or more favour it
-    const bool full = (double)g.nx >= 0.77 * 128.0 * (double)((g.nx + 127) / 128);
+    const bool full = fill(g.nx, 128) >= 0.77;
     switch (mode) {
         case Z_F32:  // full rows 5e5 nodes 3.0 / 2.9, 1e6 4.1 / 3.7; 192^3 13.1 / 14.3, 200^3 16 / 16;
                      // ragged 205^3 20.8 / 21.7, 211^3 25.5 / 23.8
             return n <= (aligned ? (full ? 6e5 : 7.5e6) : 8.8e6);
         case Z_F32_COMP:  // 160^3 14 / 19, 176^3 25 / 25; full rows 128^3 9.4 / 10.9, 368 x 112 x 72
-                          // 12.0 / 10.8; odd rows (zcomp_rag.cu) 2.1e6 nodes 11.3 / 9.9, rows that
-                          // leave lanes idle 173^3 24 / 25, 177^3 30 / 26, 163 x 150 x 200 26 / 25
-            // (also where the column kernel's 32-column CTAs leave as many idle: 99 x 150 x 200 15.3 / 13.3)
+                          // 12.0 / 10.8
             if (!aligned) {
-                const int64_t x = g.nx - 2, tiled = (x + 127) / 128 * 128, columns = (x + 31) / 32 * 32;
-                return n <= (tiled == columns || (double)x >= 0.85 * (double)tiled ? 2e6 : 5.2e6);
+                // odd rows (zcomp_rag.cu), by the useful lanes of its 128 x 16 tiles against the column
+                // kernel's 32 x 8: 113 x 18 x 588 (0.9) 7.2 / 6.2, 2717 x 48 x 20 (1) 11.2 / 10.7, 225 x 205 x 80
+                // (0.87) 13.3 / 14.7, 437 x 734 x 16 (0.87) 22 / 18.5, 1079 x 8 x 408 (0.5) 12 / 19
+                return n <= (comp_ragged_share(g) >= 0.9 ? 2e6 : 5.2e6);
             }
             return n <= (full ? 2.2e6 : 4.3e6);
-        case Z_F64_EMU_ANISO:  // 192^3 37 / 41, 200^3 53 / 49; ragged 219^3 61 / 64, 227^3 71 / 69
-            return n <= (aligned ? 7.5e6 : 1.05e7);
+        case Z_F64_EMU_ANISO:  // 192^3 37 / 41, 200^3 53 / 49; ragged 219^3 61 / 64, 227^3 71 / 69, 93 x 512 x
+                               // 257 (0.75 of the column kernel's useful lanes) 80 / 117
+            return n <= (aligned ? 7.5e6 : (fill(g.nx - 2, 64) >= 0.8 * fill(g.nx - 2, 32) ? 1.05e7 : 1.3e7));
+        case Z_F64_EMU_ISO:  // odd rows (aligned ones above): 369 x 160 x 112 (1) 38 / 41, 303 x 250 x 160 (1) 74 / 71,
+                             // 213 x 407 x 192 (0.88) 95 / 107, 797 x 20 x 1559 (0.96) 168 / 141
+            return n <= (fill(g.nx - 2, 64) >= 0.94 * fill(g.nx - 2, 32) ? 7.5e6 : 2e7);
         default: {
             // by the share of useful lanes in the march's 64-node tiles (four nodes per thread:
             // where as good): 128 x 321 x 75 (1) 23 / 21, 128^3 (1) 10 / 15; 160^3 (0.83) 21 / 24,
             // 176^3 (0.92) 32 / 29; 200^3 (0.78) 50 / 45
-            const double lanes = aligned ? (double)g.nx / (64.0 * (double)((g.nx + 63) / 64))
-                                         : (double)(g.nx - 2) / (64.0 * (double)((g.nx - 2 + 63) / 64));
-            return n <= (lanes >= 0.87 ? 2.2e6 : (lanes >= 0.8 ? 4.3e6 : 7.5e6));
+            if (aligned) {
+                const double lanes = fill(g.nx, 64);
+                return n <= (lanes >= 0.87 ? 2.2e6 : (lanes >= 0.8 ? 4.3e6 : 7.5e6));
+            }
+            // odd rows, whose march is slower, by that share against the column kernel's (32 nodes wide):
+            // 191 x 8 x 1793 (1) 12 / 15, 919 x 15 x 261 (0.97) 17 / 22, 125 x 128 x 352 (1) 33 / 32; 225 x 205 x 80
+            // (0.87) 17 / 23, 199 x 104 x 353 (0.82) 45 / 45; 75 x 148 x 320 (0.76) 21 / 31, 93 x 512 x 257 (0.75) 69 / 77
+            const double share = fill(g.nx - 2, 64) / fill(g.nx - 2, 32);
+            return n <= (share >= 0.9 ? 4.5e6 : (share >= 0.8 ? 7.5e6 : 1.3e7));
         }
     }
 }
 
 bool step_ragged_ok(Grid3 g, int esz, const void *a, const void *b, const void *c) {
     if (launch_override(PS_OVERRIDE_STEP_PLAIN) == 1 || (g.nx * esz) % 16 == 0) return false;
-    // FP32 rows that leave more than 40% of its 128-node tiles idle: the column kernel is as
-    // fast (151 x 367 x 271, 0.58 in use: 44.5 us a step here, 43.6 there)
-    if (esz == 4 && (double)(g.nx - 2) < 0.6 * 128.0 * (double)((g.nx - 2 + 127) / 128) &&
-        launch_override(PS_OVERRIDE_KCHUNK) <= 0)
+    // FP32 grids that leave more than 40% of its 128 x 8 tiles idle: the column kernel is as
+    // fast (151 x 367 x 271, 0.58 in use: 44.5 us a step here, 43.6 there; 391 x 8 x 3059, 0.57: 24 and 18)
+    if (esz == 4 && fill(g.nx - 2, 128) * fill(g.ny - 2, 8) < 0.6 && launch_override(PS_OVERRIDE_KCHUNK) <= 0)
         return false;
     return ragged_supported(g, a, b, c);
 }
 
+double comp_ragged_share(Grid3 g) {
+    return fill(g.nx - 2, 128) * fill(g.ny - 2, 16) / (fill(g.nx - 2, 32) * fill(g.ny - 2, 8));
+}
+
 bool comp_ragged_ok(Grid3 g, const void *a, const void *b, const void *c) {
     if (launch_override(PS_OVERRIDE_STEP_PLAIN) == 1 || g.nx % 4 == 0) return false;
-    // rows that leave more than half of the 128-node tiles idle: the column kernel (us a step, column
-    // / here: 67 x 400 x 400, 0.51 in use, 86 / 55; 131 x 300 x 300, 0.50, 85 / 60)
-    if ((double)(g.nx - 2) < 0.5 * 128.0 * (double)((g.nx - 2 + 127) / 128)) return false;
+    // less than 0.45 of the column kernel's useful lanes: that kernel (us a step, column / here: 391 x 8 x 3059
+    // (0.4) 41 / 55, 1061 x 6 x 4776 (0.47) 228 / 184, 67 x 400 x 400 (0.75) 86 / 55)
+    if (comp_ragged_share(g) < 0.45 && launch_override(PS_OVERRIDE_KCHUNK) <= 0) return false;
     return ragged_supported(g, a, b, c);
 }
 
@@ -334,7 +354,7 @@ static cudaError_t launch_rag_t(void *T2, const void *T, const void *Ci, Grid3 g
     if (kchunk <= 0) {
         constexpr WaveCost ragged{0.5, 0.4, 0.1, 3, 12};
         kchunk = step_kchunk(sizeof(E), g, tiles, 3,
-                             MODE == Z_F64_SCALED || MODE == Z_F64_EMU_ISO_DMUL ? &ragged : nullptr);
+                             MODE == Z_F64_SCALED || MODE == Z_F64_EMU_ISO ? &ragged : nullptr);
     }
     kchunk = grid_chunk(g.nz, kchunk);
     const int64_t gz = (g.nz - 2 + kchunk - 1) / kchunk;
@@ -360,8 +380,10 @@ cudaError_t launch_zmarch_ragged(int mode, void *T2, const void *T, const void *
                                  cudaStream_t s, bool write_bnd) {
     const ZParams p = make_params(c);
     switch (mode) {
-        case Z_F64_EMU_ISO_DMUL:
-            return launch_rag_b<Z_F64_EMU_ISO_DMUL, 2, 8, 3>(T2, T, Ci, g, p, s, write_bnd);
+        // K*S, bit for bit the column kernel's, which takes smaller grids (257^3 91 us a step, 85 with Ci*K
+        // multiplied first, whose last bit depends on which nodes share a warp; column kernel 99)
+        case Z_F64_EMU_ISO:
+            return launch_rag_b<Z_F64_EMU_ISO, 2, 8, 3>(T2, T, Ci, g, p, s, write_bnd);
         case Z_F64_EMU_ANISO:
             if (p.ek.axes == AX_SPREAD)
                 return launch_rag_b<Z_F64_EMU_ANISO_SPREAD, 2, 8, 3>(T2, T, Ci, g, p, s, write_bnd);

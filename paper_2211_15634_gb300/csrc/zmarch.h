@@ -53,9 +53,12 @@ struct RagMaps {
 };
 // Planes per chunk of the FP32 pair kernels for `tiles` tiles on `slots` resident CTAs.
 int pair_kchunk(Grid3 g, int64_t tiles, int64_t slots);
-// Grids whose steps inside a time loop take the column kernels (stencil_basic.cuh); mode:
-// Z_F32, Z_F32_COMP, Z_F64_SCALED or Z_F64_EMU_ANISO (any unequal spacings).
-bool step_small(Grid3 g, int mode);
+// Grids whose steps take the column kernels (stencil_basic.cuh), aligned ones inside a time loop only; mode:
+// Z_F32, Z_F32_COMP, Z_F64_SCALED, Z_F64_EMU_ISO (Ci as given, equal spacings) or Z_F64_EMU_ANISO (any
+// unequal spacings).
+bool step_small(Grid3 g, int mode, bool in_loop);
+// Useful lanes of the staged two-float step on odd rows against the column kernel's.
+double comp_ragged_share(Grid3 g);
 // Whether fused FP32 pairs (zpair.cu) beat single steps in a loop on this grid; states: a
 // loop that keeps every state.
 bool pairs_pay(Grid3 g, bool states);
@@ -93,7 +96,7 @@ bool emu_ok(StepCoef c);
 // boundary nodes of planes 1 .. nz-2 as copies of T's (not with Z_F32_COMP).
 cudaError_t launch_zmarch(int mode, void *T2, const void *T, void *E2, const void *Ein, const void *Ci,
                           StepCoef c, Grid3 g, cudaStream_t s, bool write_bnd = false);
-// The same on ragged rows (mode: Z_F64_EMU_ISO_DMUL, Z_F64_EMU_ANISO, Z_F64_SCALED or Z_F32;
+// The same on ragged rows (mode: Z_F64_EMU_ISO, Z_F64_EMU_ANISO, Z_F64_SCALED or Z_F32;
 // the caller has checked step_ragged_ok).
 cudaError_t launch_zmarch_ragged(int mode, void *T2, const void *T, const void *Ci, StepCoef c, Grid3 g,
                                  cudaStream_t s, bool write_bnd = false);

@@ -184,7 +184,7 @@ __device__ __forceinline__ void zrag_tile(const CUtensorMap *tmT, const CUtensor
             if constexpr (kF64) {
                 constexpr int kAx = MODE == Z_F64_EMU_ANISO ? AX_COMMON
                                     : MODE == Z_F64_EMU_ANISO_SPREAD ? AX_SPREAD : AX_ISO;
-                constexpr bool kDmul = MODE == Z_F64_EMU_ISO_DMUL, kScaled = MODE == Z_F64_SCALED;
+                constexpr bool kScaled = MODE == Z_F64_SCALED;
                 unsigned long long c[PX], xm[PX], xp[PX], ym[PX], yp[PX], zm[PX], zp[PX];
                 double ci[PX];
                 unsigned hw[7 * PX - 1];
@@ -226,7 +226,7 @@ __device__ __forceinline__ void zrag_tile(const CUtensorMap *tmT, const CUtensor
                         if constexpr (kScaled)
                             out[i] = emu_fast_node_scaled(c[i], xm[i], xp[i], ym[i], yp[i], zm[i], zp[i], ci[i]);
                         else
-                            out[i] = emu_fast_node<kAx, kDmul>(c[i], xm[i], xp[i], ym[i], yp[i], zm[i], zp[i],
+                            out[i] = emu_fast_node<kAx, false>(c[i], xm[i], xp[i], ym[i], yp[i], zm[i], zp[i],
                                                                ci[i], p.ek);
                     }
                 } else {

@@ -35,3 +35,52 @@ def test_fp32_pairs_by_the_rows_they_use(launch_override, shape, pairs):
     for a, b in zip(got, run()):
         assert np.array_equal(a, b)
     assert api.device_error() == 0
+
+
+@pytest.mark.parametrize("form", ["f32", "comp", "scaled", "equal", "unequal"])
+@pytest.mark.parametrize("shape", [(75, 31, 40), (129, 5, 60), (191, 25, 33)])
+def test_odd_rows_the_same_bits_by_every_route(launch_override, shape, form):
+    """Single steps, the loop, and both with the march or the column kernel asked for."""
+    dtype = torch.float32 if form in ("f32", "comp") else torch.float64
+    T, C = fields(shape, dtype)
+    T[:T.shape[0] // 2, ::3] -= 1.5  # both signs below, one binade above
+    inv = (3.0, 2.0, 2.5) if form == "unequal" else (2.0, 2.0, 2.0)
+    dt, nt, scaled = 0.01, 3, form == "scaled"
+    if scaled:
+        C = api.scale_ci(C, 1.0, dt, inv)
+
+    def loop():
+        A, B = T.clone(), torch.empty_like(T)
+        comp = api.compensation_fields(T) if form == "comp" else None
+        out = api.run(A, B, C, 1.0, dt, inv, nt, comp=comp, ci_scaled=scaled)
+        return torch.stack([out, comp[nt % 2]]) if form == "comp" else out
+
+    def steps():
+        A, B = T.clone(), T.clone()
+        E = [torch.zeros_like(T) for _ in range(2)] if form == "comp" else None
+        for i in range(nt):
+            if form == "comp":
+                api.step_compensated(B, A, E[1 - i % 2], E[i % 2], C, 1.0, dt, inv)
+            else:
+                api.step(B, A, C, 1.0, dt, inv, ci_scaled=scaled)
+            A, B = B, A
+        return torch.stack([A, E[nt % 2]]) if form == "comp" else A
+
+    want = loop()
+    for override in (dict(), dict(kchunk=3), dict(kchunk=0, step_plain=1)):
+        launch_override(**override)
+        assert torch.equal(loop(), want)
+        assert torch.equal(steps(), want)
+    assert api.device_error() == 0
+
+
+@pytest.mark.parametrize("form,shape,name", [
+    ("f32", (161, 265, 96), "k_step_basic<float>"), ("f32", (257, 257, 257), "k_zmarch_rag<F32>"),
+    ("f32", (391, 8, 3059), "k_step_basic<float>"), ("scaled", (75, 148, 320), "k_step_basic_emu"),
+    ("scaled", (257, 257, 257), "k_zmarch_rag<F64_SCALED>"), ("equal", (213, 407, 192), "k_step_basic_emu"),
+    ("equal", (257, 257, 257), "k_zmarch_rag<F64_EMU_ISO>"), ("unequal", (93, 512, 257), "k_step_basic_emu"),
+    ("unequal", (257, 257, 257), "k_zmarch_rag<F64_EMU_ANISO>")])
+def test_odd_rows_kernel_of_a_single_step(form, shape, name):
+    T, C = fields(shape, torch.float32 if form == "f32" else torch.float64)
+    inv = (1.0, 1.5, 1.2) if form == "unequal" else (1.0, 1.0, 1.0)
+    assert api.step_kernel_name(torch.empty_like(T), T, C, 1.0, 0.1, inv, ci_scaled=form == "scaled") == name
