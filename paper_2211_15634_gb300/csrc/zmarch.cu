@@ -309,10 +309,10 @@ bool tma_encoder_available() { return encode_fn() != nullptr; }
 
 bool f64_scaled_wide(Grid3 g, const void *T2, const void *T, const void *Ci) {
     if (launch_override(PS_OVERRIDE_F64_PX2) == 1) return false;
-    // 128-node tiles, unless 64-node ones leave fewer lanes past the row's end (us a step, four
-    // / two per thread: 192^3 41 / 34, 320^3 150 / 132, 448^3 357 / 330; equal widths 256^3 71 /
-    // 71, 384^3 212 / 216).  Below a million nodes the launch counts, not the lanes.
-    if (64 * ((g.nx + 63) / 64) < 128 * ((g.nx + 127) / 128) && (double)g.n() >= 1e6) return false;
+    // 128 x 4 tiles, unless 64 x 8 ones leave fewer lanes past the grid's edges (us a step, four
+    // / two per thread: 192^3 41 / 34, 320^3 150 / 132, 448^3 357 / 330, 3000 x 3 x 300 14 / 18; equal
+    // widths 256^3 71 / 71, 384^3 212 / 216).  Below a million nodes the launch counts, not the lanes.
+    if (fill(g.nx, 64) * fill(g.ny, 8) > fill(g.nx, 128) * fill(g.ny, 4) && (double)g.n() >= 1e6) return false;
     return g.nx % 4 == 0 && ((((uintptr_t)T2 | (uintptr_t)T | (uintptr_t)Ci) & 31u) == 0);
 }
 

@@ -84,3 +84,10 @@ def test_odd_rows_kernel_of_a_single_step(form, shape, name):
     T, C = fields(shape, torch.float32 if form == "f32" else torch.float64)
     inv = (1.0, 1.5, 1.2) if form == "unequal" else (1.0, 1.0, 1.0)
     assert api.step_kernel_name(torch.empty_like(T), T, C, 1.0, 0.1, inv, ci_scaled=form == "scaled") == name
+
+
+@pytest.mark.parametrize("shape,name", [((3000, 3, 300), "k_zmarch<F64_SCALED4>"), ((192, 192, 192), "k_zmarch<F64_SCALED>"),
+                                        ((256, 100, 100), "k_zmarch<F64_SCALED4>")])
+def test_tile_shape_of_the_pre_scaled_step(shape, name):
+    T, C = fields(shape, torch.float64)
+    assert api.step_kernel_name(torch.empty_like(T), T, C, 1.0, 0.1, (1.0,) * 3, ci_scaled=True) == name
