@@ -72,10 +72,10 @@ struct EmuCoef {
 };
 
 // How a node's Laplacian combines its axes: one K (equal spacings); one K per axis as integers at the
-// highest exponent (AX_COMMON: the K within a factor of 2^2, to the bit of their exponents, i.e.
-// spacings within 2 to 2.8 of each other); the sums at the lowest exponent instead (AX_SPREAD: within 2^8,
-// spacings within 16), for which AX_COMMON's K would keep too few bits; or a rounded product for each
-// (AX_FAR), beyond which the shifted sums would not fit 64 bits.
+// highest exponent (AX_COMMON: the K's exponents within 2, i.e. spacings within 2 to 2.8 of each other); the
+// same with the sums brought to lower exponents too (AX_SPREAD: within 8, spacings within 16), as the K
+// alone would keep too few bits; or a rounded product for each (AX_FAR), beyond which the shifted sums
+// would not fit 64 bits.
 enum EmuAxes { AX_COMMON = 0, AX_ISO = 1, AX_FAR = 2, AX_SPREAD = 3 };
 
 // Sets axes, re, r_d and h_d from the three K.
@@ -84,15 +84,19 @@ __host__ __device__ inline void emu_set_common(EmuCoef &c) {
     const int lxy = c.kx.e < c.ky.e ? c.kx.e : c.ky.e, l = lxy < c.kz.e ? lxy : c.kz.e;
     const int gap = e - l;
     c.axes = (signed char)(gap <= 2 ? AX_COMMON : (gap <= 8 ? AX_SPREAD : AX_FAR));
-    const bool up = c.axes == AX_COMMON;
-    c.re = up ? e : l;
-    // mantissas are multiples of 2^10: after a shift by at most 2 still of 4 (emu_L_common)
-    c.rx = up ? c.kx.m >> (e - c.kx.e) : c.kx.m;
-    c.ry = up ? c.ky.m >> (e - c.ky.e) : c.ky.m;
-    c.rz = up ? c.kz.m >> (e - c.kz.e) : c.kz.m;
-    c.hx = (signed char)(up ? 0 : c.kx.e - l);
-    c.hy = (signed char)(up ? 0 : c.ky.e - l);
-    c.hz = (signed char)(up ? 0 : c.kz.e - l);
+    // The finest axis's sums are shifted left by h, a coarser axis's by that much less, and its K right by what
+    // is left: by two bits at most (mantissas are multiples of 2^10: still of 4, emu_L_common), up to a gap of
+    // 5 so that h <= 3 and any sums fit; beyond, by none, where sums have to be looked at anyway.
+    const int h = gap <= 2 ? 0 : (gap <= 5 ? gap - 2 : gap);
+    c.re = e - h;
+    auto axis = [&](const EmuK &k, unsigned long long *r, signed char *s) {
+        const int d = h - (e - k.e);
+        *r = d < 0 ? k.m >> (-d & 63) : k.m;
+        *s = (signed char)(d > 0 ? d : 0);
+    };
+    axis(c.kx, &c.rx, &c.hx);
+    axis(c.ky, &c.ry, &c.hy);
+    axis(c.kz, &c.rz, &c.hz);
 }
 
 // K_d = dtlam * a_d (positive normal, or the emulated forms are not run).
@@ -231,20 +235,19 @@ __device__ __forceinline__ unsigned long long emu_pack_any(unsigned long long a,
 }
 
 // sum_d K_d * S_d * 2^sc for exact per-axis sums, with one rounding.  kSmall: |S_d| < 2^53 (differences of
-// one binade's bit patterns), else |S_d| <= 2^59.
+// one binade's bit patterns), else |S_d| < 2^59.
 //
 // The sums are shifted left together until the largest fills 62 bits, biased by 2^62 to be unsigned,
 // multiplied by the 63-bit r_d keeping the top 64 bits of each product (three 32 x 32-bit multiplies with
 // the accumulation inside; the dropped low product is below one unit), added, unbiased
 // (sum r_d / 4, exact as r_d % 4 == 0) and converted once: one rounding to 53 bits of a value
 // known to six units of 2^-59 (three axes, two each) of the product of the largest sum and the largest
-// r.  With AX_COMMON that is up to 2^2 times the largest term there is, so the value is known to 2^-54.4 of
-// its largest term, or 2^-56 where one axis alone varies (a rounding for each axis: 2^-53 for each).
-// AX_SPREAD first brings the sums to the lowest exponent (S_d * 2^h_d, the largest of which then
-// belongs to the largest term, to within a factor of two): 2^-56.4 of the largest term at any ratio
-// (0.07 units of 2^-53 found), at three more 64-bit shifts where the sums are small and some 25
-// instructions where their length has to be looked at (larger ones may not fit: bits below 2^-60 of the
-// largest are dropped).  A node needs two FP64-pipe instructions (the
+// r.  With K shifted right by up to two bits that is up to 2^2 times the largest term there is, so the value is
+// known to 2^-54.4 of its largest term, or 2^-56 where one axis alone varies (a rounding for each axis:
+// 2^-53 for each).  AX_SPREAD shifts the sums left before (S_d * 2^h_d), at three more 64-bit shifts, and where
+// the exponents are more than 5 apart leaves the K whole, which keeps 2^-56.4 of the largest term (0.07 units
+// of 2^-53 found); sums that may not fit are then looked at first, at some 25 instructions (bits below 2^-60
+// of the largest are dropped).  A node needs two FP64-pipe instructions (the
 // conversion and the final DFMA), which the pipe serves in about the time HBM needs, and
 // about 110 integer ones, which bind.  Measured, us a step: 512 x 384 x 256 nodes 271 (443
 // with one product, pack and FP64 sum per axis, three FP64 instructions and less exact; 307
@@ -255,7 +258,7 @@ __device__ __forceinline__ unsigned long long emu_pack_any(unsigned long long a,
 template <int kDim, bool kSpread, bool kSmall>
 __device__ __forceinline__ double emu_L_common(long long sx, long long sy, long long sz, int sc,
                                                unsigned long long flip, const EmuCoef &k) {
-    if (kSpread && kSmall) {
+    if (kSpread && (kSmall || (k.hx | k.hy | k.hz) <= 3)) {
         sx <<= k.hx;
         sy <<= k.hy;
         if (kDim == 3) sz <<= k.hz;

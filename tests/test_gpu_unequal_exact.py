@@ -4,8 +4,8 @@ with Ci = 1 gives L(T) where T = 0.
 
 L is one rounding of a sum whose products are cut at 2^-59 of the largest (two units each, three axes), so
 |error| <= 2^-53 |L| + 6 * 2^-59 max_d |K_d S_d|, along whichever axes the field varies and at every ratio of
-the spacings; where the K lie within 2^2 they are brought to the highest exponent, which costs that many
-bits of the second term.  (A rounding for each axis: 2^-53 of each term.)  Below the normal range half a unit
+the spacings; where the K's exponents lie within 5 they are shifted right by up to two bits, which costs that
+many of the second term.  (A rounding for each axis: 2^-53 of each term.)  Below the normal range half a unit
 of 2^-1074 takes the place of the first term."""
 import math
 from fractions import Fraction as F
@@ -22,7 +22,7 @@ pytestmark = [pytest.mark.gpu,
               pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
 
 # 1 / spacing per axis, up to the factor of 16 within which the axes share one integer sum
-RATIOS = [(1.0, 1.3, 1.0), (2.0, 1.5, 1.0), (4.1, 1.0, 3.7), (9.1, 1.0, 2.9), (15.99, 1.0, 1.0), (15.99, 1.0, 15.3)]
+RATIOS = [(1.0, 1.3, 1.0), (2.0, 1.5, 1.0), (4.1, 1.0, 3.7), (5.1, 1.0, 2.9), (9.1, 1.0, 2.9), (15.99, 1.0, 1.0), (15.99, 1.0, 15.3)]
 DT = 0.1
 FIELDS = ["binade", "window", "signed", "x", "y", "z", "pair"]
 
@@ -34,7 +34,7 @@ def coefficients(dt, inv):
 def cut(K):
     e = [math.frexp(float(k))[1] for k in K]
     gap = max(e) - min(e)
-    return F(6, 2 ** (59 - gap if gap <= 2 else 59))
+    return F(6, 2 ** (59 - min(gap, 2) if gap <= 5 else 59))
 
 
 def field(kind, shape, seed):
@@ -121,7 +121,7 @@ def test_steps(launch_override, nx, ratio, kind):
 
 
 @pytest.mark.parametrize("kind", FIELDS)
-@pytest.mark.parametrize("inv", [(9.1, 1.0, 2.9), (1.0, 15.3, 15.99), (3.0, 8.0, 1.0)])
+@pytest.mark.parametrize("inv", [(5.1, 1.0, 2.9), (9.1, 1.0, 2.9), (1.0, 15.3, 15.99), (3.0, 8.0, 1.0)])
 def test_same_bits_on_every_kernel(launch_override, inv, kind):
     """Wide spreads: the march on even and odd rows, the column kernel, the batch."""
     for nx in (67, 68):
