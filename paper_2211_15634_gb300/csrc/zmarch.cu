@@ -235,10 +235,10 @@ static int step_kchunk(int esz, Grid3 g, int64_t tiles, int per_sm, const WaveCo
     // FP32 is fastest at 8 planes; FP64 at 8 planes on small grids, at 13-18 at 320^3 and at 24
     // at 448^3 to 640^3 (1% ahead of 32), so about 32 CTAs per SM between 8 and 24 planes (with
     // 64: 320^3 134 us a step / 130, 321^3 150 / 144, 384^3 216 / 212).
-    // FP32 grids up to 3 million nodes in whole tiles (a few CTAs per SM): 3 planes (128^3 5.1 against 5.6 us), the
-    // two-float state up to 2.5 (384 x 96 x 64 10.4 against 11.5, but 400 x 140 x 52 13.7 against 11.5 and
-    // 52 x 197 x 141 13.2 against 10.5).
-    if (esz == 4 && (double)tiles * 1024.0 * (double)g.nz <= (comp ? 2.5e6 : 3e6)) return 3;
+    // FP32 grids up to 3 million nodes (a few CTAs per SM): 3 planes (128^3 5.1 against 5.6 us, 192 x 67 x 184
+    // 8.6 and 11.4).  The two-float state up to 2.5 million in whole tiles (384 x 96 x 64 10.4 against 11.5, but
+    // 400 x 140 x 52 13.7 against 11.5 and 52 x 197 x 141 13.2 against 10.5).
+    if (esz == 4 && (comp ? (double)tiles * 1024.0 * (double)g.nz <= 2.5e6 : (double)g.n() <= 3e6)) return 3;
     const int64_t target = 32LL * sm_count();
     const int64_t kmax = esz == 8 ? 24 : 8;
     const int64_t kc = (g.nz - 2) * tiles / target;
