@@ -55,8 +55,8 @@ __device__ __forceinline__ void batch_item(const BatchItem &item, const BatchPro
             }
         } else if constexpr (sizeof(F) == 8) {
             const unsigned long long *__restrict__ Tb = (const unsigned long long *)T;
-            EmuCoef k{EmuK{P.kxm, P.kxe}, EmuK{P.kym, P.kye}, EmuK{P.kzm, P.kze},
-                            P.dtlam, P.ax, P.ay, P.az, 0.0, 0ull, 0ull, 0ull, 0, 0, 0, 0, 0};
+            EmuCoef k{EmuK{P.kxm, P.kxe, 0}, EmuK{P.kym, P.kye, 0}, EmuK{P.kzm, P.kze, 0},
+                            P.dtlam, P.ax, P.ay, P.az, 0.0, 0ull, 0ull, 0ull, 0, 0};
             unsigned long long tm = Tb[p - sz], tc = Tb[p];
             if (P.iso) {
                 for (int kk = k0; kk < k1; ++kk, p += sz) {

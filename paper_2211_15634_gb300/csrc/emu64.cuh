@@ -43,10 +43,10 @@
 
 namespace psd {
 
-// K = m * 2^e with m in [2^62, 2^63).
+// K = m * 2^e with m in [2^62, 2^63); h: emu_set_common.
 struct EmuK {
     unsigned long long m;
-    int e;
+    int e, h;
 };
 
 __host__ __device__ inline EmuK emu_const(double K) {
@@ -55,20 +55,19 @@ __host__ __device__ inline EmuK emu_const(double K) {
     memcpy(&b, &K, 8);
     const int k = (int)((b >> 52) & 0x7ff) - 1023;
     const unsigned long long man = (b & 0xfffffffffffffull) | (1ull << 52);
-    return EmuK{man << 10, k - 62};
+    return EmuK{man << 10, k - 62, 0};
 }
 
 struct EmuCoef {
     EmuK kx, ky, kz;  // dt*lam*_d^2 per axis as integer mantissa and exponent
     double dtlam, ax, ay, az;
     double Kx;        // dt*lam*_dx^2 (the kDmul variant, iso grids)
-    // the K as integers at one exponent (emu_set_common): K_d = r_d * 2^(re + h_d), h_d = 0 but with
-    // AX_SPREAD; axes: which of AX_COMMON, AX_SPREAD, AX_FAR serves them
-    // (bytes: a node's general path takes the record by value, and a longer one cost 2-D fields of
-    // both signs a third of their time)
+    // the K as integers at one exponent (emu_set_common): K_d = r_d * 2^(re + k_d.h), h = 0 but with AX_SPREAD;
+    // axes: which of AX_COMMON, AX_SPREAD, AX_FAR serves them.  (120 bytes: a node's general path takes the
+    // record by value, and 136 cost 2-D fields of both signs a third of their time.  h whole words, which a
+    // shift takes from the constant bank: as bytes they were loaded for each node, transposed 256^3 267 us, 252 so.)
     unsigned long long rx, ry, rz;
-    int re;
-    signed char hx, hy, hz, axes;
+    int re, axes;
 };
 
 // How a node's Laplacian combines its axes: one K (equal spacings); one K per axis as integers at the
@@ -83,26 +82,26 @@ __host__ __device__ inline void emu_set_common(EmuCoef &c) {
     const int exy = c.kx.e > c.ky.e ? c.kx.e : c.ky.e, e = exy > c.kz.e ? exy : c.kz.e;
     const int lxy = c.kx.e < c.ky.e ? c.kx.e : c.ky.e, l = lxy < c.kz.e ? lxy : c.kz.e;
     const int gap = e - l;
-    c.axes = (signed char)(gap <= 2 ? AX_COMMON : (gap <= 8 ? AX_SPREAD : AX_FAR));
+    c.axes = gap <= 2 ? AX_COMMON : (gap <= 8 ? AX_SPREAD : AX_FAR);
     // The finest axis's sums are shifted left by h, a coarser axis's by that much less, and its K right by what
     // is left: by two bits at most (mantissas are multiples of 2^10: still of 4, emu_L_common), up to a gap of
     // 5 so that h <= 3 and any sums fit; beyond, by none, where sums have to be looked at anyway.
     const int h = gap <= 2 ? 0 : (gap <= 5 ? gap - 2 : gap);
     c.re = e - h;
-    auto axis = [&](const EmuK &k, unsigned long long *r, signed char *s) {
+    auto axis = [&](EmuK &k, unsigned long long *r) {
         const int d = h - (e - k.e);
         *r = d < 0 ? k.m >> (-d & 63) : k.m;
-        *s = (signed char)(d > 0 ? d : 0);
+        k.h = d > 0 ? d : 0;
     };
-    axis(c.kx, &c.rx, &c.hx);
-    axis(c.ky, &c.ry, &c.hy);
-    axis(c.kz, &c.rz, &c.hz);
+    axis(c.kx, &c.rx);
+    axis(c.ky, &c.ry);
+    axis(c.kz, &c.rz);
 }
 
 // K_d = dtlam * a_d (positive normal, or the emulated forms are not run).
 inline EmuCoef emu_coef(double dtlam, double ax, double ay, double az) {
     EmuCoef c{emu_const(dtlam * ax), emu_const(dtlam * ay), emu_const(dtlam * az), dtlam, ax, ay, az,
-              dtlam * ax, 0ull, 0ull, 0ull, 0, 0, 0, 0, 0};
+              dtlam * ax, 0ull, 0ull, 0ull, 0, 0};
     emu_set_common(c);
     return c;
 }
@@ -251,26 +250,27 @@ __device__ __forceinline__ unsigned long long emu_pack_any(unsigned long long a,
 // conversion and the final DFMA), which the pipe serves in about the time HBM needs, and
 // about 110 integer ones, which bind.  Measured, us a step: 512 x 384 x 256 nodes 271 (443
 // with one product, pack and FP64 sum per axis, three FP64 instructions and less exact; 307
-// with the integer pack in place of the conversion; 285 as AX_SPREAD); 2-D 8192 x 6000 247 (878 in plain
-// FP64, ten FP64 instructions per node; 253 as AX_SPREAD).
+// with the integer pack in place of the conversion); 2-D 8192 x 6000 242 (878 in plain
+// FP64, ten FP64 instructions per node).  AX_SPREAD / AX_COMMON: 256^3 115 / 101, transposed 252 / 243, columns of
+// 150^3 23.6 / 23.0.
 // The same real sums at another scale 2^sc give the same result, bit for bit, and so does every path of
 // a node.  kDim = 2: the z sum is not there.
 template <int kDim, bool kSpread, bool kSmall>
 __device__ __forceinline__ double emu_L_common(long long sx, long long sy, long long sz, int sc,
                                                unsigned long long flip, const EmuCoef &k) {
-    if (kSpread && (kSmall || (k.hx | k.hy | k.hz) <= 3)) {
-        sx <<= k.hx;
-        sy <<= k.hy;
-        if (kDim == 3) sz <<= k.hz;
+    if (kSpread && (kSmall || (k.kx.h | k.ky.h | k.kz.h) <= 3)) {
+        sx <<= k.kx.h;
+        sy <<= k.ky.h;
+        if (kDim == 3) sz <<= k.kz.h;
     } else if (kSpread) {  // to 61 bits
         auto bits = [](long long s) { return 64 - __clzll(s ^ (s >> 63)); };
-        int b = max(bits(sx) + k.hx, bits(sy) + k.hy);
-        if (kDim == 3) b = max(b, bits(sz) + k.hz);
+        int b = max(bits(sx) + k.kx.h, bits(sy) + k.ky.h);
+        if (kDim == 3) b = max(b, bits(sz) + k.kz.h);
         const int q = max(b - 61, 0);
         auto shift = [](long long s, int h) { return h >= 0 ? s << h : s >> -h; };
-        sx = shift(sx, k.hx - q);
-        sy = shift(sy, k.hy - q);
-        if (kDim == 3) sz = shift(sz, k.hz - q);
+        sx = shift(sx, k.kx.h - q);
+        sy = shift(sy, k.ky.h - q);
+        if (kDim == 3) sz = shift(sz, k.kz.h - q);
         sc += q;
     }
     unsigned long long m = (unsigned long long)(sx ^ (sx >> 63)) | (unsigned long long)(sy ^ (sy >> 63));
