@@ -295,15 +295,17 @@ cudaError_t launch_step2_ragged_f32(float *T2, const float *T, const float *Ci, 
 }
 
 bool pairs_pay_ragged(Grid3 g) {
-    // By the share of useful nodes in 128 x 14 tiles.  Up to 8.8 million nodes single steps are the column
-    // kernel's, whose fields stay in L2, so pairs need well-filled tiles; from there on both read HBM
-    // (us a step, single steps / pairs, share): 103^3 (0.71) 5.4 / 4.7, 159^3 (0.57) 8.9 / 10.9, 299 x 256 x 64
-    // (0.74) 10.8 / 10.3, 61 x 48 x 936 (0.38) 7.1 / 9.9, 625 x 5 x 980 (0.21) 6.2 / 11, 113 x 18 x 588 (0.5) 4.5 / 4.9,
-    // 1697 x 12 x 800 (0.68) 39 / 27, 129 x 18 x 4932 (0.57) 24.6 / 23, 1061 x 6 x 4776 (0.26) 65 / 79, 143 x 250 x 250
-    // (0.55) 24.7 / 21.3, 255^3 33.4 / 22.5.  Over 186 shapes 0.4% off the better of the two on average.
+    // By the useful nodes of 128 x 14 tiles.  Up to 8.8 million nodes single steps are the column kernel's, whose
+    // fields stay in L2, so pairs need rows that fill three quarters of a tile and 0.6 of
+    // its height; from there on both read HBM (us a step, single steps / pairs, shares in x
+    // and y): 103^3 (0.79, 0.90) 5.4 / 4.7, 102 x 75 x 208 (0.78, 0.87) 5.6 / 5.1, 159^3 (0.61, 0.93) 8.9 / 10.9, 299 x
+    // 256 x 64 (0.77, 0.95) 10.8 / 10.3, 87 x 128 x 387 (0.66, 1) 9.5 / 10, 625 x 5 x 980 (0.97, 0.21) 6.2 / 11, 113 x 18 x
+    // 588 (0.87, 0.57) 4.5 / 4.9, 1697 x 12 x 800 (0.95, 0.71) 39 / 27, 129 x 18 x 4932 (0.99, 0.57) 24.6 / 23, 1061 x 6 x
+    // 4776 (0.92, 0.29) 65 / 79, 143 x 250 x 250 (0.55, 0.98) 24.7 / 21.3, 255^3 33.4 / 22.5.  Over 186 shapes 0.3%
+    // off the better of the two on average.
     const double n = (double)g.n(), x = (double)(g.nx - 2) / (128.0 * (double)((g.nx - 2 + 127) / 128)),
-                 share = x * (double)(g.ny - 2) / (14.0 * (double)((g.ny - 2 + 13) / 14));
-    return n > 8.8e6 ? share >= 0.5 : share >= 0.7 && n * share * share > 6e5;
+                 y = (double)(g.ny - 2) / (14.0 * (double)((g.ny - 2 + 13) / 14)), share = x * y;
+    return n > 8.8e6 ? share >= 0.5 : x >= 0.75 && y >= 0.6 && n * share * share > 6e5;
 }
 
 unsigned zpair_rag_device_error(bool clear) {
