@@ -74,9 +74,10 @@ def state_pairs_default(T0) -> bool:
     """Whether the loops that keep states run fused step pairs that write both states
     (``api.run_states(temporal2=True)``: FP32 only; bit for bit the same states; single
     steps where pairs would not be faster).  Measured at 256^3, nt = 200: 200 states in
-    5.39 against 6.84 ms, the gradient with every state kept 18.1 against 19.5 ms.  The
-    recomputes run beside the transposed steps: 192^3, nt = 60, a checkpoint every 8 steps
-    3.28 ms against 3.40, 256^3, 49, every 7 5.07 against 5.16, 160^3, 64, 8 2.51 and 2.49."""
+    4.35 against 6.68 ms, the gradient with every state kept 17.1 against 19.4 ms.  With
+    checkpoints pairs serve the checkpoint pass and the recomputes too, which run beside the
+    transposed steps: 256^3, nt = 200, a checkpoint every 15 steps 19.5 ms against 23.3,
+    192^3, 60, every 8 3.13 against 3.64, 160^3, 64, 8 2.41 against 2.69."""
     return T0.dtype == torch.float32
 
 

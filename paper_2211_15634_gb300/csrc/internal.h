@@ -43,8 +43,8 @@ int api_fail(int status, const char *msg);
 int api_cuda_fail(cudaError_t e, const char *where);
 
 // ---- forward step kernels (step_f64.cu, step_f32.cu) ----
-// in_loop: one step of a time loop, which may take the column kernel on a small grid (bit for
-// bit the same).  write_bnd: where the TMA march serves the step (step_takes_march) it also
+// in_loop: one step of a time loop, which may take the column kernel on a small grid of aligned
+// rows (bit for bit the same; rows that are no multiple of 16 bytes may take it in any case).  write_bnd: where the TMA march serves the step (step_takes_march) it also
 // stores the x and y boundary nodes of planes 1 .. nz-2 as copies of T's.
 cudaError_t launch_step_f64_native(double *T2, const double *T, const double *Ci, StepCoef c,
                                    Grid3 g, cudaStream_t s);
@@ -140,7 +140,7 @@ struct BatchHeader {
     int32_t dtype, tile_x, tile_y, tile_z;
     int64_t problems_offset, items_offset;  // byte offsets from the table start
     // kernel 0: column march (batch.cu); 1: TMA z-march (batch_tma.cu) in step mode
-    // zmode, with a ZParams record and three tensor maps per problem at these offsets
+    // zmode, with a ZParams record and twelve tensor maps per problem at these offsets
     int32_t kernel, zmode;
     int64_t zparams_offset, maps_offset;
     // z-march tables built for fused step pairs (PS_BATCH_TEMPORAL2): a second work list

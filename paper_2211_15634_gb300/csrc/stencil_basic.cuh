@@ -2,14 +2,15 @@
 // marching along z with a three-value register queue.  x/y neighbours are
 // read through the L1/L2 caches.
 //
-// They serve two kinds of grid.  Small ones inside a time loop (step_small, zmarch.cu): a
-// march of 1 .. 16 planes per thread keeps a step at a few memory round trips, where the TMA
-// z-march waits for 8 planes of copies one after the other.  Measured, us a step in a
-// captured loop (march as it was / this): FP64 pre-scaled 32^3 7.4 / 1.5, 64^3 7.4 / 3.0, 96^3
-// 8.9 / 6.1, 128^3 14.8 / 10.4, 192^3 41 / 39, 208^3 48 / 52; FP32 32^3 4.2 / 1.5, 64^3
-// 4.3 / 2.2, 96^3 4.4 / 3.6, 160^3 10.9 / 8.8, 192^3 14.3 / 13.7, 208^3 19 / 22.  And grids
-// that the march cannot take (2^31 nodes and more on ragged rows, spacings more than 16
-// apart on odd nx, plain FP64, the two-float step on ragged rows).
+// They serve two kinds of grid.  Small ones (step_small, zmarch.cu; rows of a multiple of 16
+// bytes inside a time loop only): a march of 1 .. 16 planes per thread keeps a step at a few
+// memory round trips, where the TMA z-march waits for 8 planes of copies one after the other.
+// Measured, us a step in a captured loop (march of 8 planes / this): FP64 pre-scaled 32^3 7.6 /
+// 1.7, 64^3 7.6 / 3.2, 96^3 9.1 / 6.3, 128^3 14.9 / 10.5; FP32 32^3 4.2 / 1.5, 64^3 4.3 / 2.2,
+// 96^3 4.4 / 3.6, 160^3 10.9 / 8.8, 192^3 14.3 / 13.7, 208^3 19 / 22.  And grids
+// that the march cannot take or would be slower on (2^31 nodes and more on ragged rows, spacings
+// more than 16 apart on odd nx, plain FP64; FP32 grids on ragged rows that leave many lanes of
+// its tiles idle: step_ragged_ok, comp_ragged_ok).
 // They never store boundary nodes: x faces stored beside the interior cost more than the
 // boundary copy they save (127^3 FP32 states: 10.1 us a step against 8.3).
 // The next step's CTAs are let in at the end of the march, not at its start: with one wave of

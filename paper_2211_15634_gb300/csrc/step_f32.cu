@@ -1,6 +1,7 @@
 // FP32 forward step dispatch (deviation storage D = T - T_ref): TMA z-march when nx is a
 // multiple of 4, else its row-by-row form (zrag_tile.cuh; the two-float state zcomp_rag.cu) below
-// 2^31 nodes, else the plain column march.  Small grids inside a time loop take the column march (stencil_basic.cuh).
+// 2^31 nodes, else the plain column march.  Small grids take the column march (stencil_basic.cuh): on aligned
+// rows inside a time loop only, on other rows a single step too.
 #include "internal.h"
 #include "stencil_basic.cuh"
 #include "zmarch.h"

@@ -1,8 +1,9 @@
 // FP64 forward step dispatch.
 //   fast:   TMA z-march with one-DFMA emulated arithmetic (even nx), its row-by-row form
 //           (odd nx below 2^31 nodes, spacings within 16 of each other), else the plain
-//           column march with the same arithmetic;
-//           Small grids inside a time loop take the column march (stencil_basic.cuh).
+//           column march with the same arithmetic.  Small grids take the column march
+//           (stencil_basic.cuh): even nx inside a time loop only (and not Ci as given on equal
+//           spacings), odd nx a single step too.
 //   native: plain column march with ordinary FP64 instructions.
 #include "internal.h"
 #include "stencil_basic.cuh"

@@ -7,8 +7,8 @@
 // of two rows) with packed FP32 arithmetic (f32x2, the same roundings as f32_node), shares the
 // first differences along x between neighbours and along z between planes, and its loop's own
 // instructions count for eight nodes.  Measured (us a step): 512^3 130.9, 384^3 57.4, 256^3
-// 18.8, where the four-node form with a scalar ring around the tile (zmarch2_tile.cuh, 83
-// instructions per node and pass against 53) took 179, 82.8 and 27.6.  Four nodes per thread
+// 18.8, where the four-node form with a scalar ring around the tile (zmarch2_tile.cuh, 95
+// instructions per node and pass against 45) took 179, 82.8 and 27.6.  Four nodes per thread
 // with halo rows and columns in whole warps and lanes took 188 at 512^3 (the 120 columns that
 // leaves waste a seventh of the lanes), and passes of three and four steps in that form 215
 // and 372 per step's share: more levels cost more instructions than the memory they save.
@@ -366,7 +366,7 @@ bool pairs_pay(Grid3 g, bool states) {
     if (y < 0.6) return false;
     const double n = (double)g.n(), useful = n * x * y;
     // loops that keep every state (us a step, single steps / pairs): 128^3 6.0 / 7.1, 160^3 (0.63) 13.1
-    // / 11.0, 256^3 33.8 / 27.1
+    // / 9.9, 256^3 33.8 / 22.7
     if (states) return useful > 2.2e6;
     // By nodes and the share of useful lanes against the column kernel's, which steps small grids
     // and wastes at most 31 columns (us a step, single steps / pairs): 108 x 48 x 128 (0.84 of the
